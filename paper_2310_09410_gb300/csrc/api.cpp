@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "opf_internal.h"
+#include "persist_plan.h"
 #include "warp_place.h"
 
 namespace opf {
@@ -50,8 +51,9 @@ int launch_cluster_engine(const IterArgs<T> &g, const ClusterLayout &lay, const 
                           int n_iters, int check_every, DevStatus *st, double rho,
                           cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
 template <typename T> int cluster_occupancy(const ClusterLayout &lay);
-template <typename T> int prepare_persist_engine(unsigned bytes);
-template <typename T> int persist_occupancy(int threads, unsigned bytes);
+template <typename T> int prepare_persist_engine(const PersistLayout &lay);
+template <typename T> int persist_occupancy(const PersistLayout &lay);
+template <typename T> size_t persist_exchange_bytes(int L);
 template <typename T>
 int launch_persist_engine(const IterArgs<T> &g, const PersistLayout &lay, const PersistPtrs &pp, T *U,
                           int bar_extra, int n_iters, int check_every, DevStatus *st, double rho,
@@ -300,7 +302,7 @@ static int build_layout(opf_handle *h) {
     TRY(dalloc(h, &h->w32.d_fbig, h->S + 1));
     TRY(dalloc(h, &h->w32.d_F2, h->nF));
     for (PersistPlan *pp : {&h->p32, &h->p64}) {
-        TRY(dalloc(h, &pp->d_pr, 5 * (kPersistMaxP + 1)));
+        TRY(dalloc(h, &pp->d_pr, 7 * (kPersistMaxP + 1)));
         TRY(dalloc(h, &pp->d_srec, h->S + 1));
         TRY(dalloc(h, &pp->d_items, std::max<long long>(items_cap, 1)));
         TRY(dalloc(h, &pp->d_meta, h->L));
@@ -723,110 +725,128 @@ static int get_cluster_plan(opf_handle *h, ClusterPlan *cp, int requested, int t
     return OPF_OK;
 }
 
-// Partition the instance over P co-resident CTAs of the persistent grid
-// engine: contiguous subsystem ranges balanced by work (the same cost as the
-// cluster plan), part-relative records, and the shared-memory layout.  Leaves
-// pp->ok false when a part does not fit one CTA or P CTAs cannot be resident.
+// Partition the instance over P co-resident CTAs of the persistent grid engine
+// and lay out its shared memory: parts of a depth-first order for the local
+// form, else (more slots or columns than threads, or no room) runs of the
+// size-sorted order.  Leaves pp->ok false when a part does not fit one CTA or
+// P CTAs cannot be resident.
 template <typename T>
-static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm) {
+static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local) {
     pp->ok = false;
     pp->P = P;
     if (P < 1 || P > kPersistMaxP) return OPF_OK;
     const int S = h->S, L = h->L;
     std::vector<double> cost(S);
-    double total = 0;
-    for (int s = 0; s < S; ++s) {
+    for (int s = 0; s < S; ++s)
         cost[s] = 6.0 * h->h_sn[s] + (double)h->h_sf[s] * h->h_npad[s] + (double)h->h_sn[s] * h->h_sf[s];
-        total += cost[s];
+    std::vector<int> order(S);
+    if (local) {
+        std::vector<int> start(S);           // new trees begin in canonical order
+        for (int d = 0; d < S; ++d) start[h->dev_to_canon_sub[d]] = d;
+        order = persist_order(S, h->h_soff, h->h_gk, h->h_gstart, h->h_uslot, start);
+    } else {
+        std::iota(order.begin(), order.end(), 0);
     }
-    std::vector<int> sp(P + 1, S);
-    sp[0] = 0;
-    {
-        double acc = 0;
-        int p = 1;
-        for (int s = 0; s < S && p < P; ++s) {
-            acc += cost[s];
-            while (p < P && acc >= total * p / P) sp[p++] = s + 1;
-        }
-        for (int p2 = 1; p2 <= P; ++p2) sp[p2] = std::max(sp[p2], sp[p2 - 1]);
-        sp[P] = S;
-    }
+    const PersistParts parts = persist_parts(P, S, order, cost, h->h_soff, h->h_gk, h->h_pk, h->h_gstart, h->h_uslot);
     const int P1 = P + 1;
-    std::vector<int> pr(5 * P1);
+    std::vector<int> pr(7 * P1, 0);
     auto PR = [&](int field, int p) -> int & { return pr[field * P1 + p]; };
-    for (int p = 0; p <= P; ++p) {
-        const int s = sp[p];
-        PR(0, p) = h->h_soff[s];
-        PR(1, p) = s;
-        PR(2, p) = h->h_tpre[s];
-        PR(3, p) = h->h_foff[s];
-        PR(4, p) = h->h_vpre[s];
-    }
-    // factors staged per part with column stride npad (+ 4 when npad % 8 == 0)
+    // per part: factors staged with column stride npad (+ 4 when npad % 8 == 0)
     std::vector<int4> srec(S + 1, make_int4(0, 0, 0, 0));
-    std::vector<int> items, meta(L);
-    std::vector<long long> fpart(P, 0);
+    std::vector<int> items, meta;
+    meta.reserve(L);
+    long long mf = 0, ms = 0, mj = 0, mk = 0, mv = 0, mr = 0, ml = 0;
     for (int p = 0; p < P; ++p) {
-        for (int s = sp[p]; s < sp[p + 1]; ++s) {
-            const int npad = h->h_npad[s], cs = npad + ((npad & 7) == 0 ? 4 : 0);
-            srec[s] = make_int4((int)fpart[p], h->h_vpre[s] - PR(4, p), h->h_tpre[s] - PR(2, p),
-                                (h->h_sf[s] << 10) | (npad << 1) | (h->h_mode[s] & 1));
-            fpart[p] += (long long)h->h_sf[s] * cs;
-            for (int c = 0; c < h->h_sf[s]; ++c) items.push_back(((s - sp[p]) << 8) | c);
-            for (int r = 0; r < h->h_sn[s]; ++r) meta[h->h_soff[s] + r] = ((s - sp[p]) << 8) | r;
+        const int s0 = parts.s0[p];
+        long long f = 0, v = 0, t = 0;
+        for (int i = s0; i < parts.s0[p + 1]; ++i) {
+            const int d = parts.sub[i], npad = h->h_npad[d], cs = npad + ((npad & 7) == 0 ? 4 : 0);
+            srec[i] = make_int4((int)f, (int)v, (int)t, (h->h_sf[d] << 10) | (npad << 1) | (h->h_mode[d] & 1));
+            for (int c = 0; c < h->h_sf[d]; ++c) items.push_back(((i - s0) << 8) | c);
+            for (int r = 0; r < h->h_sn[d]; ++r) meta.push_back(((i - s0) << 8) | r);
+            f += (long long)h->h_sf[d] * cs;
+            v += npad;
+            t += h->h_sf[d];
         }
-    }
-    long long mf = 0, ms = 0, mj = 0, mk = 0, mv = 0;
-    for (int p = 0; p < P; ++p) {
-        mk = std::max<long long>(mk, PR(0, p + 1) - PR(0, p));
-        ms = std::max<long long>(ms, PR(1, p + 1) - PR(1, p));
-        mj = std::max<long long>(mj, PR(2, p + 1) - PR(2, p));
-        mf = std::max<long long>(mf, fpart[p]);
-        mv = std::max<long long>(mv, PR(4, p + 1) - PR(4, p));
+        PR(0, p + 1) = parts.k0[p + 1];
+        PR(1, p + 1) = parts.s0[p + 1];
+        PR(2, p + 1) = (int)items.size();
+        PR(4, p + 1) = PR(4, p) + (int)v;
+        PR(5, p + 1) = parts.r0[p + 1];
+        PR(6, p + 1) = parts.l0[p + 1];
+        mf = std::max(mf, f);
+        mv = std::max(mv, v);
+        mj = std::max(mj, t);
+        mk = std::max<long long>(mk, parts.k0[p + 1] - parts.k0[p]);
+        ms = std::max<long long>(ms, parts.s0[p + 1] - s0);
+        mr = std::max<long long>(mr, parts.r0[p + 1] - parts.r0[p]);
+        ml = std::max<long long>(ml, parts.l0[p + 1] - parts.l0[p]);
     }
     PersistLayout &c = pp->lay;
     c = PersistLayout{};
     c.P = P;
     c.L = L;
+    c.local = local ? 1 : 0;
+    c.threads = (int)std::min<long long>(kPersistMaxThreads, std::max<long long>(64, (std::max(mk, mj) + 31) / 32 * 32));
+    if (local && (std::max(mk, mj) > c.threads || mk + mr > 0xffff)) return OPF_OK;
+    // plans of small CTAs (one or a few subsystems each: the 123-bus feeder)
+    // run phase B with each factor column on 4 lanes, given threads for it;
+    // large ones keep one lane per column (the split measured slower there)
+    if (local && c.threads <= 128) {
+        c.split = 1;
+        c.threads = (int)std::max<long long>(c.threads, (4 * mj + 31) / 32 * 32);
+    }
     size_t off = 0;
     auto take = [&](unsigned *o, size_t bytes) { *o = (unsigned)off; off = align16u(off + bytes); };
     take(&c.off_F, (size_t)mf * sizeof(T));
     take(&c.off_srec, (size_t)ms * sizeof(int4));
-    take(&c.off_items, (size_t)mj * sizeof(int));
-    take(&c.off_meta, (size_t)mk * sizeof(int));
-    take(&c.off_segp, (size_t)mk * sizeof(int));
-    take(&c.off_pk, (size_t)mk * sizeof(int));
-    take(&c.off_bt, (size_t)mk * sizeof(T));
-    take(&c.off_ds, (size_t)mk * sizeof(T));
-    take(&c.off_mu, (size_t)mk * sizeof(T));
-    take(&c.off_ct, (size_t)mk * sizeof(T));
-    take(&c.off_lbt, (size_t)mk * sizeof(T));
-    take(&c.off_ubt, (size_t)mk * sizeof(T));
-    take(&c.off_vbx, (size_t)mv * sizeof(T));
-    take(&c.off_vbw, (size_t)mv * sizeof(T));
+    if (local) {
+        take(&c.off_list, (size_t)ml * sizeof(int));
+        take(&c.off_rem, (size_t)mr * sizeof(int));
+        take(&c.off_ul, (size_t)(mk + mr) * sizeof(T));
+    } else {
+        take(&c.off_items, (size_t)mj * sizeof(int));
+        take(&c.off_slots, (size_t)mk * persist_slot_bytes(sizeof(T)));
+        take(&c.off_r, (size_t)mk * sizeof(T));
+        take(&c.off_rn, 256 * sizeof(T));
+    }
+    take(&c.off_vb, (size_t)mv * sizeof(T));
     take(&c.off_tb, (size_t)mj * sizeof(T));
-    take(&c.off_recip, 256 * sizeof(T));
     take(&c.off_xrs, (size_t)mk * sizeof(double));
     take(&c.off_lrs, (size_t)mk * sizeof(double));
     take(&c.off_cobj, (size_t)mk * sizeof(double));
     // flags (16 B), a DevStatus copy, the [32][6] block-sum scratch
     take(&c.off_misc, 16 + ((sizeof(DevStatus) + 15) & ~(size_t)15) + 32 * 6 * sizeof(double));
     c.bytes = (unsigned)off;
-    c.threads = (int)std::min<long long>(kPersistMaxThreads, std::max<long long>(64, (std::max(mk, mj) + 31) / 32 * 32));
-    // plans of small CTAs (one or a few subsystems each: the 123-bus feeder)
-    // run phase B with each factor column on 4 lanes, given threads for it;
-    // large ones keep one lane per column (the split measured slower there)
-    c.split = 0;
-    if (c.threads <= 128) {
-        c.split = 1;
-        c.threads = (int)std::min<long long>(kPersistMaxThreads, std::max<long long>(c.threads, (4 * mj + 31) / 32 * 32));
-    }
     int optin = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
-    if ((long long)c.bytes > optin) return OPF_OK;
-    if (prepare_persist_engine<T>(c.bytes)) { cudaGetLastError(); return OPF_OK; }
-    const int occ = persist_occupancy<T>(c.threads, c.bytes);
+    if ((long long)off > optin) return OPF_OK;
+    if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
+    const int occ = persist_occupancy<T>(c);
     if ((long long)occ * n_sm < P) { cudaGetLastError(); return OPF_OK; }
+    pp->S = S;
+    pp->L = L;
+    if (!pp->d_xu) TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(L) / sizeof(unsigned long long)));
+    if (local) {
+        if (!pp->d_parts) TRY(dalloc(h, &pp->d_parts, (size_t)S + 3 * (size_t)L));
+        pp->list_len = parts.list.size();
+        const size_t need = parts.list.size() + parts.rem.size();
+        if (need > pp->n_lists) {
+            TRY(dalloc(h, &pp->d_lists, need));
+            pp->n_lists = need;
+        }
+        int *at = pp->d_parts;
+        for (const std::vector<int> *v : {&parts.sub, &parts.slot, &parts.seg, &parts.out}) {
+            CUDA_TRY(cudaMemcpyAsync(at, v->data(), v->size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+            at += v->size();
+        }
+        at = pp->d_lists;
+        for (const std::vector<int> *v : {&parts.list, &parts.rem}) {
+            if (!v->empty())
+                CUDA_TRY(cudaMemcpyAsync(at, v->data(), v->size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+            at += v->size();
+        }
+    }
     CUDA_TRY(cudaMemcpyAsync(pp->d_pr, pr.data(), pr.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(cudaMemcpyAsync(pp->d_srec, srec.data(), srec.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
     if (!items.empty())
@@ -846,10 +866,15 @@ static int get_persist_plan(opf_handle *h, PersistPlan *pp, int requested) {
     const int n_sm = stream_sm_count(h->stream, h->device);
     pp->tried = true;
     pp->req = requested;
-    if (requested > 0) return build_persist_plan<T>(h, pp, requested, n_sm);
+    auto build = [&](int P) -> int {
+        TRY(build_persist_plan<T>(h, pp, P, n_sm, true));
+        if (!pp->ok) TRY(build_persist_plan<T>(h, pp, P, n_sm, false));
+        return OPF_OK;
+    };
+    if (requested > 0) return build(requested);
     const int cap = std::max(1, (h->L + 31) / 32);
     for (int per : {2, 1}) {
-        TRY(build_persist_plan<T>(h, pp, std::min(per * n_sm, cap), n_sm));
+        TRY(build(std::min(per * n_sm, cap)));
         if (pp->ok) return OPF_OK;
     }
     return OPF_OK;
@@ -1248,8 +1273,6 @@ static int fault_error(opf_handle *h) {
 static int run_persist64(opf_handle *h, const opf_solve_opts &o) {
     const double rho = o.rho;
     TRY(set_recip(h, rho));
-    launch_make_u<double>(h->L, h->d_pk, h->d_ds64, h->d_mu64, rho, h->d_u64, nullptr, h->stream);
-    CUDA_TRY(cudaGetLastError());
     const PersistPlan &pp = h->p64;
     IterArgs<double> a = with_persist(iter_args<double>(h, rho), pp);
     const int k = o.check_every;
@@ -1314,7 +1337,8 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                            h->d_gseg, h->d_uslot, h->d_c64, h->d_lb64, h->d_ub64, h->d_ct32, h->d_lbt32,
                            h->d_ubt32, h->d_sub, h->d_sub2, h->d_F64, h->d_bbar64, rho, h->d_bt32,
                            nullptr, h->stream);
-    launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, nullptr, h->stream);
+    // (the persistent engine forms u itself)
+    if (eng != 4) launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, nullptr, h->stream);
     CUDA_TRY(cudaGetLastError());
 
     const int kind = eng + (recenter ? 0 : 8);
@@ -1346,7 +1370,8 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                                    h->d_lbt32, h->d_ubt32, h->d_sub, h->d_sub2, h->d_F64, h->d_bbar64, rho,
                                    h->d_bt32, h->d_st, h->stream);
             launch_copy_if_running(G, h->d_xr2, h->d_xr, h->d_st, h->stream);
-            launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, h->d_st, h->stream);
+            if (eng != 4)
+                launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, h->d_st, h->stream);
     };
     const int planP = eng == 4 ? 10000 + h->p32.P : eng == 3 ? 100 + h->w32.P : eng == 2 ? h->c32.P : 0;
     if (h->gmix.kind != kind || h->gmix.rho != rho || h->gmix.k != k || h->gmix.R != R ||

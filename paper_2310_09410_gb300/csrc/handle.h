@@ -49,12 +49,22 @@ struct PersistPlan {
     bool tried = false;          // built (ok or not) for the current factors and request
     int req = 0;                 // requested CTA count of that build (0: automatic)
     PersistLayout lay{};
-    int *d_pr = nullptr;         // 5 * (kPersistMaxP + 1)
+    int *d_pr = nullptr;         // 7 * (kPersistMaxP + 1)
     int4 *d_srec = nullptr;
     int *d_items = nullptr, *d_meta = nullptr;
     double *d_part = nullptr;    // 6 * kPersistMaxP
     unsigned long long *d_sync = nullptr;
-    PersistPtrs ptrs() const { return PersistPtrs{d_pr, d_part, d_sync}; }
+    // allocated with the first plan that fits
+    unsigned long long *d_xu = nullptr;   // exchange buffer
+    // local plans: subsystem, slot, seg and out per part-order position (S + 3 L),
+    // then the lists and remote entries (capacity n_lists)
+    int *d_parts = nullptr, *d_lists = nullptr;
+    size_t n_lists = 0, list_len = 0;
+    int S = 0, L = 0;
+    PersistPtrs ptrs() const {
+        return PersistPtrs{d_pr, d_part, d_sync, d_xu, d_parts, d_parts + S, d_parts + S + L, d_parts + S + 2 * L,
+                           d_lists, d_lists + list_len};
+    }
 };
 
 // Warp-engine plan for one precision: warp slots of the CTAs of one cluster.

@@ -154,19 +154,27 @@ struct ClusterLayout {
 constexpr int kPersistMaxThreads = 512;
 struct PersistLayout {
     int P, L, threads;
-    int split;                     // phase B: a factor column on 4 lanes (plans of small CTAs)
-    unsigned off_F, off_srec, off_items, off_meta, off_segp, off_pk, off_bt, off_ds, off_mu;
-    unsigned off_ct, off_lbt, off_ubt, off_vbx, off_vbw, off_tb, off_recip, off_xrs, off_lrs, off_cobj;
-    unsigned off_misc;
+    int local;                     // k_persist_local (one slot and one factor column per thread), else k_persist_engine
+    int split;                     // phase B: a factor column on 4 lanes (local plans of small CTAs)
+    unsigned off_F, off_srec, off_vb, off_tb, off_xrs, off_lrs, off_cobj, off_misc;
+    unsigned off_list, off_rem, off_ul;                 // local plans
+    unsigned off_items, off_slots, off_r, off_rn;       // the others
     unsigned bytes;
 };
 
 // Device arrays of a persistent grid engine plan.
 struct PersistPtrs {
-    const int *pr;                 // part ranges, 5 fields x (P + 1)
+    const int *pr;                 // part ranges, 7 fields x (P + 1)
     double *part;                  // Sec. III-C partial sums, P x 6
     unsigned long long *sync;      // grid barrier counter
+    unsigned long long *xu;        // exchange of u: two buffers of L stamped entries
+    // local plans (persist_plan.h): subsystems and slots in part order, the
+    // slots' lists of copies and exports, the remote entries
+    const int *sub, *slot, *seg, *out, *list, *rem;
 };
+
+// Bytes of a slot's record in a plan with several slots per thread (persist.cu).
+constexpr size_t persist_slot_bytes(size_t word) { return 6 * word + 8; }
 
 // Shared-memory image of one CTA of the warp engine, byte offsets.
 struct WarpLayout {
