@@ -302,10 +302,6 @@ static int build_layout(opf_handle *h) {
     TRY(dalloc(h, &h->w32.d_fbig, h->S + 1));
     TRY(dalloc(h, &h->w32.d_F2, h->nF));
     for (PersistPlan *pp : {&h->p32, &h->p64}) {
-        TRY(dalloc(h, &pp->d_pr, 7 * (kPersistMaxP + 1)));
-        TRY(dalloc(h, &pp->d_srec, h->S + 1));
-        TRY(dalloc(h, &pp->d_items, std::max<long long>(items_cap, 1)));
-        TRY(dalloc(h, &pp->d_meta, h->L));
         TRY(dalloc(h, &pp->d_part, 6 * kPersistMaxP));
         TRY(dalloc(h, &pp->d_sync, 1));
     }
@@ -456,10 +452,10 @@ extern "C" int opf_precompute(opf_handle *h) {
     CUDA_TRY(cudaEventRecord(h->ev[0], h->stream));
     h->have_pinv = false;
     TRY(launch_precompute_kernel(h, false));
-    std::vector<int> status(h->S);
-    h->h_sf.resize(h->S);
+    std::vector<int> status(h->S), sf(h->S), mode(h->S);
     CUDA_TRY(cudaMemcpyAsync(status.data(), h->d_pstatus, h->S * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(h->h_sf.data(), h->d_sf, h->S * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(sf.data(), h->d_sf, h->S * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(mode.data(), h->d_smode, h->S * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     for (int s = 0; s < h->S; ++s)
         if (status[s]) {
@@ -468,35 +464,56 @@ extern "C" int opf_precompute(opf_handle *h) {
             return OPF_E_INFEASIBLE_LOCAL;
         }
     // iteration layout: per subsystem (first slot, n, f, mode) and (factor
-    // offset, npad, padded-v prefix, f prefix); factor columns padded to npad
-    h->h_mode.resize(h->S);
-    CUDA_TRY(cudaMemcpyAsync(h->h_mode.data(), h->d_smode, h->S * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    std::vector<int4> sub(h->S + 1), sub2(h->S + 1);
-    h->h_tpre.assign(h->S + 1, 0); h->h_vpre.assign(h->S + 1, 0); h->h_foff.assign(h->S + 1, 0);
-    h->h_npad.assign(h->S, 0);
-    std::vector<int> items;
-    long long fo = 0, vpre = 0, tpre = 0;
-    h->sum_nf = 0;
-    for (int s = 0; s < h->S; ++s) {
-        const int n = h->h_sn[s], f = h->h_sf[s], npad = round4(n);
-        sub[s] = make_int4(h->h_soff[s], n, f, h->h_mode[s]);
-        sub2[s] = make_int4((int)fo, npad, (int)vpre, (int)tpre);
-        h->h_foff[s] = (int)fo; h->h_vpre[s] = (int)vpre; h->h_tpre[s] = (int)tpre; h->h_npad[s] = npad;
-        for (int c = 0; c < f; ++c) items.push_back((s << 8) | c);
-        fo += (long long)f * npad;
-        vpre += npad;
-        tpre += f;
-        h->sum_nf += (long long)n * f;
+    // offset, npad, padded-v prefix, f prefix); factor columns padded to npad.
+    // These tables, the engine plans and their solve graphs follow from the
+    // subsystems' slots, factor ranks and modes alone: new loads leave those as
+    // they were (a new A_s may change a rank), and then only the factors and
+    // bbar are new.  (8500 buses: a solve with new loads 55.9 ms the first time,
+    // 51.2 ms with the plans kept; with a partition built for each precision
+    // and each solve it was 61.6 ms.)
+    if (!h->have_layout || sf != h->h_sf || mode != h->h_mode) {
+        h->h_sf = sf;
+        h->h_mode = mode;
+        h->have_layout = false;
+        std::vector<int4> sub(h->S + 1), sub2(h->S + 1);
+        h->h_tpre.assign(h->S + 1, 0); h->h_vpre.assign(h->S + 1, 0); h->h_foff.assign(h->S + 1, 0);
+        h->h_npad.assign(h->S, 0);
+        std::vector<int> items;
+        long long fo = 0, vpre = 0, tpre = 0;
+        h->sum_nf = 0;
+        for (int s = 0; s < h->S; ++s) {
+            const int n = h->h_sn[s], f = h->h_sf[s], npad = round4(n);
+            sub[s] = make_int4(h->h_soff[s], n, f, h->h_mode[s]);
+            sub2[s] = make_int4((int)fo, npad, (int)vpre, (int)tpre);
+            h->h_foff[s] = (int)fo; h->h_vpre[s] = (int)vpre; h->h_tpre[s] = (int)tpre; h->h_npad[s] = npad;
+            for (int c = 0; c < f; ++c) items.push_back((s << 8) | c);
+            fo += (long long)f * npad;
+            vpre += npad;
+            tpre += f;
+            h->sum_nf += (long long)n * f;
+        }
+        sub[h->S] = make_int4(h->L, 0, 0, 0);
+        h->h_foff[h->S] = (int)fo; h->h_vpre[h->S] = (int)vpre; h->h_tpre[h->S] = (int)tpre;
+        sub2[h->S] = make_int4((int)fo, 0, (int)vpre, (int)tpre);
+        h->nitems = (long long)items.size();
+        h->nF = std::max<long long>(fo, 4);
+        CUDA_TRY(cudaMemcpyAsync(h->d_sub, sub.data(), sub.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+        CUDA_TRY(cudaMemcpyAsync(h->d_sub2, sub2.data(), sub2.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
+        if (!items.empty())
+            CUDA_TRY(cudaMemcpyAsync(h->d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+        TRY(make_tiling(h, &h->t64, 64, 64));
+        TRY(make_tiling(h, &h->t32, 256, 128));
+        CUDA_TRY(cudaStreamSynchronize(h->stream));      // the uploads read local vectors
+        h->c32.P = h->c64.P = 0;
+        h->c32.ok = h->c64.ok = false;
+        h->p32.P = h->p64.P = 0;
+        h->p32.ok = h->p64.ok = h->p32.tried = h->p64.tried = false;
+        h->p32.tab.reset();
+        h->p64.tab.reset();
+        h->g64.reset();
+        h->gmix.reset();
+        h->have_layout = true;
     }
-    sub[h->S] = make_int4(h->L, 0, 0, 0);
-    h->h_foff[h->S] = (int)fo; h->h_vpre[h->S] = (int)vpre; h->h_tpre[h->S] = (int)tpre;
-    sub2[h->S] = make_int4((int)fo, 0, (int)vpre, (int)tpre);
-    h->nitems = (long long)items.size();
-    CUDA_TRY(cudaMemcpyAsync(h->d_sub, sub.data(), sub.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(h->d_sub2, sub2.data(), sub2.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
-    if (!items.empty())
-        CUDA_TRY(cudaMemcpyAsync(h->d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     launch_pack_factors(h->S, h->d_sub, h->d_sub2, h->d_fcap, h->d_Fcap, h->d_F64, h->d_F32, h->stream);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaEventRecord(h->ev[1], h->stream));
@@ -504,18 +521,10 @@ extern "C" int opf_precompute(opf_handle *h) {
     float ms = 0;
     cudaEventElapsedTime(&ms, h->ev[0], h->ev[1]);
     h->timing[0] = ms;
-    h->nF = std::max<long long>(fo, 4);
-    TRY(make_tiling(h, &h->t64, 64, 64));
-    TRY(make_tiling(h, &h->t32, 256, 128));
-    h->c32.P = h->c64.P = 0;
-    h->c32.ok = h->c64.ok = false;
-    h->p32.P = h->p64.P = 0;
-    h->p32.ok = h->p64.ok = h->p32.tried = h->p64.tried = false;
+    // the warp engine's plans hold copies of the factors
     h->w32.built = h->w32.ok = false;
     h->w64.built = h->w64.ok = false;
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    h->g64.reset();
-    h->gmix.reset();
+    if ((h->gmix.kind & 7) == 3) h->gmix.reset();
     h->precomputed = true;
     return reset_state(h);
 }
@@ -725,48 +734,47 @@ static int get_cluster_plan(opf_handle *h, ClusterPlan *cp, int requested, int t
     return OPF_OK;
 }
 
-// Partition the instance over P co-resident CTAs of the persistent grid engine
-// and lay out its shared memory: parts of a depth-first order for the local
-// form, else (more slots or columns than threads, or no room) runs of the
-// size-sorted order.  Leaves pp->ok false when a part does not fit one CTA or
-// P CTAs cannot be resident.
-template <typename T>
-static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local) {
-    pp->ok = false;
-    pp->P = P;
-    if (P < 1 || P > kPersistMaxP) return OPF_OK;
+// The partition of the instance over P CTAs: parts of a depth-first order for
+// the local form, else runs of the size-sorted order.
+static int build_persist_tables(opf_handle *h, int P, bool local, std::shared_ptr<PersistTables> *out) {
     const int S = h->S, L = h->L;
     std::vector<double> cost(S);
     for (int s = 0; s < S; ++s)
         cost[s] = 6.0 * h->h_sn[s] + (double)h->h_sf[s] * h->h_npad[s] + (double)h->h_sn[s] * h->h_sf[s];
-    std::vector<int> order(S);
+    std::vector<int> order;
     if (local) {
-        std::vector<int> start(S);           // new trees begin in canonical order
-        for (int d = 0; d < S; ++d) start[h->dev_to_canon_sub[d]] = d;
-        order = persist_order(S, h->h_soff, h->h_gk, h->h_gstart, h->h_uslot, start);
+        if (h->persist_order.empty()) {
+            std::vector<int> start(S);           // new trees begin in canonical order
+            for (int d = 0; d < S; ++d) start[h->dev_to_canon_sub[d]] = d;
+            h->persist_order = persist_order(S, h->h_soff, h->h_gk, h->h_gstart, h->h_uslot, start);
+        }
+        order = h->persist_order;
     } else {
+        order.resize(S);
         std::iota(order.begin(), order.end(), 0);
     }
     const PersistParts parts = persist_parts(P, S, order, cost, h->h_soff, h->h_gk, h->h_pk, h->h_gstart, h->h_uslot);
+    auto t = std::make_shared<PersistTables>();
+    t->P = P; t->S = S; t->L = L;
+    t->local = local;
     const int P1 = P + 1;
-    std::vector<int> pr(7 * P1, 0);
+    std::vector<int> pr(7 * P1, 0), items, meta;
     auto PR = [&](int field, int p) -> int & { return pr[field * P1 + p]; };
     // per part: factors staged with column stride npad (+ 4 when npad % 8 == 0)
-    std::vector<int4> srec(S + 1, make_int4(0, 0, 0, 0));
-    std::vector<int> items, meta;
+    std::vector<int4> srec(S);
     meta.reserve(L);
-    long long mf = 0, ms = 0, mj = 0, mk = 0, mv = 0, mr = 0, ml = 0;
+    items.reserve(h->nitems);
     for (int p = 0; p < P; ++p) {
         const int s0 = parts.s0[p];
-        long long f = 0, v = 0, t = 0;
+        long long f = 0, v = 0, c0 = 0;
         for (int i = s0; i < parts.s0[p + 1]; ++i) {
             const int d = parts.sub[i], npad = h->h_npad[d], cs = npad + ((npad & 7) == 0 ? 4 : 0);
-            srec[i] = make_int4((int)f, (int)v, (int)t, (h->h_sf[d] << 10) | (npad << 1) | (h->h_mode[d] & 1));
+            srec[i] = make_int4((int)f, (int)v, (int)c0, (h->h_sf[d] << 10) | (npad << 1) | (h->h_mode[d] & 1));
             for (int c = 0; c < h->h_sf[d]; ++c) items.push_back(((i - s0) << 8) | c);
             for (int r = 0; r < h->h_sn[d]; ++r) meta.push_back(((i - s0) << 8) | r);
             f += (long long)h->h_sf[d] * cs;
             v += npad;
-            t += h->h_sf[d];
+            c0 += h->h_sf[d];
         }
         PR(0, p + 1) = parts.k0[p + 1];
         PR(1, p + 1) = parts.s0[p + 1];
@@ -774,47 +782,86 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
         PR(4, p + 1) = PR(4, p) + (int)v;
         PR(5, p + 1) = parts.r0[p + 1];
         PR(6, p + 1) = parts.l0[p + 1];
-        mf = std::max(mf, f);
-        mv = std::max(mv, v);
-        mj = std::max(mj, t);
-        mk = std::max<long long>(mk, parts.k0[p + 1] - parts.k0[p]);
-        ms = std::max<long long>(ms, parts.s0[p + 1] - s0);
-        mr = std::max<long long>(mr, parts.r0[p + 1] - parts.r0[p]);
-        ml = std::max<long long>(ml, parts.l0[p + 1] - parts.l0[p]);
+        t->mf = std::max(t->mf, f);
+        t->mv = std::max(t->mv, v);
+        t->mj = std::max(t->mj, c0);
+        t->mk = std::max<long long>(t->mk, parts.k0[p + 1] - parts.k0[p]);
+        t->ms = std::max<long long>(t->ms, parts.s0[p + 1] - s0);
+        t->mr = std::max<long long>(t->mr, parts.r0[p + 1] - parts.r0[p]);
+        t->ml = std::max<long long>(t->ml, parts.l0[p + 1] - parts.l0[p]);
     }
+    // one allocation and one upload
+    std::vector<int> all(4 * (size_t)S);
+    memcpy(all.data(), srec.data(), 4 * (size_t)S * sizeof(int));
+    std::vector<std::pair<int **, size_t>> at;
+    auto add = [&](int **p, const std::vector<int> &v) {
+        at.push_back({p, all.size()});
+        all.insert(all.end(), v.begin(), v.end());
+    };
+    add(&t->pr, pr); add(&t->items, items); add(&t->meta, meta);
+    add(&t->sub, parts.sub);
+    if (local) {
+        add(&t->slot, parts.slot); add(&t->seg, parts.seg); add(&t->out, parts.out);
+        add(&t->list, parts.list); add(&t->rem, parts.rem);
+    }
+    void *q = nullptr;
+    CUDA_TRY(cudaMalloc(&q, std::max<size_t>(all.size(), 1) * sizeof(int)));
+    t->mem = (int *)q;
+    t->srec = (int4 *)q;
+    for (auto &e : at) *e.first = t->mem + e.second;
+    CUDA_TRY(cudaMemcpyAsync(t->mem, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    *out = t;
+    return OPF_OK;
+}
+
+// Plan of the persistent grid engine on P CTAs: the partition and its
+// shared-memory layout.  Leaves pp->ok false when a part does not fit one CTA
+// (local form: also when it has more slots or columns than threads) or P CTAs
+// cannot be resident.
+template <typename T>
+static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local) {
+    pp->ok = false;
+    pp->P = P;
+    if (P < 1 || P > kPersistMaxP) return OPF_OK;
+    PersistPlan &other = pp == &h->p32 ? h->p64 : h->p32;
+    if (other.tab && other.tab->P == P && other.tab->local == local) pp->tab = other.tab;
+    else if (!pp->tab || pp->tab->P != P || pp->tab->local != local) TRY(build_persist_tables(h, P, local, &pp->tab));
+    const PersistTables &t = *pp->tab;
     PersistLayout &c = pp->lay;
     c = PersistLayout{};
     c.P = P;
-    c.L = L;
+    c.L = h->L;
     c.local = local ? 1 : 0;
-    c.threads = (int)std::min<long long>(kPersistMaxThreads, std::max<long long>(64, (std::max(mk, mj) + 31) / 32 * 32));
-    if (local && (std::max(mk, mj) > c.threads || mk + mr > 0xffff)) return OPF_OK;
+    c.threads = (int)std::min<long long>(kPersistMaxThreads,
+                                         std::max<long long>(64, (std::max(t.mk, t.mj) + 31) / 32 * 32));
+    if (local && (std::max(t.mk, t.mj) > c.threads || t.mk + t.mr > 0xffff)) return OPF_OK;
     // plans of small CTAs (one or a few subsystems each: the 123-bus feeder)
     // run phase B with each factor column on 4 lanes, given threads for it;
     // large ones keep one lane per column (the split measured slower there)
     if (local && c.threads <= 128) {
         c.split = 1;
-        c.threads = (int)std::max<long long>(c.threads, (4 * mj + 31) / 32 * 32);
+        c.threads = (int)std::max<long long>(c.threads, (4 * t.mj + 31) / 32 * 32);
     }
     size_t off = 0;
     auto take = [&](unsigned *o, size_t bytes) { *o = (unsigned)off; off = align16u(off + bytes); };
-    take(&c.off_F, (size_t)mf * sizeof(T));
-    take(&c.off_srec, (size_t)ms * sizeof(int4));
+    take(&c.off_F, (size_t)t.mf * sizeof(T));
+    take(&c.off_srec, (size_t)t.ms * sizeof(int4));
     if (local) {
-        take(&c.off_list, (size_t)ml * sizeof(int));
-        take(&c.off_rem, (size_t)mr * sizeof(int));
-        take(&c.off_ul, (size_t)(mk + mr) * sizeof(T));
+        take(&c.off_list, (size_t)t.ml * sizeof(int));
+        take(&c.off_rem, (size_t)t.mr * sizeof(int));
+        take(&c.off_ul, (size_t)(t.mk + t.mr) * sizeof(T));
     } else {
-        take(&c.off_items, (size_t)mj * sizeof(int));
-        take(&c.off_slots, (size_t)mk * persist_slot_bytes(sizeof(T)));
-        take(&c.off_r, (size_t)mk * sizeof(T));
+        take(&c.off_items, (size_t)t.mj * sizeof(int));
+        take(&c.off_slots, (size_t)t.mk * persist_slot_bytes(sizeof(T)));
+        take(&c.off_r, (size_t)t.mk * sizeof(T));
         take(&c.off_rn, 256 * sizeof(T));
     }
-    take(&c.off_vb, (size_t)mv * sizeof(T));
-    take(&c.off_tb, (size_t)mj * sizeof(T));
-    take(&c.off_xrs, (size_t)mk * sizeof(double));
-    take(&c.off_lrs, (size_t)mk * sizeof(double));
-    take(&c.off_cobj, (size_t)mk * sizeof(double));
+    take(&c.off_vb, (size_t)t.mv * sizeof(T));
+    take(&c.off_tb, (size_t)t.mj * sizeof(T));
+    take(&c.off_xrs, (size_t)t.mk * sizeof(double));
+    take(&c.off_lrs, (size_t)t.mk * sizeof(double));
+    take(&c.off_cobj, (size_t)t.mk * sizeof(double));
     // flags (16 B), a DevStatus copy, the [32][6] block-sum scratch
     take(&c.off_misc, 16 + ((sizeof(DevStatus) + 15) & ~(size_t)15) + 32 * 6 * sizeof(double));
     c.bytes = (unsigned)off;
@@ -824,36 +871,7 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
     const int occ = persist_occupancy<T>(c);
     if ((long long)occ * n_sm < P) { cudaGetLastError(); return OPF_OK; }
-    pp->S = S;
-    pp->L = L;
-    if (!pp->d_xu) TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(L) / sizeof(unsigned long long)));
-    if (local) {
-        if (!pp->d_parts) TRY(dalloc(h, &pp->d_parts, (size_t)S + 3 * (size_t)L));
-        pp->list_len = parts.list.size();
-        const size_t need = parts.list.size() + parts.rem.size();
-        if (need > pp->n_lists) {
-            TRY(dalloc(h, &pp->d_lists, need));
-            pp->n_lists = need;
-        }
-        int *at = pp->d_parts;
-        for (const std::vector<int> *v : {&parts.sub, &parts.slot, &parts.seg, &parts.out}) {
-            CUDA_TRY(cudaMemcpyAsync(at, v->data(), v->size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-            at += v->size();
-        }
-        at = pp->d_lists;
-        for (const std::vector<int> *v : {&parts.list, &parts.rem}) {
-            if (!v->empty())
-                CUDA_TRY(cudaMemcpyAsync(at, v->data(), v->size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-            at += v->size();
-        }
-    }
-    CUDA_TRY(cudaMemcpyAsync(pp->d_pr, pr.data(), pr.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(pp->d_srec, srec.data(), srec.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
-    if (!items.empty())
-        CUDA_TRY(cudaMemcpyAsync(pp->d_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice,
-                                 h->stream));
-    CUDA_TRY(cudaMemcpyAsync(pp->d_meta, meta.data(), L * sizeof(int), cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    if (!pp->d_xu) TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(h->L) / sizeof(unsigned long long)));
     pp->ok = true;
     return OPF_OK;
 }
@@ -882,7 +900,7 @@ static int get_persist_plan(opf_handle *h, PersistPlan *pp, int requested) {
 
 template <typename T>
 static IterArgs<T> with_persist(IterArgs<T> a, const PersistPlan &pp) {
-    a.srec = pp.d_srec; a.citems = pp.d_items; a.cmeta = pp.d_meta;
+    a.srec = pp.tab->srec; a.citems = pp.tab->items; a.cmeta = pp.tab->meta;
     return a;
 }
 

@@ -6,6 +6,7 @@
 
 #include <atomic>
 #include <cstring>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -40,8 +41,25 @@ struct ClusterPlan {
     int *d_items = nullptr, *d_meta = nullptr, *d_udst = nullptr, *d_gsegp = nullptr, *d_cdst = nullptr;
 };
 
-// Persistent grid engine plan for one precision: P co-resident CTAs, part
-// ranges, part-relative records, the partial sums and the barrier counter.
+// Partition of the persistent grid engine over P CTAs (persist_plan.h) on the
+// device; the plans of both precisions share it while they agree on P and form.
+struct PersistTables {
+    int P = 0, S = 0, L = 0;
+    bool local = false;
+    long long mf = 0, ms = 0, mj = 0, mk = 0, mv = 0, mr = 0, ml = 0;   // largest part: factor words, subsystems,
+                                                                        // columns, slots, vector rows, remote, list
+    int *mem = nullptr;          // one allocation: the arrays below
+    int *pr = nullptr, *items = nullptr, *meta = nullptr;   // ranges, 7 x (P + 1); per column; per slot
+    int *sub = nullptr, *slot = nullptr, *seg = nullptr, *out = nullptr, *list = nullptr, *rem = nullptr;
+    int4 *srec = nullptr;
+    PersistTables() = default;
+    PersistTables(const PersistTables &) = delete;
+    PersistTables &operator=(const PersistTables &) = delete;
+    ~PersistTables() { if (mem) cudaFree(mem); }
+};
+
+// Persistent grid engine plan for one precision: P co-resident CTAs, the
+// partition, the partial sums and the barrier counter.
 constexpr int kPersistMaxP = 2048;
 struct PersistPlan {
     int P = 0;
@@ -49,21 +67,12 @@ struct PersistPlan {
     bool tried = false;          // built (ok or not) for the current factors and request
     int req = 0;                 // requested CTA count of that build (0: automatic)
     PersistLayout lay{};
-    int *d_pr = nullptr;         // 7 * (kPersistMaxP + 1)
-    int4 *d_srec = nullptr;
-    int *d_items = nullptr, *d_meta = nullptr;
+    std::shared_ptr<PersistTables> tab;
     double *d_part = nullptr;    // 6 * kPersistMaxP
     unsigned long long *d_sync = nullptr;
-    // allocated with the first plan that fits
-    unsigned long long *d_xu = nullptr;   // exchange buffer
-    // local plans: subsystem, slot, seg and out per part-order position (S + 3 L),
-    // then the lists and remote entries (capacity n_lists)
-    int *d_parts = nullptr, *d_lists = nullptr;
-    size_t n_lists = 0, list_len = 0;
-    int S = 0, L = 0;
+    unsigned long long *d_xu = nullptr;   // exchange buffer, allocated with the first plan that fits
     PersistPtrs ptrs() const {
-        return PersistPtrs{d_pr, d_part, d_sync, d_xu, d_parts, d_parts + S, d_parts + S + L, d_parts + S + 2 * L,
-                           d_lists, d_lists + list_len};
+        return PersistPtrs{tab->pr, d_part, d_sync, d_xu, tab->sub, tab->slot, tab->seg, tab->out, tab->list, tab->rem};
     }
 };
 
@@ -125,6 +134,7 @@ struct opf_handle {
     Tiling t64, t32;
     // bookkeeping
     bool precomputed = false;
+    bool have_layout = false;    // the iteration tables and plans belong to h_sf, h_mode
     bool have_prev_u = false;    // d_u64 + L holds the u that produced the last global update
     double last_rho = 100.0, recip_rho = -1.0;
     // Stop for solves whose body the host relaunches (OPF_SOLVE_HOST_LOOP):
@@ -142,6 +152,7 @@ struct opf_handle {
     GraphCache g64, gmix;
     ClusterPlan c32, c64;
     PersistPlan p32, p64;
+    std::vector<int> persist_order;      // depth-first order of the subsystems (computed with the first plan)
     bool persist_graph_failed = false;   // the cooperative launch could not be captured in a graph
     WarpPlan w32, w64;
     std::vector<int> h_tpre, h_vpre, h_foff, h_npad, h_pk, h_gk, h_gstart, h_uslot;

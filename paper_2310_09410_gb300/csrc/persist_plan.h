@@ -54,14 +54,20 @@ inline std::vector<int> persist_order(int S, const std::vector<int> &soff, const
             seen[d] = 1;
             order.push_back(d);
             // the globals with the fewest copies pushed last, so followed first
-            by_count.assign(gk.begin() + soff[d], gk.begin() + soff[d + 1]);
-            std::stable_sort(by_count.begin(), by_count.end(), [&](int a, int b) {
-                return gstart[a + 1] - gstart[a] > gstart[b + 1] - gstart[b];
-            });
+            by_count.clear();
+            for (int k = soff[d]; k < soff[d + 1]; ++k) {
+                const int g = gk[k], cnt = gstart[g + 1] - gstart[g];
+                if (cnt < 2 || walked[g]) continue;      // no other copy, or all on the stack or seen
+                walked[g] = cnt > 2;
+                size_t at = by_count.size();             // insertion sort: few and short
+                by_count.push_back(g);
+                while (at > 0 && gstart[by_count[at - 1] + 1] - gstart[by_count[at - 1]] < cnt) {
+                    by_count[at] = by_count[at - 1];
+                    --at;
+                }
+                by_count[at] = g;
+            }
             for (int g : by_count) {
-                if (walked[g]) continue;      // its copies' subsystems are on the stack or seen
-                const int cnt = gstart[g + 1] - gstart[g];
-                if (cnt > 2) walked[g] = 1;
                 for (int q = gstart[g + 1] - 1; q >= gstart[g]; --q)
                     if (!seen[sub_of[uslot[q]]]) stack.push_back(sub_of[uslot[q]]);
             }
@@ -77,6 +83,8 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
                                   const std::vector<int> &uslot) {
     PersistParts t;
     const int L = (int)gk.size(), G = (int)gstart.size() - 1;
+    t.slot.reserve(L);
+    t.list.reserve(2 * (size_t)L);
     t.s0.assign(P + 1, S);
     t.s0[0] = 0;
     double total = 0, acc = 0;
@@ -107,6 +115,7 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
     t.r0.assign(P + 1, 0);
     t.l0.assign(P + 1, 0);
     std::vector<int> done(G, -1), where(G, 0);
+    std::vector<char> read(L, 0);                // per slot: another part reads it
     for (int q = 0; q < P; ++q) {
         const int nk = t.k0[q + 1] - t.k0[q];
         for (int j = t.k0[q]; j < t.k0[q + 1]; ++j) {
@@ -121,16 +130,17 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
                     } else {
                         t.list.push_back(nk + (int)t.rem.size() - t.r0[q]);
                         t.rem.push_back(c);
+                        read[o] = 1;
                     }
                 }
             }
             t.seg[j] = ((cnt > 1 ? where[g] : 0) << 8) | cnt;
-            for (int c = c0; c < c0 + cnt; ++c)
-                if (part_of[uslot[c]] != q) t.out[j] = pk[k];
         }
         t.r0[q + 1] = (int)t.rem.size();
         t.l0[q + 1] = (int)t.list.size();
     }
+    for (int j = 0; j < L; ++j)
+        if (read[t.slot[j]]) t.out[j] = pk[t.slot[j]];
     return t;
 }
 

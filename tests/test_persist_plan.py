@@ -149,3 +149,29 @@ def test_engine_forms_match_oracle(ctas, precision):
     for got, want in ((xs, ref.xs), (lam, ref.lam), (x, ref.x)):
         scale = max(1.0, float(np.abs(want).max()))
         assert np.max(np.abs(got - want)) <= (1e-10 if precision == "fp64" else 1e-4) * scale
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_kept_plans_serve_new_loads(precision):
+    """Tables, plans and solve graphs kept over opf_precompute: a handle given
+    new loads twice returns what a fresh handle of those loads returns."""
+    from paper_2310_09410_gb300 import opf, synth
+
+    base = synth.preset_feeder("123", 2001)
+    prec = opf.PREC_FP64 if precision == "fp64" else opf.PREC_MIXED
+
+    def solved(s):
+        s.precompute()
+        s.solve(eps_rel=0.0, max_iter=1500, check_every=50, precision=prec)
+        return s.solution()
+
+    with opf.Solver.from_feeder(base) as s:
+        solved(s)
+        for seed in (7200, 7201):
+            f = synth.load_scenario(base, seed)
+            s.set_loads(f["load_a"], f["load_b"])
+            x, obj = solved(s)
+            with opf.Solver.from_feeder(f) as fresh:
+                y, want = solved(fresh)
+            assert np.array_equal(x, y) and obj == want
