@@ -84,8 +84,6 @@ BATCH_ENGINE_TRAFFIC_SOURCE = "profiles/k_batch_engine_123bus_x1024.md"
 # its 4000 iterations x 1024 instances (copied; None for other shapes).
 BATCH_ENGINE_INST_PER_INSTANCE_ITER = 16.7984e9 / (4000 * 1024)
 BATCH_ENGINE_INST_SHAPE = {"k_inst": 8, "warps": 16, "tmem": 1}
-WARP_ENGINE_TRAFFIC_PER_LAUNCH = 516864 + 768
-PERSIST_ENGINE_TRAFFIC_PER_LAUNCH = 8708352 + 313088
 ITERS_PER_LAUNCH = 1000
 
 
@@ -485,27 +483,32 @@ def max_over_ranks(value: float, world: int, device) -> float:
 
 
 def warp_engine_fp64(sizes):
-    """The library's automatic choice runs FP64 iterations on the warp engine
-    for instances of at most 64 subsystems of at most 64 slots."""
+    """The library's automatic choice runs FP64 iterations in one thread-block
+    cluster (one launch per solve) for instances of at most 64 subsystems of at
+    most 64 slots: those the FP64 warp engine holds with 4 warps per CTA."""
     return sizes["n_sub"] <= 64 and sizes["max_ns"] <= 64
 
 
-def count_launches_single(stats, precision, k=50, R=1000, persistent=False, warp64=False, per_launch=20000):
+def count_launches_single(stats, precision, k=50, R=1000, persistent=False, warp64=False, per_launch=20000,
+                          own_u=False):
     """Kernels of ours per single-instance step: precompute (3) + solve + objective read (1).
-    FP64 iterations: the warp engine (one launch) for small instances, else the
-    persistent engine (one launch per 20000 iterations); whole-grid kernels
-    (k + 1 per chunk of k) only where neither holds the instance."""
+    FP64 iterations: one launch for small instances, else the persistent grid
+    engine (one launch per 20000 iterations); whole-grid kernels (k + 1 per
+    chunk of k) only where neither holds the instance.  own_u: the engine forms
+    u = rho x_s - lambda itself (the persistent engine in both its forms), so
+    no kernel does before each of its launches."""
     n = 3 + 1
+    u = 0 if own_u else 1
 
     def fp64(iters):
         if warp64:
-            return 1 + 1
-        return 1 + (-(-iters // per_launch) if persistent else (iters // k) * (k + 1))
+            return u + 1
+        return u + (-(-iters // per_launch) if persistent else (iters // k) * (k + 1))
     if precision == "fp64":
         return n + fp64(stats["main_iters"])
     main, pol = stats["main_iters"], stats["polish_iters"]
     bodies = -(-main // R)
-    return n + 8 + bodies * 7 + 1 + fp64(pol)
+    return n + 7 + u + bodies * (6 + u) + 1 + fp64(pol)
 
 
 def count_launches_batch(t):
@@ -582,8 +585,8 @@ def plain_fp64_reference(opf, f, device, stream, n=2):
                          "peak_source": "measured in this run: FP64 FMA probe (opf_probe_dfma)",
                          "note": "latency-bound: one instance's iteration is a chain of small dependent "
                                  "products and a grid barrier"},
-            "path": "single instance, FP64 iterations on the engine opf_solve_ex picks (warp engine up to 64 "
-                    "subsystems, else the persistent grid engine)"}
+            "path": "single instance, FP64 iterations on the engine opf_solve_ex picks (the persistent engine, in "
+                    "one cluster up to 64 subsystems, else on the grid)"}
 
 
 def run_batch(args, rank, world, local):
@@ -812,7 +815,7 @@ def run_single(args, rank, world, local):
         it_main += st["main_iters"]
         it_pol += st["polish_iters"]
         launches += count_launches_single(st, args.precision, persistent=not warp_engine_fp64(sizes),
-                                          warp64=warp_engine_fp64(sizes))
+                                          warp64=warp_engine_fp64(sizes), own_u=True)
         if not ok:
             raise SystemExit("a timed solve did not converge")
     torch.cuda.synchronize()
@@ -844,20 +847,13 @@ def run_single(args, rank, world, local):
     peak, peak_kind = measured_peak()
     mixed = args.precision == "mixed"
     big = sizes["n_slots"] > 4096
-    if mixed and not big:
-        kern, traffic = ("k_warp_engine<float> (FP32 iterations; one warp per subsystem, factors in registers, "
-                         "instance resident in one thread-block cluster)"), WARP_ENGINE_TRAFFIC_PER_LAUNCH
-    elif big:
-        kern = ("k_persist_engine<%s> (%s iterations; cooperative launch over two CTAs per SM, instance "
-                "resident in their shared memory, one grid barrier per iteration)"
-                % (("float", "FP32") if mixed else ("double", "FP64")))
-        traffic = PERSIST_ENGINE_TRAFFIC_PER_LAUNCH if mixed else None
-    elif warp_engine_fp64(sizes):
-        kern, traffic = ("k_warp_engine<double> (FP64 iterations; one warp per subsystem, factors in shared "
-                         "memory, instance resident in one thread-block cluster)"), None
-    else:
-        kern, traffic = ("k_persist_engine<double> (FP64 iterations; cooperative launch, instance resident in "
-                         "the CTAs' shared memory, one grid barrier per iteration)"), None
+    one = ("k_persist_local<%s> (%s iterations; instance resident in one thread-block cluster, u stamped with its "
+           "iteration in the readers' shared memory)")
+    grid = ("k_persist_local<%s> (%s iterations; cooperative launch, instance resident in the CTAs' shared memory, "
+            "u stamped with its iteration in L2, no barrier between iterations)")
+    kern = (one if (mixed and not big) or (not mixed and warp_engine_fp64(sizes)) else grid) % (
+        ("float", "FP32") if mixed else ("double", "FP64"))
+    traffic = None          # the captures in profiles/ are of the kernels before these
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak,
             "traffic": traffic,

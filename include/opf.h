@@ -127,7 +127,8 @@ typedef struct opf_solve_opts {
                                            of at most 32 slots in registers, FP64 factors in
                                            shared memory),
                                        4 = persistent grid (cooperative launch, instance resident in
-                                       the shared memory of all CTAs, one grid barrier per iteration) */
+                                       the shared memory of all CTAs, u exchanged between them through
+                                       L2 with its iteration's number) */
     int32_t flags;                  /* OPF_SOLVE_* bits */
     int32_t cluster;                /* engine 2: CTAs per cluster (1, 2, 4, 8, 16; 0 = automatic);
                                        engine 3: CTAs of the cluster (1 .. 16, at most 12
@@ -189,12 +190,15 @@ int opf_solve(opf_handle *h, double rho, double eps, int32_t max_iter);
 
 /* Same with every option (NULL = defaults: rho 100, eps_rel 1e-8,
  * eps_abs_pres 1e-4, max_iter 1e6, check_every 50, FP64).  Automatic engine
- * choice: FP32 / mixed iterations on the warp engine, else the cluster
- * engine, else the persistent grid engine, else whole-grid kernels; FP64
- * iterations (and the polish) on the warp engine when the instance fits it
- * with at most 4 warps per CTA (at most 64 subsystems), else on the
- * persistent grid engine when its plan fits, else whole-grid kernels.  The persistent engine's grid
- * barrier waits at most 1 s; past that the solve returns OPF_E_TIMEOUT. */
+ * choice: instances that the warp engine can hold (FP64 with at most 4 warps
+ * per CTA: at most 64 subsystems) run on the persistent engine's one-cluster
+ * form (the instance in one cluster of at most 16 CTAs, u written straight into
+ * the readers' shared memory).  FP32 / mixed iterations of others: the
+ * persistent grid engine when most copies of its parts' globals are their own,
+ * else the cluster engine, else the persistent grid engine, else whole-grid
+ * kernels; FP64 iterations (and the polish) of others: the persistent grid
+ * engine when its plan fits, else whole-grid kernels.  The persistent engine's
+ * waits last at most 1 s each; past that the solve returns OPF_E_TIMEOUT. */
 int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts);
 
 /* Exactly n_iters FP64 iterations with penalty rho, no stopping test. */

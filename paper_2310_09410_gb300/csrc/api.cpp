@@ -52,7 +52,7 @@ int launch_cluster_engine(const IterArgs<T> &g, const ClusterLayout &lay, const 
                           cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
 template <typename T> int cluster_occupancy(const ClusterLayout &lay);
 template <typename T> int prepare_persist_engine(const PersistLayout &lay);
-template <typename T> int persist_occupancy(const PersistLayout &lay);
+template <typename T> long long persist_resident(const PersistLayout &lay, int n_sm);
 template <typename T> size_t persist_exchange_bytes(int L);
 template <typename T>
 int launch_persist_engine(const IterArgs<T> &g, const PersistLayout &lay, const PersistPtrs &pp, T *U,
@@ -247,6 +247,7 @@ static int build_layout(opf_handle *h) {
     for (int i = 0; i < h->G; ++i) gseg[i] = make_int2(gstart[i], cnt[i]);
     for (int k = 0; k < h->L; ++k) segp[k] = (gstart[gk[k]] << 8) | cnt[gk[k]];
     h->h_pk = pk;
+    h->h_segp = segp;
     h->h_gk = gk;
     h->h_gstart = gstart;
     h->h_uslot = uslot;
@@ -302,7 +303,7 @@ static int build_layout(opf_handle *h) {
     TRY(dalloc(h, &h->w32.d_fbig, h->S + 1));
     TRY(dalloc(h, &h->w32.d_F2, h->nF));
     for (PersistPlan *pp : {&h->p32, &h->p64}) {
-        TRY(dalloc(h, &pp->d_part, 6 * kPersistMaxP));
+        TRY(dalloc(h, &pp->d_part, 24 * kPersistMaxP));
         TRY(dalloc(h, &pp->d_sync, 1));
     }
     for (ClusterPlan *cp : {&h->c32, &h->c64}) {
@@ -506,10 +507,11 @@ extern "C" int opf_precompute(opf_handle *h) {
         CUDA_TRY(cudaStreamSynchronize(h->stream));      // the uploads read local vectors
         h->c32.P = h->c64.P = 0;
         h->c32.ok = h->c64.ok = false;
-        h->p32.P = h->p64.P = 0;
-        h->p32.ok = h->p64.ok = h->p32.tried = h->p64.tried = false;
-        h->p32.tab.reset();
-        h->p64.tab.reset();
+        for (PersistPlan *pp : {&h->p32, &h->p64, &h->k32, &h->k64}) {
+            pp->P = 0;
+            pp->ok = pp->tried = false;
+            pp->tab.reset();
+        }
         h->g64.reset();
         h->gmix.reset();
         h->have_layout = true;
@@ -734,9 +736,33 @@ static int get_cluster_plan(opf_handle *h, ClusterPlan *cp, int requested, int t
     return OPF_OK;
 }
 
+constexpr int kWarpEngineWarps = 12;
+// Warps per CTA when the cluster has room: one per SM sub-partition, so that
+// the largest subsystems' warps do not share an FP64 pipe (FP64 iterations)
+// or an issue slot (FP32: 5 % faster than 12 warps on the 13- and 34-bus feeders)
+constexpr int kWarpEngineWarps64 = 4;
+
+// Warps per subsystem in the warp engine: the largest are split over two while
+// the warps stay within 4 per CTA of the cluster (16 CTAs, or req_P): in FP64
+// those of more than 16 slots; in FP32 those of more than 32 (the ones whose
+// factor is in shared memory), up to 12 warps per CTA.
+static std::vector<int> warp_parts(const opf_handle *h, bool fp32, int req_P) {
+    const int S = h->S, min_n = fp32 ? 32 : 16;
+    std::vector<int> nparts(S, 1), big_first;
+    for (int s = 0; s < S; ++s)
+        if (h->h_sn[s] > min_n) big_first.push_back(s);
+    std::stable_sort(big_first.begin(), big_first.end(), [&](int x, int y) {
+        return h->h_sn[x] * (h->h_sf[x] + 4) > h->h_sn[y] * (h->h_sf[y] + 4);
+    });
+    const int per_cta = fp32 ? kWarpEngineWarps : kWarpEngineWarps64;
+    const int budget = (req_P > 0 ? req_P : 16) * per_cta - S;
+    for (int i = 0; i < (int)big_first.size() && i < budget; ++i) nparts[big_first[i]] = 2;
+    return nparts;
+}
+
 // The partition of the instance over P CTAs: parts of a depth-first order for
-// the local form, else runs of the size-sorted order.
-static int build_persist_tables(opf_handle *h, int P, bool local, std::shared_ptr<PersistTables> *out) {
+// the local forms, else runs of the size-sorted order.
+static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, std::shared_ptr<PersistTables> *out) {
     const int S = h->S, L = h->L;
     std::vector<double> cost(S);
     for (int s = 0; s < S; ++s)
@@ -746,17 +772,25 @@ static int build_persist_tables(opf_handle *h, int P, bool local, std::shared_pt
         if (h->persist_order.empty()) {
             std::vector<int> start(S);           // new trees begin in canonical order
             for (int d = 0; d < S; ++d) start[h->dev_to_canon_sub[d]] = d;
-            h->persist_order = persist_order(S, h->h_soff, h->h_gk, h->h_gstart, h->h_uslot, start);
+            h->persist_order = persist_order(S, h->h_soff, h->h_segp, h->h_pk, start);
         }
         order = h->persist_order;
     } else {
         order.resize(S);
         std::iota(order.begin(), order.end(), 0);
     }
-    const PersistParts parts = persist_parts(P, S, order, cost, h->h_soff, h->h_gk, h->h_pk, h->h_gstart, h->h_uslot);
+    const PersistParts parts = persist_parts(P, S, order, cost, h->h_soff, h->h_segp, h->h_pk);
     auto t = std::make_shared<PersistTables>();
     t->P = P; t->S = S; t->L = L;
     t->local = local;
+    t->cluster = cluster;
+    t->fits = parts.ok;
+    t->remote = (long long)parts.rem.size();
+    // cluster form: a subsystem whose FP32 column products go by halves (in the
+    // order of the warp engine's two warps) has its second half start at a
+    // multiple of 4 rows, for 16-byte loads
+    std::vector<int> two = cluster ? warp_parts(h, true, 0) : std::vector<int>(S, 1);
+    std::vector<int> halves(S, 0);
     const int P1 = P + 1;
     std::vector<int> pr(7 * P1, 0), items, meta;
     auto PR = [&](int field, int p) -> int & { return pr[field * P1 + p]; };
@@ -766,16 +800,30 @@ static int build_persist_tables(opf_handle *h, int P, bool local, std::shared_pt
     items.reserve(h->nitems);
     for (int p = 0; p < P; ++p) {
         const int s0 = parts.s0[p];
-        long long f = 0, v = 0, c0 = 0;
+        long long f = 0, v = 0, c0 = 0, j = 0, nbig = 0;
+        int nmax = 0, fmax = 0;
         for (int i = s0; i < parts.s0[p + 1]; ++i) {
-            const int d = parts.sub[i], npad = h->h_npad[d], cs = npad + ((npad & 7) == 0 ? 4 : 0);
+            const int d = parts.sub[i], n = h->h_sn[d], hn = two[d] == 2 ? (n + 1) / 2 : 0;
+            const int gap = round4(hn) - hn, npad = hn ? round4(hn) + round4(n - hn) : h->h_npad[d];
+            const int cs = npad + ((npad & 7) == 0 ? 4 : 0), fp = local ? round4(h->h_sf[d]) : h->h_sf[d];
+            halves[i] = hn;
             srec[i] = make_int4((int)f, (int)v, (int)c0, (h->h_sf[d] << 10) | (npad << 1) | (h->h_mode[d] & 1));
             for (int c = 0; c < h->h_sf[d]; ++c) items.push_back(((i - s0) << 8) | c);
-            for (int r = 0; r < h->h_sn[d]; ++r) meta.push_back(((i - s0) << 8) | r);
-            f += (long long)h->h_sf[d] * cs;
+            for (int r = 0; r < n; ++r) meta.push_back(((i - s0) << 8) | (hn && r >= hn ? r + gap : r));
+            f += (long long)fp * cs;
             v += npad;
-            c0 += h->h_sf[d];
+            c0 += fp;
+            j += h->h_sf[d];
+            if (n > 32) nbig = j;
+            nmax = std::max(nmax, n);
+            fmax = std::max(fmax, h->h_sf[d]);
         }
+        t->nj.push_back((int)j);
+        t->nk.push_back(parts.k0[p + 1] - parts.k0[p]);
+        t->nmax.push_back(nmax);
+        t->fmax.push_back(fmax);
+        t->rows32 = t->rows32 && fmax <= 32;
+        t->mpair = std::max(t->mpair, ((2 * nbig + 31) & ~31LL) + j - nbig);
         PR(0, p + 1) = parts.k0[p + 1];
         PR(1, p + 1) = parts.s0[p + 1];
         PR(2, p + 1) = (int)items.size();
@@ -784,30 +832,38 @@ static int build_persist_tables(opf_handle *h, int P, bool local, std::shared_pt
         PR(6, p + 1) = parts.l0[p + 1];
         t->mf = std::max(t->mf, f);
         t->mv = std::max(t->mv, v);
-        t->mj = std::max(t->mj, c0);
+        t->mj = std::max(t->mj, j);
+        t->mt = std::max(t->mt, c0);
         t->mk = std::max<long long>(t->mk, parts.k0[p + 1] - parts.k0[p]);
         t->ms = std::max<long long>(t->ms, parts.s0[p + 1] - s0);
         t->mr = std::max<long long>(t->mr, parts.r0[p + 1] - parts.r0[p]);
         t->ml = std::max<long long>(t->ml, parts.l0[p + 1] - parts.l0[p]);
     }
-    // one allocation and one upload
-    std::vector<int> all(4 * (size_t)S);
-    memcpy(all.data(), srec.data(), 4 * (size_t)S * sizeof(int));
-    std::vector<std::pair<int **, size_t>> at;
-    auto add = [&](int **p, const std::vector<int> &v) {
-        at.push_back({p, all.size()});
-        all.insert(all.end(), v.begin(), v.end());
+    // one allocation and one upload, every array from a multiple of 16 bytes
+    std::vector<int> all;
+    std::vector<std::pair<void **, size_t>> at;
+    auto add = [&](void *slot, const void *data, size_t bytes) {
+        at.push_back({(void **)slot, all.size()});
+        const size_t n = (bytes + 15) / 16 * 4, o = all.size();
+        all.resize(o + n, 0);
+        if (bytes) memcpy(all.data() + o, data, bytes);
     };
-    add(&t->pr, pr); add(&t->items, items); add(&t->meta, meta);
-    add(&t->sub, parts.sub);
+    auto addv = [&](int **slot, const std::vector<int> &v) { add(slot, v.data(), v.size() * sizeof(int)); };
+    add(&t->srec, srec.data(), srec.size() * sizeof(int4));
+    addv(&t->pr, pr); addv(&t->items, items); addv(&t->meta, meta); addv(&t->sub, parts.sub);
     if (local) {
-        add(&t->slot, parts.slot); add(&t->seg, parts.seg); add(&t->out, parts.out);
-        add(&t->list, parts.list); add(&t->rem, parts.rem);
+        addv(&t->slot, parts.slot); addv(&t->seg, parts.seg); addv(&t->out, parts.out); addv(&t->rem, parts.rem);
+        add(&t->list, parts.list.data(), parts.list.size() * sizeof(unsigned short));
+    }
+    if (cluster) {
+        const PersistDests d = persist_dests(P, parts, h->h_uslot);
+        t->fits = t->fits && d.ok;
+        t->md = d.most;
+        addv(&t->dst, d.dst); addv(&t->dr, d.d0); addv(&t->dseg, d.dseg); addv(&t->halves, halves);
     }
     void *q = nullptr;
-    CUDA_TRY(cudaMalloc(&q, std::max<size_t>(all.size(), 1) * sizeof(int)));
+    CUDA_TRY(cudaMalloc(&q, std::max<size_t>(all.size(), 4) * sizeof(int)));
     t->mem = (int *)q;
-    t->srec = (int4 *)q;
     for (auto &e : at) *e.first = t->mem + e.second;
     CUDA_TRY(cudaMemcpyAsync(t->mem, all.data(), all.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
@@ -820,37 +876,75 @@ static int build_persist_tables(opf_handle *h, int P, bool local, std::shared_pt
 // (local form: also when it has more slots or columns than threads) or P CTAs
 // cannot be resident.
 template <typename T>
-static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local) {
+static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local, bool cluster) {
     pp->ok = false;
     pp->P = P;
     if (P < 1 || P > kPersistMaxP) return OPF_OK;
-    PersistPlan &other = pp == &h->p32 ? h->p64 : h->p32;
-    if (other.tab && other.tab->P == P && other.tab->local == local) pp->tab = other.tab;
-    else if (!pp->tab || pp->tab->P != P || pp->tab->local != local) TRY(build_persist_tables(h, P, local, &pp->tab));
+    PersistPlan &other = pp == &h->p32 ? h->p64 : pp == &h->p64 ? h->p32 : pp == &h->k32 ? h->k64 : h->k32;
+    auto same = [&](const std::shared_ptr<PersistTables> &t) {
+        return t && t->P == P && t->local == local && t->cluster == cluster;
+    };
+    if (!same(pp->tab)) {
+        if (same(other.tab)) pp->tab = other.tab;
+        else TRY(build_persist_tables(h, P, local, cluster, &pp->tab));
+    }
     const PersistTables &t = *pp->tab;
     PersistLayout &c = pp->lay;
     c = PersistLayout{};
     c.P = P;
     c.L = h->L;
     c.local = local ? 1 : 0;
+    c.cluster = cluster ? 1 : 0;
+    c.tcap = (int)t.mt;
     c.threads = (int)std::min<long long>(kPersistMaxThreads,
                                          std::max<long long>(64, (std::max(t.mk, t.mj) + 31) / 32 * 32));
-    if (local && (std::max(t.mk, t.mj) > c.threads || t.mk + t.mr > 0xffff)) return OPF_OK;
-    // plans of small CTAs (one or a few subsystems each: the 123-bus feeder)
-    // run phase B with each factor column on 4 lanes, given threads for it;
-    // large ones keep one lane per column (the split measured slower there)
-    if (local && c.threads <= 128) {
+    if (local && (std::max(t.mk, t.mj) > c.threads || !t.fits)) return OPF_OK;
+    // a thread per remote entry, two when that takes more threads than it has
+    if (local && !cluster)
+        c.threads = (int)std::max<long long>(c.threads, std::min<long long>(kPersistMaxThreads, (t.mr + 31) / 32 * 32));
+    if (cluster && sizeof(T) == 4) {
+        if (!t.rows32 || t.mpair > kPersistMaxThreads) return OPF_OK;
+        c.threads = (int)std::max<long long>(c.threads, (t.mpair + 31) / 32 * 32);
+    }
+    // FP64, small CTAs: lanes per column and per row that give the slowest
+    // CTA's sub-partitions the fewest FP64 instructions, about 64 cycles each
+    // (a column of n rows: n / lanes + log2 lanes; a row of f columns: its
+    // global update, f / lanes + log2 lanes, the dual update; once for every
+    // 128 threads, 4 warps)
+    if (local && sizeof(T) == 8 && std::max(t.mk, t.mj) <= 256) {
+        auto pick = [&](const std::vector<int> &items, const std::vector<int> &longest, int most, int fixed) {
+            int best = 1;
+            long long cost = -1;
+            for (int l = 1, lg = 0; l <= most; l *= 2, ++lg) {
+                long long worst = 0;
+                bool fit = true;
+                for (int p = 0; p < P; ++p) {
+                    const long long thr = (long long)l * items[p];
+                    if (thr > kPersistMaxThreads) fit = false;
+                    worst = std::max(worst, (thr + 127) / 128 * (fixed + (longest[p] + l - 1) / l + lg));
+                }
+                if (fit && (cost < 0 || worst < cost)) { cost = worst; best = l; }
+            }
+            return best;
+        };
         c.split = 1;
-        c.threads = (int)std::max<long long>(c.threads, (4 * t.mj + 31) / 32 * 32);
+        c.clanes = pick(t.nj, t.nmax, 8, 0);
+        c.rlanes = pick(t.nk, t.fmax, 4, 8);
+        c.threads = (int)std::max<long long>(c.threads, (std::max(c.clanes * t.mj, c.rlanes * t.mk) + 31) / 32 * 32);
     }
     size_t off = 0;
     auto take = [&](unsigned *o, size_t bytes) { *o = (unsigned)off; off = align16u(off + bytes); };
     take(&c.off_F, (size_t)t.mf * sizeof(T));
     take(&c.off_srec, (size_t)t.ms * sizeof(int4));
     if (local) {
-        take(&c.off_list, (size_t)t.ml * sizeof(int));
-        take(&c.off_rem, (size_t)t.mr * sizeof(int));
-        take(&c.off_ul, (size_t)(t.mk + t.mr) * sizeof(T));
+        take(&c.off_list, (size_t)t.ml * sizeof(uint4));
+        take(&c.off_rem, (size_t)(cluster ? t.md : t.mr) * sizeof(int));
+        if (cluster) {
+            c.xcap = (int)std::max<long long>(t.mr, 1);
+            take(&c.off_xw, (size_t)2 * c.xcap * (sizeof(T) == 4 ? 8 : 16));
+            take(&c.off_tw, (size_t)12 * P * 16);
+        }
+        take(&c.off_ul, (size_t)(t.mk + t.mr + 1) * sizeof(T));
     } else {
         take(&c.off_items, (size_t)t.mj * sizeof(int));
         take(&c.off_slots, (size_t)t.mk * persist_slot_bytes(sizeof(T)));
@@ -858,26 +952,32 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
         take(&c.off_rn, 256 * sizeof(T));
     }
     take(&c.off_vb, (size_t)t.mv * sizeof(T));
-    take(&c.off_tb, (size_t)t.mj * sizeof(T));
+    take(&c.off_tb, (size_t)t.mt * sizeof(T));
     take(&c.off_xrs, (size_t)t.mk * sizeof(double));
     take(&c.off_lrs, (size_t)t.mk * sizeof(double));
     take(&c.off_cobj, (size_t)t.mk * sizeof(double));
-    // flags (16 B), a DevStatus copy, the [32][6] block-sum scratch
-    take(&c.off_misc, 16 + ((sizeof(DevStatus) + 15) & ~(size_t)15) + 32 * 6 * sizeof(double));
+    // flags (16 B), a DevStatus copy, the test's sums (48 B), per warp (16 warps)
+    take(&c.off_misc, 64 + ((sizeof(DevStatus) + 15) & ~(size_t)15) + kPersistMaxThreads / 32 * 6 * sizeof(double));
     c.bytes = (unsigned)off;
     int optin = 0;
     CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     if ((long long)off > optin) return OPF_OK;
     if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
-    const int occ = persist_occupancy<T>(c);
-    if ((long long)occ * n_sm < P) { cudaGetLastError(); return OPF_OK; }
-    if (!pp->d_xu) TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(h->L) / sizeof(unsigned long long)));
+    if (persist_resident<T>(c, n_sm) < P) { cudaGetLastError(); return OPF_OK; }
+    if (!cluster && !pp->d_xu) TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(h->L) / sizeof(unsigned long long)));
     pp->ok = true;
     return OPF_OK;
 }
 
+// More than 4 copies per global on average (feeders have 1.5 to 1.8; consensus
+// instances of overlapping blocks more): parts then read mostly other parts'
+// entries.
+static bool many_copies(const opf_handle *h) { return (long long)h->L > 4LL * h->G; }
+
 // CTA count: the requested one, else two per SM of the stream's SMs (one per
-// SM when two do not fit), at most one CTA per 32 slots.
+// SM when two do not fit, or with many copies per global: 240 blocks over 900
+// globals, 14 copies each, FP64 14.8 us per iteration on 304 CTAs, 8.7 on
+// 152), at most one CTA per 32 slots.
 template <typename T>
 static int get_persist_plan(opf_handle *h, PersistPlan *pp, int requested) {
     if (pp->tried && pp->req == requested) return OPF_OK;
@@ -885,17 +985,39 @@ static int get_persist_plan(opf_handle *h, PersistPlan *pp, int requested) {
     pp->tried = true;
     pp->req = requested;
     auto build = [&](int P) -> int {
-        TRY(build_persist_plan<T>(h, pp, P, n_sm, true));
-        if (!pp->ok) TRY(build_persist_plan<T>(h, pp, P, n_sm, false));
+        TRY(build_persist_plan<T>(h, pp, P, n_sm, true, false));
+        if (!pp->ok) TRY(build_persist_plan<T>(h, pp, P, n_sm, false, false));
         return OPF_OK;
     };
+
     if (requested > 0) return build(requested);
     const int cap = std::max(1, (h->L + 31) / 32);
     for (int per : {2, 1}) {
+        if (per == 2 && many_copies(h)) continue;
         TRY(build(std::min(per * n_sm, cap)));
         if (pp->ok) return OPF_OK;
     }
     return OPF_OK;
+}
+
+// Plan of the one-cluster form for instances that the warp engine can hold:
+// CTAs by size, at most 16.  FP32 one per 80 slots (13 buses, 271 slots: 1 /
+// 4 / 8 CTAs 1.02 / 0.92 / 1.10 us per iteration; 34 buses, 620 slots: 2 / 8 /
+// 16 CTAs 1.12 / 1.00 / 1.08; 123 buses, 2665 slots: 8 / 16 CTAs 1.28 / 1.11);
+// FP64 one per 24 slots, at most 12 (13 buses: 4 / 8 / 12 CTAs 2.48 / 1.99 /
+// 1.98; 34 buses: 4 / 8 / 12 CTAs 2.74 / 2.24 / 2.31).
+template <typename T>
+static int get_one_cluster_plan(opf_handle *h, PersistPlan *pp) {
+    if (pp->tried) return OPF_OK;
+    pp->tried = true;
+    if (h->max_ns > 64) return OPF_OK;
+    for (int f : h->h_sf)
+        if (f > 32) return OPF_OK;
+    int warps = 0;
+    for (int n : warp_parts(h, sizeof(T) == 4, 0)) warps += n;
+    if (warps > 16 * (sizeof(T) == 4 ? kWarpEngineWarps : kWarpEngineWarps64)) return OPF_OK;
+    const int per = sizeof(T) == 4 ? 80 : 24, most = sizeof(T) == 4 ? 16 : 12;
+    return build_persist_plan<T>(h, pp, std::min(most, (h->L + per - 1) / per), 0, true, true);
 }
 
 template <typename T>
@@ -903,12 +1025,6 @@ static IterArgs<T> with_persist(IterArgs<T> a, const PersistPlan &pp) {
     a.srec = pp.tab->srec; a.citems = pp.tab->items; a.cmeta = pp.tab->meta;
     return a;
 }
-
-constexpr int kWarpEngineWarps = 12;
-// Warps per CTA when the cluster has room: one per SM sub-partition, so that
-// the largest subsystems' warps do not share an FP64 pipe (FP64 iterations)
-// or an issue slot (FP32: 5 % faster than 12 warps on the 13- and 34-bus feeders)
-constexpr int kWarpEngineWarps64 = 4;
 
 // Warp-engine plan for precision T.  Work items are warps: one per subsystem,
 // or in FP64 two for the largest subsystems of more than 16 slots, as many as
@@ -929,23 +1045,7 @@ static int build_warp_plan(opf_handle *h, WarpPlan &wp, int req_P) {
     if (h->max_ns > 64) return OPF_OK;
     for (int s = 0; s < S; ++s)
         if (h->h_sf[s] > 32) return OPF_OK;
-    // split the largest subsystems over two warps while the warps stay within
-    // 4 per CTA of the cluster (16 CTAs, or req_P): in FP64 those of more than
-    // 16 slots; in FP32 those of more than 32 (the ones whose factor is in
-    // shared memory), up to 12 warps per CTA
-    std::vector<int> nparts(S, 1);
-    {
-        const int min_n = REG ? 32 : 16;
-        std::vector<int> big_first;
-        for (int s = 0; s < S; ++s)
-            if (h->h_sn[s] > min_n) big_first.push_back(s);
-        std::stable_sort(big_first.begin(), big_first.end(), [&](int x, int y) {
-            return h->h_sn[x] * (h->h_sf[x] + 4) > h->h_sn[y] * (h->h_sf[y] + 4);
-        });
-        const int per_cta = REG ? kWarpEngineWarps : kWarpEngineWarps64;
-        const int budget = (req_P > 0 ? req_P : 16) * per_cta - S;
-        for (int i = 0; i < (int)big_first.size() && i < budget; ++i) nparts[big_first[i]] = 2;
-    }
+    const std::vector<int> nparts = warp_parts(h, REG, req_P);
     int W = 0;
     for (int s = 0; s < S; ++s) W += nparts[s];
     int P = (W + kWarpEngineWarps - 1) / kWarpEngineWarps;
@@ -1288,10 +1388,9 @@ static int fault_error(opf_handle *h) {
 }
 
 // FP64 iterations by the persistent grid engine until the test or max_iter.
-static int run_persist64(opf_handle *h, const opf_solve_opts &o) {
+static int run_persist64(opf_handle *h, const opf_solve_opts &o, const PersistPlan &pp) {
     const double rho = o.rho;
     TRY(set_recip(h, rho));
-    const PersistPlan &pp = h->p64;
     IterArgs<double> a = with_persist(iter_args<double>(h, rho), pp);
     const int k = o.check_every;
     const int per = std::max(k, (kPersistLaunchIters / k) * k);
@@ -1328,16 +1427,18 @@ static int run_warp64(opf_handle *h, const opf_solve_opts &o) {
     return OPF_OK;
 }
 
-// FP64 iterations on the engine chosen for the solve: 4 persistent grid,
-// 3 warp engine, else whole-grid kernels.
+// FP64 iterations on the engine chosen for the solve: 5 the persistent engine's
+// one-cluster form, 4 persistent grid, 3 warp engine, else whole-grid kernels.
 static int run_fp64(opf_handle *h, const opf_solve_opts &o, int e64) {
-    if (e64 == 4 && h->p64.ok) return run_persist64(h, o);
+    if (e64 == 5 && h->k64.ok) return run_persist64(h, o, h->k64);
+    if (e64 == 4 && h->p64.ok) return run_persist64(h, o, h->p64);
     if (e64 == 3 && h->w64.ok) return run_warp64(h, o);
     return run_grid64(h, o);
 }
 
 // FP32 iterations in the shifted frame, re-centred in FP64 every R iterations.
-// eng: 1 whole-grid kernels, 2 cluster engine, 3 warp engine, 4 persistent grid
+// eng: 1 whole-grid kernels, 2 cluster engine, 3 warp engine, 4 persistent
+// grid, 5 its one-cluster form
 static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recenter) {
     const double rho = o.rho;
     TRY(set_recip(h, rho));
@@ -1356,18 +1457,19 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                            h->d_ubt32, h->d_sub, h->d_sub2, h->d_F64, h->d_bbar64, rho, h->d_bt32,
                            nullptr, h->stream);
     // (the persistent engine forms u itself)
-    if (eng != 4) launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, nullptr, h->stream);
+    if (eng < 4) launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, nullptr, h->stream);
     CUDA_TRY(cudaGetLastError());
 
     const int kind = eng + (recenter ? 0 : 8);
     bool hl = (o.flags & OPF_SOLVE_HOST_LOOP) != 0 || (eng == 4 && h->persist_graph_failed);
     IterArgs<float> a = eng == 3   ? with_warp_plan(h, iter_args<float>(h, rho), h->w32)
                         : eng == 4 ? with_persist(iter_args<float>(h, rho), h->p32)
+                        : eng == 5 ? with_persist(iter_args<float>(h, rho), h->k32)
                                    : with_plan(iter_args<float>(h, rho), h->c32);
     int launch_rc = 0;
     auto body = [&](cudaGraphConditionalHandle c, int use) {
-            if (eng == 4) {
-                const PersistPlan &pp = h->p32;
+            if (eng >= 4) {
+                const PersistPlan &pp = eng == 4 ? h->p32 : h->k32;
                 launch_rc |= launch_persist_engine<float>(a, pp.lay, pp.ptrs(), h->d_u32, bar_extra(o), R, k,
                                                           h->d_st, rho, c, use, h->stream);
             } else if (eng == 3) {
@@ -1388,10 +1490,15 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                                    h->d_lbt32, h->d_ubt32, h->d_sub, h->d_sub2, h->d_F64, h->d_bbar64, rho,
                                    h->d_bt32, h->d_st, h->stream);
             launch_copy_if_running(G, h->d_xr2, h->d_xr, h->d_st, h->stream);
-            if (eng != 4)
+            if (eng < 4)
                 launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, h->d_st, h->stream);
     };
-    const int planP = eng == 4 ? 10000 + h->p32.P : eng == 3 ? 100 + h->w32.P : eng == 2 ? h->c32.P : 0;
+    // (the test hook of the bounded waits is an argument of the captured launch)
+    const int planP = (eng == 5   ? 20000 + h->k32.P
+                       : eng == 4 ? 10000 + h->p32.P
+                       : eng == 3 ? 100 + h->w32.P
+                       : eng == 2 ? h->c32.P
+                                  : 0) + 1000000 * bar_extra(o);
     if (h->gmix.kind != kind || h->gmix.rho != rho || h->gmix.k != k || h->gmix.R != R ||
         h->gmix.host_loop != hl || h->gmix.P != planP) {
         int rc = build_while_graph(h, &h->gmix, body, hl);
@@ -1451,24 +1558,29 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
     h->last_rho = o.rho;
     TRY(set_status(h, o, false));
     CUDA_TRY(cudaEventRecord(h->ev[1], h->stream));
-    // FP64 iterations (plain solves and the polish): on the warp engine when
-    // asked for, or automatically when the instance fits one cluster of it
-    // with at most 4 warps per CTA (with more, the warps of an SM queue on its
-    // FP64 pipe); else on the persistent grid engine when asked for, or
-    // automatically when its plan fits (123 buses: 5.5 us per iteration
-    // against 7.3 us for whole-grid kernels); else whole-grid kernels
-    bool w64 = false, p64 = false;
-    if (o.precision != OPF_PREC_FP32 && (o.engine == 0 || o.engine == 3)) {
+    // FP64 iterations (plain solves and the polish).  Automatic: instances the
+    // warp engine would hold with at most 4 warps per CTA (with more, the warps
+    // of an SM queue on its FP64 pipe) on the persistent engine's one-cluster
+    // form (13 / 34 buses 2.00 / 2.31 us per iteration against 2.92 / 3.03 on
+    // the warp engine), else on the warp engine; others on the persistent grid
+    // engine when its plan fits, else whole-grid kernels (123 buses: 2.9
+    // against 7.3 us).
+    bool w64 = false, p64 = false, k64 = false;
+    if (o.precision != OPF_PREC_FP32 && o.engine == 0) {
+        TRY(get_one_cluster_plan<double>(h, &h->k64));
+        k64 = h->k64.ok;
+    }
+    if (o.precision != OPF_PREC_FP32 && !k64 && (o.engine == 0 || o.engine == 3)) {
         const int req = o.engine == 3 ? o.cluster : 0;
         if (!h->w64.built || h->w64.req != req) TRY(build_warp_plan<double>(h, h->w64, req));
         w64 = h->w64.ok && (o.engine == 3 || h->w64.lay.warps <= kWarpEngineWarps64);
     }
-    if (!w64 && (o.engine == 4 || (o.engine == 0 && o.precision != OPF_PREC_FP32))) {
+    if (!k64 && !w64 && (o.engine == 4 || (o.engine == 0 && o.precision != OPF_PREC_FP32))) {
         TRY(get_persist_plan<double>(h, &h->p64, o.engine == 4 ? o.cluster : 0));
         if (!h->p64.ok && o.engine == 4 && o.cluster > 0) TRY(get_persist_plan<double>(h, &h->p64, 0));
         p64 = h->p64.ok;
     }
-    const int e64 = w64 ? 3 : p64 ? 4 : 1;
+    const int e64 = k64 ? 5 : w64 ? 3 : p64 ? 4 : 1;
     if (o.precision == OPF_PREC_FP64) {
         bool cl = false;
         if (o.engine == 2) {
@@ -1488,11 +1600,27 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
         CUDA_TRY(cudaEventRecord(h->ev[2], h->stream));
         CUDA_TRY(cudaEventRecord(h->ev[3], h->stream));
     } else {
+        // FP32 iterations.  Automatic: instances the warp engine would hold on
+        // the persistent engine's one-cluster form, else on the warp engine;
+        // others on the persistent grid engine when its parts take the local
+        // form and read at most one remote entry per slot (200 / 400 / 1000
+        // buses: 2.2 / 2.6 / 2.5 us per iteration against 3.1 / 3.5 / 4.6 on the
+        // cluster engine, the same iterates bit for bit; blocks over random
+        // globals, 2.5 copies each: 3.1-3.5 against 2.7-2.9, 14 copies each: 6.9
+        // against 6.6), else the cluster engine, else the persistent grid engine.
         int eng = 1;
-        if (o.engine == 0 || o.engine == 3) {
+        if (o.engine == 0) {
+            TRY(get_one_cluster_plan<float>(h, &h->k32));
+            if (h->k32.ok) eng = 5;
+        }
+        if (eng == 1 && (o.engine == 0 || o.engine == 3)) {
             const int req = o.engine == 3 ? o.cluster : 0;
             if (!h->w32.built || h->w32.req != req) TRY(build_warp_plan<float>(h, h->w32, req));
             if (h->w32.ok) eng = 3;
+        }
+        if (eng == 1 && o.engine == 0 && !many_copies(h)) {
+            TRY(get_persist_plan<float>(h, &h->p32, 0));
+            if (h->p32.ok && h->p32.lay.local && h->p32.tab->remote <= h->L) eng = 4;
         }
         if (eng == 1 && (o.engine == 0 || o.engine == 2)) {
             TRY(get_cluster_plan<float>(h, &h->c32, o.cluster, 192));

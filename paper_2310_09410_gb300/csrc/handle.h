@@ -45,12 +45,22 @@ struct ClusterPlan {
 // device; the plans of both precisions share it while they agree on P and form.
 struct PersistTables {
     int P = 0, S = 0, L = 0;
-    bool local = false;
-    long long mf = 0, ms = 0, mj = 0, mk = 0, mv = 0, mr = 0, ml = 0;   // largest part: factor words, subsystems,
-                                                                        // columns, slots, vector rows, remote, list
+    bool local = false, cluster = false;
+    // largest part: factor words, subsystems, columns, products (columns
+    // rounded up to 4 per subsystem), slots, vector rows, remote entries,
+    // lists, destinations
+    long long mf = 0, ms = 0, mj = 0, mt = 0, mk = 0, mv = 0, mr = 0, ml = 0, md = 0;
+    // per part the columns and slots and the longest of each (FP64 lane splits);
+    // most threads of the FP32 cluster form's columns; its factors fit registers
+    std::vector<int> nj, nk, nmax, fmax;
+    long long mpair = 0, remote = 0;     // remote: entries read from other parts, over all parts
+    bool rows32 = true;
+    bool fits = true;            // indices and counts fit their fields
     int *mem = nullptr;          // one allocation: the arrays below
     int *pr = nullptr, *items = nullptr, *meta = nullptr;   // ranges, 7 x (P + 1); per column; per slot
-    int *sub = nullptr, *slot = nullptr, *seg = nullptr, *out = nullptr, *list = nullptr, *rem = nullptr;
+    int *sub = nullptr, *slot = nullptr, *seg = nullptr, *out = nullptr, *rem = nullptr;
+    uint4 *list = nullptr;
+    int *dst = nullptr, *dr = nullptr, *dseg = nullptr, *halves = nullptr;
     int4 *srec = nullptr;
     PersistTables() = default;
     PersistTables(const PersistTables &) = delete;
@@ -68,11 +78,12 @@ struct PersistPlan {
     int req = 0;                 // requested CTA count of that build (0: automatic)
     PersistLayout lay{};
     std::shared_ptr<PersistTables> tab;
-    double *d_part = nullptr;    // 6 * kPersistMaxP
+    unsigned long long *d_part = nullptr;   // 24 * kPersistMaxP
     unsigned long long *d_sync = nullptr;
     unsigned long long *d_xu = nullptr;   // exchange buffer, allocated with the first plan that fits
     PersistPtrs ptrs() const {
-        return PersistPtrs{tab->pr, d_part, d_sync, d_xu, tab->sub, tab->slot, tab->seg, tab->out, tab->list, tab->rem};
+        return PersistPtrs{tab->pr, d_part, d_sync, d_xu, tab->sub, tab->slot, tab->seg, tab->out, tab->rem, tab->list,
+                           tab->dst, tab->dr, tab->dseg, tab->halves};
     }
 };
 
@@ -152,10 +163,11 @@ struct opf_handle {
     GraphCache g64, gmix;
     ClusterPlan c32, c64;
     PersistPlan p32, p64;
+    PersistPlan k32, k64;                // its one-cluster form (small instances)
     std::vector<int> persist_order;      // depth-first order of the subsystems (computed with the first plan)
     bool persist_graph_failed = false;   // the cooperative launch could not be captured in a graph
     WarpPlan w32, w64;
-    std::vector<int> h_tpre, h_vpre, h_foff, h_npad, h_pk, h_gk, h_gstart, h_uslot;
+    std::vector<int> h_tpre, h_vpre, h_foff, h_npad, h_pk, h_segp, h_gk, h_gstart, h_uslot;
     std::vector<int> h_boff;                 // device subsystem -> first row (device row order)
     std::vector<int> dev_to_canon_sub;       // device subsystem -> canonical subsystem
     std::vector<int> canon_row_to_dev;       // canonical row -> device row

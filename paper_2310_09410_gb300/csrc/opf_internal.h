@@ -155,9 +155,13 @@ constexpr int kPersistMaxThreads = 512;
 struct PersistLayout {
     int P, L, threads;
     int local;                     // k_persist_local (one slot and one factor column per thread), else k_persist_engine
-    int split;                     // phase B: a factor column on 4 lanes (local plans of small CTAs)
+    int split, clanes, rlanes;     // FP64 local plans of small CTAs: lanes per factor column and per row
+    int cluster;                   // local plans: the CTAs are one thread-block cluster, u goes through its shared memory
+    int xcap;                      // cluster plans: stamped words per buffer (the most remote entries of a part)
+    int tcap;                      // local plans: products per part (columns rounded up to 4 per subsystem)
     unsigned off_F, off_srec, off_vb, off_tb, off_xrs, off_lrs, off_cobj, off_misc;
     unsigned off_list, off_rem, off_ul;                 // local plans
+    unsigned off_xw, off_tw;                            // cluster plans
     unsigned off_items, off_slots, off_r, off_rn;       // the others
     unsigned bytes;
 };
@@ -165,12 +169,18 @@ struct PersistLayout {
 // Device arrays of a persistent grid engine plan.
 struct PersistPtrs {
     const int *pr;                 // part ranges, 7 fields x (P + 1)
-    double *part;                  // Sec. III-C partial sums, P x 6
+    unsigned long long *part;      // Sec. III-C partial sums, stamped FP64 words, 2 x P x 6
     unsigned long long *sync;      // grid barrier counter
     unsigned long long *xu;        // exchange of u: two buffers of L stamped entries
     // local plans (persist_plan.h): subsystems and slots in part order, the
     // slots' lists of copies and exports, the remote entries
-    const int *sub, *slot, *seg, *out, *list, *rem;
+    const int *sub, *slot, *seg, *out, *rem;
+    const uint4 *list;             // 8 16-bit indices each
+    // cluster plans: destinations of the exported u (rank << 16 | word of the
+    // reader), part p's from dr[p]; per slot (first << 8 | count); per
+    // subsystem (part order) the rows of the first half when the FP32 column
+    // products go by halves, else 0
+    const int *dst, *dr, *dseg, *halves;
 };
 
 // Bytes of a slot's record in a plan with several slots per thread (persist.cu).

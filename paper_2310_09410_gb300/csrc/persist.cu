@@ -48,15 +48,29 @@
 // cycles), so the FP64 forms below count FP64 instructions: the clip compares
 // integers, the global update is one FMA, a column is one chain over its own
 // rows.
-// Measured per iteration with a test every 50, before (every copy of u through
-// L2 behind a grid barrier, parts of the size-sorted order, FP64 sums of the
-// test by butterflies) and now: 8500 buses FP32 4.23 -> 3.10 us, FP64 10.5 ->
-// 7.7 us; 123 buses FP64 4.7 -> 3.04 us.  Of the 8500-bus steps: stamped
+// One cluster (CL, instances of the warp engine's size): the stamped words lie
+// in the readers' shared memory and the writer stores into them directly
+// (distributed shared memory), so an exchange is one remote store.  FP32 keeps
+// the warp engine's order of every sum (the iterates are its, bit for bit) with
+// the factor rows in registers, columns on one lane each and those of more than
+// 32 rows on two.  FP64 (SPLIT) spreads columns and rows over lanes while each
+// warp has a sub-partition of its own.
+// Measured per iteration with a test every 50, grid form, before (every copy of
+// u through L2 behind a grid barrier, parts of the size-sorted order, FP64 sums
+// of the test by butterflies) and now: 8500 buses FP32 4.23 -> 3.0 us, FP64
+// 10.5 -> 7.7 us; 123 buses FP64 4.7 -> 2.9 us.  Of the 8500-bus steps: stamped
 // entries alone, all copies through L2, 6.1 us FP32 (every slot polls, and the
 // polls fill the L1) and 8.4 us FP64; local parts 3.6 and 8.8 us; the copies'
 // places in registers, loops unrolled, long warps of co-resident CTAs on
 // different sub-partitions, and the test's sums spread over lanes and warps
 // 3.1 and 7.7 us (a test cost some 40 us, now 12).
+// One-cluster form against the warp engine: FP32 13 / 34 / 123 buses 0.92 /
+// 1.00 / 1.11 us against 1.71 / 1.80 / 2.31; FP64 13 / 34 buses 1.98 / 2.31
+// against 2.92 / 3.03.  Its FP32 phases before the last changes (123 buses,
+// 1.91 us): column products 1950 of 3700 cycles (scalar reads of strided
+// columns, 8-way bank conflicts; 16-byte reads, all of a column's in flight),
+// local update 940 (the row from registers, the products as 16-byte reads).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -68,6 +82,8 @@
 
 namespace opf {
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr unsigned long long kBarrierLimitNs = 1000000000ull;   // 1 s
 
@@ -119,18 +135,30 @@ __device__ __forceinline__ void stage(T *dst, const T *src, int n) {
     for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
 }
 
-// <f, v> over the first n rows of a zero-padded column (FP32: n rounded up to
-// 4 rows, two chains; FP64: to 2 rows, one chain, no add at the end).
+// <f, v> over the first n rows of a zero-padded column.  FP32: two chains, the
+// 16-byte loads of CH row vectors in flight together (vectors past n as zeros,
+// which leave the chains as they are).  FP64: rows rounded up to 2, one chain,
+// no add at the end.
+template <int CH>
 __device__ __forceinline__ float dot_fv(const float *__restrict__ f, const float *__restrict__ v, int n) {
     float a0 = 0.0f, a1 = 0.0f;
-#pragma unroll 4
-    for (int r = 0; r < n; r += 4) {
-        const float4 a = *reinterpret_cast<const float4 *>(f + r);
-        const float4 b = *reinterpret_cast<const float4 *>(v + r);
-        a0 = fmaf(a.x, b.x, a0);
-        a1 = fmaf(a.y, b.y, a1);
-        a0 = fmaf(a.z, b.z, a0);
-        a1 = fmaf(a.w, b.w, a1);
+    for (int r = 0; r < n; r += 4 * CH) {
+        float4 a[CH], b[CH];
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            a[k] = b[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (r + 4 * k < n) {
+                a[k] = *reinterpret_cast<const float4 *>(f + r + 4 * k);
+                b[k] = *reinterpret_cast<const float4 *>(v + r + 4 * k);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < CH; ++k) {
+            a0 = fmaf(a[k].x, b[k].x, a0);
+            a1 = fmaf(a[k].y, b[k].y, a1);
+            a0 = fmaf(a[k].z, b[k].z, a0);
+            a1 = fmaf(a[k].w, b[k].w, a1);
+        }
     }
     return a0 + a1;
 }
@@ -147,41 +175,16 @@ __device__ __forceinline__ double dot_fv(const double *__restrict__ f, const dou
     return acc;
 }
 
-// Part `part` (0..3) of <f, v> over the zero-padded column: 4-row vectors at
-// rows 4 part, 4 part + 16, ...
-template <typename T>
-__device__ __forceinline__ T dot_fv_part(const T *__restrict__ f, const T *__restrict__ v, int npad, int part);
+__device__ __forceinline__ float dot_col(const float *f, const float *v, int n) { return dot_fv<2>(f, v, n); }
+__device__ __forceinline__ double dot_col(const double *f, const double *v, int n) { return dot_fv(f, v, n); }
 
-template <>
-__device__ __forceinline__ float dot_fv_part<float>(const float *__restrict__ f, const float *__restrict__ v,
-                                                    int npad, int part) {
-    float a0 = 0.0f, a1 = 0.0f;
-    for (int r = 4 * part; r < npad; r += 16) {
-        const float4 a = *reinterpret_cast<const float4 *>(f + r);
-        const float4 b = *reinterpret_cast<const float4 *>(v + r);
-        a0 = fmaf(a.x, b.x, a0);
-        a1 = fmaf(a.y, b.y, a1);
-        a0 = fmaf(a.z, b.z, a0);
-        a1 = fmaf(a.w, b.w, a1);
-    }
-    return a0 + a1;
-}
-
-template <>
-__device__ __forceinline__ double dot_fv_part<double>(const double *__restrict__ f, const double *__restrict__ v,
-                                                      int npad, int part) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int r = 4 * part; r < npad; r += 16) {
-        const double2 a = *reinterpret_cast<const double2 *>(f + r);
-        const double2 b = *reinterpret_cast<const double2 *>(v + r);
-        const double2 c = *reinterpret_cast<const double2 *>(f + r + 2);
-        const double2 d = *reinterpret_cast<const double2 *>(v + r + 2);
-        a0 = fma(a.x, b.x, a0);
-        a1 = fma(a.y, b.y, a1);
-        a0 = fma(c.x, d.x, a0);
-        a1 = fma(c.y, d.y, a1);
-    }
-    return a0 + a1;
+// Rows part, part + lanes, .. of <f, v> (one chain: two chains and their add
+// measured slower, 2.24 -> 2.72 us per iteration on the 34-bus feeder).
+__device__ __forceinline__ double dot_rows(const double *f, const double *v, int n, int part, int lanes) {
+    double acc = 0.0;
+#pragma unroll 4
+    for (int r = part; r < n; r += lanes) acc = fma(f[r], v[r], acc);
+    return acc;
 }
 
 // Column stride of a staged factor with npad rows: npad, plus 4 words when
@@ -220,6 +223,32 @@ __device__ __forceinline__ bool xis(const Word2 &w, unsigned stamp) {
 __device__ __forceinline__ float xval(const Word1 &w) { return __uint_as_float((unsigned)w.a); }
 __device__ __forceinline__ double xval(const Word2 &w) { return __hiloint2double((int)(unsigned)w.b, (int)(unsigned)w.a); }
 
+// The same words in the shared memory of a CTA of the cluster: addr is the
+// word's address there (mapa), reads are of the CTA's own.
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ unsigned at_rank(unsigned addr, int rank) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void sput(unsigned addr, float u, unsigned stamp) {
+    const u64 w = ((u64)stamp << 32) | __float_as_uint(u);
+    asm volatile("st.relaxed.cluster.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(w) : "memory");
+}
+__device__ __forceinline__ void sput(unsigned addr, double u, unsigned stamp) {
+    const u64 s = (u64)stamp << 32;
+    const u64 w0 = s | (unsigned)__double2loint(u), w1 = s | (unsigned)__double2hiint(u);
+    asm volatile("st.relaxed.cluster.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(addr), "l"(w0), "l"(w1) : "memory");
+}
+__device__ __forceinline__ void sget(unsigned addr, Word1 &w) {
+    asm volatile("ld.relaxed.cluster.shared::cta.u64 %0, [%1];" : "=l"(w.a) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void sget(unsigned addr, Word2 &w) {
+    asm volatile("ld.relaxed.cluster.shared::cta.v2.u64 {%0, %1}, [%2];" : "=l"(w.a), "=l"(w.b) : "r"(addr) : "memory");
+}
+template <typename T>
+using WordOf = typename std::conditional<sizeof(T) == 4, Word1, Word2>::type;
+
 // One more unsuccessful poll; true when the wait has to end: a fault of this
 // CTA, or the limit (which makes it one).
 __device__ __forceinline__ bool wait_over(unsigned &polls, u64 &t0, volatile int *fault) {
@@ -230,17 +259,26 @@ __device__ __forceinline__ bool wait_over(unsigned &polls, u64 &t0, volatile int
     return true;
 }
 
-// The u of entry i that iteration `stamp` reads.
-template <typename T>
-__device__ __forceinline__ T xwait(const u64 *X, int i, unsigned stamp, volatile int *fault) {
-    typename std::conditional<sizeof(T) == 4, Word1, Word2>::type w;
+// The values that iteration `stamp` reads of N words, get(j, w) loading word j
+// (those with live(j)): the loads of all in flight together, until every
+// number is there.
+template <typename T, int N, typename Get, typename Live>
+__device__ __forceinline__ void wait_words(T (&v)[N], Get get, Live live, unsigned stamp, volatile int *fault) {
+    WordOf<T> w[N];
     unsigned polls = 0;
     u64 t0 = 0;
     for (;;) {
-        xget(X, i, w);
-        if (xis(w, stamp) || wait_over(polls, t0, fault)) break;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (live(j)) get(j, w[j]);
+        bool ok = true;
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (live(j)) ok = ok && xis(w[j], stamp);
+        if (ok || wait_over(polls, t0, fault)) break;
     }
-    return xval(w);
+#pragma unroll
+    for (int j = 0; j < N; ++j) v[j] = live(j) ? xval(w[j]) : T(0);
 }
 
 // Sum over the cnt >= 2 copies of a global (entries us .. us + cnt - 1, in
@@ -249,28 +287,17 @@ __device__ __forceinline__ T xwait(const u64 *X, int i, unsigned stamp, volatile
 template <typename T>
 __device__ __forceinline__ T copy_sum(const u64 *X, int us, int cnt, int own, T u, unsigned stamp,
                                       volatile int *fault) {
-    using W = typename std::conditional<sizeof(T) == 4, Word1, Word2>::type;
     constexpr int SEGW = 4;
     T sum = T(0);
     for (int q0 = 0; q0 < cnt; q0 += SEGW) {
-        W w[SEGW];
-        unsigned polls = 0;
-        u64 t0 = 0;
-        for (;;) {
-#pragma unroll
-            for (int j = 0; j < SEGW; ++j)
-                if (q0 + j < cnt && q0 + j != own) xget(X, us + q0 + j, w[j]);
-            bool ok = true;
-#pragma unroll
-            for (int j = 0; j < SEGW; ++j)
-                if (q0 + j < cnt && q0 + j != own) ok = ok && xis(w[j], stamp);
-            if (ok || wait_over(polls, t0, fault)) break;
-        }
+        T v[SEGW];
+        wait_words<T, SEGW>(v, [&](int j, WordOf<T> &w) { xget(X, us + q0 + j, w); },
+                            [&](int j) { return q0 + j < cnt && q0 + j != own; }, stamp, fault);
 #pragma unroll
         for (int j = 0; j < SEGW; ++j)
             if (q0 + j < cnt) {
-                const T v = q0 + j == own ? u : xval(w[j]);
-                sum = q0 + j == 0 ? v : sum + v;
+                const T t = q0 + j == own ? u : v[j];
+                sum = q0 + j == 0 ? t : sum + t;
             }
     }
     return sum;
@@ -286,14 +313,17 @@ __device__ __forceinline__ T copy_sum(const u64 *X, int us, int cnt, int own, T 
 //   is one FMA with c~ / N, and the clip compares order-preserving integers (a
 //   double's bits, the lower 63 flipped when negative): an FP64 compare costs
 //   as much as an FP64 FMA.  NaN stays NaN.
-template <typename T>
+// CL (one cluster, FP32): the rounding of the warp engine, which ran these
+// instances before: v = x + lambda / rho is one FMA.
+template <typename T, bool CL>
 struct Slot;
 
-template <>
-struct Slot<float> {
+template <bool CL>
+struct Slot<float, CL> {
     float lam, xs, u;                // lambda - lambda_ref, x_s - x_ref, u
-    float r, v, w;                   // x of this iteration, v = x + lambda / rho, lambda / rho
+    float r, v, w;                   // x of this iteration, v = x + lambda / rho, lambda / rho (not CL)
     float bt, ct, rn, lo, hi;        // bbar~, c~, 1 / (rho N), bounds - x_ref
+    float fr[CL ? 32 : 1];           // CL: the slot's row of the factor (at most 32 columns)
     int frow, trow, fcm, pos;        // F offset of the row, t offset, f | column stride << 8 | mode << 20, V position
 
     __device__ __forceinline__ void load(const IterArgs<float> &g, int kk, int gi, int cnt) {
@@ -304,7 +334,7 @@ struct Slot<float> {
         hi = g.ubt[gi];
         lam = g.mu[kk];
         xs = g.ds[kk];
-        w = __fmul_rn(lam, g.inv_rho);
+        w = CL ? g.inv_rho : __fmul_rn(lam, g.inv_rho);
         u = g.rho * xs - lam;
         r = v = 0.0f;
     }
@@ -313,23 +343,51 @@ struct Slot<float> {
         if (x < lo) x = lo;
         if (x > hi) x = hi;
         r = x;
-        v = x + w;
+        v = CL ? fmaf(lam, w, x) : x + w;
     }
-    __device__ __forceinline__ void local_update(const float *F, const float *tb, const IterArgs<float> &g) {
+    template <bool PAD4, bool SPLIT>
+    __device__ __forceinline__ void local_update(const float *F, const float *tb, const IterArgs<float> &g, int, int) {
         const float *Fr = F + frow, *tt = tb + trow;
         const int f = fcm & 255, cs = (fcm >> 8) & 0xfff;
         float y0 = 0.0f, y1 = 0.0f;      // two chains for latency
-        int c = 0;
+        if constexpr (CL) {              // row in registers, the products' loads in flight together
+            float4 t[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                t[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (4 * k < f) t[k] = *reinterpret_cast<const float4 *>(tt + 4 * k);
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                y0 += fr[4 * k] * t[k].x;
+                y1 += fr[4 * k + 1] * t[k].y;
+                y0 += fr[4 * k + 2] * t[k].z;
+                y1 += fr[4 * k + 3] * t[k].w;
+            }
+        } else if constexpr (PAD4) {     // columns and products padded with zeros to a multiple of 4
 #pragma unroll 2
-        for (; c + 1 < f; c += 2) {
-            y0 += Fr[c * cs] * tt[c];
-            y1 += Fr[(c + 1) * cs] * tt[c + 1];
+            for (int c = 0; c < f; c += 4) {
+                const float4 t = *reinterpret_cast<const float4 *>(tt + c);
+                const float f0 = Fr[0], f1 = Fr[cs], f2 = Fr[2 * cs], f3 = Fr[3 * cs];
+                Fr += 4 * cs;
+                y0 += f0 * t.x;
+                y1 += f1 * t.y;
+                y0 += f2 * t.z;
+                y1 += f3 * t.w;
+            }
+        } else {
+            int c = 0;
+#pragma unroll 2
+            for (; c + 1 < f; c += 2) {
+                y0 += Fr[c * cs] * tt[c];
+                y1 += Fr[(c + 1) * cs] * tt[c + 1];
+            }
+            if (c < f) y0 += Fr[c * cs] * tt[c];
         }
-        if (c < f) y0 += Fr[c * cs] * tt[c];
         xs = ((fcm >> 20) ? (y0 + y1) : v - (y0 + y1)) + bt;
         const float res = r - xs;
         lam = lam + g.rho * res;
-        w = __fmul_rn(lam, g.inv_rho);
+        if constexpr (!CL) w = __fmul_rn(lam, g.inv_rho);
         u = g.rho * xs - lam;
     }
     __device__ __forceinline__ float state() const { return xs; }
@@ -354,8 +412,8 @@ struct Slot<float> {
     }
 };
 
-template <>
-struct Slot<double> {
+template <bool CL>
+struct Slot<double, CL> {
     double lam, rx, u;               // lambda - lambda_ref, rho (x_s - x_ref), u
     double r, v;                     // rho x of this iteration, V = r + lam
     double rbt, ct, rn;              // +-rho bbar~ (mode 1 / 0), c~ / N, 1 / N
@@ -388,12 +446,18 @@ struct Slot<double> {
         }
         v = r + lam;
     }
-    __device__ __forceinline__ void local_update(const double *F, const double *tb, const IterArgs<double> &) {
+    // SPLIT: the row on `lanes` lanes (columns part, part + lanes, ..), each of
+    // which ends with the whole slot
+    template <bool PAD4, bool SPLIT>
+    __device__ __forceinline__ void local_update(const double *F, const double *tb, const IterArgs<double> &, int part,
+                                                 int lanes) {
         const double *Fr = F + frow, *tt = tb + trow;
         const int f = fcm & 255, cs = (fcm >> 8) & 0xfff;
-        double y = rbt;
+        double y = part == 0 ? rbt : 0.0;
 #pragma unroll 4
-        for (int c = 0; c < f; ++c) y += Fr[c * cs] * tt[c];
+        for (int c = part; c < f; c += SPLIT ? lanes : 1) y += Fr[c * cs] * tt[c];
+        if constexpr (SPLIT)
+            for (int o = 1; o < lanes; o <<= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
         rx = (fcm >> 20) ? y : v - y;
         lam = v - rx;
         u = rx - lam;
@@ -420,8 +484,8 @@ struct Slot<double> {
 };
 
 // Geometry of a slot from its part's subsystem record r and its row.
-template <typename T>
-__device__ __forceinline__ void place(Slot<T> &s, const int4 r, int row) {
+template <typename S>
+__device__ __forceinline__ void place(S &s, const int4 r, int row) {
     const int f = r.w >> 10, npad = (r.w >> 1) & 0x1ff;
     s.frow = r.x + row;
     s.trow = r.z;
@@ -439,19 +503,19 @@ struct SlotRec {
 static_assert(sizeof(SlotRec<float>) == persist_slot_bytes(4) && sizeof(SlotRec<double>) == persist_slot_bytes(8),
               "the layout reserves this much per slot");
 
-__device__ __forceinline__ void pack(SlotRec<float> &q, const Slot<float> &s) {
+__device__ __forceinline__ void pack(SlotRec<float> &q, const Slot<float, false> &s) {
     q.f[0] = s.lam; q.f[1] = s.xs; q.f[2] = s.bt; q.f[3] = s.ct; q.f[4] = s.lo; q.f[5] = s.hi;
 }
-__device__ __forceinline__ void pack(SlotRec<double> &q, const Slot<double> &s) {
+__device__ __forceinline__ void pack(SlotRec<double> &q, const Slot<double, false> &s) {
     q.f[0] = s.lam; q.f[1] = s.rx; q.f[2] = s.rbt; q.f[3] = s.ct;
     q.f[4] = __longlong_as_double(s.lo); q.f[5] = __longlong_as_double(s.hi);
 }
-__device__ __forceinline__ void unpack(Slot<float> &s, const SlotRec<float> &q, const IterArgs<float> &g) {
+__device__ __forceinline__ void unpack(Slot<float, false> &s, const SlotRec<float> &q, const IterArgs<float> &g) {
     s.lam = q.f[0]; s.xs = q.f[1]; s.bt = q.f[2]; s.ct = q.f[3]; s.lo = q.f[4]; s.hi = q.f[5];
     s.w = __fmul_rn(s.lam, g.inv_rho);
     s.u = g.rho * s.xs - s.lam;
 }
-__device__ __forceinline__ void unpack(Slot<double> &s, const SlotRec<double> &q, const IterArgs<double> &) {
+__device__ __forceinline__ void unpack(Slot<double, false> &s, const SlotRec<double> &q, const IterArgs<double> &) {
     s.lam = q.f[0]; s.rx = q.f[1]; s.rbt = q.f[2]; s.ct = q.f[3];
     s.lo = __double_as_longlong(q.f[4]); s.hi = __double_as_longlong(q.f[5]);
     s.u = s.rx - s.lam;
@@ -461,33 +525,56 @@ __device__ __forceinline__ void unpack(Slot<double> &s, const SlotRec<double> &q
 struct Misc {
     volatile int *flags;             // [0] fault, [1] stop
     DevStatus *loc;
-    double (*red)[6];
+    double *sum;                     // the six sums over all CTAs
+    double (*red)[6];                // per warp
     __device__ __forceinline__ explicit Misc(unsigned char *m)
         : flags(reinterpret_cast<volatile int *>(m)), loc(reinterpret_cast<DevStatus *>(m + 16)),
-          red(reinterpret_cast<double(*)[6]>(m + 16 + ((sizeof(DevStatus) + 15) & ~15))) {}
+          sum(reinterpret_cast<double *>(m + 16 + ((sizeof(DevStatus) + 15) & ~15))),
+          red(reinterpret_cast<double(*)[6]>(m + 64 + ((sizeof(DevStatus) + 15) & ~15))) {}
 };
 
-// The test of iteration `it`: the CTA's sums out, grid barrier number nb, the
-// P partials summed, the decision.  False: leave the loop (stopped or fault).
-__device__ __forceinline__ bool test_iteration(const Misc &m, const PersistPtrs &pp, double acc[6], int it,
-                                               int check_every, int P, int bar_extra, unsigned long long nb,
-                                               DevStatus *st, double rho_d) {
+// The test of iteration `it`, test number nb of the launch: the CTA's six sums
+// out as stamped FP64 words, every CTA's taken and added in the same order, the
+// decision.  The words of a test are overwritten two tests later, when every
+// CTA has published (so read) the one between.  False: leave the loop
+// (stopped, or a wait ran out).  CL: the words in every CTA's shared memory at
+// tw (2 x P x 6), else in pp.part.
+template <bool CL>
+__device__ __forceinline__ bool test_iteration(const Misc &m, const PersistPtrs &pp, unsigned tw, double acc[6],
+                                               int it, int check_every, int P, unsigned nb, DevStatus *st,
+                                               double rho_d) {
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = (int)(blockDim.x >> 5), rank = (int)blockIdx.x;
+    const unsigned stamp = (unsigned)it + 1u;
+    const int base = (int)(nb & 1u) * P * 6;
     const double mine = cta_sum6(acc, m.red);
-    if (tid < 6) __stcg(pp.part + rank * 6 + tid, mine);
-    if (!grid_barrier(pp.sync, nb * (unsigned long long)(P + bar_extra), m.flags)) return false;
-    // the partials of one quantity per warp, in the same order in every CTA
+    if (tid < 6) {
+        if constexpr (CL) {
+            for (int r = 0; r < P; ++r) sput(at_rank(tw + 16u * (base + rank * 6 + tid), r), mine, stamp);
+        } else {
+            xput(pp.part, base + rank * 6 + tid, mine, stamp);
+        }
+    }
+    // one quantity per warp, lane l the CTAs l, l + 32, ..
     for (int q = w; q < 6; q += nw) {
         double v = 0.0;
-        for (int r = lane; r < P; r += 32) v += __ldcg(pp.part + r * 6 + q);
+        for (int r = lane; r < P; r += 32)
+        {
+            double t[1];
+            wait_words<double, 1>(t, [&](int, Word2 &x) {
+                if constexpr (CL) sget(tw + 16u * (base + r * 6 + q), x);
+                else xget(pp.part, base + r * 6 + q, x);
+            }, [](int) { return true; }, stamp, m.flags);
+            v += t[0];
+        }
         v = warp_sum_d(v);
-        if (lane == 0) m.red[0][q] = v;
+        if (lane == 0) m.sum[q] = v;
     }
     __syncthreads();
+    if (m.flags[0]) return false;
     if (w == 0) {
         DevStatus *loc = m.loc;
         const int since = ((it + 1) % check_every) == 0 ? check_every : ((it + 1) % check_every);
-        apply_test_warp(loc, m.red[0], rho_d, since);
+        apply_test_warp(loc, m.sum, rho_d, since);
         if (lane == 0) {
             m.flags[1] = loc->done;
             if (rank == 0) {
@@ -516,26 +603,70 @@ __device__ __forceinline__ void leave(const Misc &m, DevStatus *st, cudaGraphCon
     if (use_cond && blockIdx.x == 0) cudaGraphSetConditional(cond, (m.flags[0] || m.flags[1]) ? 0u : 1u);
 }
 
-// Factors of the part: one warp per own subsystem, columns re-strided.
-template <typename T>
-__device__ __forceinline__ void stage_factors(T *F, const IterArgs<T> &g, const int4 *srec, const int *subs, int s0,
-                                              int ns) {
+// Factors of the part: one warp per own subsystem, columns re-strided.  The
+// local forms keep zero columns up to a multiple of 4 and, where half[i] = hn
+// > 0, rows hn and up from the next multiple of 4.
+template <typename T, bool LOCAL>
+__device__ __forceinline__ void stage_factors(T *F, const IterArgs<T> &g, const int4 *srec, const int *subs,
+                                              const int *half, int s0, int ns) {
     for (int i = threadIdx.x >> 5; i < ns; i += blockDim.x >> 5) {
         const int4 r = srec[i];
         const int f = r.w >> 10, npad = (r.w >> 1) & 0x1ff, cs = fstride(npad);
-        const T *src = g.F + g.sub2[subs ? subs[s0 + i] : s0 + i].x;
-        for (int e = threadIdx.x & 31; e < f * npad; e += 32) {
-            const int c = e / npad;
-            F[r.x + c * cs + (e - c * npad)] = src[e];
+        const int4 q = g.sub2[LOCAL ? subs[s0 + i] : s0 + i];
+        const int hn = LOCAL && half ? half[s0 + i] : 0, h4 = (hn + 3) & ~3;
+        const T *src = g.F + q.x;
+        const int fc = LOCAL ? (f + 3) & ~3 : f;
+        for (int e = threadIdx.x & 31; e < fc * npad; e += 32) {
+            const int c = e / npad, row = e - c * npad;
+            int from = row;                      // row of the packed factor, -1: padding
+            if (hn) from = row < hn ? row : row < h4 ? -1 : row - h4 + hn;
+            F[r.x + c * cs + row] = c < f && from >= 0 && from < q.y ? src[c * q.y + from] : T(0);
         }
     }
 }
 
-// SPLIT: small CTAs, each factor column on 4 lanes (rows 4 p, 4 p + 16, .. of
-// lane p, then a shuffle sum), so the longest column is no longer one lane's
-// dependent chain; otherwise one lane per column.
-template <typename T, bool SPLIT>
-__global__ void __launch_bounds__(kPersistMaxThreads, SPLIT ? 1 : 2)
+// Column products of the one-cluster FP32 form in the warp engine's order
+// (rows in two chains up to 32 rows, dot_fv; above, in four chains over the
+// column or over each of its halves, the rows past a multiple of 4 last in the
+// first chain).
+__device__ __forceinline__ float dot_rows4(const float *f, const float *v, int n) {
+    float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+    const int full = n & ~3;
+    for (int r = 0; r < full; r += 16) {
+        float4 a[4], b[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            a[k] = b[k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (r + 4 * k < full) {
+                a[k] = *reinterpret_cast<const float4 *>(f + r + 4 * k);
+                b[k] = *reinterpret_cast<const float4 *>(v + r + 4 * k);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            a0 = fmaf(a[k].x, b[k].x, a0);
+            a1 = fmaf(a[k].y, b[k].y, a1);
+            a2 = fmaf(a[k].z, b[k].z, a2);
+            a3 = fmaf(a[k].w, b[k].w, a3);
+        }
+    }
+    if (full < n) {                       // the padding rows are zeros: they leave the chain as it is
+        const float4 a = *reinterpret_cast<const float4 *>(f + full);
+        const float4 b = *reinterpret_cast<const float4 *>(v + full);
+        a0 = fmaf(a.x, b.x, a0);
+        a0 = fmaf(a.y, b.y, a0);
+        a0 = fmaf(a.z, b.z, a0);
+    }
+    return (a0 + a1) + (a2 + a3);
+}
+
+// SPLIT (FP64, small CTAs): each factor column on lay.clanes lanes and each row
+// on lay.rlanes, so that the longest one is no longer one lane's dependent
+// chain while the CTA's warps still have a sub-partition each.
+// CL: the CTAs are one thread-block cluster of at most 16; u goes straight into
+// the readers' shared memory (stamped words there, no L2 on the way).
+template <typename T, bool SPLIT, bool CL>
+__global__ void __launch_bounds__(kPersistMaxThreads, SPLIT || CL ? 1 : 2)
 k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_extra, int n_iters, int check_every,
                 DevStatus *st, double rho_d, cudaGraphConditionalHandle cond, int use_cond) {
     extern __shared__ __align__(16) unsigned char sm[];
@@ -548,7 +679,7 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
     // A part's first slots and columns are its longest, so work item 0 starts
     // at another warp in CTAs that share an SM (b and b + the number of SMs, or
     // neighbours): their long warps then sit on different sub-partitions.
-    const int turn = 32 * (((rank & 1) + (2 * rank >= P ? 2 : 0)) % (nthr >> 5));
+    const int turn = CL ? 0 : 32 * (((rank & 1) + (2 * rank >= P ? 2 : 0)) % (nthr >> 5));
     const int tid = (int)threadIdx.x >= turn ? (int)threadIdx.x - turn : (int)threadIdx.x - turn + nthr;
     const int *pr = pp.pr;
     auto range = [&](int f, int &a, int &n) { a = pr[f * P1 + rank]; n = pr[f * P1 + rank + 1] - a; };
@@ -557,127 +688,249 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
     range(GR_R, r0, nrem); range(GR_L, l0, nl);
     T *F = reinterpret_cast<T *>(sm + lay.off_F);
     int4 *srec = reinterpret_cast<int4 *>(sm + lay.off_srec);
-    int *list = reinterpret_cast<int *>(sm + lay.off_list);
-    int *rem = reinterpret_cast<int *>(sm + lay.off_rem);
-    T *ul = reinterpret_cast<T *>(sm + lay.off_ul);                // u of the own slots, then of the remote entries
+    uint4 *list = reinterpret_cast<uint4 *>(sm + lay.off_list);
+    int *rem = reinterpret_cast<int *>(sm + lay.off_rem);          // remote entries (CL: destinations of the exports)
+    T *ul = reinterpret_cast<T *>(sm + lay.off_ul);                // u of the own slots, the remote entries, a zero
     T *vb = reinterpret_cast<T *>(sm + lay.off_vb);
     T *tb = reinterpret_cast<T *>(sm + lay.off_tb);
     double *xrs = reinterpret_cast<double *>(sm + lay.off_xrs);    // x_ref of each slot's global
     double *lrs = reinterpret_cast<double *>(sm + lay.off_lrs);    // lambda_ref of each slot
     double *cobj = reinterpret_cast<double *>(sm + lay.off_cobj);  // c of the global on its first copy, else 0
     const Misc m(sm + lay.off_misc);
+    // CL: stamped words of the remote entries, two buffers of xcap, and of the tests
+    constexpr unsigned XB = sizeof(T) == 4 ? 8 : 16;               // bytes per word
+    const unsigned xw = smem_addr(sm + lay.off_xw), xbuf = XB * (unsigned)lay.xcap, tw = smem_addr(sm + lay.off_tw);
 
     stage<int4>(srec, g.srec + s0, ns);
-    stage<int>(list, pp.list + l0, nl);
-    stage<int>(rem, pp.rem + r0, nrem);
+    stage<uint4>(list, pp.list + l0, nl);
+    if constexpr (CL) stage<int>(rem, pp.dst + pp.dr[rank], pp.dr[rank + 1] - pp.dr[rank]);
+    else stage<int>(rem, pp.rem + r0, nrem);
     for (int i = tid; i < nv; i += nthr) vb[i] = T(0);
+    for (int i = tid; i < lay.tcap; i += nthr) tb[i] = T(0);
     if (tid == 0) {
+        ul[nk + nrem] = T(0);
         m.flags[0] = 0;
         m.flags[1] = 0;
         *m.loc = *st;
     }
+    if constexpr (CL) {
+        for (int i = tid; i < 2 * lay.xcap; i += nthr) sput(xw + XB * i, T(0), 0xffffffffu);
+        for (int i = tid; i < 12 * P; i += nthr) sput(tw + 16u * i, 0.0, 0xffffffffu);
+    }
     __syncthreads();
-    stage_factors<T>(F, g, srec, pp.sub, s0, ns);
-    constexpr int XW = sizeof(T) == 4 ? 1 : 2;          // words per exchange entry
+    stage_factors<T, true>(F, g, srec, pp.sub, CL ? pp.halves : nullptr, s0, ns);
+    constexpr int XW = XB / 8;                          // 8-byte words per exchange entry
     u64 *X0 = pp.xu, *X1 = pp.xu + (size_t)XW * L;      // read by even / odd iterations
-    // the thread's slot; its first u out, its entry of iteration 1 marked unwritten
-    const bool have = tid < nk;
-    Slot<T> s;
+    // the thread's slot (lay.rlanes threads of one in SPLIT)
+    const int ks = SPLIT ? tid / lay.rlanes : tid, rpart = SPLIT ? tid & (lay.rlanes - 1) : 0;
+    const bool have = ks < nk, lead = have && rpart == 0;
+    Slot<T, CL> s;
     int seg = 0, out = -1, kk = 0;
+    s.fcm = s.frow = s.trow = s.pos = 0;
+    if constexpr (CL) __syncthreads();       // the staged factors are read here
     if (have) {
-        kk = pp.slot[k0 + tid];
-        const int mt = g.cmeta[k0 + tid], gi = g.gk[kk];
-        seg = pp.seg[k0 + tid];
-        out = pp.out[k0 + tid];
+        kk = pp.slot[k0 + ks];
+        const int mt = g.cmeta[k0 + ks], gi = g.gk[kk];
+        seg = pp.seg[k0 + ks];
         place(s, srec[mt >> 8], mt & 255);
         s.load(g, kk, gi, seg & 255);
-        xrs[tid] = g.xr[gi];
-        lrs[tid] = g.lamr[kk];
-        cobj[tid] = g.pk[kk] == (g.segp[kk] >> 8) ? g.c64[gi] : 0.0;
-        ul[tid] = s.u;
-        if (out >= 0) {
-            xput(X0, out, s.u, 0u);
-            xput(X1, out, T(0), 0xffffffffu);
+        if constexpr (CL && sizeof(T) == 4) {
+            const int f4 = ((s.fcm & 255) + 3) & ~3, cs = (s.fcm >> 8) & 0xfff;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) s.fr[c] = c < f4 ? F[s.frow + c * cs] : 0.0f;
+        }
+        if (lead) {
+            out = CL ? pp.dseg[k0 + ks] : pp.out[k0 + ks];
+            xrs[ks] = g.xr[gi];
+            lrs[ks] = g.lamr[kk];
+            cobj[ks] = g.pk[kk] == (g.segp[kk] >> 8) ? g.c64[gi] : 0.0;
+            ul[ks] = s.u;
         }
     }
-    // the thread's factor column
-    const int part4 = SPLIT ? tid & 3 : 0, jcol = SPLIT ? tid >> 2 : tid;
+    // CL: the readers of the slot's u, out = first << 8 | count in the list of
+    // destinations (rank << 16 | word, made mapped addresses here); the first
+    // two in registers
+    unsigned da0 = 0, da1 = 0;
+    int nd = 0;
+    if constexpr (CL) {
+        const int n = pp.dr[rank + 1] - pp.dr[rank];
+        for (int i = tid; i < n; i += nthr) rem[i] = (int)at_rank(xw + XB * (rem[i] & 0xffff), rem[i] >> 16);
+        __syncthreads();
+        nd = lead ? out & 255 : 0;
+        if (nd > 0) da0 = (unsigned)rem[out >> 8];
+        if (nd > 1) da1 = (unsigned)rem[(out >> 8) + 1];
+    }
+    auto publish = [&](int it) {         // u for iteration `it`
+        if constexpr (CL) {
+            const unsigned off = (it & 1) ? xbuf : 0u;
+            if (nd > 0) sput(da0 + off, s.u, (unsigned)it);
+            if (nd > 1) sput(da1 + off, s.u, (unsigned)it);
+            for (int i = 2; i < nd; ++i) sput((unsigned)rem[(out >> 8) + i] + off, s.u, (unsigned)it);
+        } else {
+            if (out >= 0) xput((it & 1) ? X1 : X0, out, s.u, (unsigned)it);
+        }
+    };
+    // the thread's factor column.  FP32 cluster form: those of more than 32
+    // rows first, on two lanes each (a lane per half, the second idle when the
+    // column is one piece) and in warps of their own.
+    constexpr bool PAIRS = CL && sizeof(T) == 4;
+    int jcol, part = 0, nbig = 0;
+    if constexpr (PAIRS) {
+        for (nbig = 0; nbig < nj && g.sub[pp.sub[s0 + (g.citems[j0 + nbig] >> 8)]].y > 32;) ++nbig;
+        const int wide = (2 * nbig + 31) & ~31;
+        jcol = tid < wide ? (tid < 2 * nbig ? tid >> 1 : nj) : tid - wide + nbig;
+        part = tid < wide ? tid & 1 : 0;
+    } else {
+        jcol = SPLIT ? tid / lay.clanes : tid;
+        part = SPLIT ? tid & (lay.clanes - 1) : 0;
+    }
+    const bool big = PAIRS && tid < ((2 * nbig + 31) & ~31);
     const T *Fcol = F, *vcol = vb;
-    int ncol = 0;
+    int ncol = 0, tcol = 0;
     if (jcol < nj) {
-        const int itm = g.citems[j0 + jcol];
-        const int4 r = srec[itm >> 8];
-        const int npad = (r.w >> 1) & 0x1ff;
+        const int itm = g.citems[j0 + jcol], i = itm >> 8;
+        const int4 r = srec[i];
+        const int npad = (r.w >> 1) & 0x1ff, n = g.sub[pp.sub[s0 + i]].y;
         Fcol = F + r.x + (itm & 255) * fstride(npad);
         vcol = vb + r.y;
-        ncol = SPLIT || sizeof(T) == 4 ? npad : (g.sub[pp.sub[s0 + (itm >> 8)]].y + 1) & ~1;
+        tcol = r.z + (itm & 255);
+        ncol = sizeof(T) == 4 ? npad : SPLIT ? n : (n + 1) & ~1;
+        if constexpr (CL) {
+            const int hn = pp.halves[s0 + i], h4 = (hn + 3) & ~3;
+            if (sizeof(T) == 8 && hn) ncol = npad;
+            if (big) {
+                ncol = hn ? (part ? n - hn : hn) : (part ? 0 : n);
+                if (part) { Fcol += h4; vcol += h4; }
+            }
+        }
     }
-    // the first four copies' places in the u array in registers, later ones in the list
-    const int cnt = seg & 255, *lst = list + (seg >> 8);
-    unsigned at01 = 0, at23 = 0;
-    if (cnt > 1) {
-        at01 = (unsigned)lst[0] | ((unsigned)lst[1] << 16);
-        at23 = (cnt > 2 ? (unsigned)lst[2] : 0u) | ((cnt > 3 ? (unsigned)lst[3] : 0u) << 16);
+    // the first eight copies' places in the u array in registers, later ones in the list
+    const int cnt = seg & 255, wmax = __reduce_max_sync(0xffffffffu, cnt);
+    const uint4 *lst = list + (seg >> 8);
+    uint4 at = make_uint4(0, 0, 0, 0);
+    if (cnt > 1) at = lst[0];
+    bool running = true;
+    if constexpr (CL) {
+        cg::this_cluster().sync();           // every CTA's words are marked unwritten
+        publish(0);
+        // (the test hook of the bounded waits: a word that nobody writes)
+        if (bar_extra && tid == 0) {
+            double t[1];
+            wait_words<double, 1>(t, [&](int, Word2 &x) { sget(tw, x); }, [](int) { return true; }, 0u, m.flags);
+        }
+        __syncthreads();
+        running = m.flags[0] == 0;
+    } else {
+        if (lead && out >= 0) xput(X1, out, T(0), 0xffffffffu);
+        if (tid < 12) xput(pp.part, (tid / 6) * P * 6 + rank * 6 + tid % 6, 0.0, 0xffffffffu);
+        publish(0);
+        running = grid_barrier(pp.sync, (unsigned long long)(P + bar_extra), m.flags);
     }
-    unsigned long long nb = 1;
-    bool running = grid_barrier(pp.sync, nb * (unsigned long long)(P + bar_extra), m.flags);
+    unsigned nb = 0;
+    constexpr int WAITS = CL ? 1 : 2;        // remote entries of a thread taken together
     // one iteration (CHK: tested); false: leave the loop
     auto iteration = [&](int it, auto tested) -> bool {
         constexpr bool CHK = decltype(tested)::value;
-        const u64 *Xin = (it & 1) ? X1 : X0;
-        u64 *Xout = (it & 1) ? X0 : X1;
         double acc[6] = {0, 0, 0, 0, 0, 0};
         // remote entries: the threads of the smallest subsystems first (they
         // finish the previous iteration first)
-        for (int i = nthr - 1 - tid; i < nrem; i += nthr) ul[nk + i] = xwait<T>(Xin, rem[i], (unsigned)it, m.flags);
+        for (int i0 = nthr - 1 - tid; i0 < nrem; i0 += WAITS * nthr) {
+            T v[WAITS];
+            auto live = [&](int j) { return j == 0 || i0 + j * nthr < nrem; };
+            wait_words<T, WAITS>(v, [&](int j, WordOf<T> &w) {
+                const int i = i0 + j * nthr;
+                if constexpr (CL) sget(xw + ((it & 1) ? xbuf : 0u) + XB * i, w);
+                else xget((it & 1) ? X1 : X0, rem[i], w);
+            }, live, (unsigned)it, m.flags);
+#pragma unroll
+            for (int j = 0; j < WAITS; ++j)
+                if (live(j)) ul[nk + i0 + j * nthr] = v[j];
+        }
         __syncthreads();
         if (m.flags[0]) return false;       // written in the waits above only, so every thread reads the same
         if (have) {
             T sigma = s.u;
             if (cnt > 1) {
-                const T a0 = ul[at01 & 0xffffu], a1 = ul[at01 >> 16], a2 = ul[at23 & 0xffffu], a3 = ul[at23 >> 16];
-                sigma = a0 + a1;
-                if (cnt > 2) sigma += a2;
-                if (cnt > 3) sigma += a3;
+                if constexpr (sizeof(T) == 8) {      // no add past the last copy
+                    const T c0 = ul[at.x & 0xffffu], c1 = ul[at.x >> 16], c2 = ul[at.y & 0xffffu], c3 = ul[at.y >> 16];
+                    sigma = c0 + c1;
+                    if (cnt > 2) sigma += c2;
+                    if (cnt > 3) sigma += c3;
+                    const unsigned short *l = reinterpret_cast<const unsigned short *>(lst);
 #pragma unroll 4
-                for (int q = 4; q < cnt; ++q) sigma += ul[lst[q]];
+                    for (int q = 4; q < cnt; ++q) sigma += ul[l[q]];
+                } else {                             // the places past the last copy hold zeros
+                    T c0 = ul[at.x & 0xffffu], c1 = ul[at.x >> 16], c2 = ul[at.y & 0xffffu], c3 = ul[at.y >> 16];
+                    T d0 = T(0), d1 = T(0), d2 = T(0), d3 = T(0);
+                    if (wmax > 4) {
+                        d0 = ul[at.z & 0xffffu]; d1 = ul[at.z >> 16]; d2 = ul[at.w & 0xffffu]; d3 = ul[at.w >> 16];
+                    }
+                    if constexpr (CL) {              // four chains
+                        c0 += d0; c1 += d1; c2 += d2; c3 += d3;
+                        for (int q = 8; q < cnt; q += 8) {
+                            const uint4 l = lst[q >> 3];
+                            c0 += ul[l.x & 0xffffu]; c1 += ul[l.x >> 16]; c2 += ul[l.y & 0xffffu]; c3 += ul[l.y >> 16];
+                            c0 += ul[l.z & 0xffffu]; c1 += ul[l.z >> 16]; c2 += ul[l.w & 0xffffu]; c3 += ul[l.w >> 16];
+                        }
+                        sigma = (c0 + c1) + (c2 + c3);
+                    } else {                         // copy order
+                        sigma = ((((((c0 + c1) + c2) + c3) + d0) + d1) + d2) + d3;
+                        for (int q = 8; q < cnt; q += 8) {
+                            const uint4 l = lst[q >> 3];
+                            sigma += ul[l.x & 0xffffu]; sigma += ul[l.x >> 16];
+                            sigma += ul[l.y & 0xffffu]; sigma += ul[l.y >> 16];
+                            sigma += ul[l.z & 0xffffu]; sigma += ul[l.z >> 16];
+                            sigma += ul[l.w & 0xffffu]; sigma += ul[l.w >> 16];
+                        }
+                    }
+                }
             }
             s.global_update(sigma);
-            vb[s.pos] = s.v;
+            if (lead) vb[s.pos] = s.v;
             if constexpr (CHK) {
-                s.test_global(acc, g, xrs[tid], cobj[tid]);
-                U[(size_t)L + g.pk[kk]] = s.u;      // the u behind this global update, for the solution
+                if (lead) {
+                    s.test_global(acc, g, xrs[ks], cobj[ks]);
+                    U[(size_t)L + g.pk[kk]] = s.u;      // the u behind this global update, for the solution
+                }
             }
         }
         __syncthreads();
         if constexpr (SPLIT) {
             T a = T(0);
-            if (jcol < nj) a = dot_fv_part<T>(Fcol, vcol, ncol, part4);
-            a += __shfl_xor_sync(0xffffffffu, a, 1);
-            a += __shfl_xor_sync(0xffffffffu, a, 2);
-            if (jcol < nj && part4 == 0) tb[jcol] = a;
-        } else {
-            if (jcol < nj) tb[jcol] = dot_fv(Fcol, vcol, ncol);
+            if (jcol < nj) a = dot_rows(Fcol, vcol, ncol, part, lay.clanes);
+            for (int o = 1; o < lay.clanes; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (jcol < nj && part == 0) tb[tcol] = a;
+        } else if (big) {
+            if constexpr (PAIRS) {
+                const float t0 = dot_rows4(Fcol, vcol, ncol), t1 = __shfl_xor_sync(0xffffffffu, t0, 1);
+                if (jcol < nj && part == 0) tb[tcol] = t0 + t1;
+            }
+        } else if (jcol < nj) {
+            if constexpr (PAIRS) tb[tcol] = dot_fv<4>(Fcol, vcol, ncol);
+            else tb[tcol] = dot_col(Fcol, vcol, ncol);
         }
         __syncthreads();
-        if (have) {
+        if (have || SPLIT) {
             const T old = s.state();
-            s.local_update(F, tb, g);
-            if (out >= 0) xput(Xout, out, s.u, (unsigned)it + 1u);
-            ul[tid] = s.u;
-            if constexpr (CHK) {
-                s.test_slot(acc, g, old, xrs[tid], lrs[tid]);
-                U[g.pk[kk]] = s.u;
+            s.template local_update<true, SPLIT>(F, tb, g, rpart, lay.rlanes);
+            if (lead) {
+                publish(it + 1);
+                ul[ks] = s.u;
+                if constexpr (CHK) {
+                    s.test_slot(acc, g, old, xrs[ks], lrs[ks]);
+                    U[g.pk[kk]] = s.u;
+                }
             }
         }
-        if constexpr (CHK) return test_iteration(m, pp, acc, it, check_every, P, bar_extra, ++nb, st, rho_d);
+        if constexpr (CHK) return test_iteration<CL>(m, pp, tw, acc, it, check_every, P, nb++, st, rho_d);
         return true;
     };
     for (int it = 0; it < n_iters && running; ++it) {
         if (((it + 1) % check_every) == 0 || it == n_iters - 1) running = iteration(it, std::true_type{});
         else running = iteration(it, std::false_type{});
     }
-    if (have) s.save(g, kk);
+    if (lead) s.save(g, kk);
+    if constexpr (CL) cg::this_cluster().sync();         // no CTA leaves while others may write to its words
     leave(m, st, cond, use_cond);
 }
 
@@ -719,12 +972,12 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
         *m.loc = *st;
     }
     __syncthreads();
-    stage_factors<T>(F, g, srec, nullptr, s0, ns);
+    stage_factors<T, false>(F, g, srec, nullptr, nullptr, s0, ns);
     constexpr int XW = sizeof(T) == 4 ? 1 : 2;
     u64 *X0 = pp.xu, *X1 = pp.xu + (size_t)XW * L;
     for (int k = tid; k < nk; k += nthr) {
         const int kk = k0 + k, gi = g.gk[kk], mt = g.cmeta[kk], seg = g.segp[kk], own = g.pk[kk] - (seg >> 8);
-        Slot<T> s;
+        Slot<T, false> s;
         place(s, srec[mt >> 8], mt & 255);
         s.load(g, kk, gi, seg & 255);
         pack(slots[k], s);
@@ -738,7 +991,7 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
             xput(X1, g.pk[kk], T(0), 0xffffffffu);
         }
     }
-    auto fetch = [&](Slot<T> &s, int k, int &seg, int &own) {
+    auto fetch = [&](Slot<T, false> &s, int k, int &seg, int &own) {
         const SlotRec<T> q = slots[k];
         seg = q.seg;
         own = (int)((unsigned)q.mo >> 24);
@@ -748,14 +1001,15 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
         s.r = rb[k];
         s.v = vb[s.pos];
     };
-    unsigned long long nb = 1;
-    bool running = grid_barrier(pp.sync, nb * (unsigned long long)(P + bar_extra), m.flags);
+    if (tid < 12) xput(pp.part, (tid / 6) * P * 6 + rank * 6 + tid % 6, 0.0, 0xffffffffu);
+    bool running = grid_barrier(pp.sync, (unsigned long long)(P + bar_extra), m.flags);
+    unsigned nb = 0;
     auto iteration = [&](int it, auto tested) -> bool {
         constexpr bool CHK = decltype(tested)::value;
         const u64 *Xin = (it & 1) ? X1 : X0;
         u64 *Xout = (it & 1) ? X0 : X1;
         double acc[6] = {0, 0, 0, 0, 0, 0};
-        Slot<T> s;
+        Slot<T, false> s;
         int seg, own;
         for (int k = tid; k < nk; k += nthr) {
             fetch(s, k, seg, own);
@@ -776,13 +1030,13 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
             const int itm = items[j];
             const int4 r = srec[itm >> 8];
             const int npad = (r.w >> 1) & 0x1ff;
-            tb[j] = dot_fv(F + r.x + (itm & 255) * fstride(npad), vb + r.y, npad);
+            tb[j] = dot_col(F + r.x + (itm & 255) * fstride(npad), vb + r.y, npad);
         }
         __syncthreads();
         for (int k = tid; k < nk; k += nthr) {
             fetch(s, k, seg, own);
             const T old = s.state();
-            s.local_update(F, tb, g);
+            s.template local_update<false, false>(F, tb, g, 0, 1);
             pack(slots[k], s);
             if ((seg & 255) > 1) xput(Xout, (seg >> 8) + own, s.u, (unsigned)it + 1u);
             if constexpr (CHK) {
@@ -790,7 +1044,7 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
                 U[(seg >> 8) + own] = s.u;
             }
         }
-        if constexpr (CHK) return test_iteration(m, pp, acc, it, check_every, P, bar_extra, ++nb, st, rho_d);
+        if constexpr (CHK) return test_iteration<false>(m, pp, 0u, acc, it, check_every, P, nb++, st, rho_d);
         return true;
     };
     for (int it = 0; it < n_iters && running; ++it) {
@@ -798,7 +1052,7 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
         else running = iteration(it, std::false_type{});
     }
     for (int k = tid; k < nk; k += nthr) {
-        Slot<T> s;
+        Slot<T, false> s;
         int seg, own;
         fetch(s, k, seg, own);
         s.save(g, k0 + k);
@@ -810,24 +1064,55 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
 template <typename T>
 const void *persist_fn(const PersistLayout &lay) {
     if (!lay.local) return (const void *)k_persist_engine<T>;
-    return lay.split ? (const void *)k_persist_local<T, true> : (const void *)k_persist_local<T, false>;
+    if constexpr (sizeof(T) == 8) {
+        if (lay.split)
+            return lay.cluster ? (const void *)k_persist_local<T, true, true> : (const void *)k_persist_local<T, true, false>;
+    }
+    return lay.cluster ? (const void *)k_persist_local<T, false, true> : (const void *)k_persist_local<T, false, false>;
 }
 
 }  // namespace
 
-template <typename T>
-int prepare_persist_engine(const PersistLayout &lay) {
-    return cudaFuncSetAttribute(persist_fn<T>(lay), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes) ==
-                   cudaSuccess ? 0 : -1;
+static void fill_cfg(const PersistLayout &lay, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, cudaStream_t s) {
+    memset(cfg, 0, sizeof(*cfg));
+    cfg->gridDim = dim3(lay.P, 1, 1);
+    cfg->blockDim = dim3(lay.threads, 1, 1);
+    cfg->dynamicSmemBytes = lay.bytes;
+    cfg->stream = s;
+    if (lay.cluster) {
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = lay.P;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+    } else {
+        attr[0].id = cudaLaunchAttributeCooperative;
+        attr[0].val.cooperative = 1;
+    }
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
 }
 
-// CTAs per SM.
 template <typename T>
-int persist_occupancy(const PersistLayout &lay) {
+int prepare_persist_engine(const PersistLayout &lay) {
+    const void *fn = persist_fn<T>(lay);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes) != cudaSuccess) return -1;
+    if (lay.cluster && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return -1;
+    return 0;
+}
+
+// CTAs that can be resident on n_sm SMs (a cluster: its own P, or 0).
+template <typename T>
+long long persist_resident(const PersistLayout &lay, int n_sm) {
     int n = 0;
+    if (lay.cluster) {
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[1];
+        fill_cfg(lay, &cfg, attr, 0);
+        return cudaOccupancyMaxActiveClusters(&n, persist_fn<T>(lay), &cfg) == cudaSuccess && n > 0 ? lay.P : 0;
+    }
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, persist_fn<T>(lay), lay.threads, lay.bytes) != cudaSuccess)
         return 0;
-    return n;
+    return (long long)n * n_sm;
 }
 
 // Bytes of a plan's exchange buffer: two buffers of L entries.
@@ -839,29 +1124,20 @@ int launch_persist_engine(const IterArgs<T> &g, const PersistLayout &lay, const 
                           int bar_extra, int n_iters, int check_every, DevStatus *st, double rho,
                           cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {
     // the barrier counter starts at 0 in every launch
-    if (cudaMemsetAsync(pp.sync, 0, sizeof(unsigned long long), s) != cudaSuccess) return -1;
+    if (!lay.cluster && cudaMemsetAsync(pp.sync, 0, sizeof(unsigned long long), s) != cudaSuccess) return -1;
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(lay.P, 1, 1);
-    cfg.blockDim = dim3(lay.threads, 1, 1);
-    cfg.dynamicSmemBytes = lay.bytes;
-    cfg.stream = s;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    fill_cfg(lay, &cfg, attr, s);
     IterArgs<T> ga = g;
     PersistLayout la = lay;
     PersistPtrs pa = pp;
     void *args[] = {&ga, &la, &pa, &U, &bar_extra, &n_iters, &check_every, &st, &rho, &cond, &use_cond};
-    const cudaError_t e = cudaLaunchKernelExC(&cfg, persist_fn<T>(lay), args);
-    return e == cudaSuccess ? 0 : -1;
+    return cudaLaunchKernelExC(&cfg, persist_fn<T>(lay), args) == cudaSuccess ? 0 : -1;
 }
 
 #define OPF_PERSIST_INST(T)                                                                                   \
     template int prepare_persist_engine<T>(const PersistLayout &);                                                        \
-    template int persist_occupancy<T>(const PersistLayout &);     template size_t persist_exchange_bytes<T>(int);                                                        \
+    template long long persist_resident<T>(const PersistLayout &, int);   template size_t persist_exchange_bytes<T>(int);                                                        \
     template int launch_persist_engine<T>(const IterArgs<T> &, const PersistLayout &, const PersistPtrs &,  \
                                           T *, int, int, int, DevStatus *, double,                            \
                                           cudaGraphConditionalHandle, int, cudaStream_t);

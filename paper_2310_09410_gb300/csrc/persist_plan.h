@@ -19,31 +19,71 @@ namespace opf {
 
 // Part p owns the subsystems sub[s0[p] .. s0[p+1]) and, in that order, their
 // slots slot[k0[p] .. k0[p+1]).  A part sees u through an array of its own
-// slots (index = position in the part) followed by the entries it reads from
-// other parts, rem[r0[p] .. r0[p+1]) (positions in the global-major copy
-// order).  For every global of the part with two or more copies, list[l0[p]
-// ..] holds the array index of each copy in copy order; seg[k] = (offset of the
-// list in the part's << 8) | copies of the slot's global (offset 0 for a
-// single copy), out[k] = the slot's position in the copy order when another
-// part reads it, else -1.
+// slots (index = position in the part), then the entries it reads from other
+// parts, rem[r0[p] .. r0[p+1]) (positions in the global-major copy order), then
+// one zero.  For every global of the part with two or more copies, list (16-bit
+// entries, part p's from 8 l0[p]) holds the array index of each copy in copy
+// order, padded with the zero's index to a multiple of 8; seg[k] = (number of
+// the list's first 8 entries in the part << 8) | copies of the slot's global
+// (list 0 for a single copy), out[k] = the slot's position in the copy order
+// when another part reads it, else -1.  ok: the indices fit 16 bits.
 struct PersistParts {
     std::vector<int> s0, k0, r0, l0;
-    std::vector<int> sub, slot, rem, list, seg, out;
+    std::vector<int> sub, slot, rem, seg, out;
+    std::vector<unsigned short> list;
+    bool ok = true;
 };
 
+// Destinations of the exported u when the parts' readers are written to
+// directly: per position j of slot[] a list dst[..] of part << 16 | index in
+// the reader's remote entries, dseg[j] = (offset in the part's lists << 8) |
+// count, part p's lists from d0[p].
+struct PersistDests {
+    std::vector<int> d0, dst, dseg;
+    int most = 0;                     // longest part's lists
+    bool ok = true;                   // counts and indices fit their fields
+};
+
+inline PersistDests persist_dests(int P, const PersistParts &t, const std::vector<int> &uslot) {
+    const int L = (int)t.slot.size();
+    PersistDests d;
+    std::vector<int> pos(L), n(L, 0);            // position of a slot
+    for (int j = 0; j < L; ++j) pos[t.slot[j]] = j;
+    for (int c : t.rem) ++n[pos[uslot[c]]];
+    d.dseg.assign(L, 0);
+    d.d0.assign(P + 1, 0);
+    std::vector<int> fill(L);
+    int at = 0;
+    for (int p = 0; p < P; ++p) {
+        for (int j = t.k0[p]; j < t.k0[p + 1]; ++j) {
+            if (n[j] > 255 || at - d.d0[p] >= (1 << 22)) d.ok = false;
+            d.dseg[j] = ((at - d.d0[p]) << 8) | (n[j] & 255);
+            fill[j] = at;
+            at += n[j];
+        }
+        d.d0[p + 1] = at;
+        d.most = std::max(d.most, at - d.d0[p]);
+    }
+    d.dst.assign(at, 0);
+    for (int p = 0; p < P; ++p) {
+        if (t.r0[p + 1] - t.r0[p] > 0xffff) d.ok = false;
+        for (int i = t.r0[p]; i < t.r0[p + 1]; ++i) d.dst[fill[pos[uslot[t.rem[i]]]]++] = (p << 16) | ((i - t.r0[p]) & 0xffff);
+    }
+    return d;
+}
+
 // Depth-first order of the S subsystems.  Slots of subsystem d are
-// [soff[d], soff[d + 1]) with global gk[k]; the copies of global i are
-// uslot[gstart[i] .. gstart[i + 1]).  start: the order in which unvisited
-// subsystems begin a new tree.
-inline std::vector<int> persist_order(int S, const std::vector<int> &soff, const std::vector<int> &gk,
-                                      const std::vector<int> &gstart, const std::vector<int> &uslot,
-                                      const std::vector<int> &start) {
-    std::vector<int> sub_of(gk.size()), order, stack;
+// [soff[d], soff[d + 1]); segp[k] = (first copy of the slot's global in the
+// global-major copy order << 8) | copies, pk[k] the slot's own position there.
+// start: the order in which unvisited subsystems begin a new tree.
+inline std::vector<int> persist_order(int S, const std::vector<int> &soff, const std::vector<int> &segp,
+                                      const std::vector<int> &pk, const std::vector<int> &start) {
+    std::vector<int> sub_of(pk.size()), order, stack;        // subsystem of a copy
     for (int d = 0; d < S; ++d)
-        for (int k = soff[d]; k < soff[d + 1]; ++k) sub_of[k] = d;
-    std::vector<char> seen(S, 0), walked(gstart.size(), 0);
+        for (int k = soff[d]; k < soff[d + 1]; ++k) sub_of[pk[k]] = d;
+    std::vector<char> seen(S, 0), walked(pk.size(), 0);      // walked: by first copy
     order.reserve(S);
-    std::vector<int> by_count;
+    std::vector<int> by_count;                                // globals of a subsystem (segp words)
     for (int first : start) {
         if (seen[first]) continue;
         stack.push_back(first);
@@ -56,35 +96,32 @@ inline std::vector<int> persist_order(int S, const std::vector<int> &soff, const
             // the globals with the fewest copies pushed last, so followed first
             by_count.clear();
             for (int k = soff[d]; k < soff[d + 1]; ++k) {
-                const int g = gk[k], cnt = gstart[g + 1] - gstart[g];
-                if (cnt < 2 || walked[g]) continue;      // no other copy, or all on the stack or seen
-                walked[g] = cnt > 2;
-                size_t at = by_count.size();             // insertion sort: few and short
-                by_count.push_back(g);
-                while (at > 0 && gstart[by_count[at - 1] + 1] - gstart[by_count[at - 1]] < cnt) {
+                const int sp = segp[k], cnt = sp & 255;
+                if (cnt < 2 || walked[sp >> 8]) continue;    // no other copy, or all on the stack or seen
+                walked[sp >> 8] = cnt > 2;
+                size_t at = by_count.size();                 // insertion sort: few and short
+                by_count.push_back(sp);
+                while (at > 0 && (by_count[at - 1] & 255) < cnt) {
                     by_count[at] = by_count[at - 1];
                     --at;
                 }
-                by_count[at] = g;
+                by_count[at] = sp;
             }
-            for (int g : by_count) {
-                for (int q = gstart[g + 1] - 1; q >= gstart[g]; --q)
-                    if (!seen[sub_of[uslot[q]]]) stack.push_back(sub_of[uslot[q]]);
-            }
+            for (int sp : by_count)
+                for (int c = (sp >> 8) + (sp & 255) - 1; c >= sp >> 8; --c)
+                    if (!seen[sub_of[c]]) stack.push_back(sub_of[c]);
         }
     }
     return order;
 }
 
-// P parts of the given order, balanced by cost[d].
+// P parts of the given order, balanced by cost[d].  Subsystems are numbered in
+// decreasing size (so a part's are sorted by number).
 inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, const std::vector<double> &cost,
-                                  const std::vector<int> &soff, const std::vector<int> &gk,
-                                  const std::vector<int> &pk, const std::vector<int> &gstart,
-                                  const std::vector<int> &uslot) {
+                                  const std::vector<int> &soff, const std::vector<int> &segp,
+                                  const std::vector<int> &pk) {
     PersistParts t;
-    const int L = (int)gk.size(), G = (int)gstart.size() - 1;
-    t.slot.reserve(L);
-    t.list.reserve(2 * (size_t)L);
+    const int L = (int)pk.size();
     t.s0.assign(P + 1, S);
     t.s0[0] = 0;
     double total = 0, acc = 0;
@@ -95,52 +132,64 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
         while (p < P && acc >= total * p / P) t.s0[p++] = i + 1;
     }
     t.sub = order;
-    for (int q = 0; q < P; ++q)
-        std::stable_sort(t.sub.begin() + t.s0[q], t.sub.begin() + t.s0[q + 1], [&](int a, int b) {
-            return soff[a + 1] - soff[a] > soff[b + 1] - soff[b];
-        });
-    std::vector<int> part_of(L), at(L);          // per slot: part, position in it
+    for (int q = 0; q < P; ++q) std::sort(t.sub.begin() + t.s0[q], t.sub.begin() + t.s0[q + 1]);
+    // per copy (in copy order) its part and position there, so that a list
+    // reads one run of memory
+    struct Place { int part, at; };
+    std::vector<Place> place(L);
     t.k0.assign(P + 1, 0);
-    for (int q = 0; q < P; ++q) {
+    t.slot.resize(L);
+    for (int q = 0, j = 0; q < P; ++q) {
         for (int i = t.s0[q]; i < t.s0[q + 1]; ++i)
-            for (int k = soff[t.sub[i]]; k < soff[t.sub[i] + 1]; ++k) {
-                part_of[k] = q;
-                at[k] = (int)t.slot.size() - t.k0[q];
-                t.slot.push_back(k);
+            for (int k = soff[t.sub[i]]; k < soff[t.sub[i] + 1]; ++k, ++j) {
+                place[pk[k]] = {q, j - t.k0[q]};
+                t.slot[j] = k;
             }
-        t.k0[q + 1] = (int)t.slot.size();
+        t.k0[q + 1] = j;
     }
-    t.seg.assign(L, 0);
+    t.seg.resize(L);
     t.out.assign(L, -1);
+    t.list.reserve(4 * (size_t)L);
     t.r0.assign(P + 1, 0);
     t.l0.assign(P + 1, 0);
-    std::vector<int> done(G, -1), where(G, 0);
-    std::vector<char> read(L, 0);                // per slot: another part reads it
+    std::vector<int> where(L, -1);               // by first copy: number of the part's list, or below l0[part]
     for (int q = 0; q < P; ++q) {
-        const int nk = t.k0[q + 1] - t.k0[q];
+        const int nk = t.k0[q + 1] - t.k0[q], l0 = t.l0[q], r0 = t.r0[q];
         for (int j = t.k0[q]; j < t.k0[q + 1]; ++j) {
-            const int k = t.slot[j], g = gk[k], c0 = gstart[g], cnt = gstart[g + 1] - c0;
-            if (cnt > 1 && done[g] != q) {
-                done[g] = q;
-                where[g] = (int)t.list.size() - t.l0[q];
-                for (int c = c0; c < c0 + cnt; ++c) {
-                    const int o = uslot[c];
-                    if (part_of[o] == q) {
-                        t.list.push_back(at[o]);
-                    } else {
-                        t.list.push_back(nk + (int)t.rem.size() - t.r0[q]);
-                        t.rem.push_back(c);
-                        read[o] = 1;
+            const int sp = segp[t.slot[j]], c0 = sp >> 8, cnt = sp & 255;
+            if (cnt == 1) {
+                t.seg[j] = 1;
+                continue;
+            }
+            if (where[c0] < l0) {
+                where[c0] = (int)(t.list.size() / 8);
+                unsigned short e[8];
+                for (int c = c0, n = 0; c < c0 + cnt || n; ++c) {
+                    e[n] = 0xffff;               // past the last copy: the zero, below
+                    if (c < c0 + cnt) {
+                        if (place[c].part == q) {
+                            e[n] = (unsigned short)place[c].at;
+                        } else {
+                            e[n] = (unsigned short)(nk + (int)t.rem.size() - r0);
+                            t.rem.push_back(c);
+                            t.out[t.k0[place[c].part] + place[c].at] = c;
+                        }
+                    }
+                    if (++n == 8) {
+                        t.list.insert(t.list.end(), e, e + 8);
+                        n = 0;
                     }
                 }
             }
-            t.seg[j] = ((cnt > 1 ? where[g] : 0) << 8) | cnt;
+            t.seg[j] = ((where[c0] - l0) << 8) | cnt;
         }
         t.r0[q + 1] = (int)t.rem.size();
-        t.l0[q + 1] = (int)t.list.size();
+        t.l0[q + 1] = (int)(t.list.size() / 8);
+        const int zero = nk + t.r0[q + 1] - r0;
+        if (zero >= 0xffff) t.ok = false;
+        for (size_t i = 8 * (size_t)l0; i < t.list.size(); ++i)
+            if (t.list[i] == 0xffff) t.list[i] = (unsigned short)zero;
     }
-    for (int j = 0; j < L; ++j)
-        if (read[t.slot[j]]) t.out[j] = pk[t.slot[j]];
     return t;
 }
 

@@ -3,8 +3,9 @@ with g++ and checked on the CPU: on random consensus structures and part
 counts (one part, more parts than subsystems), every subsystem and slot in
 exactly one part and in decreasing size there, every global's copy list
 reading exactly its copies in copy order through the part's own slots and its
-remote entries, and the exported slots exactly those another part reads.  A
-planted wrong list entry fails it.
+remote entries (padded with the zero's index), the exported slots exactly those
+another part reads, and an export's destinations exactly its readers' entries.
+A planted wrong list entry fails it.
 
 On the GPU: the engine's two forms (one slot per thread; several, where a
 part has more than 512 slots) on consensus instances with wide, rank-deficient
@@ -26,6 +27,22 @@ DRIVER = r"""
 #include <random>
 using namespace opf;
 static int fail(const char *what, int seed) { std::printf("FAIL %s seed %d\n", what, seed); return 1; }
+
+static int check_dests(const PersistParts &t, int P, const std::vector<int> &uslot, int seed) {
+    const PersistDests d = persist_dests(P, t, uslot);
+    size_t n = 0;
+    for (int p = 0; p < P; ++p)
+        for (int j = t.k0[p]; j < t.k0[p + 1]; ++j) {
+            const int o = d.d0[p] + (d.dseg[j] >> 8), cnt = d.dseg[j] & 255;
+            if (o + cnt > d.d0[p + 1] || (cnt > 0) != (t.out[j] >= 0)) return fail("destination range", seed);
+            for (int i = o; i < o + cnt; ++i, ++n) {
+                const int r = d.dst[i] >> 16, e = d.dst[i] & 0xffff;
+                if (r == p || t.r0[r] + e >= t.r0[r + 1] || uslot[t.rem[t.r0[r] + e]] != t.slot[j])
+                    return fail("destination", seed);
+            }
+        }
+    return n == t.rem.size() && d.ok ? 0 : fail("destination count", seed);
+}
 
 static int check(const PersistParts &t, int P, int S, const std::vector<int> &soff, const std::vector<int> &gk,
                  const std::vector<int> &pk, const std::vector<int> &gstart, const std::vector<int> &uslot, int seed) {
@@ -55,9 +72,11 @@ static int check(const PersistParts &t, int P, int S, const std::vector<int> &so
             if ((t.seg[j] & 255) != cnt) return fail("copies", seed);
             if (cnt == 1) continue;
             const int o = t.seg[j] >> 8;
-            if (o < 0 || o + cnt > nl) return fail("list range", seed);
+            if (o < 0 || 8 * o + cnt > 8 * nl) return fail("list range", seed);
+            for (int q = cnt; q % 8; ++q)
+                if (t.list[8 * (t.l0[p] + o) + q] != nk + nr) return fail("list padding", seed);
             for (int q = 0; q < cnt; ++q) {
-                const int e = t.list[t.l0[p] + o + q];
+                const int e = t.list[8 * (t.l0[p] + o) + q];
                 if (e < 0 || e >= nk + nr) return fail("list entry range", seed);
                 const int c = e < nk ? pk[t.slot[t.k0[p] + e]] : t.rem[t.r0[p] + e - nk];
                 if (c != gstart[g] + q) return fail("list entry", seed);
@@ -101,11 +120,14 @@ int main() {
         for (int i = 0; i < G; ++i) gstart[i + 1] += gstart[i];
         std::vector<int> fill(gstart.begin(), gstart.end() - 1);
         for (int k = 0; k < L; ++k) { pk[k] = fill[gk[k]]++; uslot[pk[k]] = k; }
-        std::vector<int> order = persist_order(S, soff, gk, gstart, uslot, start);
+        std::vector<int> segp(L);
+        for (int k = 0; k < L; ++k) segp[k] = (gstart[gk[k]] << 8) | (gstart[gk[k] + 1] - gstart[gk[k]]);
+        std::vector<int> order = persist_order(S, soff, segp, pk, start);
         if ((int)order.size() != S) return fail("order", seed);
         const int P = seed % 5 == 0 ? 1 : 1 + (int)(rng() % (S + 5));
-        PersistParts t = persist_parts(P, S, order, cost, soff, gk, pk, gstart, uslot);
-        if (check(t, P, S, soff, gk, pk, gstart, uslot, seed)) return 1;
+        PersistParts t = persist_parts(P, S, order, cost, soff, segp, pk);
+        if (!t.ok || check(t, P, S, soff, gk, pk, gstart, uslot, seed)) return 1;
+        if (check_dests(t, P, uslot, seed)) return 1;
         if (seed == 7 && t.list.size() > 1) {
             PersistParts bad = t;
             bad.list[0] ^= 1;
@@ -175,3 +197,51 @@ def test_kept_plans_serve_new_loads(precision):
             with opf.Solver.from_feeder(f) as fresh:
                 y, want = solved(fresh)
             assert np.array_equal(x, y) and obj == want
+
+
+def one_cluster_instances():
+    from paper_2310_09410_gb300 import opf, synth
+
+    out = [lambda n=n, s=s: opf.Solver.from_feeder(synth.preset_feeder(n, s))
+           for n, s in (("13", 1001), ("34", 5034), ("123", 2001))]
+    out.append(lambda: opf.Solver.from_feeder(synth.make_feeder(2, 1, 1, seed=3)))
+    # blocks up to 63 slots (two warps in the warp engine, odd halves), rank-deficient, free variables
+    for seed, n, subs, widest in ((41, 90, 20, 63), (42, 40, 3, 39), (43, 200, 150, 9)):
+        g = synth.random_generic(seed, n_global=n, n_sub=subs, max_n=widest, p_free=0.3)
+        out.append(lambda g=g: opf.Solver.from_generic(g["c"], g["lb"], g["ub"], g["subs"]))
+    return out
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("case", range(7))
+def test_one_cluster_form_equals_warp_engine(case):
+    """FP32 iterates of the one-cluster form (the automatic choice at these
+    sizes) are the warp engine's bit for bit."""
+    from paper_2310_09410_gb300 import opf
+
+    got = []
+    for engine in (opf.ENGINE_AUTO, opf.ENGINE_WARP):
+        with one_cluster_instances()[case]() as s:
+            s.precompute()
+            s.solve(eps_rel=0.0, max_iter=700, check_every=50, precision=opf.PREC_FP32, engine=engine)
+            got.append(s.locals() + s.solution())
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.gpu
+def test_one_cluster_bounded_wait():
+    """A wait that can never end (the test hook) gives OPF_E_TIMEOUT, and the
+    handle iterates afterwards."""
+    from paper_2310_09410_gb300 import opf, synth
+
+    with opf.Solver.from_feeder(synth.preset_feeder("13", 1001)) as s:
+        s.precompute()
+        for precision in (opf.PREC_FP64, opf.PREC_FP32):
+            with pytest.raises(opf.OPFError) as e:
+                s.solve(eps_rel=0.0, max_iter=100, check_every=50, precision=precision,
+                        flags=opf.SOLVE_TEST_BARRIER_TIMEOUT)
+            assert e.value.code == opf.OPF_E_TIMEOUT
+            s.reset()
+            s.solve(eps_rel=0.0, max_iter=100, check_every=50, precision=precision)
+            assert s.residuals()["iters"] == 100
