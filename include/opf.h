@@ -259,8 +259,8 @@ int opf_get_timing(opf_handle *h, double *ms, int n);
  *   objective  device, 1 double out: c^T x
  *   stream     cudaStream_t (NULL = legacy default stream); the call only
  *              enqueues work, synchronise the stream before reading outputs.
- * Scratch is a fixed device array of OPF_STATIC_MAX_BLOCKS doubles, one per
- * block of 256 globals, held by every device that loads the library until
+ * Scratch is a fixed device array of OPF_STATIC_MAX_BLOCKS doubles (a partial
+ * sum per block of threads), held by every device that loads the library until
  * the process exits.  The first call in a CUDA context (the stream's; a
  * stream of an SM partition has its own) is the set-up: it looks up the
  * array's address in that context, and the CUDA driver may load the

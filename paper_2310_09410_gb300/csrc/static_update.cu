@@ -5,11 +5,12 @@
 // allocation once they run (an allocation may block or fail at any time), and
 // hosts whose device memory is handed out only by their own allocator (a
 // framework's caching allocator that owns the whole device).  Its scratch (one
-// FP64 objective partial per block of 256 globals) is a file-scope __device__
+// FP64 objective partial per block) is a file-scope __device__
 // array instead of memory from a handle, so the call allocates nothing.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <map>
 #include <mutex>
@@ -20,46 +21,99 @@
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kOneBlock = 512;       // up to so many globals run in one block, which sums the objective itself
+                                     // (181 / 408 globals 7.6 / 7.9 us a call against 9.6 with a second kernel,
+                                     // 1024 globals 10.3 against 9.6)
+constexpr int kBlocks = 8 * 152;     // resident blocks of the GPU: more globals than threads go round by round
+constexpr int kRecip = 16;           // 1 / (rho N) by copy count below this
 
 // Per-block partial sums of c^T x.  Shared by every call in a CUDA context and
 // kept between calls; each call writes the entries it later reads.
 static __device__ __align__(256) double g_static_partials[OPF_STATIC_MAX_BLOCKS];
 
-// x_i = clip((sum of u over the copies of global i - c_i) / (rho N_i), lb_i, ub_i)
-// and the block's share of c^T x.
-__global__ void __launch_bounds__(kThreads) k_global_update_static(int n, const int *seg_off, const double *u,
-                                                                   const double *c, const double *lb,
-                                                                   const double *ub, double rho, double *x,
-                                                                   double *partials) {
-    __shared__ double red[kThreads];
-    const int i = blockIdx.x * kThreads + threadIdx.x;
-    double o = 0.0;
-    if (i < n) {
-        const int a = seg_off[i], b = seg_off[i + 1];
-        double sigma = 0.0;
-        for (int q = a; q < b; ++q) sigma += u[q];
-        double xv = (sigma - c[i]) / (rho * (double)(b - a));
-        if (xv < lb[i]) xv = lb[i];
-        if (xv > ub[i]) xv = ub[i];
-        x[i] = xv;
-        o = c[i] * xv;
-    }
-    red[threadIdx.x] = o;
-    __syncthreads();
-    for (int w = kThreads >> 1; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partials[blockIdx.x] = red[0];
+struct Recips {
+    double r[kRecip];                // 1 / (rho N), 0 where that is not a normal number (then the division is done)
+};
+
+// What bounds these kernels: the FP64 pipe (a warp's FP64 instruction occupies
+// its sub-partition's for about 64 cycles; 2 million globals in 15 us of memory
+// traffic), so the forms below count FP64 instructions.
+
+// num / den: one multiply by den's reciprocal and one correction step (the
+// quotient's residual by FMA) instead of the 20-odd instructions of a division;
+// the same to the last bit but one.  Infinite and NaN quotients are the
+// multiply's.
+__device__ __forceinline__ double quotient(double num, double den, double rcp) {
+    const double q = num * rcp;
+    if ((__double2hiint(q) & 0x7ff00000) == 0x7ff00000) return q;
+    return fma(fma(-q, den, num), rcp, q);
 }
 
-// Objective: the block partials summed in block order by one thread.
-__global__ void k_sum_partials_static(int nblk, const double *partials, double *objective) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += partials[b];
-        *objective = s;
+// Order-preserving integer of a double that is not NaN.
+__device__ __forceinline__ long long ordered(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// x_i = clip((sum of u over the copies of global i - c_i) / (rho N_i), lb_i, ub_i)
+__device__ __forceinline__ double global_update(int a, int b, const double *u, double c, double lb, double ub,
+                                                double rho, const Recips &rc) {
+    const int cnt = b - a;
+    double sigma = cnt > 0 ? u[a] : 0.0;
+    for (int q = a + 1; q < b; ++q) sigma += u[q];
+    const double num = sigma - c;
+    const double rcp = cnt > 0 && cnt < kRecip ? rc.r[cnt] : 0.0;
+    double x = rcp != 0.0 ? quotient(num, rho * (double)cnt, rcp) : num / (rho * (double)cnt);
+    if ((unsigned long long)(__double_as_longlong(x) << 1) <= 0xffe0000000000000ull) {   // NaN stays NaN
+        if (ordered(x) < ordered(lb)) x = lb;
+        if (ordered(x) > ordered(ub)) x = ub;
     }
+    return x;
+}
+
+// Sum over a block in a fixed order, in thread 0.
+__device__ __forceinline__ double block_sum(double v) {
+    __shared__ double red[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) red[w] = v;
+    __syncthreads();
+    if (w == 0) {
+        v = lane < nw ? red[lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    return v;
+}
+
+// The update of every global (round by round when there are more than threads)
+// and each block's share of c^T x in out[block] (one block: the objective).
+__global__ void __launch_bounds__(kOneBlock) k_global_update_static(int n, const int *seg_off, const double *u,
+                                                                    const double *c, const double *lb,
+                                                                    const double *ub, double rho, Recips rc, double *x,
+                                                                    double *out) {
+    double o = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const double ci = c[i];
+        const double xv = global_update(seg_off[i], seg_off[i + 1], u, ci, lb[i], ub[i], rho, rc);
+        x[i] = xv;
+        o = fma(ci, xv, o);
+    }
+    o = block_sum(o);
+    if (threadIdx.x == 0) out[blockIdx.x] = o;
+}
+
+// Objective: the block partials summed in a fixed order by one block.  (By one
+// thread, 248 dependent adds took 15 of the 24.6 us of a 63,405-global call;
+// with the block sum and the forms above a call takes 10.6 us, most of it the
+// two launches, and one of 2 million globals 61 us, where 1 million took 250.)
+__global__ void __launch_bounds__(kThreads) k_sum_partials_static(int nblk, const double *partials,
+                                                                  double *objective) {
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += kThreads) s += partials[b];
+    s = block_sum(s);
+    if (threadIdx.x == 0) *objective = s;
 }
 
 // Driver entry points fetched through the runtime (no link-time dependency
@@ -119,8 +173,7 @@ extern "C" int opf_global_update_static(int32_t n, const int32_t *seg_off, const
                                         double *objective, void *stream) {
     if (n < 1 || !seg_off || !u || !c || !lb || !ub || !x || !objective || !(rho > 0.0))
         return fail(OPF_E_INVALID, "need n >= 1, rho > 0 and non-null device pointers");
-    const long long nblk = ((long long)n + kThreads - 1) / kThreads;
-    if (nblk > OPF_STATIC_MAX_BLOCKS)
+    if (n > OPF_STATIC_MAX_GLOBALS)
         return fail(OPF_E_CAPACITY, "n = " + std::to_string(n) + " exceeds OPF_STATIC_MAX_GLOBALS (" +
                                         std::to_string(OPF_STATIC_MAX_GLOBALS) + ")");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -165,8 +218,19 @@ extern "C" int opf_global_update_static(int32_t n, const int32_t *seg_off, const
             g_dev_ptr[id] = partials;
         }
     }
-    k_global_update_static<<<(unsigned)nblk, kThreads, 0, s>>>(n, seg_off, u, c, lb, ub, rho, x, partials);
-    k_sum_partials_static<<<1, 32, 0, s>>>((int)nblk, partials, objective);
+    Recips rc;
+    for (int k = 0; k < kRecip; ++k) {
+        const double den = rho * (double)k, r = k ? 1.0 / den : 0.0;
+        rc.r[k] = std::isnormal(r) && std::isnormal(den) ? r : 0.0;
+    }
+    if (n <= kOneBlock) {
+        k_global_update_static<<<1, (unsigned)((n + 31) / 32 * 32), 0, s>>>(n, seg_off, u, c, lb, ub, rho, rc, x,
+                                                                            objective);
+    } else {
+        const int nblk = std::min((n + kThreads - 1) / kThreads, kBlocks);
+        k_global_update_static<<<(unsigned)nblk, kThreads, 0, s>>>(n, seg_off, u, c, lb, ub, rho, rc, x, partials);
+        k_sum_partials_static<<<1, kThreads, 0, s>>>(nblk, partials, objective);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(OPF_E_CUDA, std::string("launch: ") + cudaGetErrorString(e));
     return OPF_OK;
