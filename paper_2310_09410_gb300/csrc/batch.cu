@@ -65,9 +65,17 @@ __device__ __forceinline__ void st4(double *p, const Q4<double> &q) {
     *reinterpret_cast<double2 *>(p + 2) = make_double2(q.v[2], q.v[3]);
 }
 
-template <typename T>
-__device__ __forceinline__ T clampT(T x, T lo, T hi) {
-    return x < lo ? lo : (x > hi ? hi : x);
+__device__ __forceinline__ float clampT(float x, float lo, float hi) { return x < lo ? lo : (x > hi ? hi : x); }
+// FP64: compared as order-preserving integers (a double's bits, the lower 63
+// flipped when negative); an FP64 compare occupies a sub-partition's FP64 pipe
+// for about 64 cycles, as an FMA does.  NaN stays NaN.
+__device__ __forceinline__ long long ordered(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double clampT(double x, double lo, double hi) {
+    if (((unsigned long long)__double_as_longlong(x) << 1) > 0xffe0000000000000ull) return x;
+    return ordered(x) < ordered(lo) ? lo : (ordered(x) > ordered(hi) ? hi : x);
 }
 
 }  // namespace
@@ -251,7 +259,7 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const T *Fs, T *
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            y[4 * q + e] = TM ? b4.v[e] : rho * b4.v[e];
+            y[4 * q + e] = TM || sizeof(T) == 8 ? b4.v[e] : rho * b4.v[e];   // (FP64 arrays hold rho bbar~)
             v[4 * q + e] = us[upos<K>(ch, e, sc)] + m4.v[e];
         }
     }
@@ -304,10 +312,13 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const T *Fs, T *
             m4.v[e] = mun;
             u4.v[e] = rx - mun;
         }
-        // x_s~ (written on wds iterations, test terms); computed on every
-        // iteration: a branch here measured 6 % slower per launch
+        // x_s~ (written on wds iterations, test terms); in FP32 computed on
+        // every iteration (a branch here measured 6 % slower per launch), in
+        // FP64, where a multiply costs 64 cycles, only when it is used
+        if (sizeof(T) == 4 || wds) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) x4.v[e] = r4.v[e] * inv_rho;
+            for (int e = 0; e < 4; ++e) x4.v[e] = r4.v[e] * inv_rho;
+        }
         if (check) {
             const int4 g4 = __ldg(chg + ch);
             const int gg[4] = {g4.x, g4.y, g4.z, g4.w};
@@ -517,13 +528,17 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
             for (int j = 0; j < GB; ++j) {
                 const int cnt = gtj[j].z & 0xff;
+                if constexpr (sizeof(T) == 8) {          // no add of the first copy to zero
+                    if (cnt > 0) load_row<T, KQ, false>(sum[j], us + row0[j]);
+                } else {
 #pragma unroll
-                for (int k = 0; k < KQ; ++k) sum[j].v[k] = T(0);
-                if (cnt > 0) {
-                    RowK<T, KQ> u0;
-                    load_row<T, KQ, false>(u0, us + row0[j]);
+                    for (int k = 0; k < KQ; ++k) sum[j].v[k] = T(0);
+                    if (cnt > 0) {
+                        RowK<T, KQ> u0;
+                        load_row<T, KQ, false>(u0, us + row0[j]);
 #pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] += u0.v[k];
+                        for (int k = 0; k < KQ; ++k) sum[j].v[k] += u0.v[k];
+                    }
                 }
                 if (cnt > 1) {
                     RowK<T, KQ> u1;
@@ -913,7 +928,9 @@ __device__ __forceinline__ void bref_one(int in, bool valid, int d, int l0, int 
         const size_t e = (((size_t)cta * NCH + (p >> 2)) * K + sc) * 4 + (p & 3);
         const double btv = mv + bi[k] - xg;
         const double dg = dr[gk[k]];
-        bt[e] = (T)(mode ? btv : -btv);      // the engine starts y at this value
+        // the engine starts y at rho times this; the FP64 arrays hold the product
+        const double yv0 = mode ? btv : -btv;
+        bt[e] = sizeof(T) == 8 ? (T)(rho * yv0) : (T)yv0;
         ds[e] = (T)(xi[k] - xg);
         mu[e] = (T)dg;
         lref[e] = (T)(li[k] - dg);

@@ -341,16 +341,26 @@ int run_loop(opf_batch *b, BPlan &p, double rho, int R, int k, bool host_loop) {
 }
 
 // Plans: FP32 shapes tried on the batch (fastest wins) unless fixed by
-// opf_batch_set_shape; FP64 uses the largest K <= 4 that fits.
+// opf_batch_set_shape; FP64 spreads the instances over the SMs (below).
 int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
     BPlan &p = dbl ? b->p64 : b->p32;
     if (p.ok) return OPF_OK;
     opf_handle *h = b->h;
     if (dbl) {
-        // factors in shared memory when they fit, else read through L1/L2 (the
-        // FP64 iteration is bound by the FP64 FMA rate either way)
-        const int fk = b->force_k64, fw = b->force_w64 > 0 ? b->force_w64 : 16;
-        const int ks[] = {4, 2, 1};
+        // The FP64 iteration is bound by the FP64 pipes of the SMs it runs on, so
+        // the instances are spread over the SMs: as few per CTA as give every SM
+        // at most one CTA (1 / 2 / 4 per CTA take 32 / 48 / 90 us per iteration
+        // on the 123-bus feeder, 14 / 17 / 26 on the 34-bus one, as long as there
+        // is an SM per CTA; 1024 instances of 123 buses 190 / 184 / 181 us), 4
+        // beyond that.  8 warps: 16 measured 0.3 % faster to 28 % slower.
+        // Factors in shared memory when they fit, else read through L1/L2.
+        const int fk = b->force_k64, fw = b->force_w64 > 0 ? b->force_w64 : 8;
+        const int n_sm = stream_sm_count(h->stream, h->device);
+        int want = 4;
+        while (want > 1 && (b->n + want / 2 - 1) / (want / 2) <= n_sm) want /= 2;
+        std::vector<int> ks = {want};
+        for (int K : {4, 2, 1})
+            if (K != want) ks.push_back(K);
         for (int fg = 0; fg < 2; ++fg)
             for (int K : ks) {
                 if (fk && K != fk) continue;

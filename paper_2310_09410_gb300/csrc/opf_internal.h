@@ -220,7 +220,8 @@ constexpr int kBatchRecip = 256;   // copy counts of a global are below this (th
 
 // Arguments of one batched-engine launch.  Instance column sc of CTA c holds
 // instance inst[c * K + sc] (-1: empty).  Engine arrays (type T):
-//   per slot      [c][NCH][K][4]   mu, ds, bt (+bbar~ if M = F^T F, else -bbar~), lref (lambda_ref)
+//   per slot      [c][NCH][K][4]   mu, ds, bt (+bbar~ if M = F^T F, else -bbar~; FP64: rho times that),
+//                                  lref (lambda_ref)
 //   per global    [c][G][K]        xrf (x_ref), xo (x~ at the end)
 //   per bounded   [c][NB][K]       lbt, ubt (bounds - x_ref), cbt (c~)
 // The reference lambda_ref of the shifted frame makes c~ = c + sum lambda_ref
