@@ -142,18 +142,37 @@ __device__ __forceinline__ void st4cg(double *p, const Q4<double> &q) {
     __stcg(reinterpret_cast<double2 *>(p + 2), make_double2(q.v[2], q.v[3]));
 }
 
-// One warp task with exactly NQT chunks per position.  chg holds g * K per
-// slot (-1: padding); bt holds +bbar~ for members with M = F^T F and -bbar~
-// for M = I - F^T F, so that y = bt + F^T w gives x_s = y or v - y.
-// Shared-memory slot array: chunk ch, slot e, column sc at
-// (ch * 4 + (e ^ (ch & 3))) * K + sc.  Between the two phases of an
-// iteration it holds, at every slot, x of the slot's global (written there by
-// the global update); otherwise u = rho x_s - lambda of the slot.  The
-// swizzle e ^ (ch & 3) puts the four member positions of a warp (consecutive
-// chunks) on distinct banks.  Padding slots hold 0.
+// One warp task with exactly NQT chunks per position.  bt holds +bbar~ for
+// members with M = F^T F and -bbar~ for M = I - F^T F, so that y = bt + F^T w
+// gives x_s = y or v - y.
+// Adds a task's test sums over its J member positions to the warp's sums of the
+// column, quantities 0, 1, 3, 4, spread over the positions as they are added:
+// at K = 8 FP64 adds of 4 instead of 12 (each occupies the sub-partition's FP64
+// pipe for about 64 cycles, and the tasks' were a third of a tested iteration).
 template <int K>
+__device__ __forceinline__ void add_column_sums(double *redw, int sc, int jpos, double c0, double c1, double c3,
+                                                double c4) {
+    static_assert(K <= 8, "four member positions at least");
+    const bool b0 = jpos & 1, b1 = jpos & 2;
+    const double p0 = (b0 ? c3 : c0) + __shfl_xor_sync(0xffffffffu, b0 ? c0 : c3, K);
+    const double p1 = (b0 ? c4 : c1) + __shfl_xor_sync(0xffffffffu, b0 ? c1 : c4, K);
+    double r = (b1 ? p1 : p0) + __shfl_xor_sync(0xffffffffu, b1 ? p0 : p1, 2 * K);
+#pragma unroll
+    for (int o = 4 * K; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if (jpos < 4) redw[sc * 6 + 3 * (jpos & 1) + (jpos >> 1)] += r;
+}
+
+// Shared-memory slot array: chunk ch, slot e, column sc at slot_row(ch, e) * K
+// + sc.  Between the two phases of an iteration it holds, at every slot, x of
+// the slot's global (written there by the global update); otherwise
+// u = rho x_s - lambda of the slot.  slot_row swizzles the four slots of a
+// chunk so that the lanes that share a shared-memory transaction (consecutive
+// chunks, one slot each) fall on distinct banks at each row width (K = 2 in
+// FP32 with the swizzle of 32-byte rows: 4-way conflicts, the loads of u at the
+// start of a task 840 cycles).  Padding slots hold 0.
+template <typename T, int K>
 __device__ __forceinline__ int upos(int ch, int e, int sc) {
-    return (ch * 4 + (e ^ (ch & 3))) * K + sc;
+    return slot_row(ch, e, K * (int)sizeof(T)) * K + sc;
 }
 
 // ---- tensor memory (tcgen05, tmem.cuh): lambda and bbar~ of the tasks,
@@ -228,55 +247,44 @@ __device__ __forceinline__ void tm_stage_out(const BatchTask &tk, unsigned tl, f
 
 // The slot array holds rho x_g at every slot when the task starts (the global
 // update wrote it; a one-copy unbounded global's slot holds its u, which is
-// that value) and gets u at the end; y starts at +-rho bbar~ (tensor-memory
-// plans stage it scaled, the others scale it on load).
-template <typename T, int K, int NQT, bool TM>
-__device__ __forceinline__ void batch_task(const BatchTask &tk, const T *Fs, T *us, T *mu_c, const T *bt_c,
-                                           T *ds_c, const T *lr_c, const T *xr_c, const int4 *chg, int jpos,
-                                           int sc, T rho, T inv_rho, bool check, bool act, bool wds,
-                                           double *redw, unsigned tl) {
+// that value) and gets u at the end; y starts at +-rho bbar~ (the FP64 arrays
+// hold it scaled, FP32 tensor-memory plans stage it scaled, the other FP32
+// ones scale it on load).  FP64 form:
+template <int K, int NQT, bool>
+__device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs, double *us, double *mu_c,
+                                           const double *bt_c, double *ds_c, const double *lr_c, const double *xs_c,
+                                           int jpos, int sc, double, double inv_rho, bool check, bool act, bool wds,
+                                           double *redw, unsigned) {
     constexpr int J = 32 / K;
     const int mode1 = (tk.modes >> (jpos >> tk.lp)) & 1;
-    T v[4 * NQT], y[4 * NQT];
+    double v[4 * NQT], y[4 * NQT];
     double c0 = 0.0, c1 = 0.0, c3 = 0.0, c4 = 0.0;
-    // FP32 plans: a lane's test terms (FP32 already) summed over the task's
-    // chunks in FP32 and added to the FP64 sums once per task (FP64 adds
-    // cost this part 64 FP32 ones)
-    float f0 = 0.f, f1 = 0.f, f3 = 0.f, f4 = 0.f;
     const int ch0 = tk.ch0 + jpos;
-    const unsigned tcol = tl + (unsigned)(tk.tm >> 2);
 #pragma unroll
     for (int q = 0; q < NQT; ++q) {
         const int ch = ch0 + q * J;
         const int off = (ch * K + sc) * 4;
-        Q4<T> m4, b4;
-        if constexpr (TM) {
-            tm_ld8(tcol + 8 * q, m4, b4);
-            tm_wait_ld();
-        } else {
-            m4 = ld4cg(mu_c + off);
-            b4 = ld4cg(bt_c + off);
-        }
+        const Q4<double> m4 = ld4cg(mu_c + off), b4 = ld4cg(bt_c + off);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            y[4 * q + e] = TM || sizeof(T) == 8 ? b4.v[e] : rho * b4.v[e];   // (FP64 arrays hold rho bbar~)
-            v[4 * q + e] = us[upos<K>(ch, e, sc)] + m4.v[e];
+            y[4 * q + e] = b4.v[e];
+            v[4 * q + e] = us[upos<double, K>(ch, e, sc)] + m4.v[e];
         }
     }
     // rho x_s = M V + rho bbar~ over the factor rows, two rows per step
     const int rstride = NQT * J * 4;
-    const T *F0 = Fs + tk.foff + jpos * 4;
+    const double *F0 = Fs + tk.foff + jpos * 4;
     const int red_top = tk.p * K;
     // (the task's row count is even: a member's missing rows are zero)
     for (int r = 0; r < tk.f; r += 2, F0 += 2 * rstride) {
-        const T *F1 = F0 + rstride;
+        const double *F1 = F0 + rstride;
         // one accumulation chain per row (four partial sums and their adds
         // measured 4.5 % slower per launch: more instructions)
-        T s0 = T(0), s1 = T(0);
+        double s0 = 0.0, s1 = 0.0;
 #pragma unroll
         for (int q = 0; q < NQT; ++q) {
-            const Q4<T> f0 = ld4(F0 + q * J * 4);
-            const Q4<T> f1 = ld4(F1 + q * J * 4);
+            const Q4<double> f0 = ld4(F0 + q * J * 4);
+            const Q4<double> f1 = ld4(F1 + q * J * 4);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 s0 += f0.v[e] * v[4 * q + e];
@@ -289,8 +297,8 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const T *Fs, T *
         }
 #pragma unroll
         for (int q = 0; q < NQT; ++q) {
-            const Q4<T> f0 = ld4(F0 + q * J * 4);
-            const Q4<T> f1 = ld4(F1 + q * J * 4);
+            const Q4<double> f0 = ld4(F0 + q * J * 4);
+            const Q4<double> f1 = ld4(F1 + q * J * 4);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 y[4 * q + e] += f0.v[e] * s0;
@@ -302,84 +310,254 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const T *Fs, T *
     for (int q = 0; q < NQT; ++q) {
         const int ch = ch0 + q * J;
         const int off = (ch * K + sc) * 4;
-        Q4<T> x4, m4, u4, r4;
+        Q4<double> x4, m4, u4, r4;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const T vv = v[4 * q + e];
-            const T rx = mode1 ? y[4 * q + e] : vv - y[4 * q + e];     // rho x_s
-            const T mun = vv - rx;
+            const double vv = v[4 * q + e];
+            const double rx = mode1 ? y[4 * q + e] : vv - y[4 * q + e];     // rho x_s
+            const double mun = vv - rx;
             r4.v[e] = rx;
             m4.v[e] = mun;
             u4.v[e] = rx - mun;
         }
-        // x_s~ (written on wds iterations, test terms); in FP32 computed on
-        // every iteration (a branch here measured 6 % slower per launch), in
-        // FP64, where a multiply costs 64 cycles, only when it is used
-        if (sizeof(T) == 4 || wds) {
+        // x_s~ (written on wds iterations, test terms) only when it is used: a
+        // multiply costs 64 cycles
+        if (wds) {
 #pragma unroll
             for (int e = 0; e < 4; ++e) x4.v[e] = r4.v[e] * inv_rho;
         }
         if (check) {
-            const int4 g4 = __ldg(chg + ch);
-            const int gg[4] = {g4.x, g4.y, g4.z, g4.w};
-            const Q4<T> o4 = ld4cg(ds_c + off);
-            const Q4<T> l4 = ld4cg(lr_c + off);
-            T t0 = T(0), t1 = T(0), t3 = T(0), t4 = T(0);
+            const Q4<double> o4 = ld4cg(ds_c + off);
+            const Q4<double> l4 = ld4cg(lr_c + off);
+            const Q4<double> g4 = ld4cg(xs_c + off);
+            double t0 = 0.0, t1 = 0.0, t3 = 0.0, t4 = 0.0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                if (gg[e] < 0) continue;
-                const T d0 = (us[upos<K>(ch, e, sc)] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
-                const T xa = x4.v[e] + __ldcg(xr_c + gg[e]);
-                const T la = m4.v[e] + l4.v[e];
+                const double d0 = (us[upos<double, K>(ch, e, sc)] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
+                const double xa = x4.v[e] + g4.v[e];
+                const double la = m4.v[e] + l4.v[e];
                 t0 += d0 * d0;
                 t1 += d1 * d1;
                 t3 += xa * xa;
                 t4 += la * la;
             }
-            if constexpr (sizeof(T) == 4) {
-                f0 += t0;
-                f1 += t1;
-                f3 += t3;
-                f4 += t4;
-            } else {
-                c0 += (double)t0;
-                c1 += (double)t1;
-                c3 += (double)t3;
-                c4 += (double)t4;
-            }
+            c0 += t0;
+            c1 += t1;
+            c3 += t3;
+            c4 += t4;
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) us[upos<K>(ch, e, sc)] = u4.v[e];
-        if constexpr (TM) {
-            // every lane (a frozen column keeps iterating in tensor memory;
-            // its lambda went to the engine array when it froze)
-            tm_st4(tcol + 8 * q, m4);
-            if (act && wds) st4cg(ds_c + off, x4);
-        } else if (act) {
+        for (int e = 0; e < 4; ++e) us[upos<double, K>(ch, e, sc)] = u4.v[e];
+        if (act) {
             st4cg(mu_c + off, m4);
             if (wds) st4cg(ds_c + off, x4);
         }
     }
     if (check) {
-        if constexpr (sizeof(T) == 4) {
-            c0 = (double)f0;
-            c1 = (double)f1;
-            c3 = (double)f3;
-            c4 = (double)f4;
+        add_column_sums<K>(redw, sc, jpos, c0, c1, c3, c4);
+    }
+}
+
+// ---- FP32: packed pairs (two values per 64-bit register)
+// What bounds an FP32 iteration: with every SM's CTA full (K = 8) issue slots
+// and shared-memory transactions, with few instances (K = 2) the latency of
+// the longest task and of the global update.  Hence one instruction per two
+// multiply-adds; a row's sum over a member's lanes with its levels unrolled (a
+// loop over them took 90 cycles per level, twice the shuffle and the add);
+// every tensor-memory load of a task before one wait; a slot array free of
+// bank conflicts at each K; global-update items sorted so that a warp's lanes
+// take the same branches.  us per iteration with a test every 50, before and
+// now: 123 buses, 20 instances (K = 2) 4.11 -> 3.37; 34 buses, 201 instances
+// (K = 2) 2.47 -> 1.98; 123 buses, 1024 instances (K = 8) 6.57 -> 6.41, of
+// which the tests take 0.42 -> 0.26.  Tried and slower: four rows per step
+// (K = 8 6.19 -> 7.4), 20 or 24 warps (6.24 -> 6.46, 7.42), the next rows'
+// factors prefetched (spills), two chains per row (K = 2 3.19 -> 3.35).
+using u64 = unsigned long long;
+__device__ __forceinline__ u64 pk(float a, float b) {
+    u64 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpk(u64 p, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p)); }
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
+    u64 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) {
+    u64 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ u64 add2(u64 a, u64 b) {
+    u64 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// R factor rows of a task whose members span 2^LP lanes: w_r = <F_r, V> over
+// the member's lanes, y += w_r F_r.  A row's product is two chains (the even
+// and the odd slots of a lane), added at the end.
+template <int K, int NQT, int R, int LP>
+__device__ __forceinline__ void rows(const float *F0, int rstride, const u64 (&v)[2 * NQT], u64 (&y)[2 * NQT]) {
+    constexpr int J = 32 / K;
+    u64 s[R];
+#pragma unroll
+    for (int q = 0; q < NQT; ++q)
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(F0 + i * rstride + q * J * 4);
+            s[i] = q == 0 ? mul2(a.x, v[0]) : fma2(a.x, v[2 * q], s[i]);
+            s[i] = fma2(a.y, v[2 * q + 1], s[i]);
         }
-        // per instance column: sum over the J member positions, in lane order
-        for (int o = K; o < 32; o <<= 1) {
-            c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-            c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            c3 += __shfl_xor_sync(0xffffffffu, c3, o);
-            c4 += __shfl_xor_sync(0xffffffffu, c4, o);
+    float t[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+        float e, o;
+        unpk(s[i], e, o);
+        t[i] = e + o;
+    }
+#pragma unroll
+    for (int o = K; o < (K << LP); o <<= 1)
+#pragma unroll
+        for (int i = 0; i < R; ++i) t[i] += __shfl_xor_sync(0xffffffffu, t[i], o);
+#pragma unroll
+    for (int i = 0; i < R; ++i) s[i] = pk(t[i], t[i]);
+#pragma unroll
+    for (int q = 0; q < NQT; ++q)
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+            const ulonglong2 a = *reinterpret_cast<const ulonglong2 *>(F0 + i * rstride + q * J * 4);
+            y[2 * q] = fma2(a.x, s[i], y[2 * q]);
+            y[2 * q + 1] = fma2(a.y, s[i], y[2 * q + 1]);
         }
-        if (jpos == 0) {
-            redw[sc * 6 + 0] += c0;
-            redw[sc * 6 + 1] += c1;
-            redw[sc * 6 + 3] += c3;
-            redw[sc * 6 + 4] += c4;
+}
+
+// The f rows (an even number: a member's missing rows are zero), two per step.
+template <int K, int NQT, int LP>
+__device__ __forceinline__ void task_rows(const float *F0, int rstride, int f, const u64 (&v)[2 * NQT],
+                                          u64 (&y)[2 * NQT]) {
+    constexpr int R = 2;
+#pragma unroll 1
+    for (int r = 0; r < f; r += R, F0 += R * rstride) rows<K, NQT, R, LP>(F0, rstride, v, y);
+}
+
+// Keeps uses of the values after the point where it stands (a tensor-memory wait).
+__device__ __forceinline__ void tie(Q4<float> &q) {
+    asm volatile("" : "+f"(q.v[0]), "+f"(q.v[1]), "+f"(q.v[2]), "+f"(q.v[3]));
+}
+
+// batch_task in FP32 with packed pairs: the same arithmetic, the factor rows by rows().
+template <int K, int NQT, bool TM>
+__device__ __forceinline__ void batch_task(const BatchTask &tk, const float *Fs, float *us, float *mu_c,
+                                           const float *bt_c, float *ds_c, const float *lr_c, const float *xs_c,
+                                           int jpos, int sc, float rho, float inv_rho, bool check,
+                                           bool act, bool wds, double *redw, unsigned tl) {
+    constexpr int J = 32 / K;
+    const bool mode1 = (tk.modes >> (jpos >> tk.lp)) & 1;
+    u64 v[2 * NQT], y[2 * NQT];
+    float f0 = 0.f, f1 = 0.f, f3 = 0.f, f4 = 0.f;     // test terms, FP32 over the task's chunks
+    const int ch0 = tk.ch0 + jpos;
+    const unsigned tcol = tl + (unsigned)(tk.tm >> 2);
+    {
+        Q4<float> m4[NQT], b4[NQT];
+#pragma unroll
+        for (int q = 0; q < NQT; ++q) {
+            if constexpr (TM) {
+                tm_ld8(tcol + 8 * q, m4[q], b4[q]);
+            } else {
+                const int off = ((ch0 + q * J) * K + sc) * 4;
+                m4[q] = ld4cg(mu_c + off);
+                b4[q] = ld4cg(bt_c + off);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) b4[q].v[e] *= rho;
+            }
         }
+        if constexpr (TM) {                  // every load of the task in flight, one wait
+            tm_wait_ld();
+#pragma unroll
+            for (int q = 0; q < NQT; ++q) {
+                tie(m4[q]);
+                tie(b4[q]);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < NQT; ++q) {
+            const int ch = ch0 + q * J;
+            y[2 * q] = pk(b4[q].v[0], b4[q].v[1]);
+            y[2 * q + 1] = pk(b4[q].v[2], b4[q].v[3]);
+            v[2 * q] = add2(pk(us[upos<float, K>(ch, 0, sc)], us[upos<float, K>(ch, 1, sc)]), pk(m4[q].v[0], m4[q].v[1]));
+            v[2 * q + 1] = add2(pk(us[upos<float, K>(ch, 2, sc)], us[upos<float, K>(ch, 3, sc)]), pk(m4[q].v[2], m4[q].v[3]));
+        }
+    }
+    // rho x_s = M V + rho bbar~ over the factor rows, two per step
+    const int rstride = NQT * J * 4;
+    const float *F0 = Fs + tk.foff + jpos * 4;
+    switch (tk.lp) {
+        case 0: task_rows<K, NQT, 0>(F0, rstride, tk.f, v, y); break;
+        case 1: task_rows<K, NQT, 1>(F0, rstride, tk.f, v, y); break;
+        case 2: task_rows<K, NQT, 2>(F0, rstride, tk.f, v, y); break;
+        case 3: if constexpr (J >= 8) task_rows<K, NQT, 3>(F0, rstride, tk.f, v, y); break;
+        default: if constexpr (J >= 16) task_rows<K, NQT, 4>(F0, rstride, tk.f, v, y); break;
+    }
+    // rho x_s = y or V - y, as ca V + cb y with exact coefficients
+    const float ca = mode1 ? 0.0f : 1.0f, cb = mode1 ? 1.0f : -1.0f;
+    const u64 ca2 = pk(ca, ca), cb2 = pk(cb, cb), neg = pk(-1.0f, -1.0f), ir2 = pk(inv_rho, inv_rho);
+#pragma unroll
+    for (int q = 0; q < NQT; ++q) {
+        const int ch = ch0 + q * J;
+        const int off = (ch * K + sc) * 4;
+        Q4<float> m4, u4;
+        u64 rx[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            rx[h] = fma2(y[2 * q + h], cb2, mul2(v[2 * q + h], ca2));
+            const u64 mun = fma2(rx[h], neg, v[2 * q + h]);
+            const u64 un = fma2(mun, neg, rx[h]);
+            unpk(mun, m4.v[2 * h], m4.v[2 * h + 1]);
+            unpk(un, u4.v[2 * h], u4.v[2 * h + 1]);
+        }
+        if (check) {
+            // x_s~ before, lambda_ref, x_ref (padding slots hold 0)
+            const Q4<float> o4 = ld4cg(ds_c + off), l4 = ld4cg(lr_c + off), g4 = ld4cg(xs_c + off);
+            float t0 = 0.f, t1 = 0.f, t3 = 0.f, t4 = 0.f;
+            Q4<float> r4, x4;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                unpk(rx[h], r4.v[2 * h], r4.v[2 * h + 1]);
+                unpk(mul2(rx[h], ir2), x4.v[2 * h], x4.v[2 * h + 1]);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float d0 = (us[upos<float, K>(ch, e, sc)] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
+                const float xa = x4.v[e] + g4.v[e];
+                const float la = m4.v[e] + l4.v[e];
+                t0 += d0 * d0;
+                t1 += d1 * d1;
+                t3 += xa * xa;
+                t4 += la * la;
+            }
+            f0 += t0;
+            f1 += t1;
+            f3 += t3;
+            f4 += t4;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) us[upos<float, K>(ch, e, sc)] = u4.v[e];
+        // (tensor memory: every lane; a frozen column keeps iterating there,
+        // its lambda went to the engine array when it froze)
+        if constexpr (TM) tm_st4(tcol + 8 * q, m4);
+        else if (act) st4cg(mu_c + off, m4);
+        if (act && wds) {
+            Q4<float> x4;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) unpk(mul2(rx[h], ir2), x4.v[2 * h], x4.v[2 * h + 1]);
+            st4cg(ds_c + off, x4);
+        }
+    }
+    if (check) {
+        double c0 = (double)f0, c1 = (double)f1, c3 = (double)f3, c4 = (double)f4;
+        add_column_sums<K>(redw, sc, jpos, c0, c1, c3, c4);
     }
 }
 
@@ -450,13 +628,13 @@ __global__ void __launch_bounds__(512, 1)
         bnd[(b * 3 + 2) * K + col] = __ldcg(a.cbt + bb + idx);              // c~
     }
     T *mu_c = a.mu + sb, *ds_c = a.ds + sb;
-    const T *bt_c = a.bt + sb, *lr_c = a.lref + sb;
+    const T *bt_c = a.bt + sb, *lr_c = a.lref + sb, *xs_c = a.xsr + sb;
     // u = rho d - mu into the swizzled slot array
     for (int idx = tid; idx < a.NCH * K; idx += nthr) {
         const int ch = idx >> KS, col = idx & (K - 1);
         const Q4<T> d = ld4cg(ds_c + (size_t)idx * 4), m = ld4cg(mu_c + (size_t)idx * 4);
 #pragma unroll
-        for (int e = 0; e < 4; ++e) us[upos<K>(ch, e, col)] = a.rho * d.v[e] - m.v[e];
+        for (int e = 0; e < 4; ++e) us[upos<T, K>(ch, e, col)] = a.rho * d.v[e] - m.v[e];
     }
     const int sc = tid & (K - 1);
     const int jpos = lane >> KS;
@@ -483,7 +661,6 @@ __global__ void __launch_bounds__(512, 1)
     }
     __syncthreads();
     if constexpr (TM) tm_fence_after();
-    const T *xr_c = a.xrf + gb + sc;
     const T rho = a.rho, inv_rho = a.inv_rho;
     double *redw = red + (size_t)w * K * 6;      // this warp's test sums per column
     int last_check = 0;
@@ -508,7 +685,10 @@ __global__ void __launch_bounds__(512, 1)
         // whose table entry names their bounded index; elsewhere c~ = 0),
         // 1 / N, clip to rho (bounds - x_ref), and rho x stored into every
         // copy's slot; GB items per thread
-        for (int b0 = tid; b0 < GQ; b0 += GB * nthr) {
+        // (items of many copies come first; the last round, when it is not
+        // full, goes to the last threads, which had none of those)
+        auto item_of = [&](int base) { return base + (base + nthr > GQ ? nthr - 1 - tid : tid); };
+        for (int b0 = 0; b0 < GQ; b0 += GB * nthr) {
             // the GB items of this thread advance stage by stage, so that the
             // loads of one stage are in flight together: the table entries
             // (with the first two copies' rows), their u; further copies
@@ -518,7 +698,7 @@ __global__ void __launch_bounds__(512, 1)
             int row0[GB], row1[GB];
 #pragma unroll
             for (int j = 0; j < GB; ++j) {
-                const int item = b0 + j * nthr;
+                const int item = item_of(b0 + j * nthr);
                 gtj[j] = make_int4(0, 0, 0, -1);
                 if (item < GQ) gtj[j] = gts[item >> QS];
                 const int hq = (item & (NQD - 1)) * KQ;
@@ -549,16 +729,25 @@ __global__ void __launch_bounds__(512, 1)
             }
 #pragma unroll
             for (int j = 0; j < GB; ++j) {
-                const int item = b0 + j * nthr;
+                const int item = item_of(b0 + j * nthr);
                 if (item >= GQ) continue;
                 const int h = item & (NQD - 1);
                 const int4 gt = gtj[j];
-                const int cnt = gt.z & 0xff, st0 = (gt.z >> 8) - 2;    // usg[st0 + q]: copy q >= 2
-                for (int q = 2; q < cnt; ++q) {
-                    RowK<T, KQ> uq;
-                    load_row<T, KQ, false>(uq, us + usg[st0 + q] + h * KQ);
+                const int cnt = gt.z & 0xff;
+                const int st0 = (gt.z >> 8) - 2;              // usg[st0 + q]: copy q >= 2
+                for (int q = 2; q < cnt; q += 4) {            // four copies' loads in flight
+                    int rr[4];
 #pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] += uq.v[k];
+                    for (int c = 0; c < 4; ++c) rr[c] = q + c < cnt ? usg[st0 + q + c] : 0;
+                    RowK<T, KQ> uq[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (q + c < cnt) load_row<T, KQ, false>(uq[c], us + rr[c] + h * KQ);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (q + c < cnt)
+#pragma unroll
+                            for (int k = 0; k < KQ; ++k) sum[j].v[k] += uq[c].v[k];
                 }
                 const T rcp = rcs[cnt];
                 if (gt.w >= 0) {
@@ -576,7 +765,14 @@ __global__ void __launch_bounds__(512, 1)
                 }
                 if (cnt > 0) store_row<T, KQ>(us + row0[j], sum[j]);
                 if (cnt > 1) store_row<T, KQ>(us + row1[j], sum[j]);
-                for (int q = 2; q < cnt; ++q) store_row<T, KQ>(us + usg[st0 + q] + h * KQ, sum[j]);
+                for (int q = 2; q < cnt; q += 4) {
+                    int rr[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) rr[c] = q + c < cnt ? usg[st0 + q + c] : 0;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        if (q + c < cnt) store_row<T, KQ>(us + rr[c] + h * KQ, sum[j]);
+                }
             }
         }
         __syncthreads();
@@ -588,22 +784,38 @@ __global__ void __launch_bounds__(512, 1)
             // FP64 from the warp sums on; FP64 plans: FP64 throughout)
             double c2 = 0.0, c5 = 0.0;
             T p2 = T(0), p5 = T(0);
-            for (int item = tid; item < GK; item += nthr) {
-                const int j = item >> KS;
-                const int2 gt = make_int2(__ldg(a.gx + j), 0);   // first copy's row | copies << 24
-                const int i = __ldg(a.gperm + j);
-                const size_t gi = gb + (size_t)i * K + sc;
-                const T xv = us[(gt.x & 0xffffff) + sc] * a.inv_rho;
-                if (flags[sc]) a.xo[gi] = xv;
-                if (check) {
-                    if constexpr (sizeof(T) == 4) {
-                        const T xa = xv + __ldcg(a.xrf + gi);
-                        p2 += (T)((unsigned)gt.x >> 24) * xa * xa;
-                        p5 += __ldg(a.cost + i) * xa;
-                    } else {
-                        const double xa = (double)xv + (double)__ldcg(a.xrf + gi);
-                        c2 += (double)((unsigned)gt.x >> 24) * xa * xa;
-                        c5 += (double)__ldg(a.cost + i) * xa;
+            constexpr int XB = 4;        // items whose loads are in flight together
+            for (int i0 = tid; i0 < GK; i0 += XB * nthr) {
+                int gx[XB], gi[XB];
+                T xr[XB], cost[XB];
+#pragma unroll
+                for (int q = 0; q < XB; ++q) {
+                    const int item = i0 + q * nthr;
+                    gx[q] = item < GK ? __ldg(a.gx + (item >> KS)) : 0;      // first copy's row | copies << 24
+                    gi[q] = item < GK ? __ldg(a.gperm + (item >> KS)) : -1;
+                }
+                if (check)
+#pragma unroll
+                    for (int q = 0; q < XB; ++q) {
+                        xr[q] = gi[q] >= 0 ? __ldcg(a.xrf + gb + (size_t)gi[q] * K + sc) : T(0);
+                        cost[q] = gi[q] >= 0 ? __ldg(a.cost + gi[q]) : T(0);
+                    }
+#pragma unroll
+                for (int q = 0; q < XB; ++q) {
+                    if (gi[q] < 0) continue;
+                    const T xv = us[(gx[q] & 0xffffff) + sc] * a.inv_rho;
+                    if (flags[sc]) a.xo[gb + (size_t)gi[q] * K + sc] = xv;
+                    if (check) {
+                        const unsigned n = (unsigned)gx[q] >> 24;
+                        if constexpr (sizeof(T) == 4) {
+                            const T xa = xv + xr[q];
+                            p2 += (T)n * xa * xa;
+                            p5 += cost[q] * xa;
+                        } else {
+                            const double xa = (double)xv + (double)xr[q];
+                            c2 += (double)n * xa * xa;
+                            c5 += (double)cost[q] * xa;
+                        }
                     }
                 }
             }
@@ -612,14 +824,10 @@ __global__ void __launch_bounds__(512, 1)
                 c5 = (double)p5;
             }
             if (check) {
-                for (int o = K; o < 32; o <<= 1) {
-                    c2 += __shfl_xor_sync(0xffffffffu, c2, o);
-                    c5 += __shfl_xor_sync(0xffffffffu, c5, o);
-                }
-                if (lane < K) {
-                    redw[lane * 6 + 2] += c2;
-                    redw[lane * 6 + 5] += c5;
-                }
+                const bool b0 = jpos & 1;
+                double r = (b0 ? c5 : c2) + __shfl_xor_sync(0xffffffffu, b0 ? c2 : c5, K);
+                for (int o = 2 * K; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+                if (jpos < 2) redw[sc * 6 + (b0 ? 5 : 2)] += r;
             }
             __syncthreads();      // the slots still hold x: read before phase L overwrites them
         }
@@ -640,16 +848,16 @@ __global__ void __launch_bounds__(512, 1)
                 if (!check && lane == 0) claim = atomicAdd(cnt, 1);
                 const BatchTask tk = tks[t];
                 switch (tk.nq) {
-                    case 1: batch_task<T, K, 1, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xr_c, a.chg, jpos, sc, rho,
+                    case 1: batch_task<K, 1, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c, jpos, sc, rho,
                                                     inv_rho, check, act, wds, redw, tl); break;
-                    case 2: if constexpr (NQ >= 2) batch_task<T, K, 2, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xr_c,
-                                                                           a.chg, jpos, sc, rho, inv_rho, check, act,
+                    case 2: if constexpr (NQ >= 2) batch_task<K, 2, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c,
+                                                                           jpos, sc, rho, inv_rho, check, act,
                                                                            wds, redw, tl); break;
-                    case 3: if constexpr (NQ >= 3) batch_task<T, K, 3, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xr_c,
-                                                                           a.chg, jpos, sc, rho, inv_rho, check, act,
+                    case 3: if constexpr (NQ >= 3) batch_task<K, 3, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c,
+                                                                           jpos, sc, rho, inv_rho, check, act,
                                                                            wds, redw, tl); break;
-                    default: if constexpr (NQ >= 4) batch_task<T, K, 4, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xr_c,
-                                                                            a.chg, jpos, sc, rho, inv_rho, check, act,
+                    default: if constexpr (NQ >= 4) batch_task<K, 4, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c,
+                                                                            jpos, sc, rho, inv_rho, check, act,
                                                                             wds, redw, tl); break;
                 }
                 t = check ? t + t_step : __shfl_sync(0xffffffffu, claim, 0);
@@ -662,26 +870,29 @@ __global__ void __launch_bounds__(512, 1)
         if (check) {
             __syncthreads();
             if constexpr (TM) tm_fence_after();
-            // one thread per (column, quantity) sums the warps' parts in warp
-            // order into warp 0's slot, then one thread per column tests
-            if (tid < 6 * K) {
-                const int col = tid / 6, q = tid - 6 * col;
-                double sum = 0.0;
-                for (int ww = 0; ww < n_warps; ++ww) sum += red[((size_t)ww * K + col) * 6 + q];
-                red[col * 6 + q] = sum;
-            }
-            __syncthreads();
-            if (tid < K) {
-                flags[K + tid] = 0;
-                if (flags[tid]) {
-                    const int in = a.inst[c * K + tid];
-                    double s6[6];
+            // eight lanes per column: lane q sums quantity q of the warps' parts
+            // in warp order and takes its square root (5 in turn by one thread
+            // took some 7000 cycles), the first decides
+            for (int c0 = 4 * w; c0 < K; c0 += 4 * n_warps) {
+                const int col = c0 + (lane >> 3), q = lane & 7;
+                double sum = 0.0, root[5], s6[6];
+                if (col < K && q < 6)
+                    for (int ww = 0; ww < n_warps; ++ww) sum += red[((size_t)ww * K + col) * 6 + q];
+                const double mine = q < 5 ? sqrt(sum) : 0.0;
 #pragma unroll
-                    for (int q = 0; q < 6; ++q) s6[q] = red[tid * 6 + q];
-                    apply_test(&a.st[in], s6, a.rho_d, check_every);
-                    if (a.st[in].done) {
-                        flags[tid] = 0;
-                        flags[K + tid] = 1;
+                for (int i = 0; i < 6; ++i) {
+                    s6[i] = __shfl_sync(0xffffffffu, sum, i, 8);
+                    if (i < 5) root[i] = __shfl_sync(0xffffffffu, mine, i, 8);
+                }
+                if (col < K && q == 0) {
+                    flags[K + col] = 0;
+                    if (flags[col]) {
+                        const int in = a.inst[c * K + col];
+                        apply_roots(&a.st[in], s6, root, a.rho_d, check_every);
+                        if (a.st[in].done) {
+                            flags[col] = 0;
+                            flags[K + col] = 1;
+                        }
                     }
                 }
             }
@@ -900,7 +1111,7 @@ __device__ __forceinline__ void bref_one(int in, bool valid, int d, int l0, int 
                                          const int *sch, double rho, const double *xref, const double *dref,
                                          const double *xsv, const double *lam, const double *bbar, int G, int L,
                                          int K, int kshift, int NCH, double *v, double *tt, T *bt, T *ds, T *mu,
-                                         T *lref) {
+                                         T *lref, T *xsr) {
     const int so = h.x, n = h.y, f = h.z, mode = h.w, npad = q2.y;
     const double *Fs = F64 + q2.x;
     const int ll = lane - l0;
@@ -934,6 +1145,7 @@ __device__ __forceinline__ void bref_one(int in, bool valid, int d, int l0, int 
         ds[e] = (T)(xi[k] - xg);
         mu[e] = (T)dg;
         lref[e] = (T)(li[k] - dg);
+        if (xsr) xsr[e] = (T)xg;
     }
 }
 
@@ -949,7 +1161,8 @@ __global__ void __launch_bounds__(128) k_bref_slots(int S, int n_inst, int G, in
                                                     const double *F64, const int *gk, const int *sch,
                                                     double rho, const double *xref, const double *dref,
                                                     const double *xsv, const double *lam, const double *bbar,
-                                                    const DevStatus *st, T *bt, T *ds, T *mu, T *lref) {
+                                                    const DevStatus *st, T *bt, T *ds, T *mu, T *lref,
+                                                    T *xsr) {
     __shared__ double buf[4][2][OPF_MAX_NS];
     const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long task = (long long)blockIdx.x * 4 + wl;
@@ -961,14 +1174,15 @@ __global__ void __launch_bounds__(128) k_bref_slots(int S, int n_inst, int G, in
         const int half = lane >> 4, in = 2 * pair + half;
         const bool valid = in < n_inst && !st[in].done && ipos[in] >= 0;
         bref_one<T>(in, valid, d, half * 16, 16, lane, h, q2, F64, ipos, gk, sch, rho, xref, dref, xsv, lam, bbar,
-                    G, L, K, kshift, NCH, buf[wl][0] + half * 128, buf[wl][1] + half * 128, bt, ds, mu, lref);
+                    G, L, K, kshift, NCH, buf[wl][0] + half * 128, buf[wl][1] + half * 128, bt, ds, mu, lref,
+                    xsr);
     } else {
         for (int q = 0; q < 2; ++q) {
             const int in = 2 * pair + q;
             if (in >= n_inst) break;
             const bool valid = !st[in].done && ipos[in] >= 0;
             bref_one<T>(in, valid, d, 0, 32, lane, h, q2, F64, ipos, gk, sch, rho, xref, dref, xsv, lam, bbar, G,
-                        L, K, kshift, NCH, buf[wl][0], buf[wl][1], bt, ds, mu, lref);
+                        L, K, kshift, NCH, buf[wl][0], buf[wl][1], bt, ds, mu, lref, xsr);
             __syncwarp();
         }
     }
@@ -1175,14 +1389,14 @@ void launch_bref(int n_inst, int S, int G, int L, int K, int kshift, int NCH, in
                  const double *ub, double rho, const double *xsv, const double *lam, DevStatus *st,
                  double *xref, double *dref, T *ct, T *xrf, T *lbt, T *ubt, T *cbt, const int4 *sub,
                  const int4 *sub2, const double *F64, const int *gk, const int *sch, const double *bbar, T *bt,
-                 T *ds, T *mu, T *lref, cudaStream_t s) {
+                 T *ds, T *mu, T *lref, T *xsr, cudaStream_t s) {
     k_bref_globals<T><<<bl((long long)n_inst * G, 256), 256, 0, s>>>(n_inst, G, L, K, kshift, NB, ipos, gseg, uslot,
                                                                     bidx, c64, lb, ub, rho, xsv, lam, st, xref,
                                                                     dref, ct, xrf, lbt, ubt, cbt);
     const long long warps = (long long)S * ((n_inst + 1) / 2);
     k_bref_slots<T><<<(int)((warps + 3) / 4), 128, 0, s>>>(S, n_inst, G, L, K, kshift, NCH, ipos, sub, sub2, F64,
                                                            gk, sch, rho, xref, dref, xsv, lam, bbar, st, bt, ds, mu,
-                                                           lref);
+                                                           lref, xsr);
 }
 
 template <typename T>
@@ -1199,13 +1413,13 @@ template void launch_bref<float>(int, int, int, int, int, int, int, int, const i
                                  const double *, const double *, DevStatus *, double *, double *, float *,
                                  float *, float *, float *, float *, const int4 *, const int4 *, const double *,
                                  const int *, const int *, const double *, float *, float *, float *, float *,
-                                 cudaStream_t);
+                                 float *, cudaStream_t);
 template void launch_bref<double>(int, int, int, int, int, int, int, int, const int *, const int2 *, const int *,
                                   const int *, const double *, const double *, const double *, double,
                                   const double *, const double *, DevStatus *, double *, double *, double *,
                                   double *, double *, double *, double *, const int4 *, const int4 *, const double *,
                                   const int *, const int *, const double *, double *, double *, double *,
-                                  double *, cudaStream_t);
+                                  double *, double *, cudaStream_t);
 template void launch_bunshift<float>(int, int, int, int, int, int, const int *, const int *, const int *,
                                      const double *, const double *, const float *, const float *, const float *,
                                      const DevStatus *, double *, double *, double *, cudaStream_t);

@@ -48,7 +48,7 @@ void launch_bref(int n_inst, int S, int G, int L, int K, int kshift, int NCH, in
                  const double *ub, double rho, const double *xsv, const double *lam, DevStatus *st,
                  double *xref, double *dref, T *ct, T *xrf, T *lbt, T *ubt, T *cbt, const int4 *sub,
                  const int4 *sub2, const double *F64, const int *gk, const int *sch, const double *bbar, T *bt,
-                 T *ds, T *mu, T *lref, cudaStream_t s);
+                 T *ds, T *mu, T *lref, T *xsr, cudaStream_t s);
 template <typename T>
 void launch_bunshift(int n_inst, int G, int L, int K, int kshift, int NCH, const int *ipos, const int *gk,
                      const int *sch, const double *xref, const double *dref, const T *ds, const T *mu, const T *xo,
@@ -91,9 +91,6 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
     if (trc) { set_last_error("batch plan: slot without a chunk"); return OPF_E_INVALID; }
     std::vector<BatchTask> &tasks = tp.tasks;
     std::vector<int> &memb = tp.memb, &sch = tp.sch;
-    std::vector<int4> chg(tp.chg.size() / 4);
-    for (size_t c = 0; c < chg.size(); ++c)
-        chg[c] = make_int4(tp.chg[4 * c], tp.chg[4 * c + 1], tp.chg[4 * c + 2], tp.chg[4 * c + 3]);
     p->tm = tp.tm;
     p->tm_cols = tp.tm_cols;
     for (int q = 0; q < 5; ++q) p->qstart[q] = tp.qstart[q];
@@ -108,7 +105,7 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
         for (int q = 0; q < cnt; ++q) {
             const int pos = sch[h->h_uslot[s0 + q]];
             const int ch = pos >> 2, e = pos & 3;
-            crow[s0 + q] = (ch * 4 + (e ^ (ch & 3))) * K;
+            crow[s0 + q] = slot_row(ch, e, K * (int)sz) * K;
         }
     }
     // global-update tables (batch_tables.h): gperm, the computed globals'
@@ -118,6 +115,7 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
         set_last_error("batch plan: global table");
         return OPF_E_CAPACITY;
     }
+    sort_global_items(&gt);
     p->Gs = gt.Gs;
     std::vector<int4> gtab(std::max(p->Gs, 1), make_int4(0, 0, 0, -1));
     for (int j = 0; j < p->Gs; ++j)
@@ -152,7 +150,6 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
     BTRY(bupload(A, &p->d_sch, sch, st));
     BTRY(bupload(A, &p->d_uxt, uxt, st));
     BTRY(bupload(A, &p->d_gx, gx, st));
-    BTRY(bupload(A, &p->d_chg, chg, st));
     BTRY(bupload(A, &p->d_gtab, gtab, st));
     BTRY(bupload(A, &p->d_gperm, gperm, st));
     BTRY(bupload(A, &p->d_inst, inst, st));
@@ -169,6 +166,7 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
     BTRY(arr(&p->d_recip, (size_t)kBatchRecip));
     BTRY(arr(&p->d_cost, (size_t)G));
     BTRY(arr(&p->mu, nslot)); BTRY(arr(&p->ds, nslot)); BTRY(arr(&p->bt, nslot)); BTRY(arr(&p->lref, nslot));
+    BTRY(arr(&p->xsr, nslot));
     BTRY(arr(&p->xo, nglob)); BTRY(arr(&p->ct, nglob)); BTRY(arr(&p->xrf, nglob));
     BTRY(arr(&p->lbt, nbnd)); BTRY(arr(&p->ubt, nbnd)); BTRY(arr(&p->cbt, nbnd));
     if (dbl) launch_bpack<double>(p->n_tasks, J, p->d_tasks, p->d_memb, h->d_sub, h->d_sub2, h->d_F64,
@@ -224,11 +222,11 @@ BatchArgs<T> engine_args(opf_batch *b, const BPlan &p, double rho) {
     a.off_u = p.off_u; a.off_gt = p.off_gt; a.off_rc = p.off_rc; a.off_task = p.off_task; a.off_useg = p.off_useg;
     a.off_bnd = p.off_bnd;
     a.off_red = p.off_red; a.off_flag = p.off_flag;
-    a.tasks = p.d_tasks; a.chg = p.d_chg; a.gtab = p.d_gtab; a.gperm = p.d_gperm; a.Gs = p.Gs;
+    a.tasks = p.d_tasks; a.gtab = p.d_gtab; a.gperm = p.d_gperm; a.Gs = p.Gs;
     a.uxt = p.d_uxt; a.gx = p.d_gx; a.n_uxt = p.n_uxt;
     a.Fpk = (const T *)p.d_F; a.cost = (const T *)p.d_cost;
     a.mu = (T *)p.mu; a.ds = (T *)p.ds; a.xo = (T *)p.xo;
-    a.bt = (const T *)p.bt; a.lref = (const T *)p.lref; a.xrf = (const T *)p.xrf;
+    a.bt = (const T *)p.bt; a.lref = (const T *)p.lref; a.xsr = (const T *)p.xsr; a.xrf = (const T *)p.xrf;
     a.lbt = (const T *)p.lbt; a.ubt = (const T *)p.ubt; a.cbt = (const T *)p.cbt;
     a.inst = p.d_inst; a.st = b->d_st;
     a.rho = (T)rho; a.inv_rho = (T)(1.0 / rho); a.rho_d = rho;
@@ -249,7 +247,7 @@ void enqueue_body(opf_batch *b, BPlan &p, double rho, int n_iters, int check_eve
     launch_bref<T>(b->n, h->S, b->G, b->L, p.K, p.ks, p.NCH, p.NB, p.d_ipos, h->d_gseg, h->d_uslot, b->d_bidx,
                    h->d_c64, h->d_lb64, h->d_ub64, rho, b->d_xs, b->d_lam, b->d_st, b->d_xref, b->d_dref, (T *)p.ct,
                    (T *)p.xrf, (T *)p.lbt, (T *)p.ubt, (T *)p.cbt, h->d_sub, h->d_sub2, h->d_F64, h->d_gk, p.d_sch,
-                   b->d_bbar, (T *)p.bt, (T *)p.ds, (T *)p.mu, (T *)p.lref, s);
+                   b->d_bbar, (T *)p.bt, (T *)p.ds, (T *)p.mu, (T *)p.lref, (T *)p.xsr, s);
     if (e0) cudaEventRecord(e0, s);
     const int grid = ctas >= 0 ? std::min(ctas, p.C) : p.C;
     if (p.lane) {
@@ -403,7 +401,7 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
                            b->d_dref, (float *)p.ct, (float *)p.xrf, (float *)p.lbt, (float *)p.ubt, (float *)p.cbt,
                            h->d_sub, h->d_sub2,
                            h->d_F64, h->d_gk, p.d_sch, b->d_bbar, (float *)p.bt, (float *)p.ds, (float *)p.mu,
-                           (float *)p.lref, h->stream);
+                           (float *)p.lref, (float *)p.xsr, h->stream);
         auto run = [&](int n_it) {
             if (p.lane) lane_engine_launch(lane_args(b, p, rho), p.C, p.threads, p.bytes, n_it, 0, h->stream);
             else batch_engine_launch<float>(engine_args<float>(b, p, rho), p.nq, false, p.C, p.threads, p.bytes,

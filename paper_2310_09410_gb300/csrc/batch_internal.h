@@ -22,9 +22,10 @@ struct BPlan {
     int *d_memb = nullptr, *d_sch = nullptr, *d_uxt = nullptr, *d_gx = nullptr;
     int n_uxt = 0;
     int *d_inst = nullptr, *d_ipos = nullptr, *d_gperm = nullptr;
-    int4 *d_chg = nullptr, *d_gtab = nullptr;
+    int4 *d_gtab = nullptr;
     void *d_F = nullptr, *d_recip = nullptr, *d_cost = nullptr;
     void *mu = nullptr, *ds = nullptr, *xo = nullptr, *bt = nullptr, *lref = nullptr;
+    void *xsr = nullptr;              // not in lane-engine plans
     void *ct = nullptr, *xrf = nullptr, *lbt = nullptr, *ubt = nullptr, *cbt = nullptr;
     // lane-engine plans (K = kLaneInst, C = tiles of K instances)
     bool lane = false;
@@ -38,6 +39,7 @@ struct BPlan {
         graph.reset();
         for (void *p : allocs) cudaFree(p);
         allocs.clear();
+        xsr = nullptr;
         ok = false;
         lane = false;
     }

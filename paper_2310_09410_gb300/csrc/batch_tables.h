@@ -19,6 +19,7 @@
 
 #include <algorithm>
 #include <numeric>
+#include <tuple>
 #include <vector>
 
 namespace opf {
@@ -244,6 +245,23 @@ inline bool build_global_tables(int G, const std::vector<int> &gstart, const std
         for (int q = 2; q < cnt; ++q) t->uxt.push_back(crow[s0 + q]);
     }
     return true;
+}
+
+// The computed globals' entries by decreasing number of copies, the bounded
+// ones first, then by the first copy's row, so that the threads of a warp take
+// the same branches and read neighbouring rows.  (The order of the entries is
+// free: gperm and gx list the globals of the test on their own.)
+inline void sort_global_items(GlobalTables *t) {
+    const std::vector<int> was(t->gtab);
+    std::vector<int> ord(t->Gs);
+    std::iota(ord.begin(), ord.end(), 0);
+    auto key = [&](int j) {
+        const int *e = &was[4 * (size_t)j];
+        return std::make_tuple(-(e[2] & 255), e[3] < 0, e[0]);
+    };
+    std::sort(ord.begin(), ord.end(), [&](int a, int b) { return key(a) < key(b); });
+    for (int j = 0; j < t->Gs; ++j)
+        for (int e = 0; e < 4; ++e) t->gtab[4 * (size_t)j + e] = was[4 * (size_t)ord[j] + e];
 }
 
 }  // namespace opf

@@ -215,13 +215,23 @@ inline int32_t cap_at_tests(int32_t max_iter, int32_t k) {
     return (int32_t)(r < top ? r : top);
 }
 
+// Row of slot e of chunk ch in the shared-memory slot array whose rows (one
+// slot, K columns) take `bytes`: 32-byte rows swizzle by the chunk, 16-byte
+// rows by its pair, 8-byte rows by its group of four.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+constexpr int slot_row(int ch, int e, int bytes) {
+    return ch * 4 + (e ^ ((ch >> (bytes >= 32 ? 0 : bytes >= 16 ? 1 : 2)) & 3));
+}
+
 constexpr int kBatchRecip = 256;   // copy counts of a global are below this (the 8-bit count field)
 
 
 // Arguments of one batched-engine launch.  Instance column sc of CTA c holds
 // instance inst[c * K + sc] (-1: empty).  Engine arrays (type T):
 //   per slot      [c][NCH][K][4]   mu, ds, bt (+bbar~ if M = F^T F, else -bbar~; FP64: rho times that),
-//                                  lref (lambda_ref)
+//                                  lref (lambda_ref), xsr (x_ref of the slot's global)
 //   per global    [c][G][K]        xrf (x_ref), xo (x~ at the end)
 //   per bounded   [c][NB][K]       lbt, ubt (bounds - x_ref), cbt (c~)
 // The reference lambda_ref of the shifted frame makes c~ = c + sum lambda_ref
@@ -240,8 +250,7 @@ struct BatchArgs {
     // [qstart[q], qstart[q + 1]) and run only on warps w with w % 4 == q.
     int tm, tm_cols, qstart[5];
     const BatchTask *tasks;    // [n_tasks] in decreasing cost
-    const int4 *chg;           // [NCH] g * K of each chunk's 4 slots (-1: padding)
-    // slot-array row of a copy: (ch * 4 + (e ^ (ch & 3))) * K
+    // slot-array row of a copy: slot_row(ch, e, K * sizeof(T)) * K
     const int4 *gtab;          // [Gs] (row of copy 0, row of copy 1, copies | first later copy in uxt << 8,
                                //       bounded index or -1)
     const int *uxt;            // [n_uxt] rows of the third and later copies
@@ -251,7 +260,7 @@ struct BatchArgs {
     const T *Fpk;              // [nF] factors, task-interleaved
     const T *cost;             // [G] c_i
     T *mu, *ds, *xo;
-    const T *bt, *lref, *xrf, *lbt, *ubt, *cbt;
+    const T *bt, *lref, *xsr, *xrf, *lbt, *ubt, *cbt;
     const int *inst;
     DevStatus *st;             // per instance
     T rho, inv_rho;
