@@ -33,7 +33,8 @@ namespace opf {
 
 
 
-int launch_precompute(const PreArgs &a, cudaStream_t st);
+size_t precompute_smem(int m, int n);
+int launch_precompute(const PreArgs &a, int max_n, cudaStream_t st);
 void launch_pack_factors(int S, const int4 *sub, const int4 *sub2, const long long *cap_off,
                          const double *src, double *dst64, float *dst32, cudaStream_t st);
 template <typename T>
@@ -223,8 +224,17 @@ static int build_layout(opf_handle *h) {
             for (int i = 0; i < sm[d]; ++i) h->canon_row_to_dev[crow0[order[d]] + i] = boff[d] + i;
     }
     h->nA = ao; h->nB = bo; h->nP = po; h->nFcap = fo; h->nF = std::max<long long>(fc, 4);
-    h->sh_m = std::min(h->sh_m, 64);
-    h->sh_n = std::min(h->max_ns, 64);
+    // The precompute's shared memory covers every subsystem when their CTAs then
+    // run in at most three waves, else those of up to 64 rows and columns (the
+    // others work in global memory, and more CTAs fit an SM): 240 blocks of up to
+    // 100 slots 1.37 against 1.88 ms, 400 of up to 110 1.55 against 2.39; 2000 of
+    // up to 80, 100 and 110 2.03, 4.25 and 4.57 against 1.93, 2.81 and 3.25.
+    h->sh_n = h->max_ns;
+    const size_t shared = precompute_smem(h->sh_m, h->sh_n), room = 220 * 1024;
+    if ((size_t)h->S > 3 * (room / shared) * (size_t)stream_sm_count(h->stream, h->device)) {
+        h->sh_m = std::min(h->sh_m, 64);
+        h->sh_n = std::min(h->sh_n, 64);
+    }
     // u segments: copies of each global contiguous, canonical slot order inside
     std::vector<int> cnt(h->G, 0);
     for (int k = 0; k < h->L; ++k) cnt[gk[k]]++;
@@ -415,7 +425,7 @@ static int launch_precompute_kernel(opf_handle *h, bool with_pinv) {
     if (with_pinv) {
         a.Tw = h->d_Tw; a.toff = h->d_toff; a.pinv = h->d_pinv; a.pioff = h->d_pioff; a.nrej = h->d_nrej;
     }
-    if (launch_precompute(a, h->stream)) { g_last_error = "cannot size the precompute kernel"; return OPF_E_CUDA; }
+    if (launch_precompute(a, h->max_ns, h->stream)) { g_last_error = "cannot size the precompute kernel"; return OPF_E_CUDA; }
     CUDA_TRY(cudaGetLastError());
     return OPF_OK;
 }

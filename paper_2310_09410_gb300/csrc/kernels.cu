@@ -1,6 +1,6 @@
 // Device kernels of the ADMM library (sm_103a).
 //
-//  k_precompute   Algorithm 1 precomputation (Sec. III-B), FP64, one warp per
+//  k_precompute   Algorithm 1 precomputation (Sec. III-B), FP64, one CTA per
 //                 subsystem: Gram-Schmidt with re-orthogonalisation on the rows
 //                 of A_s gives an orthonormal basis Q of row(A_s); the same
 //                 operations on b_s give bbar_s = A_s^+ b_s = sum_k beta_k q_k.
@@ -56,239 +56,246 @@ __device__ __forceinline__ T ld(const T *p) {
 
 // ============================================================ precompute
 
-// Coefficients c_k = <rows_k, v> for k < nr of the lane-distributed vector v
-// (entries v[t] at column lane + 32 t): per-lane partials go through a
-// shared/global transpose so the nr warp reductions run side by side.
-__device__ __forceinline__ void project_coeffs(const double *rows, int n, int nr, const double v[RMAX],
-                                               int T, int lane, double *red, double *coef) {
-    for (int k = 0; k < nr; ++k) {
-        double p = 0.0;
-#pragma unroll
-        for (int t = 0; t < RMAX; ++t) {
-            const int c = lane + 32 * t;
-            if (t < T && c < n) p += rows[(long long)k * n + c] * v[t];
-        }
-        red[k * 32 + lane] = p;
+// Zero (either sign) without an FP64 compare; an order-preserving integer.
+__device__ __forceinline__ bool is_zero(double x) { return ((unsigned long long)__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ long long ordered_key(double x) {
+    const long long b = is_zero(x) ? 0 : __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// One CTA per subsystem (n + 1 <= blockDim.x).  Rows of A_s (turned into Q in
+// place) and the null-space rows N live in shared memory when the subsystem
+// fits (m <= sh_m, n <= sh_n), else in the per-subsystem global scratch.
+// What bounds it: dependent FP64 chains (an FP64 instruction of a warp occupies
+// its sub-partition's pipe for about 64 cycles, whatever lanes are active).  So
+// the products of a row with the earlier ones are spread over the warps, a
+// column's update is one chain on its own thread (b_s is one more column), sums
+// run over the occupied lanes only, the rows' first norms are taken together at
+// the start, and the pivot compares order-preserving integers.
+// The order of every sum is that of one warp per subsystem, lane l the columns
+// l, l + 32, ..: the pivots of structured rows tie up to rounding, so another
+// order picks another basis, which the FP32 engines round differently (sums
+// spread over more lanes: opf_precompute of 13 buses 0.22 ms instead of 0.34).
+// opf_precompute of 13 / 123 / 8500 buses and of 240 blocks of up to 100 slots:
+// 0.86 / 0.70 / 1.69 / 8.98 ms with one warp per subsystem, eight predicated
+// columns per lane and rows of more than 64 columns in global memory, now 0.34 /
+// 0.27 / 0.78 / 1.99 ms.
+struct PreSpace {
+    double *Q, *N, *red, *beta, *s0;   // red: per-lane products; s0: squared norms of the rows as given
+    double *v, *coef;                  // the row being orthogonalised (v[n] its right-hand side), its coefficients
+    int rs;                            // row stride of red
+};
+
+// x - sum_k a[k as] b[k bs], k < nr, in that order, four terms' loads in flight.
+__device__ __forceinline__ double chain_sub(double x, const double *a, int as, const double *b, int bs, int nr) {
+    int k = 0;
+    for (; k + 4 <= nr; k += 4, a += 4 * as, b += 4 * bs) {
+        const double u0 = a[0], u1 = a[as], u2 = a[2 * as], u3 = a[3 * as];
+        const double v0 = b[0], v1 = b[bs], v2 = b[2 * bs], v3 = b[3 * bs];
+        x -= u0 * v0;
+        x -= u1 * v1;
+        x -= u2 * v2;
+        x -= u3 * v3;
     }
-    __syncwarp();
-    for (int k = lane; k < nr; k += 32) {
+    for (; k < nr; ++k, a += as, b += bs) x -= a[0] * b[0];
+    return x;
+}
+
+// v[c] -= sum_k <rows_k, v> rows_k[c], k < nr; with beta != nullptr the
+// right-hand side goes along (and row j of Ta, when given).
+__device__ __forceinline__ void project_out(const PreSpace &ps, const double *rows, int n, int nr, const double *beta,
+                                            double *Ta, int m, int j) {
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;
+    const int terms = n < 32 ? n : 32;
+    // a warp per row, the first 128 columns' loads in flight
+    double x[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) x[t] = lane + 32 * t < n ? ps.v[lane + 32 * t] : 0.0;
+    for (int k = tid >> 5; k < nr; k += nthr >> 5) {
+        const double *row = rows + k * n;
+        double y[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) y[t] = lane + 32 * t < n ? row[lane + 32 * t] : 0.0;
+        double p = y[0] * x[0];
+        if (n > 32) p = fma(y[1], x[1], p);
+        if (n > 64) p = fma(y[2], x[2], p);
+        if (n > 96) p = fma(y[3], x[3], p);
+        for (int c = lane + 128; c < n; c += 32) p += row[c] * ps.v[c];
+        ps.red[k * ps.rs + lane] = p;
+    }
+    __syncthreads();
+    for (int k = tid; k < nr; k += nthr) {
         double acc = 0.0;
-        for (int i = 0; i < 32; ++i) acc += red[k * 32 + i];
-        coef[k] = acc;
+#pragma unroll 8
+        for (int i = 0; i < terms; ++i) acc += ps.red[k * ps.rs + i];
+        ps.coef[k] = acc;
     }
-    __syncwarp();
+    __syncthreads();
+    if (tid < n || (tid == n && beta))       // one chain for both kinds: they share a warp
+        ps.v[tid] = chain_sub(ps.v[tid], ps.coef, 1, tid < n ? rows + tid : beta, tid < n ? n : 1, nr);
+    if (Ta)
+        for (int i = tid; i < m; i += nthr) {
+            double x = Ta[(long long)j * m + i];
+            for (int k = 0; k < nr; ++k) x -= ps.coef[k] * Ta[(long long)k * m + i];
+            Ta[(long long)j * m + i] = x;
+        }
+    __syncthreads();
 }
 
-__device__ __forceinline__ double warp_norm(const double v[RMAX]) {
-    double s = 0.0;
-#pragma unroll
-    for (int t = 0; t < RMAX; ++t) s += v[t] * v[t];
-    return sqrt(warp_sum(s));
+// || v ||^2 by a warp (every lane).
+__device__ __forceinline__ double row_norm2(const double *v, int n) {
+    const int lane = threadIdx.x & 31;
+    const double v0 = lane < n ? v[lane] : 0.0, v1 = lane + 32 < n ? v[lane + 32] : 0.0;
+    double s = fma(v0, v0, __dmul_rn(v1, v1));
+    for (int c = lane + 64; c < n; c += 32) s = fma(v[c], v[c], s);
+    return warp_sum(s);
 }
 
-// One warp per subsystem.  Rows of A_s (turned into Q in place), the null-space
-// rows N and the reduction scratch live in shared memory when the subsystem
-// fits (m <= sh_m, n <= sh_n), otherwise in the per-subsystem global scratch.
-__global__ void __launch_bounds__(32) k_precompute(PreArgs a) {
+__global__ void __launch_bounds__(288) k_precompute(PreArgs a) {
     extern __shared__ __align__(16) double shp[];
+    __shared__ double vrow[OPF_MAX_NS + 1], coefs[OPF_MAX_NS];
+    __shared__ long long wkey[9];
+    __shared__ int wcol[9];
     const int s = blockIdx.x;
-    const int lane = threadIdx.x;
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, w = tid >> 5, nw = nthr >> 5;
     if (s >= a.S) return;
     const int m = a.sm[s], n = a.sn[s];
-    const int T = (n + 31) >> 5;
-    const bool use_sh = m <= a.sh_m && n <= a.sh_n;
-    const int mm = m > 0 ? m : 1;
-    double *Q, *N, *red, *coef, *beta;
-    if (use_sh) {
-        Q = shp;
-        N = Q + a.sh_m * a.sh_n;
-        red = N + a.sh_n * a.sh_n;
-        coef = red + 32 * (a.sh_m > a.sh_n ? a.sh_m : a.sh_n);
-        beta = coef + (a.sh_m > a.sh_n ? a.sh_m : a.sh_n);
-        for (int i = lane; i < m * n; i += 32) Q[i] = a.W[a.aoff[s] + i];
-        for (int i = lane; i < m; i += 32) beta[i] = a.Bw[a.boff[s] + i];
+    PreSpace ps;
+    ps.v = vrow;
+    ps.coef = coefs;
+    if (m <= a.sh_m && n <= a.sh_n) {
+        const int big = a.sh_m > a.sh_n ? a.sh_m : a.sh_n;
+        ps.rs = 33;
+        ps.Q = shp;
+        ps.N = ps.Q + a.sh_m * a.sh_n;
+        ps.red = ps.N + (a.sh_n / 2) * a.sh_n;
+        ps.beta = ps.red + 33 * big;
+        ps.s0 = ps.beta + a.sh_m;
+        for (int i = tid; i < m * n; i += nthr) ps.Q[i] = a.W[a.aoff[s] + i];
+        for (int i = tid; i < m; i += nthr) ps.beta[i] = a.Bw[a.boff[s] + i];
     } else {
-        Q = a.W + a.aoff[s];
-        N = a.P + a.poff[s];
-        red = N + (long long)n * n;
-        coef = red + 32 * (m > n ? m : n);
-        beta = a.Bw + a.boff[s];
+        ps.rs = 32;
+        ps.Q = a.W + a.aoff[s];
+        ps.N = a.P + a.poff[s];
+        ps.red = ps.N + (long long)n * n;
+        ps.beta = a.Bw + a.boff[s];
+        ps.s0 = ps.red + 32LL * n;
     }
-    (void)mm;
-    __syncwarp();
+    double *Q = ps.Q, *N = ps.N, *beta = ps.beta;
+    const long long ld = n;
+    // T (optional): the identity under the same row operations, so that beta = T b
+    double *Ta = nullptr, *Tr = nullptr;
+    if (a.pinv) {
+        Ta = a.Tw + a.toff[s];
+        Tr = Ta + (long long)m * m;
+        for (int i = tid; i < m * m; i += nthr) Ta[i] = (i / m == i % m) ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    for (int j = w; j < m; j += nw) {
+        const double q = row_norm2(Q + j * ld, n);
+        if (lane == 0) ps.s0[j] = q;
+    }
     double bmax = 0.0;
     for (int j = lane; j < m; j += 32) bmax = fmax(bmax, fabs(beta[j]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
-    // T (optional): the identity under the same row operations, so that beta = T b
-    const bool want_t = a.pinv != nullptr;
-    double *Ta = nullptr, *Tr = nullptr;
-    if (want_t) {
-        Ta = a.Tw + a.toff[s];
-        Tr = Ta + (long long)m * m;
-        for (int i = lane; i < m * m; i += 32) Ta[i] = (i / m == i % m) ? 1.0 : 0.0;
-        __syncwarp();
-    }
     int nrj = 0;
     // classical Gram-Schmidt, applied twice, on the rows; b follows the same operations
     int r = 0, bad = 0;
     for (int j = 0; j < m; ++j) {
-        double v[RMAX];
-#pragma unroll
-        for (int t = 0; t < RMAX; ++t) {
-            const int c = lane + 32 * t;
-            v[t] = (t < T && c < n) ? Q[(long long)j * n + c] : 0.0;
-        }
-        double bj = beta[j];
-        const double n0 = warp_norm(v);
-        for (int pass = 0; pass < 2 && r > 0; ++pass) {
-            project_coeffs(Q, n, r, v, T, lane, red, coef);
-            for (int k = 0; k < r; ++k) {
-                const double ck = coef[k];
-#pragma unroll
-                for (int t = 0; t < RMAX; ++t) {
-                    const int c = lane + 32 * t;
-                    if (t < T && c < n) v[t] -= ck * Q[(long long)k * n + c];
-                }
-                bj -= ck * beta[k];
-                if (want_t)
-                    for (int i = lane; i < m; i += 32) Ta[(long long)j * m + i] -= ck * Ta[(long long)k * m + i];
-            }
-            __syncwarp();
-        }
-        const double nr = warp_norm(v);
-        if (n0 > 0.0 && nr > 1e-10 * n0) {
+        if (tid <= n) ps.v[tid] = tid < n ? Q[j * ld + tid] : beta[j];
+        __syncthreads();
+        for (int pass = 0; pass < 2 && r > 0; ++pass) project_out(ps, Q, n, r, beta, Ta, m, j);
+        // a row stays when its norm is above 1e-10 of what it was
+        const double s0 = ps.s0[j], s1 = row_norm2(ps.v, n), nr = sqrt(s1);
+        if (s0 > 0.0 && (s1 > 1.001e-20 * s0 || nr > 1e-10 * sqrt(s0))) {
             const double inv = 1.0 / nr;
-#pragma unroll
-            for (int t = 0; t < RMAX; ++t) {
-                const int c = lane + 32 * t;
-                if (t < T && c < n) Q[(long long)r * n + c] = v[t] * inv;
-            }
-            __syncwarp();
-            if (lane == 0) beta[r] = bj * inv;
-            if (want_t)
-                for (int i = lane; i < m; i += 32) Ta[(long long)r * m + i] = Ta[(long long)j * m + i] * inv;
+            if (tid < n) Q[r * ld + tid] = ps.v[tid] * inv;
+            if (tid == n) beta[r] = ps.v[n] * inv;
+            if (Ta)
+                for (int i = tid; i < m; i += nthr) Ta[(long long)r * m + i] = Ta[(long long)j * m + i] * inv;
             ++r;
         } else {
-            if (want_t) {
-                for (int i = lane; i < m; i += 32) Tr[(long long)nrj * m + i] = Ta[(long long)j * m + i];
-                ++nrj;
-            }
-            if (fabs(bj) > 1e-9 * (1.0 + bmax)) bad = 1;
+            if (Ta)
+                for (int i = tid; i < m; i += nthr) Tr[(long long)nrj * m + i] = Ta[(long long)j * m + i];
+            ++nrj;
+            if (tid == n && fabs(ps.v[n]) > 1e-9 * (1.0 + bmax)) bad = 1;
         }
-        __syncwarp();
+        __syncthreads();
     }
     // A_s^+ = Q^T T_acc (n x m)
-    if (want_t) {
+    if (Ta) {
         double *Pi = a.pinv + a.pioff[s];
-        for (int c = lane; c < n; c += 32)
-            for (int i = 0; i < m; ++i) {
-                double acc = 0.0;
-                for (int k = 0; k < r; ++k) acc += Q[(long long)k * n + c] * Ta[(long long)k * m + i];
-                Pi[(long long)c * m + i] = acc;
-            }
-        if (lane == 0) a.nrej[s] = nrj;
-        __syncwarp();
+        for (int e = tid; e < n * m; e += nthr) {
+            const int c = e / m, i = e - c * m;
+            double acc = 0.0;
+            for (int k = 0; k < r; ++k) acc += Q[k * ld + c] * Ta[(long long)k * m + i];
+            Pi[e] = acc;
+        }
+        if (tid == 0) a.nrej[s] = nrj;
     }
     // bbar = sum_k beta_k q_k
-    const int so = a.soff[s];
-    for (int c = lane; c < n; c += 32) {
+    if (tid < n) {
         double acc = 0.0;
-        for (int k = 0; k < r; ++k) acc += beta[k] * Q[(long long)k * n + c];
-        a.bbar[so + c] = acc;
+        for (int k = 0; k < r; ++k) acc += beta[k] * Q[k * ld + tid];
+        a.bbar[a.soff[s] + tid] = acc;
     }
     double *F = a.F + a.foff[s];
     if (r <= n - r) {
-        for (int k = 0; k < r; ++k)
-            for (int c = lane; c < n; c += 32) F[(long long)k * n + c] = Q[(long long)k * n + c];
-        if (lane == 0) { a.sf[s] = r; a.smode[s] = 0; }
+        for (int k = w; k < r; k += nw)
+            for (int c = lane; c < n; c += 32) F[(long long)k * n + c] = Q[k * ld + c];
+        if (tid == 0) { a.sf[s] = r; a.smode[s] = 0; }
     } else {
         // orthonormal basis of null(A_s): pivot on the column c with the largest
-        // remaining norm d_c = 1 - sum_k Q_kc^2 - sum_t N_tc^2, take
-        // e_c - Q^T Q e_c - N^T N e_c, orthogonalise once more, normalise
+        // remaining norm d_c = 1 - sum_k Q_kc^2 - sum_t N_tc^2 (the first of
+        // equal ones), take e_c - Q^T Q e_c - N^T N e_c, orthogonalise once more,
+        // normalise
         const int nf = n - r;
-        double d[RMAX];
-#pragma unroll
-        for (int t = 0; t < RMAX; ++t) {
-            const int c = lane + 32 * t;
-            double acc = 1.0;
-            if (t < T && c < n) {
-                for (int k = 0; k < r; ++k) { const double q = Q[(long long)k * n + c]; acc -= q * q; }
-            } else {
-                acc = -1.0;
-            }
-            d[t] = acc;
-        }
+        double d = 1.0;
+        if (tid < n)
+            for (int k = 0; k < r; ++k) { const double q = Q[k * ld + tid]; d -= q * q; }
         for (int st = 0; st < nf; ++st) {
-            double best = -2.0;
+            long long key = ordered_key(-2.0);
             int bc = 0x7fffffff;
-#pragma unroll
-            for (int t = 0; t < RMAX; ++t) {
-                const int c = lane + 32 * t;
-                if (t < T && c < n && d[t] > best) { best = d[t]; bc = c; }
-            }
+            if (tid < n && !(d != d) && ordered_key(d) > key) { key = ordered_key(d); bc = tid; }
+            auto take = [&](long long ok, int oc) {
+                if (ok > key || (ok == key && oc < bc)) { key = ok; bc = oc; }
+            };
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const long long ok = __shfl_xor_sync(0xffffffffu, key, o);
                 const int oc = __shfl_xor_sync(0xffffffffu, bc, o);
-                if (ob > best || (ob == best && oc < bc)) { best = ob; bc = oc; }
+                take(ok, oc);
             }
-            double v[RMAX];
-#pragma unroll
-            for (int t = 0; t < RMAX; ++t) {
-                const int c = lane + 32 * t;
-                double acc = (c == bc) ? 1.0 : 0.0;
-                if (t < T && c < n) {
-                    for (int k = 0; k < r; ++k) acc -= Q[(long long)k * n + bc] * Q[(long long)k * n + c];
-                    for (int k = 0; k < st; ++k) acc -= N[(long long)k * n + bc] * N[(long long)k * n + c];
-                } else {
-                    acc = 0.0;
+            if (lane == 0) { wkey[w] = key; wcol[w] = bc; }
+            __syncthreads();
+            for (int i = 0; i < nw; ++i) take(wkey[i], wcol[i]);
+            if (tid < n) {
+                double x = tid == bc ? 1.0 : 0.0;
+                if (bc < n) {
+                    x = chain_sub(x, Q + bc, n, Q + tid, n, r);
+                    x = chain_sub(x, N + bc, n, N + tid, n, st);
                 }
-                v[t] = acc;
+                ps.v[tid] = x;
             }
+            __syncthreads();
             // second pass against Q and the null rows found so far
-            if (r > 0) {
-                project_coeffs(Q, n, r, v, T, lane, red, coef);
-                for (int k = 0; k < r; ++k) {
-                    const double ck = coef[k];
-#pragma unroll
-                    for (int t = 0; t < RMAX; ++t) {
-                        const int c = lane + 32 * t;
-                        if (t < T && c < n) v[t] -= ck * Q[(long long)k * n + c];
-                    }
-                }
-                __syncwarp();
-            }
-            if (st > 0) {
-                project_coeffs(N, n, st, v, T, lane, red, coef);
-                for (int k = 0; k < st; ++k) {
-                    const double ck = coef[k];
-#pragma unroll
-                    for (int t = 0; t < RMAX; ++t) {
-                        const int c = lane + 32 * t;
-                        if (t < T && c < n) v[t] -= ck * N[(long long)k * n + c];
-                    }
-                }
-                __syncwarp();
-            }
-            const double nn = warp_norm(v);
+            if (r > 0) project_out(ps, Q, n, r, nullptr, nullptr, m, 0);
+            if (st > 0) project_out(ps, N, n, st, nullptr, nullptr, m, 0);
+            const double nn = sqrt(row_norm2(ps.v, n));
             const double inv = nn > 0.0 ? 1.0 / nn : 0.0;
-#pragma unroll
-            for (int t = 0; t < RMAX; ++t) {
-                const int c = lane + 32 * t;
-                if (t < T && c < n) {
-                    const double x = v[t] * inv;
-                    N[(long long)st * n + c] = x;
-                    d[t] -= x * x;
-                }
+            if (tid < n) {
+                const double x = ps.v[tid] * inv;
+                N[st * ld + tid] = x;
+                d -= x * x;
             }
-            __syncwarp();
+            __syncthreads();
         }
-        for (int k = 0; k < nf; ++k)
-            for (int c = lane; c < n; c += 32) F[(long long)k * n + c] = N[(long long)k * n + c];
-        if (lane == 0) { a.sf[s] = nf; a.smode[s] = 1; }
+        for (int k = w; k < nf; k += nw)
+            for (int c = lane; c < n; c += 32) F[(long long)k * n + c] = N[k * ld + c];
+        if (tid == 0) { a.sf[s] = nf; a.smode[s] = 1; }
     }
-    if (lane == 0) a.status[s] = bad;
+    if (tid == n) a.status[s] = bad;
 }
 
 // Factors written at capacity offsets (n x f, column stride n) are packed into
@@ -1344,13 +1351,18 @@ static inline int nblocks(long long n, int t) {
     return (int)b;
 }
 
-int launch_precompute(const PreArgs &a, cudaStream_t st) {
-    const int big = a.sh_m > a.sh_n ? a.sh_m : a.sh_n;
-    const size_t shm = sizeof(double) * ((size_t)a.sh_m * a.sh_n + (size_t)a.sh_n * a.sh_n +
-                                         33 * (size_t)big + (size_t)a.sh_m + 2);
+// Shared memory of subsystems of up to m rows and n columns.
+size_t precompute_smem(int m, int n) {
+    return sizeof(double) * ((size_t)(m + n / 2) * n + 33 * (size_t)(m > n ? m : n) + 2 * (size_t)m + 2);
+}
+
+int launch_precompute(const PreArgs &a, int max_n, cudaStream_t st) {
+    const size_t shm = precompute_smem(a.sh_m, a.sh_n);
     if (cudaFuncSetAttribute(k_precompute, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess)
         return -1;
-    k_precompute<<<a.S, 32, shm, st>>>(a);
+    // 4 warps up to 63 columns (8: 8500 buses 0.79 -> 1.23 ms), 8 above (240 blocks
+    // of up to 100: 2.18 -> 1.99 ms), and one more for the right-hand side at 256
+    k_precompute<<<a.S, 32 * (max_n < 64 ? 4 : max_n < 256 ? 8 : 9), shm, st>>>(a);
     return 0;
 }
 

@@ -53,7 +53,6 @@ int build_generic_model(int n, const double *c, const double *lb, const double *
                         const double *A, const double *b, const int *idx,
                         HostModel *out, std::string *err);
 
-constexpr int RMAX = 8;   // entries per lane in the precompute (n <= 256)
 
 // Arguments of one iteration, in precision T.  Pointers may address global or
 // shared memory (generic addressing).
