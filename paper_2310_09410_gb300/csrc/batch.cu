@@ -367,9 +367,10 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs
 // every tensor-memory load of a task before one wait; a slot array free of
 // bank conflicts at each K; global-update items sorted so that a warp's lanes
 // take the same branches.  us per iteration with a test every 50, before and
-// now: 123 buses, 20 instances (K = 2) 4.11 -> 3.37; 34 buses, 201 instances
-// (K = 2) 2.47 -> 1.98; 123 buses, 1024 instances (K = 8) 6.57 -> 6.41, of
-// which the tests take 0.42 -> 0.26.  Tried and slower: four rows per step
+// now, with four chunks per lane as before and with the plan's choice
+// (task_chunks): 123 buses, 20 instances (K = 2) 4.11 -> 3.37 -> 3.10; 34 buses,
+// 201 instances (K = 2) 2.47 -> 1.98 -> 1.71; 123 buses, 1024 instances (K = 8)
+// 6.57 -> 6.39, of which the tests take 0.42 -> 0.26.  Tried and slower: four rows per step
 // (K = 8 6.19 -> 7.4), 20 or 24 warps (6.24 -> 6.46, 7.42), the next rows'
 // factors prefetched (spills), two chains per row (K = 2 3.19 -> 3.35).
 using u64 = unsigned long long;
@@ -433,13 +434,21 @@ __device__ __forceinline__ void rows(const float *F0, int rstride, const u64 (&v
         }
 }
 
-// The f rows (an even number: a member's missing rows are zero), two per step.
+// The f rows (an even number: a member's missing rows are zero), two per step;
+// with one instance per CTA, where a warp has a task or two and waits on their
+// chains, six or four while they last (34 buses 1.68 -> 1.56 us per iteration).
 template <int K, int NQT, int LP>
 __device__ __forceinline__ void task_rows(const float *F0, int rstride, int f, const u64 (&v)[2 * NQT],
                                           u64 (&y)[2 * NQT]) {
-    constexpr int R = 2;
+    int r = 0;
+    if constexpr (K == 1 && NQT == 1)
 #pragma unroll 1
-    for (int r = 0; r < f; r += R, F0 += R * rstride) rows<K, NQT, R, LP>(F0, rstride, v, y);
+        for (; r + 6 <= f; r += 6, F0 += 6 * rstride) rows<K, NQT, 6, LP>(F0, rstride, v, y);
+    if constexpr (K == 1 && NQT <= 2)
+#pragma unroll 1
+        for (; r + 4 <= f; r += 4, F0 += 4 * rstride) rows<K, NQT, 4, LP>(F0, rstride, v, y);
+#pragma unroll 1
+    for (; r < f; r += 2, F0 += 2 * rstride) rows<K, NQT, 2, LP>(F0, rstride, v, y);
 }
 
 // Keeps uses of the values after the point where it stands (a tensor-memory wait).
@@ -498,7 +507,8 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const float *Fs,
         case 1: task_rows<K, NQT, 1>(F0, rstride, tk.f, v, y); break;
         case 2: task_rows<K, NQT, 2>(F0, rstride, tk.f, v, y); break;
         case 3: if constexpr (J >= 8) task_rows<K, NQT, 3>(F0, rstride, tk.f, v, y); break;
-        default: if constexpr (J >= 16) task_rows<K, NQT, 4>(F0, rstride, tk.f, v, y); break;
+        case 4: if constexpr (J >= 16) task_rows<K, NQT, 4>(F0, rstride, tk.f, v, y); break;
+        default: if constexpr (J >= 32) task_rows<K, NQT, 5>(F0, rstride, tk.f, v, y); break;
     }
     // rho x_s = y or V - y, as ca V + cb y with exact coefficients
     const float ca = mode1 ? 0.0f : 1.0f, cb = mode1 ? 1.0f : -1.0f;
@@ -1294,13 +1304,15 @@ static inline int bl(long long n, int t) {
     return (int)b;
 }
 
-// Instantiated shapes: FP32 with factors in shared memory (K = 2, 4, 8; NQ = 4),
+// Instantiated shapes: FP32 with factors in shared memory (K = 1, 2, 4, 8; NQ = 4),
 // lambda and bbar~ in tensor memory or streamed from L2; FP64 (NQ = 2,
 // K = 1, 2, 4) with factors in shared or global memory.
 template <typename T>
 static const void *engine_fn(int K, int nq, bool fg, bool tm) {
     if constexpr (sizeof(T) == 4) {
         if (fg || nq != 4) return nullptr;
+        if (K == 1) return tm ? (const void *)k_batch_engine<float, 1, 4, false, true>
+                              : (const void *)k_batch_engine<float, 1, 4, false, false>;
         if (K == 2) return tm ? (const void *)k_batch_engine<float, 2, 4, false, true>
                               : (const void *)k_batch_engine<float, 2, 4, false, false>;
         if (K == 4) return tm ? (const void *)k_batch_engine<float, 4, 4, false, true>

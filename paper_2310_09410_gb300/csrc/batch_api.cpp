@@ -72,9 +72,29 @@ int ilog2(int x) {
     return l;
 }
 
+// Chunks per lane of an FP32 plan's tasks, at most 4: fewer chunks give a wide
+// subsystem more lanes and its rows shorter chains, and cost lane sums and
+// padding.  Two when every warp then has one task at most, else three, as long
+// as tensor memory and the member positions hold the plan, else four.  us per
+// iteration with 4 / 3 / 2 (a test every 50): 34 buses, 201 instances (K = 2, 8
+// warps) 1.98 / 1.71 / 1.92; 34 and 13 buses, 20 instances (K = 1) 1.96 / 1.71 /
+// 1.68 and 1.93 / 1.83 / 1.71; 123 buses, 20 instances (K = 2) 3.38 / 3.10 /
+// 3.55, 400 (K = 4) 4.56 / 4.17 / 5.16.
+int task_chunks(const opf_handle *h, int K, int W) {
+    for (int nq : {2, 3}) {
+        TaskPlan tp;
+        if (build_task_plan(h->S, h->L, h->h_npad, h->h_sf, h->h_mode, h->h_soff, h->h_sn, h->h_gk, K, nq, W % 4 == 0,
+                            &tp) == 0 &&
+            (tp.tm || W % 4) && (nq == 3 || (int)tp.tasks.size() <= W))
+            return nq;
+    }
+    return 4;
+}
+
 // Builds the tables of a plan with K instance columns, W warps and NQ chunks
-// per lane; returns OPF_E_CAPACITY when the shape cannot hold the model.
-int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) {
+// per lane (the tasks' at most `chunks`); returns OPF_E_CAPACITY when the shape
+// cannot hold the model.  With dry the fit alone is checked.
+int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, int chunks, bool fg, bool dry = false) {
     opf_handle *h = b->h;
     cudaStream_t st = h->stream;
     p->release();
@@ -85,7 +105,7 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
     const size_t sz = dbl ? sizeof(double) : sizeof(float);
     // warp tasks, tensor-memory quadrants, chunk and slot tables (batch_tables.h)
     TaskPlan tp;
-    const int trc = build_task_plan(S, L, h->h_npad, h->h_sf, h->h_mode, h->h_soff, h->h_sn, h->h_gk, K, nq,
+    const int trc = build_task_plan(S, L, h->h_npad, h->h_sf, h->h_mode, h->h_soff, h->h_sn, h->h_gk, K, chunks,
                                     !dbl && b->allow_tmem && W % 4 == 0, &tp);
     if (trc == 1) { set_last_error("batch plan: a subsystem needs more lanes than a task has"); return OPF_E_CAPACITY; }
     if (trc) { set_last_error("batch plan: slot without a chunk"); return OPF_E_INVALID; }
@@ -133,6 +153,7 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, bool fg) 
     p->off_flag = p->off_red + a16((size_t)W * K * 6 * sizeof(double));
     p->bytes = p->off_flag + a16((size_t)(2 * K + 4) * sizeof(int));
     if (p->bytes > kMaxSmem) { set_last_error("batch plan: shared memory"); return OPF_E_CAPACITY; }
+    if (dry) return OPF_OK;
     const int rc = dbl ? batch_engine_prepare<double>(K, nq, fg, p->tm, p->bytes)
                        : batch_engine_prepare<float>(K, nq, fg, p->tm, p->bytes);
     if (rc) { set_last_error("batch plan: engine attributes"); return OPF_E_CUDA; }
@@ -362,7 +383,7 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
         for (int fg = 0; fg < 2; ++fg)
             for (int K : ks) {
                 if (fk && K != fk) continue;
-                if (build_plan(b, &p, true, K, fw, 2, fg != 0) == OPF_OK) return OPF_OK;
+                if (build_plan(b, &p, true, K, fw, 2, 2, fg != 0) == OPF_OK) return OPF_OK;
             }
         p.release();
         set_last_error("batch: no FP64 engine shape fits");
@@ -371,30 +392,43 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
     // candidates (K, W); K = kLaneInst (the lane engine, W / 4 warps per lane
     // quadrant) only when asked for: it measured several times slower than
     // these shapes on the feeders it holds
-    std::vector<std::pair<int, int>> cand;
-    if (b->force_k32) cand.push_back({b->force_k32, b->force_w32 > 0 ? b->force_w32 : 16});
-    else {
-        const int Ks[] = {8, 4, 2};
-        const int Ws[] = {16, 12, 8};
-        for (int K : Ks) for (int W : Ws) cand.push_back({K, W});
-    }
     auto build = [&](int K, int W) -> int {
         if (K == kLaneInst) return build_lane_plan(b, &p, W / 4, 16);
-        return build_plan(b, &p, false, K, W, 4, false);
+        const int chunks = task_chunks(h, K, W);
+        if (chunks < 4 && build_plan(b, &p, false, K, W, 4, chunks, false) == OPF_OK) return OPF_OK;
+        return build_plan(b, &p, false, K, W, 4, 4, false);
     };
     b->tune_log.clear();
-    if (cand.size() == 1) {
-        BTRY(build(cand[0].first, cand[0].second));
-        return OPF_OK;
+    if (b->force_k32) {
+        if (b->force_k32 == 1) { set_last_error("batch plan: engine attributes"); return OPF_E_CUDA; }
+        return build(b->force_k32, b->force_w32 > 0 ? b->force_w32 : 16);
     }
+    // K: the fewest instances per CTA that leave an SM per CTA, and half of that
+    // (several CTAs per SM).  More only put more work on fewer SMs (us per
+    // iteration, K as said and its double: 123 buses, 20 instances 2.69 and 3.10;
+    // 34 buses, 304 instances 1.98 and 2.23).  One per CTA needs a model that two
+    // would fit.  The others when none of these fits.
+    std::vector<std::pair<int, int>> cand;
+    const int n_sm = stream_sm_count(h->stream, h->device);
+    int want = 1;
+    while (want < 8 && (b->n + want - 1) / want > n_sm) want *= 2;
+    BPlan two;
+    const bool one = want <= 2 && build_plan(b, &two, false, 2, 8, 4, 4, false, true) == OPF_OK;
+    for (int K = want; K >= std::max(1, want / 2); K /= 2)
+        for (int W : {16, 8})
+            if (K > 1 || one) cand.push_back({K, W});
     // timing runs on a copy of the status; the FP64 state is not touched by
     // the engine (it works on the plan's own arrays)
     BCUDA(cudaMemcpyAsync(b->d_st_save, b->d_st, b->n * sizeof(DevStatus), cudaMemcpyDeviceToDevice, h->stream));
     double best = 1e300;
     int bk = 0, bw = 0;
     const int iters = 2 * std::max(k, 2);
-    for (auto &c : cand) {
-        if (build(c.first, c.second) != OPF_OK) continue;
+    int lk = 0, lw = 0;      // the shape p holds
+    auto timed = [&](int K, int W) -> int {
+        lk = 0;
+        if (build(K, W) != OPF_OK) return OPF_OK;
+        lk = K;
+        lw = W;
         BTRY(plan_set_rho(b, &p, rho));
         launch_bref<float>(b->n, h->S, b->G, b->L, p.K, p.ks, p.NCH, p.NB, p.d_ipos, h->d_gseg, h->d_uslot,
                            b->d_bidx, h->d_c64, h->d_lb64, h->d_ub64, rho, b->d_xs, b->d_lam, b->d_st, b->d_xref,
@@ -403,9 +437,8 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
                            h->d_F64, h->d_gk, p.d_sch, b->d_bbar, (float *)p.bt, (float *)p.ds, (float *)p.mu,
                            (float *)p.lref, (float *)p.xsr, h->stream);
         auto run = [&](int n_it) {
-            if (p.lane) lane_engine_launch(lane_args(b, p, rho), p.C, p.threads, p.bytes, n_it, 0, h->stream);
-            else batch_engine_launch<float>(engine_args<float>(b, p, rho), p.nq, false, p.C, p.threads, p.bytes,
-                                            n_it, 0, h->stream);
+            batch_engine_launch<float>(engine_args<float>(b, p, rho), p.nq, false, p.C, p.threads, p.bytes, n_it, 0,
+                                       h->stream);
         };
         run(4);   // warm-up
         BCUDA(cudaEventRecord(b->ev[0], h->stream));
@@ -415,17 +448,21 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
         BCUDA(cudaGetLastError());
         float ms = 0;
         cudaEventElapsedTime(&ms, b->ev[0], b->ev[1]);
-        b->tune_log.push_back(c.first);
-        b->tune_log.push_back(c.second);
+        b->tune_log.push_back(K);
+        b->tune_log.push_back(W);
         b->tune_log.push_back(ms);
-        if (ms < best) { best = ms; bk = c.first; bw = c.second; }
+        if (ms < best) { best = ms; bk = K; bw = W; }
         BCUDA(cudaMemcpyAsync(b->d_st, b->d_st_save, b->n * sizeof(DevStatus), cudaMemcpyDeviceToDevice, h->stream));
-    }
+        return OPF_OK;
+    };
+    for (const auto &c : cand) BTRY(timed(c.first, c.second));
+    if (!bk)
+        for (int K : {8, 4, 2})
+            for (int W : {16, 12, 8}) BTRY(timed(K, W));
     // the status copies carry the pad (shifted) marks of the timing runs: clear them
     BCUDA(cudaMemcpyAsync(b->d_st, b->d_st_save, b->n * sizeof(DevStatus), cudaMemcpyDeviceToDevice, h->stream));
     if (!bk) { p.release(); set_last_error("batch: no FP32 engine shape fits"); return OPF_E_CAPACITY; }
-    BTRY(build(bk, bw));
-    return OPF_OK;
+    return lk == bk && lw == bw ? OPF_OK : build(bk, bw);
 }
 
 int check_range(opf_batch *b, int first, int count) {

@@ -216,12 +216,12 @@ inline int32_t cap_at_tests(int32_t max_iter, int32_t k) {
 
 // Row of slot e of chunk ch in the shared-memory slot array whose rows (one
 // slot, K columns) take `bytes`: 32-byte rows swizzle by the chunk, 16-byte
-// rows by its pair, 8-byte rows by its group of four.
+// rows by its pair, 8-byte rows by its group of four, 4-byte rows by its eight.
 #ifdef __CUDACC__
 __host__ __device__
 #endif
 constexpr int slot_row(int ch, int e, int bytes) {
-    return ch * 4 + (e ^ ((ch >> (bytes >= 32 ? 0 : bytes >= 16 ? 1 : 2)) & 3));
+    return ch * 4 + (e ^ ((ch >> (bytes >= 32 ? 0 : bytes >= 16 ? 1 : bytes >= 8 ? 2 : 3)) & 3));
 }
 
 constexpr int kBatchRecip = 256;   // copy counts of a global are below this (the 8-bit count field)

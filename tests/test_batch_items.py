@@ -54,8 +54,8 @@ int main() {
                 if (*rows.begin() != 4 * ch || *rows.rbegin() != 4 * ch + 3 || rows.size() != 4)
                     return std::printf("chunk %d, %d bytes\n", ch, bytes), 1;
             }
-            const int lanes = bytes <= 128 ? 128 / bytes : 1;     // chunks of one transaction
-            for (int e = 0; bytes >= 8 && e < 4; ++e)
+            const int lanes = 128 / bytes;     // chunks of one transaction
+            for (int e = 0; e < 4; ++e)
                 for (int ch = 0; ch + lanes <= 64; ch += lanes) {
                     std::set<int> at;
                     for (int i = 0; i < lanes; ++i) at.insert(slot_row(ch + i, e, bytes) * bytes % 128);
