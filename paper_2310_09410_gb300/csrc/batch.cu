@@ -175,6 +175,13 @@ __device__ __forceinline__ int upos(int ch, int e, int sc) {
     return slot_row(ch, e, K * (int)sizeof(T)) * K + sc;
 }
 
+// A lane's places in a task's chunks.  A task's first chunk and the chunks of
+// its next positions are multiples of J = 32 / K apart, which the swizzle does
+// not see, so they are offsets that the lane keeps for the launch.
+struct LaneRows {
+    int at[4];
+};
+
 // ---- tensor memory (tcgen05, tmem.cuh): lambda and bbar~ of the tasks,
 // 32-bit columns.
 // 8 consecutive columns of the lane: lambda (4) then bbar~ (4) of one chunk
@@ -253,13 +260,14 @@ __device__ __forceinline__ void tm_stage_out(const BatchTask &tk, unsigned tl, f
 template <int K, int NQT, bool>
 __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs, double *us, double *mu_c,
                                            const double *bt_c, double *ds_c, const double *lr_c, const double *xs_c,
-                                           int jpos, int sc, double, double inv_rho, bool check, bool act, bool wds,
+                                           int jpos, int sc, const LaneRows &lr, double, double inv_rho, bool check, bool act, bool wds,
                                            double *redw, unsigned) {
     constexpr int J = 32 / K;
     const int mode1 = (tk.modes >> (jpos >> tk.lp)) & 1;
     double v[4 * NQT], y[4 * NQT];
     double c0 = 0.0, c1 = 0.0, c3 = 0.0, c4 = 0.0;
     const int ch0 = tk.ch0 + jpos;
+    double *ut = us + tk.ch0 * 4 * K;
 #pragma unroll
     for (int q = 0; q < NQT; ++q) {
         const int ch = ch0 + q * J;
@@ -268,7 +276,7 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             y[4 * q + e] = b4.v[e];
-            v[4 * q + e] = us[upos<double, K>(ch, e, sc)] + m4.v[e];
+            v[4 * q + e] = ut[lr.at[e] + q * J * 4 * K] + m4.v[e];
         }
     }
     // rho x_s = M V + rho bbar~ over the factor rows, two rows per step
@@ -333,7 +341,7 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs
             double t0 = 0.0, t1 = 0.0, t3 = 0.0, t4 = 0.0;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const double d0 = (us[upos<double, K>(ch, e, sc)] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
+                const double d0 = (ut[lr.at[e] + q * J * 4 * K] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
                 const double xa = x4.v[e] + g4.v[e];
                 const double la = m4.v[e] + l4.v[e];
                 t0 += d0 * d0;
@@ -347,7 +355,7 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs
             c4 += t4;
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) us[upos<double, K>(ch, e, sc)] = u4.v[e];
+        for (int e = 0; e < 4; ++e) ut[lr.at[e] + q * J * 4 * K] = u4.v[e];
         if (act) {
             st4cg(mu_c + off, m4);
             if (wds) st4cg(ds_c + off, x4);
@@ -367,12 +375,15 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs
 // every tensor-memory load of a task before one wait; a slot array free of
 // bank conflicts at each K; global-update items sorted so that a warp's lanes
 // take the same branches.  us per iteration with a test every 50, before and
-// now, with four chunks per lane as before and with the plan's choice
-// (task_chunks): 123 buses, 20 instances (K = 2) 4.11 -> 3.37 -> 3.10; 34 buses,
-// 201 instances (K = 2) 2.47 -> 1.98 -> 1.71; 123 buses, 1024 instances (K = 8)
-// 6.57 -> 6.39, of which the tests take 0.42 -> 0.26.  Tried and slower: four rows per step
+// now: 123 buses, 20 instances (K = 2) 4.11 -> 2.97; 34 buses, 201 instances
+// (K = 2) 2.47 -> 1.71; 123 buses, 1024 instances (K = 8) 6.57 -> 6.16, of which
+// the tests take 0.42 -> 0.26.  Single parts: the plan's chunks per lane
+// (task_chunks) 3.37 -> 3.10 and 1.98 -> 1.71, a lane's places in the slot array
+// kept instead of recomputed 6.39 -> 6.29, the items' rows on distinct banks
+// (sort_global_items) 6.29 -> 6.16 and 3.08 -> 2.97.  Tried and slower: four rows per step
 // (K = 8 6.19 -> 7.4), 20 or 24 warps (6.24 -> 6.46, 7.42), the next rows'
-// factors prefetched (spills), two chains per row (K = 2 3.19 -> 3.35).
+// factors prefetched (spills), two chains per row (K = 2 3.19 -> 3.35), whole rows of 8 columns
+// per global-update item (6.29 -> 7.63: two-way conflicts).
 using u64 = unsigned long long;
 __device__ __forceinline__ u64 pk(float a, float b) {
     u64 r;
@@ -460,13 +471,14 @@ __device__ __forceinline__ void tie(Q4<float> &q) {
 template <int K, int NQT, bool TM>
 __device__ __forceinline__ void batch_task(const BatchTask &tk, const float *Fs, float *us, float *mu_c,
                                            const float *bt_c, float *ds_c, const float *lr_c, const float *xs_c,
-                                           int jpos, int sc, float rho, float inv_rho, bool check,
+                                           int jpos, int sc, const LaneRows &lr, float rho, float inv_rho, bool check,
                                            bool act, bool wds, double *redw, unsigned tl) {
     constexpr int J = 32 / K;
     const bool mode1 = (tk.modes >> (jpos >> tk.lp)) & 1;
     u64 v[2 * NQT], y[2 * NQT];
     float f0 = 0.f, f1 = 0.f, f3 = 0.f, f4 = 0.f;     // test terms, FP32 over the task's chunks
     const int ch0 = tk.ch0 + jpos;
+    float *ut = us + tk.ch0 * 4 * K;
     const unsigned tcol = tl + (unsigned)(tk.tm >> 2);
     {
         Q4<float> m4[NQT], b4[NQT];
@@ -495,8 +507,8 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const float *Fs,
             const int ch = ch0 + q * J;
             y[2 * q] = pk(b4[q].v[0], b4[q].v[1]);
             y[2 * q + 1] = pk(b4[q].v[2], b4[q].v[3]);
-            v[2 * q] = add2(pk(us[upos<float, K>(ch, 0, sc)], us[upos<float, K>(ch, 1, sc)]), pk(m4[q].v[0], m4[q].v[1]));
-            v[2 * q + 1] = add2(pk(us[upos<float, K>(ch, 2, sc)], us[upos<float, K>(ch, 3, sc)]), pk(m4[q].v[2], m4[q].v[3]));
+            v[2 * q] = add2(pk(ut[lr.at[0] + q * J * 4 * K], ut[lr.at[1] + q * J * 4 * K]), pk(m4[q].v[0], m4[q].v[1]));
+            v[2 * q + 1] = add2(pk(ut[lr.at[2] + q * J * 4 * K], ut[lr.at[3] + q * J * 4 * K]), pk(m4[q].v[2], m4[q].v[3]));
         }
     }
     // rho x_s = M V + rho bbar~ over the factor rows, two per step
@@ -539,7 +551,7 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const float *Fs,
             }
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float d0 = (us[upos<float, K>(ch, e, sc)] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
+                const float d0 = (ut[lr.at[e] + q * J * 4 * K] - r4.v[e]) * inv_rho, d1 = x4.v[e] - o4.v[e];
                 const float xa = x4.v[e] + g4.v[e];
                 const float la = m4.v[e] + l4.v[e];
                 t0 += d0 * d0;
@@ -553,7 +565,7 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const float *Fs,
             f4 += t4;
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) us[upos<float, K>(ch, e, sc)] = u4.v[e];
+        for (int e = 0; e < 4; ++e) ut[lr.at[e] + q * J * 4 * K] = u4.v[e];
         // (tensor memory: every lane; a frozen column keeps iterating there,
         // its lambda went to the engine array when it froze)
         if constexpr (TM) tm_st4(tcol + 8 * q, m4);
@@ -648,6 +660,9 @@ __global__ void __launch_bounds__(512, 1)
     }
     const int sc = tid & (K - 1);
     const int jpos = lane >> KS;
+    LaneRows lr;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) lr.at[e] = upos<T, K>(jpos, e, sc);
     const int n_warps = nthr >> 5;
     const int qd = w & 3, wq = w >> 2, nwq = n_warps >> 2;     // quadrant, warp in it, warps per quadrant
     unsigned tl = 0;                                             // this warp's tensor-memory lane base
@@ -858,16 +873,16 @@ __global__ void __launch_bounds__(512, 1)
                 if (!check && lane == 0) claim = atomicAdd(cnt, 1);
                 const BatchTask tk = tks[t];
                 switch (tk.nq) {
-                    case 1: batch_task<K, 1, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c, jpos, sc, rho,
+                    case 1: batch_task<K, 1, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c, jpos, sc, lr, rho,
                                                     inv_rho, check, act, wds, redw, tl); break;
                     case 2: if constexpr (NQ >= 2) batch_task<K, 2, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c,
-                                                                           jpos, sc, rho, inv_rho, check, act,
+                                                                           jpos, sc, lr, rho, inv_rho, check, act,
                                                                            wds, redw, tl); break;
                     case 3: if constexpr (NQ >= 3) batch_task<K, 3, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c,
-                                                                           jpos, sc, rho, inv_rho, check, act,
+                                                                           jpos, sc, lr, rho, inv_rho, check, act,
                                                                            wds, redw, tl); break;
                     default: if constexpr (NQ >= 4) batch_task<K, 4, TM>(tk, Fs, us, mu_c, bt_c, ds_c, lr_c, xs_c,
-                                                                            jpos, sc, rho, inv_rho, check, act,
+                                                                            jpos, sc, lr, rho, inv_rho, check, act,
                                                                             wds, redw, tl); break;
                 }
                 t = check ? t + t_step : __shfl_sync(0xffffffffu, claim, 0);

@@ -135,7 +135,7 @@ int build_plan(opf_batch *b, BPlan *p, bool dbl, int K, int W, int nq, int chunk
         set_last_error("batch plan: global table");
         return OPF_E_CAPACITY;
     }
-    sort_global_items(&gt);
+    sort_global_items(&gt, K, std::max(1, 128 / (K * (int)sz)));
     p->Gs = gt.Gs;
     std::vector<int4> gtab(std::max(p->Gs, 1), make_int4(0, 0, 0, -1));
     for (int j = 0; j < p->Gs; ++j)

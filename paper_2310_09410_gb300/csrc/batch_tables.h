@@ -248,20 +248,41 @@ inline bool build_global_tables(int G, const std::vector<int> &gstart, const std
 }
 
 // The computed globals' entries by decreasing number of copies, the bounded
-// ones first, then by the first copy's row, so that the threads of a warp take
-// the same branches and read neighbouring rows.  (The order of the entries is
+// ones first, so that the threads of a warp take the same branches; among those
+// the `group` neighbours that share a shared-memory transaction (rows of K
+// values, 128 bytes) get first and second rows on distinct banks as far as the
+// entries allow, the smallest first row first.  (The order of the entries is
 // free: gperm and gx list the globals of the test on their own.)
-inline void sort_global_items(GlobalTables *t) {
+inline void sort_global_items(GlobalTables *t, int K, int group) {
     const std::vector<int> was(t->gtab);
+    auto entry = [&](int j) { return &was[4 * (size_t)j]; };
     std::vector<int> ord(t->Gs);
     std::iota(ord.begin(), ord.end(), 0);
-    auto key = [&](int j) {
-        const int *e = &was[4 * (size_t)j];
-        return std::make_tuple(-(e[2] & 255), e[3] < 0, e[0]);
-    };
-    std::sort(ord.begin(), ord.end(), [&](int a, int b) { return key(a) < key(b); });
-    for (int j = 0; j < t->Gs; ++j)
-        for (int e = 0; e < 4; ++e) t->gtab[4 * (size_t)j + e] = was[4 * (size_t)ord[j] + e];
+    auto kind = [&](int j) { return std::make_pair(-(entry(j)[2] & 255), entry(j)[3] < 0); };
+    std::sort(ord.begin(), ord.end(), [&](int a, int b) {
+        return std::make_tuple(kind(a), entry(a)[0]) < std::make_tuple(kind(b), entry(b)[0]);
+    });
+    std::vector<char> bank0(group), bank1(group);
+    for (int j = 0; j < t->Gs; ++j) {
+        if (j % group == 0) {
+            std::fill(bank0.begin(), bank0.end(), 0);
+            std::fill(bank1.begin(), bank1.end(), 0);
+        }
+        auto clashes = [&](int i) {
+            const int *e = entry(ord[i]);
+            return bank0[e[0] / K % group] + ((e[2] & 255) > 1 ? bank1[e[1] / K % group] : 0);
+        };
+        int best = j;
+        for (int i = j; i < t->Gs && i < j + 256 && kind(ord[i]) == kind(ord[j]); ++i) {
+            if (clashes(i) < clashes(best)) best = i;
+            if (clashes(best) == 0) break;
+        }
+        std::rotate(ord.begin() + j, ord.begin() + best, ord.begin() + best + 1);
+        const int *e = entry(ord[j]);
+        bank0[e[0] / K % group] = 1;
+        if ((e[2] & 255) > 1) bank1[e[1] / K % group] = 1;
+        for (int q = 0; q < 4; ++q) t->gtab[4 * (size_t)j + q] = e[q];
+    }
 }
 
 }  // namespace opf

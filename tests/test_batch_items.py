@@ -34,7 +34,7 @@ int main() {
             was.insert(e);
             t.gtab.insert(t.gtab.end(), e.begin(), e.end());
         }
-        sort_global_items(&t);
+        sort_global_items(&t, 4, 8);
         for (int j = 0; j < Gs; ++j) {
             const int *e = &t.gtab[4 * j], *p = e - 4;
             now.insert({e[0], e[1], e[2], e[3]});
