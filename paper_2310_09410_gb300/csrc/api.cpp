@@ -54,7 +54,7 @@ int launch_cluster_engine(const IterArgs<T> &g, const ClusterLayout &lay, const 
 template <typename T> int cluster_occupancy(const ClusterLayout &lay);
 template <typename T> int prepare_persist_engine(const PersistLayout &lay);
 template <typename T> long long persist_resident(const PersistLayout &lay, int n_sm);
-template <typename T> size_t persist_exchange_bytes(int L);
+template <typename T> size_t persist_exchange_bytes(long long n);
 template <typename T>
 int launch_persist_engine(const IterArgs<T> &g, const PersistLayout &lay, const PersistPtrs &pp, T *U,
                           int bar_extra, int n_iters, int check_every, DevStatus *st, double rho,
@@ -517,7 +517,7 @@ extern "C" int opf_precompute(opf_handle *h) {
         CUDA_TRY(cudaStreamSynchronize(h->stream));      // the uploads read local vectors
         h->c32.P = h->c64.P = 0;
         h->c32.ok = h->c64.ok = false;
-        for (PersistPlan *pp : {&h->p32, &h->p64, &h->k32, &h->k64}) {
+        for (PersistPlan *pp : {&h->p32, &h->p64, &h->k32, &h->k64, &h->o32, &h->o64}) {
             pp->P = 0;
             pp->ok = pp->tried = false;
             pp->tab.reset();
@@ -772,13 +772,14 @@ static std::vector<int> warp_parts(const opf_handle *h, bool fp32, int req_P) {
 
 // The partition of the instance over P CTAs: parts of a depth-first order for
 // the local forms, else runs of the size-sorted order.
-static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, std::shared_ptr<PersistTables> *out) {
+static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, bool own,
+                                std::shared_ptr<PersistTables> *out) {
     const int S = h->S, L = h->L;
     std::vector<double> cost(S);
     for (int s = 0; s < S; ++s)
         cost[s] = 6.0 * h->h_sn[s] + (double)h->h_sf[s] * h->h_npad[s] + (double)h->h_sn[s] * h->h_sf[s];
     std::vector<int> order;
-    if (local) {
+    if (local && !own) {
         if (h->persist_order.empty()) {
             std::vector<int> start(S);           // new trees begin in canonical order
             for (int d = 0; d < S; ++d) start[h->dev_to_canon_sub[d]] = d;
@@ -789,11 +790,17 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
         order.resize(S);
         std::iota(order.begin(), order.end(), 0);
     }
-    const PersistParts parts = persist_parts(P, S, order, cost, h->h_soff, h->h_segp, h->h_pk);
+    PersistOwners owners;
+    if (own) owners = persist_owners(P, S, h->G, cost, h->h_soff, h->h_segp, h->h_pk, h->h_gk, h->h_gstart);
+    else owners.parts = persist_parts(P, S, order, cost, h->h_soff, h->h_segp, h->h_pk);
+    const PersistParts &parts = owners.parts;
     auto t = std::make_shared<PersistTables>();
     t->P = P; t->S = S; t->L = L;
     t->local = local;
     t->cluster = cluster;
+    t->own = own;
+    t->mog = owners.most_globals;
+    t->moc = owners.most_copies;
     t->fits = parts.ok;
     t->remote = (long long)parts.rem.size();
     // cluster form: a subsystem whose FP32 column products go by halves (in the
@@ -871,6 +878,7 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
         t->md = d.most;
         addv(&t->dst, d.dst); addv(&t->dr, d.d0); addv(&t->dseg, d.dseg); addv(&t->halves, halves);
     }
+    if (own) { addv(&t->g0, owners.g0); addv(&t->gfirst, h->h_gstart); }
     void *q = nullptr;
     CUDA_TRY(cudaMalloc(&q, std::max<size_t>(all.size(), 4) * sizeof(int)));
     t->mem = (int *)q;
@@ -886,17 +894,23 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
 // (local form: also when it has more slots or columns than threads) or P CTAs
 // cannot be resident.
 template <typename T>
-static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local, bool cluster) {
+static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, bool local, bool cluster,
+                              bool own = false) {
     pp->ok = false;
     pp->P = P;
     if (P < 1 || P > kPersistMaxP) return OPF_OK;
-    PersistPlan &other = pp == &h->p32 ? h->p64 : pp == &h->p64 ? h->p32 : pp == &h->k32 ? h->k64 : h->k32;
+    PersistPlan &other = pp == &h->p32   ? h->p64
+                         : pp == &h->p64 ? h->p32
+                         : pp == &h->k32 ? h->k64
+                         : pp == &h->k64 ? h->k32
+                         : pp == &h->o32 ? h->o64
+                                         : h->o32;
     auto same = [&](const std::shared_ptr<PersistTables> &t) {
-        return t && t->P == P && t->local == local && t->cluster == cluster;
+        return t && t->P == P && t->local == local && t->cluster == cluster && t->own == own;
     };
     if (!same(pp->tab)) {
         if (same(other.tab)) pp->tab = other.tab;
-        else TRY(build_persist_tables(h, P, local, cluster, &pp->tab));
+        else TRY(build_persist_tables(h, P, local, cluster, own, &pp->tab));
     }
     const PersistTables &t = *pp->tab;
     PersistLayout &c = pp->lay;
@@ -905,6 +919,8 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     c.L = h->L;
     c.local = local ? 1 : 0;
     c.cluster = cluster ? 1 : 0;
+    c.own = own ? 1 : 0;
+    c.G = h->G;
     c.tcap = (int)t.mt;
     c.threads = (int)std::min<long long>(kPersistMaxThreads,
                                          std::max<long long>(64, (std::max(t.mk, t.mj) + 31) / 32 * 32));
@@ -912,6 +928,11 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     // a thread per remote entry, two when that takes more threads than it has
     if (local && !cluster)
         c.threads = (int)std::max<long long>(c.threads, std::min<long long>(kPersistMaxThreads, (t.mr + 31) / 32 * 32));
+    if (own) {
+        if (t.mog > kPersistMaxThreads) return OPF_OK;
+        c.threads = (int)std::max<long long>(
+            c.threads, std::min<long long>(kPersistMaxThreads, (std::max(t.moc, t.mog) + 31) / 32 * 32));
+    }
     if (cluster && sizeof(T) == 4) {
         if (!t.rows32 || t.mpair > kPersistMaxThreads) return OPF_OK;
         c.threads = (int)std::max<long long>(c.threads, (t.mpair + 31) / 32 * 32);
@@ -955,6 +976,7 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
             take(&c.off_tw, (size_t)12 * P * 16);
         }
         take(&c.off_ul, (size_t)(t.mk + t.mr + 1) * sizeof(T));
+        if (own) take(&c.off_ow, (size_t)t.moc * sizeof(T));
     } else {
         take(&c.off_items, (size_t)t.mj * sizeof(int));
         take(&c.off_slots, (size_t)t.mk * persist_slot_bytes(sizeof(T)));
@@ -974,7 +996,12 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     if ((long long)off > optin) return OPF_OK;
     if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
     if (persist_resident<T>(c, n_sm) < P) { cudaGetLastError(); return OPF_OK; }
-    if (!cluster && !pp->d_xu) TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(h->L) / sizeof(unsigned long long)));
+    if (own && !pp->d_part) {
+        TRY(dalloc(h, &pp->d_part, 24 * kPersistMaxP));
+        TRY(dalloc(h, &pp->d_sync, 1));
+    }
+    if (!cluster && !pp->d_xu)
+        TRY(dalloc(h, &pp->d_xu, persist_exchange_bytes<T>(h->L + (own ? (long long)h->G : 0)) / sizeof(unsigned long long)));
     pp->ok = true;
     return OPF_OK;
 }
@@ -1028,6 +1055,20 @@ static int get_one_cluster_plan(opf_handle *h, PersistPlan *pp) {
     if (warps > 16 * (sizeof(T) == 4 ? kWarpEngineWarps : kWarpEngineWarps64)) return OPF_OK;
     const int per = sizeof(T) == 4 ? 80 : 24, most = sizeof(T) == 4 ? 16 : 12;
     return build_persist_plan<T>(h, pp, std::min(most, (h->L + per - 1) / per), 0, true, true);
+}
+
+// Owner form: at most a CTA per subsystem; FP64 a CTA per SM of the stream (its
+// FP64 pipes bound it), FP32 one per 160 slots up to that (every CTA takes the x
+// of its own globals: 240 blocks over 900 globals 3.62 us per iteration on 152
+// CTAs, 3.44 with 160 slots each, 3.51 with 320; over 300 globals 6.37, 4.55 and
+// 3.95; 200 blocks of up to 30 3.74, 2.45 and 2.75).
+template <typename T>
+static int get_owner_plan(opf_handle *h, PersistPlan *pp) {
+    if (pp->tried) return OPF_OK;
+    pp->tried = true;
+    const int n_sm = stream_sm_count(h->stream, h->device);
+    const int want = sizeof(T) == 8 ? n_sm : std::min(n_sm, (h->L + 159) / 160);
+    return build_persist_plan<T>(h, pp, std::min(want, h->S), n_sm, true, false, true);
 }
 
 template <typename T>
@@ -1441,6 +1482,7 @@ static int run_warp64(opf_handle *h, const opf_solve_opts &o) {
 // one-cluster form, 4 persistent grid, 3 warp engine, else whole-grid kernels.
 static int run_fp64(opf_handle *h, const opf_solve_opts &o, int e64) {
     if (e64 == 5 && h->k64.ok) return run_persist64(h, o, h->k64);
+    if (e64 == 6 && h->o64.ok) return run_persist64(h, o, h->o64);
     if (e64 == 4 && h->p64.ok) return run_persist64(h, o, h->p64);
     if (e64 == 3 && h->w64.ok) return run_warp64(h, o);
     return run_grid64(h, o);
@@ -1471,15 +1513,16 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
     CUDA_TRY(cudaGetLastError());
 
     const int kind = eng + (recenter ? 0 : 8);
-    bool hl = (o.flags & OPF_SOLVE_HOST_LOOP) != 0 || (eng == 4 && h->persist_graph_failed);
+    bool hl = (o.flags & OPF_SOLVE_HOST_LOOP) != 0 || ((eng == 4 || eng == 6) && h->persist_graph_failed);
     IterArgs<float> a = eng == 3   ? with_warp_plan(h, iter_args<float>(h, rho), h->w32)
                         : eng == 4 ? with_persist(iter_args<float>(h, rho), h->p32)
                         : eng == 5 ? with_persist(iter_args<float>(h, rho), h->k32)
+                        : eng == 6 ? with_persist(iter_args<float>(h, rho), h->o32)
                                    : with_plan(iter_args<float>(h, rho), h->c32);
     int launch_rc = 0;
     auto body = [&](cudaGraphConditionalHandle c, int use) {
             if (eng >= 4) {
-                const PersistPlan &pp = eng == 4 ? h->p32 : h->k32;
+                const PersistPlan &pp = eng == 4 ? h->p32 : eng == 5 ? h->k32 : h->o32;
                 launch_rc |= launch_persist_engine<float>(a, pp.lay, pp.ptrs(), h->d_u32, bar_extra(o), R, k,
                                                           h->d_st, rho, c, use, h->stream);
             } else if (eng == 3) {
@@ -1504,7 +1547,8 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                 launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, h->d_st, h->stream);
     };
     // (the test hook of the bounded waits is an argument of the captured launch)
-    const int planP = (eng == 5   ? 20000 + h->k32.P
+    const int planP = (eng == 6   ? 30000 + h->o32.P
+                       : eng == 5 ? 20000 + h->k32.P
                        : eng == 4 ? 10000 + h->p32.P
                        : eng == 3 ? 100 + h->w32.P
                        : eng == 2 ? h->c32.P
@@ -1512,7 +1556,7 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
     if (h->gmix.kind != kind || h->gmix.rho != rho || h->gmix.k != k || h->gmix.R != R ||
         h->gmix.host_loop != hl || h->gmix.P != planP) {
         int rc = build_while_graph(h, &h->gmix, body, hl);
-        if (rc != OPF_OK && eng == 4 && !hl) {
+        if (rc != OPF_OK && (eng == 4 || eng == 6) && !hl) {
             // a cooperative launch that cannot be captured: drive it from the host
             cudaGetLastError();
             h->persist_graph_failed = true;
@@ -1575,7 +1619,7 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
     // the warp engine), else on the warp engine; others on the persistent grid
     // engine when its plan fits, else whole-grid kernels (123 buses: 2.9
     // against 7.3 us).
-    bool w64 = false, p64 = false, k64 = false;
+    bool w64 = false, p64 = false, k64 = false, o64 = false;
     if (o.precision != OPF_PREC_FP32 && o.engine == 0) {
         TRY(get_one_cluster_plan<double>(h, &h->k64));
         k64 = h->k64.ok;
@@ -1585,12 +1629,27 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
         if (!h->w64.built || h->w64.req != req) TRY(build_warp_plan<double>(h, h->w64, req));
         w64 = h->w64.ok && (o.engine == 3 || h->w64.lay.warps <= kWarpEngineWarps64);
     }
-    if (!k64 && !w64 && (o.engine == 4 || (o.engine == 0 && o.precision != OPF_PREC_FP32))) {
+    // the owner form where most copies lie in other parts and subsystems take at
+    // least half of the SMs (us per iteration, the persistent engine's other forms
+    // and this one: 240 blocks of up to 100 slots over 900 and 300 globals 8.7 /
+    // 7.4 and 15.0 / 9.6, 400 of up to 60 over 5000 7.1 / 4.9, 4000 of up to 30
+    // over 20,000 9.8 / 7.2; 60 and 15 blocks of up to 100 5.4 / 6.2 and 4.5 / 5.1;
+    // feeders, whose parts read few copies, 300 to 8500 buses 3.2 / 4.6 to 5.9 / 6.8)
+    const bool wide = o.engine == 0 && o.precision != OPF_PREC_FP32 && !k64 && !w64 &&
+                      2 * h->S >= stream_sm_count(h->stream, h->device);
+    auto owner64 = [&]() -> int {
+        TRY(get_owner_plan<double>(h, &h->o64));
+        o64 = h->o64.ok;
+        return OPF_OK;
+    };
+    if (wide && many_copies(h)) TRY(owner64());
+    if (!k64 && !w64 && !o64 && (o.engine == 4 || (o.engine == 0 && o.precision != OPF_PREC_FP32))) {
         TRY(get_persist_plan<double>(h, &h->p64, o.engine == 4 ? o.cluster : 0));
         if (!h->p64.ok && o.engine == 4 && o.cluster > 0) TRY(get_persist_plan<double>(h, &h->p64, 0));
         p64 = h->p64.ok;
+        if (wide && p64 && h->p64.tab->remote > h->L) TRY(owner64());
     }
-    const int e64 = k64 ? 5 : w64 ? 3 : p64 ? 4 : 1;
+    const int e64 = k64 ? 5 : w64 ? 3 : o64 ? 6 : p64 ? 4 : 1;
     if (o.precision == OPF_PREC_FP64) {
         bool cl = false;
         if (o.engine == 2) {
@@ -1616,8 +1675,12 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
         // form and read at most one remote entry per slot (200 / 400 / 1000
         // buses: 2.2 / 2.6 / 2.5 us per iteration against 3.1 / 3.5 / 4.6 on the
         // cluster engine, the same iterates bit for bit; blocks over random
-        // globals, 2.5 copies each: 3.1-3.5 against 2.7-2.9, 14 copies each: 6.9
-        // against 6.6), else the cluster engine, else the persistent grid engine.
+        // globals, 2.5 copies each: 3.1-3.5 against 2.7-2.9), else its owner
+        // form, again the cluster engine's iterates bit for bit (240 blocks of up
+        // to 100 slots over 900 globals 3.44 against 6.48, of up to 20 2.35
+        // against 2.70, 400 of up to 60 over 5000 3.10 against 5.52, 15 of up to
+        // 100 2.42 against 2.93), else the cluster engine, else the persistent
+        // grid engine.
         int eng = 1;
         if (o.engine == 0) {
             TRY(get_one_cluster_plan<float>(h, &h->k32));
@@ -1631,6 +1694,10 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
         if (eng == 1 && o.engine == 0 && !many_copies(h)) {
             TRY(get_persist_plan<float>(h, &h->p32, 0));
             if (h->p32.ok && h->p32.lay.local && h->p32.tab->remote <= h->L) eng = 4;
+        }
+        if (eng == 1 && o.engine == 0) {
+            TRY(get_owner_plan<float>(h, &h->o32));
+            if (h->o32.ok) eng = 6;
         }
         if (eng == 1 && (o.engine == 0 || o.engine == 2)) {
             TRY(get_cluster_plan<float>(h, &h->c32, o.cluster, 192));

@@ -45,7 +45,7 @@ struct ClusterPlan {
 // device; the plans of both precisions share it while they agree on P and form.
 struct PersistTables {
     int P = 0, S = 0, L = 0;
-    bool local = false, cluster = false;
+    bool local = false, cluster = false, own = false;
     // largest part: factor words, subsystems, columns, products (columns
     // rounded up to 4 per subsystem), slots, vector rows, remote entries,
     // lists, destinations
@@ -53,6 +53,7 @@ struct PersistTables {
     // per part the columns and slots and the longest of each (FP64 lane splits);
     // most threads of the FP32 cluster form's columns; its factors fit registers
     std::vector<int> nj, nk, nmax, fmax;
+    long long mog = 0, moc = 0;          // owner form: most globals and copies that a part owns
     long long mpair = 0, remote = 0;     // remote: entries read from other parts, over all parts
     bool rows32 = true;
     bool fits = true;            // indices and counts fit their fields
@@ -60,7 +61,7 @@ struct PersistTables {
     int *pr = nullptr, *items = nullptr, *meta = nullptr;   // ranges, 7 x (P + 1); per column; per slot
     int *sub = nullptr, *slot = nullptr, *seg = nullptr, *out = nullptr, *rem = nullptr;
     uint4 *list = nullptr;
-    int *dst = nullptr, *dr = nullptr, *dseg = nullptr, *halves = nullptr;
+    int *dst = nullptr, *dr = nullptr, *dseg = nullptr, *halves = nullptr, *g0 = nullptr, *gfirst = nullptr;
     int4 *srec = nullptr;
     PersistTables() = default;
     PersistTables(const PersistTables &) = delete;
@@ -83,7 +84,7 @@ struct PersistPlan {
     unsigned long long *d_xu = nullptr;   // exchange buffer, allocated with the first plan that fits
     PersistPtrs ptrs() const {
         return PersistPtrs{tab->pr, d_part, d_sync, d_xu, tab->sub, tab->slot, tab->seg, tab->out, tab->rem, tab->list,
-                           tab->dst, tab->dr, tab->dseg, tab->halves};
+                           tab->dst, tab->dr, tab->dseg, tab->halves, tab->g0, tab->gfirst};
     }
 };
 
@@ -164,6 +165,7 @@ struct opf_handle {
     ClusterPlan c32, c64;
     PersistPlan p32, p64;
     PersistPlan k32, k64;                // its one-cluster form (small instances)
+    PersistPlan o32, o64;                // its owner form (globals with many copies)
     std::vector<int> persist_order;      // depth-first order of the subsystems (computed with the first plan)
     bool persist_graph_failed = false;   // the cooperative launch could not be captured in a graph
     WarpPlan w32, w64;

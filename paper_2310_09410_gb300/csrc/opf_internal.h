@@ -156,11 +156,13 @@ struct PersistLayout {
     int local;                     // k_persist_local (one slot and one factor column per thread), else k_persist_engine
     int split, clanes, rlanes;     // FP64 local plans of small CTAs: lanes per factor column and per row
     int cluster;                   // local plans: the CTAs are one thread-block cluster, u goes through its shared memory
+    int own, G;                    // owner form: each global updated by the CTA that owns it; globals
     int xcap;                      // cluster plans: stamped words per buffer (the most remote entries of a part)
     int tcap;                      // local plans: products per part (columns rounded up to 4 per subsystem)
     unsigned off_F, off_srec, off_vb, off_tb, off_xrs, off_lrs, off_cobj, off_misc;
     unsigned off_list, off_rem, off_ul;                 // local plans
     unsigned off_xw, off_tw;                            // cluster plans
+    unsigned off_ow;                                    // owner form
     unsigned off_items, off_slots, off_r, off_rn;       // the others
     unsigned bytes;
 };
@@ -180,6 +182,10 @@ struct PersistPtrs {
     // subsystem (part order) the rows of the first half when the FP32 column
     // products go by halves, else 0
     const int *dst, *dr, *dseg, *halves;
+    // owner form: part p owns the globals [g0[p], g0[p + 1]), global g's copies
+    // [gfirst[g], gfirst[g + 1]) of the copy order; xu holds two buffers of G
+    // entries (x) after those of u
+    const int *g0, *gfirst;
 };
 
 // Bytes of a slot's record in a plan with several slots per thread (persist.cu).

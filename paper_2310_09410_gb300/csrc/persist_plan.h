@@ -12,7 +12,9 @@
 #pragma once
 
 #include <algorithm>
+#include <functional>
 #include <numeric>
+#include <utility>
 #include <vector>
 
 namespace opf {
@@ -191,6 +193,76 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
             if (t.list[i] == 0xffff) t.list[i] = (unsigned short)zero;
     }
     return t;
+}
+
+// Owner form (instances whose globals have many copies): P parts of balanced
+// cost, the dearest subsystems placed first, and an owner for every global, its
+// copies' entries of u one run of the copy order.  Part p owns the globals
+// [g0[p], g0[p+1]) (most copies: most); parts.rem[r0[p] .. r0[p+1]) are the
+// distinct globals of part p's slots, parts.seg[j] = (index there << 8) |
+// copies, parts.out[j] = the slot's position in the copy order.
+struct PersistOwners {
+    PersistParts parts;
+    std::vector<int> g0;
+    int most_globals = 0, most_copies = 0;
+};
+
+inline PersistOwners persist_owners(int P, int S, int G, const std::vector<double> &cost, const std::vector<int> &soff,
+                                    const std::vector<int> &segp, const std::vector<int> &pk,
+                                    const std::vector<int> &gk, const std::vector<int> &gstart) {
+    PersistOwners o;
+    PersistParts &t = o.parts;
+    const int L = (int)pk.size();
+    std::vector<int> order(S);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return cost[a] > cost[b]; });
+    std::vector<std::vector<int>> of(P);
+    std::vector<std::pair<double, int>> load(P);             // min-heap
+    for (int p = 0; p < P; ++p) load[p] = {0.0, p};
+    const auto more = std::greater<std::pair<double, int>>();
+    for (int d : order) {
+        std::pop_heap(load.begin(), load.end(), more);
+        of[load.back().second].push_back(d);
+        load.back().first += cost[d];
+        std::push_heap(load.begin(), load.end(), more);
+    }
+    t.s0.assign(P + 1, 0);
+    t.k0.assign(P + 1, 0);
+    t.r0.assign(P + 1, 0);
+    t.l0.assign(P + 1, 0);
+    std::vector<int> at(G, -1), seen(G, -1);
+    for (int p = 0; p < P; ++p) {
+        std::sort(of[p].begin(), of[p].end());               // decreasing size
+        t.sub.insert(t.sub.end(), of[p].begin(), of[p].end());
+        for (int d : of[p])
+            for (int k = soff[d]; k < soff[d + 1]; ++k) {
+                const int g = gk[k];
+                if (seen[g] != p) {
+                    seen[g] = p;
+                    at[g] = (int)t.rem.size() - t.r0[p];
+                    t.rem.push_back(g);
+                }
+                t.slot.push_back(k);
+                t.seg.push_back((at[g] << 8) | (segp[k] & 255));
+                t.out.push_back(pk[k]);
+            }
+        t.s0[p + 1] = (int)t.sub.size();
+        t.k0[p + 1] = (int)t.slot.size();
+        t.r0[p + 1] = (int)t.rem.size();
+    }
+    // a global weighs one besides its copies
+    o.g0.assign(P + 1, G);
+    o.g0[0] = 0;
+    const long long total = (long long)L + G;
+    for (int p = 1, g = 0; p < P; ++p) {
+        while (g < G && (long long)gstart[g + 1] + g + 1 <= total * p / P) ++g;
+        o.g0[p] = g;
+    }
+    for (int p = 0; p < P; ++p) {
+        o.most_globals = std::max(o.most_globals, o.g0[p + 1] - o.g0[p]);
+        o.most_copies = std::max(o.most_copies, gstart[o.g0[p + 1]] - gstart[o.g0[p]]);
+    }
+    return o;
 }
 
 }  // namespace opf
