@@ -802,6 +802,7 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
     t->mog = owners.most_globals;
     t->moc = owners.most_copies;
     t->fits = parts.ok;
+    t->s0 = parts.s0;
     t->remote = (long long)parts.rem.size();
     // cluster form: a subsystem whose FP32 column products go by halves (in the
     // order of the warp engine's two warps) has its second half start at a
@@ -818,7 +819,7 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
     for (int p = 0; p < P; ++p) {
         const int s0 = parts.s0[p];
         long long f = 0, v = 0, c0 = 0, j = 0, nbig = 0;
-        int nmax = 0, fmax = 0;
+        int fmax = 0;
         for (int i = s0; i < parts.s0[p + 1]; ++i) {
             const int d = parts.sub[i], n = h->h_sn[d], hn = two[d] == 2 ? (n + 1) / 2 : 0;
             const int gap = round4(hn) - hn, npad = hn ? round4(hn) + round4(n - hn) : h->h_npad[d];
@@ -832,13 +833,13 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
             c0 += fp;
             j += h->h_sf[d];
             if (n > 32) nbig = j;
-            nmax = std::max(nmax, n);
+            t->npad.push_back(npad);
+            t->n.push_back(n);
+            t->f.push_back(h->h_sf[d]);
             fmax = std::max(fmax, h->h_sf[d]);
         }
         t->nj.push_back((int)j);
         t->nk.push_back(parts.k0[p + 1] - parts.k0[p]);
-        t->nmax.push_back(nmax);
-        t->fmax.push_back(fmax);
         t->rows32 = t->rows32 && fmax <= 32;
         t->mpair = std::max(t->mpair, ((2 * nbig + 31) & ~31LL) + j - nbig);
         PR(0, p + 1) = parts.k0[p + 1];
@@ -937,32 +938,88 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
         if (!t.rows32 || t.mpair > kPersistMaxThreads) return OPF_OK;
         c.threads = (int)std::max<long long>(c.threads, (t.mpair + 31) / 32 * 32);
     }
-    // FP64, small CTAs: lanes per column and per row that give the slowest
-    // CTA's sub-partitions the fewest FP64 instructions, about 64 cycles each
-    // (a column of n rows: n / lanes + log2 lanes; a row of f columns: its
-    // global update, f / lanes + log2 lanes, the dual update; once for every
-    // 128 threads, 4 warps)
-    if (local && sizeof(T) == 8 && std::max(t.mk, t.mj) <= 256) {
-        auto pick = [&](const std::vector<int> &items, const std::vector<int> &longest, int most, int fixed) {
-            int best = 1;
-            long long cost = -1;
-            for (int l = 1, lg = 0; l <= most; l *= 2, ++lg) {
-                long long worst = 0;
-                bool fit = true;
-                for (int p = 0; p < P; ++p) {
-                    const long long thr = (long long)l * items[p];
-                    if (thr > kPersistMaxThreads) fit = false;
-                    worst = std::max(worst, (thr + 127) / 128 * (fixed + (longest[p] + l - 1) / l + lg));
+    // FP64: lanes for the columns, and for the rows, of subsystems above a size,
+    // such that the slowest CTA takes the shortest time.  A warp's share is a
+    // chain of FP64 instructions of about 64 cycles each (a column of n rows on l
+    // lanes: n / l + log2 l; a row of f columns: its global update, f / l + log2
+    // l, the dual update).  A CTA with an SM to itself takes its longest chain or
+    // what a sub-partition has to issue on average; one of two on an SM what its
+    // busiest sub-partition has to issue and an average CTA's on top, or, with at
+    // most 256 slots and columns, its longest chain once per 4 warps with every
+    // item alike.  us per iteration by these three / every item on the lanes of
+    // the last rule / one lane each: 34, 123 and 200 buses (an SM each) 2.07, 2.79
+    // and 2.98 / 2.31, 2.92 and 3.21 / 3.28, 4.09 and 4.82; 8500 buses 7.30 / - /
+    // 8.61; 1000 and 2500 buses by the second rule 3.86 and 4.70, by the last 3.62
+    // and 4.27.
+    std::vector<int> wide;
+    const bool shared = local && !cluster && !own && P > n_sm;      // two CTAs on an SM
+    if (local && sizeof(T) == 8) {
+        const bool small = std::max(t.mk, t.mj) <= 256;
+        struct Choice { int lanes = 1, above = 0; long long threads = 0; };
+        auto pick = [&](bool rows, int top) {
+            const int fixed = rows ? 8 : 0;
+            Choice best;
+            double cost = -1;
+            for (int l = 1, lg = 0; l <= top; l *= 2, ++lg)
+                for (int above : {0, 8, 12, 16, 24, 32, 48}) {
+                    if (above && (l == 1 || (shared && small))) break;
+                    double worst = 0;
+                    long long threads = 0;
+                    for (int p = 0; p < P; ++p) {
+                        long long at = 0, chain = 0, longest = 0, sum = 0;    // threads so far, the open warp's chain
+                        long long issue[4] = {0, 0, 0, 0};        // per sub-partition
+                        auto close = [&]() {
+                            issue[((at + 31) / 32 - 1) & 3] += chain;
+                            longest = std::max(longest, chain);
+                            sum += chain;
+                            chain = 0;
+                        };
+                        bool big = true;
+                        for (int i = t.s0[p]; i < t.s0[p + 1]; ++i) {
+                            const int items = rows ? t.n[i] : t.f[i], terms = rows ? t.f[i] : t.n[i];
+                            if (big && t.npad[i] <= above) {
+                                big = false;
+                                if (at % 32) { close(); at = (at + 31) / 32 * 32; }
+                            }
+                            const int ll = big ? l : 1;
+                            long long left = (long long)items * ll;
+                            while (left > 0) {
+                                const long long room = 32 - at % 32, n = std::min(room, left);
+                                chain = std::max<long long>(chain, fixed + (terms + ll - 1) / ll + (big ? lg : 0));
+                                at += n;
+                                left -= n;
+                                if (at % 32 == 0) close();
+                            }
+                        }
+                        if (at % 32) close();
+                        worst = std::max(worst, !shared ? std::max((double)longest, sum / 4.0)
+                                                : small ? (double)((at + 127) / 128 * longest)
+                                                        : *std::max_element(issue, issue + 4) + sum / 4.0);
+                        threads = std::max(threads, (at + 31) / 32 * 32);
+                    }
+                    if (threads <= kPersistMaxThreads && (cost < 0 || worst < cost)) {
+                        cost = worst;
+                        best.lanes = l;
+                        best.above = above;
+                        best.threads = threads;
+                    }
                 }
-                if (fit && (cost < 0 || worst < cost)) { cost = worst; best = l; }
-            }
             return best;
         };
-        c.split = 1;
-        c.clanes = pick(t.nj, t.nmax, 8, 0);
-        c.rlanes = pick(t.nk, t.fmax, 4, 8);
-        c.threads = (int)std::max<long long>(c.threads, (std::max(c.clanes * t.mj, c.rlanes * t.mk) + 31) / 32 * 32);
+        const Choice col = pick(false, 8), row = pick(true, 4);
+        c.clanes = col.lanes;
+        c.rlanes = row.lanes;
+        c.threads = (int)std::max<long long>(c.threads, std::max(col.threads, row.threads));
+        wide.assign(2 * (size_t)P, 0);
+        for (int p = 0; p < P; ++p)
+            for (int i = t.s0[p]; i < t.s0[p + 1]; ++i) {
+                if (t.npad[i] > col.above) wide[2 * p] += t.f[i];
+                if (t.npad[i] > row.above) wide[2 * p + 1] += t.n[i];
+            }
     }
+    // (64 registers a thread when two CTAs do not fit an SM otherwise: FP64 of up to
+    // 256 threads does, 1000 buses 3.62 instead of 3.89 us)
+    c.two = shared && (sizeof(T) == 4 || c.threads > 256) ? 1 : 0;
     size_t off = 0;
     auto take = [&](unsigned *o, size_t bytes) { *o = (unsigned)off; off = align16u(off + bytes); };
     take(&c.off_F, (size_t)t.mf * sizeof(T));
@@ -996,6 +1053,11 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     if ((long long)off > optin) return OPF_OK;
     if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
     if (persist_resident<T>(c, n_sm) < P) { cudaGetLastError(); return OPF_OK; }
+    if (!wide.empty()) {
+        if (!pp->d_wide) TRY(dalloc(h, &pp->d_wide, 2 * (size_t)kPersistMaxP));
+        CUDA_TRY(cudaMemcpyAsync(pp->d_wide, wide.data(), wide.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
+        CUDA_TRY(cudaStreamSynchronize(h->stream));
+    }
     if (own && !pp->d_part) {
         TRY(dalloc(h, &pp->d_part, 24 * kPersistMaxP));
         TRY(dalloc(h, &pp->d_sync, 1));
@@ -1615,7 +1677,7 @@ extern "C" int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts) {
     // FP64 iterations (plain solves and the polish).  Automatic: instances the
     // warp engine would hold with at most 4 warps per CTA (with more, the warps
     // of an SM queue on its FP64 pipe) on the persistent engine's one-cluster
-    // form (13 / 34 buses 2.00 / 2.31 us per iteration against 2.92 / 3.03 on
+    // form (13 / 34 buses 1.93 / 2.07 us per iteration against 2.92 / 3.03 on
     // the warp engine), else on the warp engine; others on the persistent grid
     // engine when its plan fits, else whole-grid kernels (123 buses: 2.9
     // against 7.3 us).

@@ -50,9 +50,10 @@ struct PersistTables {
     // rounded up to 4 per subsystem), slots, vector rows, remote entries,
     // lists, destinations
     long long mf = 0, ms = 0, mj = 0, mt = 0, mk = 0, mv = 0, mr = 0, ml = 0, md = 0;
-    // per part the columns and slots and the longest of each (FP64 lane splits);
+    // per part the columns and slots, and the subsystems' sizes (FP64 lane splits);
     // most threads of the FP32 cluster form's columns; its factors fit registers
-    std::vector<int> nj, nk, nmax, fmax;
+    std::vector<int> nj, nk;
+    std::vector<int> s0, npad, n, f;     // parts' first subsystem, and per subsystem in part order
     long long mog = 0, moc = 0;          // owner form: most globals and copies that a part owns
     long long mpair = 0, remote = 0;     // remote: entries read from other parts, over all parts
     bool rows32 = true;
@@ -81,10 +82,11 @@ struct PersistPlan {
     std::shared_ptr<PersistTables> tab;
     unsigned long long *d_part = nullptr;   // 24 * kPersistMaxP
     unsigned long long *d_sync = nullptr;
+    int *d_wide = nullptr;                  // 2 * kPersistMaxP
     unsigned long long *d_xu = nullptr;   // exchange buffer, allocated with the first plan that fits
     PersistPtrs ptrs() const {
         return PersistPtrs{tab->pr, d_part, d_sync, d_xu, tab->sub, tab->slot, tab->seg, tab->out, tab->rem, tab->list,
-                           tab->dst, tab->dr, tab->dseg, tab->halves, tab->g0, tab->gfirst};
+                           tab->dst, tab->dr, tab->dseg, tab->halves, tab->g0, tab->gfirst, d_wide};
     }
 };
 

@@ -154,7 +154,8 @@ constexpr int kPersistMaxThreads = 512;
 struct PersistLayout {
     int P, L, threads;
     int local;                     // k_persist_local (one slot and one factor column per thread), else k_persist_engine
-    int split, clanes, rlanes;     // FP64 local plans of small CTAs: lanes per factor column and per row
+    int two;                       // local plans of more CTAs than SMs
+    int clanes, rlanes;            // FP64 local plans: lanes per long factor column and per row of a large subsystem
     int cluster;                   // local plans: the CTAs are one thread-block cluster, u goes through its shared memory
     int own, G;                    // owner form: each global updated by the CTA that owns it; globals
     int xcap;                      // cluster plans: stamped words per buffer (the most remote entries of a part)
@@ -186,6 +187,7 @@ struct PersistPtrs {
     // [gfirst[g], gfirst[g + 1]) of the copy order; xu holds two buffers of G
     // entries (x) after those of u
     const int *g0, *gfirst;
+    const int *wide;               // FP64 local plans: per part the columns and the slots spread over lanes (the first)
 };
 
 // Bytes of a slot's record in a plan with several slots per thread (persist.cu).

@@ -68,19 +68,19 @@
 // (distributed shared memory), so an exchange is one remote store.  FP32 keeps
 // the warp engine's order of every sum (the iterates are its, bit for bit) with
 // the factor rows in registers, columns on one lane each and those of more than
-// 32 rows on two.  FP64 (SPLIT) spreads columns and rows over lanes while each
-// warp has a sub-partition of its own.
+// 32 rows on two.  FP64 (every form) spreads the long columns and rows over lanes.
 // Measured per iteration with a test every 50, grid form, before (every copy of
 // u through L2 behind a grid barrier, parts of the size-sorted order, FP64 sums
 // of the test by butterflies) and now: 8500 buses FP32 4.23 -> 3.0 us, FP64
-// 10.5 -> 7.7 us; 123 buses FP64 4.7 -> 2.9 us.  Of the 8500-bus steps: stamped
+// 10.5 -> 7.3 us; 123 buses FP64 4.7 -> 2.8 us.  Of the 8500-bus steps: stamped
 // entries alone, all copies through L2, 6.1 us FP32 (every slot polls, and the
 // polls fill the L1) and 8.4 us FP64; local parts 3.6 and 8.8 us; the copies'
 // places in registers, loops unrolled, long warps of co-resident CTAs on
 // different sub-partitions, and the test's sums spread over lanes and warps
-// 3.1 and 7.7 us (a test cost some 40 us, now 12).
+// 3.1 and 7.7 us (a test cost some 40 us, now 12); FP64 with the longest columns
+// and rows on several lanes in warps of their own 7.3.
 // One-cluster form against the warp engine: FP32 13 / 34 / 123 buses 0.92 /
-// 1.00 / 1.11 us against 1.71 / 1.80 / 2.31; FP64 13 / 34 buses 1.98 / 2.31
+// 1.00 / 1.11 us against 1.71 / 1.80 / 2.31; FP64 13 / 34 buses 1.93 / 2.07
 // against 2.92 / 3.03.  Its FP32 phases before the last changes (123 buses,
 // 1.91 us): column products 1950 of 3700 cycles (scalar reads of strided
 // columns, 8-way bank conflicts; 16-byte reads, all of a column's in flight),
@@ -694,16 +694,18 @@ __device__ __forceinline__ float dot_rows4(const float *f, const float *v, int n
     return (a0 + a1) + (a2 + a3);
 }
 
-// SPLIT (FP64, small CTAs): each factor column on lay.clanes lanes and each row
-// on lay.rlanes, so that the longest one is no longer one lane's dependent
-// chain while the CTA's warps still have a sub-partition each.
+// SPLIT (FP64): the longest factor columns on lay.clanes lanes each and the rows
+// of the largest subsystems on lay.rlanes, so that the longest one is no longer
+// one lane's dependent chain; how many is the plan's choice (pick in api.cpp).
 // CL: the CTAs are one thread-block cluster of at most 16; u goes straight into
 // the readers' shared memory (stamped words there, no L2 on the way).
 // OWN: the owner form.
-template <typename T, bool SPLIT, bool CL, bool OWN>
-__global__ void __launch_bounds__(kPersistMaxThreads, SPLIT || CL || OWN ? 1 : 2)
+// TWO: two CTAs per SM (64 registers).
+template <typename T, bool CL, bool OWN, bool TWO>
+__global__ void __launch_bounds__(kPersistMaxThreads, TWO ? 2 : 1)
 k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_extra, int n_iters, int check_every,
                 DevStatus *st, double rho_d, cudaGraphConditionalHandle cond, int use_cond) {
+    constexpr bool SPLIT = sizeof(T) == 8;
     extern __shared__ __align__(16) unsigned char sm[];
     const int P = lay.P, rank = (int)blockIdx.x, P1 = P + 1, L = lay.L;
     const int nthr = blockDim.x;
@@ -774,8 +776,17 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
             xput(XG + (size_t)XW * lay.G, og0 + tid, T(0), 0xffffffffu);
         }
     }
-    // the thread's slot (lay.rlanes threads of one in SPLIT)
-    const int ks = SPLIT ? tid / lay.rlanes : tid, rpart = SPLIT ? tid & (lay.rlanes - 1) : 0;
+    // the thread's slot (SPLIT: the first ones, of the largest subsystems, on
+    // lay.rlanes threads each, in warps of their own)
+    int ks = tid, rpart = 0, rl = 1;
+    if constexpr (SPLIT) {
+        const int nb = pp.wide[2 * rank + 1] * lay.rlanes, wide = (nb + 31) & ~31;
+        ks = tid < wide ? (tid < nb ? tid / lay.rlanes : nk) : nb / lay.rlanes + tid - wide;
+        if (tid < wide) {
+            rl = lay.rlanes;
+            rpart = tid & (rl - 1);
+        }
+    }
     const bool have = ks < nk, lead = have && rpart == 0;
     Slot<T, CL> s;
     int seg = 0, out = -1, kk = 0;
@@ -827,15 +838,22 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
     // rows first, on two lanes each (a lane per half, the second idle when the
     // column is one piece) and in warps of their own.
     constexpr bool PAIRS = CL && sizeof(T) == 4;
-    int jcol, part = 0, nbig = 0;
+    int jcol, part = 0, nbig = 0, cl = 1;
     if constexpr (PAIRS) {
         for (nbig = 0; nbig < nj && g.sub[pp.sub[s0 + (g.citems[j0 + nbig] >> 8)]].y > 32;) ++nbig;
         const int wide = (2 * nbig + 31) & ~31;
         jcol = tid < wide ? (tid < 2 * nbig ? tid >> 1 : nj) : tid - wide + nbig;
         part = tid < wide ? tid & 1 : 0;
     } else {
-        jcol = SPLIT ? tid / lay.clanes : tid;
-        part = SPLIT ? tid & (lay.clanes - 1) : 0;
+        jcol = tid;
+        if constexpr (SPLIT) {               // the longest columns on lay.clanes lanes
+            const int nb = pp.wide[2 * rank] * lay.clanes, wide = (nb + 31) & ~31;
+            jcol = tid < wide ? (tid < nb ? tid / lay.clanes : nj) : nb / lay.clanes + tid - wide;
+            if (tid < wide) {
+                cl = lay.clanes;
+                part = tid & (cl - 1);
+            }
+        }
     }
     const bool big = PAIRS && tid < ((2 * nbig + 31) & ~31);
     const T *Fcol = F, *vcol = vb;
@@ -996,8 +1014,8 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
         __syncthreads();
         if constexpr (SPLIT) {
             T a = T(0);
-            if (jcol < nj) a = dot_rows(Fcol, vcol, ncol, part, lay.clanes);
-            for (int o = 1; o < lay.clanes; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (jcol < nj) a = dot_rows(Fcol, vcol, ncol, part, cl);
+            for (int o = 1; o < cl; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
             if (jcol < nj && part == 0) tb[tcol] = a;
         } else if (big) {
             if constexpr (PAIRS) {
@@ -1011,7 +1029,7 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
         __syncthreads();
         if (have || SPLIT) {
             const T old = s.state();
-            s.template local_update<true, SPLIT>(F, tb, g, rpart, lay.rlanes);
+            s.template local_update<true, SPLIT>(F, tb, g, rpart, rl);
             if (lead) {
                 publish(it + 1);
                 if constexpr (!OWN) ul[ks] = s.u;
@@ -1163,14 +1181,9 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
 template <typename T>
 const void *persist_fn(const PersistLayout &lay) {
     if (!lay.local) return (const void *)k_persist_engine<T>;
-    if constexpr (sizeof(T) == 8) {
-        if (lay.split)
-            return lay.own       ? (const void *)k_persist_local<T, true, false, true>
-                   : lay.cluster ? (const void *)k_persist_local<T, true, true, false>
-                                 : (const void *)k_persist_local<T, true, false, false>;
-    }
-    return lay.own       ? (const void *)k_persist_local<T, false, false, true>
-           : lay.cluster ? (const void *)k_persist_local<T, false, true, false>
+    return lay.own       ? (const void *)k_persist_local<T, false, true, false>
+           : lay.cluster ? (const void *)k_persist_local<T, true, false, false>
+           : lay.two     ? (const void *)k_persist_local<T, false, false, true>
                          : (const void *)k_persist_local<T, false, false, false>;
 }
 
