@@ -195,9 +195,11 @@ int opf_solve(opf_handle *h, double rho, double eps, int32_t max_iter);
  * form (the instance in one cluster of at most 16 CTAs, u written straight into
  * the readers' shared memory).  FP32 / mixed iterations of others: the
  * persistent grid engine when most copies of its parts' globals are their own,
- * else the cluster engine, else the persistent grid engine, else whole-grid
- * kernels; FP64 iterations (and the polish) of others: the persistent grid
- * engine when its plan fits, else whole-grid kernels.  The persistent engine's
+ * else its owner form (every global updated by the one CTA that owns it), else
+ * the cluster engine, else the persistent grid engine, else whole-grid kernels;
+ * FP64 iterations (and the polish) of others: the owner form when most copies
+ * lie in other parts and there is a subsystem for every second SM, else the
+ * persistent grid engine when its plan fits, else whole-grid kernels.  The persistent engine's
  * waits last at most 1 s each; past that the solve returns OPF_E_TIMEOUT. */
 int opf_solve_ex(opf_handle *h, const opf_solve_opts *opts);
 
@@ -331,13 +333,14 @@ int opf_batch_step(opf_batch *b, double rho, int32_t n_iters);
 
 /* Engine shape for one precision (OPF_PREC_FP32 or OPF_PREC_FP64): k_inst
  * instances per CTA (power of two <= 32) and warps per CTA (<= 16); 0 = pick
- * (FP32: the fastest of the candidate shapes timed on the batch; FP64: the
- * k_inst of 1, 2, 4 that gives every SM at most one CTA, else 4; 8 warps).
+ * (FP32: the fastest of a few shapes timed on the batch, k_inst 1, 2, 4 or 8;
+ * 1 cannot be asked for; FP64: the k_inst of 1, 2, 4 that gives every SM at most
+ * one CTA, else 4; 8 warps).
  * FP32 k_inst = 128 selects the lane engine (never picked automatically; several times slower than the other shapes on
  * the feeders measured): one instance per lane, tiles of 128 instances, each
  * on a cluster of up to 16 CTAs that split the subsystems; warps 4, 8, 12 or
  * 16 per CTA (OPF_E_CAPACITY at the solve when the model needs more than 16
- * parts of at most 256 slots).  out (get): ok, k_inst, warps, chunks per lane, tasks,
+ * parts of at most 256 slots).  out (get): ok, k_inst, warps, chunks per lane (the most a kernel lane holds), tasks,
  * chunks per CTA (lane engine: per tile), shared bytes, CTAs (lane engine:
  * tiles), lambda and bbar~ in tensor memory (1/0), tensor-memory columns per
  * CTA, CTAs per cluster (lane engine, else 0). */

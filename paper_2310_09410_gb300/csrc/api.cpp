@@ -231,7 +231,8 @@ static int build_layout(opf_handle *h) {
     // up to 80, 100 and 110 2.03, 4.25 and 4.57 against 1.93, 2.81 and 3.25.
     h->sh_n = h->max_ns;
     const size_t shared = precompute_smem(h->sh_m, h->sh_n), room = 220 * 1024;
-    if ((size_t)h->S > 3 * (room / shared) * (size_t)stream_sm_count(h->stream, h->device)) {
+    if ((h->sh_m > 64 || h->sh_n > 64) &&
+        (size_t)h->S > 3 * (room / shared) * (size_t)stream_sm_count(h->stream, h->device)) {
         h->sh_m = std::min(h->sh_m, 64);
         h->sh_n = std::min(h->sh_n, 64);
     }

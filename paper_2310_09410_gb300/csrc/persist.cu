@@ -52,9 +52,9 @@
 // (several slots per thread): parts are runs of the size-sorted order, slot
 // records in shared memory, and every copy of u is read from the exchange.
 // On tested iterations each CTA adds the Sec. III-C sums of its slots in FP64
-// and stores them; after a grid barrier every CTA sums the P partials in the
-// same fixed order and takes the same stopping decision (rank 0 publishes
-// the status).  Every wait is bounded: past the limit the CTA records a fault
+// and publishes them as stamped words; every CTA sums the P partials in the same
+// fixed order and takes the same stopping decision (rank 0 publishes the
+// status).  Every wait is bounded: past the limit the CTA records a fault
 // in the status and leaves, and the others follow.
 //
 // What bounds it: FP32, the latency of one iteration (an L2 store and an L2
