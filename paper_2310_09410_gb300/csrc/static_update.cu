@@ -12,6 +12,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <string>
@@ -93,6 +94,7 @@ __global__ void __launch_bounds__(kOneBlock) k_global_update_static(int n, const
                                                                     const double *c, const double *lb,
                                                                     const double *ub, double rho, Recips rc, double *x,
                                                                     double *out) {
+    cudaTriggerProgrammaticLaunchCompletion();       // the sum's block may take its place and wait there
     double o = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double ci = c[i];
@@ -106,10 +108,12 @@ __global__ void __launch_bounds__(kOneBlock) k_global_update_static(int n, const
 
 // Objective: the block partials summed in a fixed order by one block.  (By one
 // thread, 248 dependent adds took 15 of the 24.6 us of a 63,405-global call;
-// with the block sum and the forms above a call takes 10.6 us, most of it the
-// two launches, and one of 2 million globals 61 us, where 1 million took 250.)
+// with the block sum and the forms above a call takes 10.9 us, 9.3 with this
+// kernel's start-up under the update, and one of 2 million globals 61 us, where
+// 1 million took 250.)
 __global__ void __launch_bounds__(kThreads) k_sum_partials_static(int nblk, const double *partials,
                                                                   double *objective) {
+    cudaGridDependencySynchronize();                 // until the update's blocks have finished
     double s = 0.0;
     for (int b = threadIdx.x; b < nblk; b += kThreads) s += partials[b];
     s = block_sum(s);
@@ -229,7 +233,20 @@ extern "C" int opf_global_update_static(int32_t n, const int32_t *seg_off, const
     } else {
         const int nblk = std::min((n + kThreads - 1) / kThreads, kBlocks);
         k_global_update_static<<<(unsigned)nblk, kThreads, 0, s>>>(n, seg_off, u, c, lb, ub, rho, rc, x, partials);
-        k_sum_partials_static<<<1, kThreads, 0, s>>>(nblk, partials, objective);
+        // launched while the update runs (programmatic dependent launch), so that
+        // its start-up does not come after it
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3(1);
+        cfg.blockDim = dim3(kThreads);
+        cfg.stream = s;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        const cudaError_t le = cudaLaunchKernelEx(&cfg, k_sum_partials_static, nblk, (const double *)partials, objective);
+        if (le != cudaSuccess) return fail(OPF_E_CUDA, std::string("launch: ") + cudaGetErrorString(le));
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(OPF_E_CUDA, std::string("launch: ") + cudaGetErrorString(e));
