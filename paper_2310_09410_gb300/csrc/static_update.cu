@@ -23,8 +23,8 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kOneBlock = 512;       // up to so many globals run in one block, which sums the objective itself
-                                     // (181 / 408 globals 7.6 / 7.9 us a call against 9.6 with a second kernel,
-                                     // 1024 globals 10.3 against 9.6)
+                                     // (between events, one block / two kernels: 181 globals 6.8 / 8.8 us, 408
+                                     // and 512 8.8 / 8.8, 800 10.9 / 8.8)
 constexpr int kBlocks = 8 * 152;     // resident blocks of the GPU: more globals than threads go round by round
 constexpr int kRecip = 16;           // 1 / (rho N) by copy count below this
 
