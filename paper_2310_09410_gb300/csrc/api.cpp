@@ -1616,8 +1616,9 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                        : eng == 3 ? 100 + h->w32.P
                        : eng == 2 ? h->c32.P
                                   : 0) + 1000000 * bar_extra(o);
-    if (h->gmix.kind != kind || h->gmix.rho != rho || h->gmix.k != k || h->gmix.R != R ||
-        h->gmix.host_loop != hl || h->gmix.P != planP) {
+    std::shared_ptr<const void> tables;
+    if (eng >= 4) tables = (eng == 4 ? h->p32 : eng == 5 ? h->k32 : h->o32).tab;
+    if (!h->gmix.matches(kind, rho, k, R, hl, planP, tables)) {
         int rc = build_while_graph(h, &h->gmix, body, hl);
         if (rc != OPF_OK && (eng == 4 || eng == 6) && !hl) {
             // a cooperative launch that cannot be captured: drive it from the host
@@ -1630,6 +1631,7 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
         TRY(rc);
         h->gmix.kind = kind; h->gmix.rho = rho; h->gmix.k = k; h->gmix.R = R;
         h->gmix.P = planP;
+        h->gmix.tables = tables;
     }
     TRY(run_graph(h, &h->gmix, body));
     if (launch_rc) {

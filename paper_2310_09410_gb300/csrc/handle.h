@@ -11,25 +11,11 @@
 #include <vector>
 
 #include "opf_internal.h"
+#include "solve_graph.h"
 
 // The handle type is declared at global scope by opf.h; the helper records
 // live beside it.
 using namespace opf;
-
-struct GraphCache {
-    cudaGraphExec_t exec = nullptr;
-    cudaGraph_t graph = nullptr;
-    bool host_loop = false;
-    double rho = 0;
-    int k = 0, R = 0, kind = -1, P = 0;
-    void reset() {
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        exec = nullptr;
-        graph = nullptr;
-        kind = -1;
-    }
-};
 
 // Cluster plan for one precision: P CTAs, part ranges and part-relative records.
 struct ClusterPlan {
