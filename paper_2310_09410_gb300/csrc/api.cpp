@@ -1372,42 +1372,20 @@ static void enqueue_grid_chunk(opf_handle *h, const IterArgs<T> &a, T *u, int k,
     launch_check(h->d_partials, t.n_tiles, h->d_st, rho, k, cond, use_cond, h->stream);
 }
 
-// Build a graph "while (!done) body" where body is enqueued by fn(cond, 1).
+// Build a graph "while (!done) body" where body is enqueued by fn(cond, 1)
+// (0, or nonzero when a launch was refused).
 // With host_loop the graph is the body alone (fn(0, 0)), relaunched by the
 // host until the device status says done (profilers see its kernel nodes).
 template <typename Fn>
 static int build_while_graph(opf_handle *h, GraphCache *gc, Fn fn, bool host_loop) {
-    gc->reset();
     if (host_loop) {
+        gc->reset();
         gc->host_loop = true;
         return OPF_OK;
     }
-    gc->host_loop = false;
-    CUDA_TRY(cudaGraphCreate(&gc->graph, 0));
-    cudaGraphConditionalHandle cond;
-    CUDA_TRY(cudaGraphConditionalHandleCreate(&cond, gc->graph, 1, cudaGraphCondAssignDefault));
-    // the parameter union has no default constructor in C++: zeroed storage
-    alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
-    memset(raw, 0, sizeof(raw));
-    cudaGraphNodeParams *cp = reinterpret_cast<cudaGraphNodeParams *>(raw);
-    cp->type = cudaGraphNodeTypeConditional;
-    cp->conditional.handle = cond;
-    cp->conditional.type = cudaGraphCondTypeWhile;
-    cp->conditional.size = 1;
-    cudaGraphNode_t node;
-    CUDA_TRY(cudaGraphAddNode(&node, gc->graph, nullptr, nullptr, 0, cp));
-    cudaGraph_t body = cp->conditional.phGraph_out[0];
-    CUDA_TRY(cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-    fn(cond, 1);
-    cudaGraph_t captured = nullptr;
-    cudaError_t ec = cudaStreamEndCapture(h->stream, &captured);
-    if (ec != cudaSuccess) {
-        g_last_error = std::string("stream capture: ") + cudaGetErrorString(ec);
-        gc->reset();
-        return OPF_E_CUDA;
-    }
-    CUDA_TRY(cudaGraphInstantiate(&gc->exec, gc->graph, 0));
-    return OPF_OK;
+    const cudaError_t e = capture_while(gc, h->stream, [&](cudaGraphConditionalHandle cond) { return fn(cond, 1); },
+                                        &g_last_error);
+    return e == cudaSuccess ? OPF_OK : e == cudaErrorMemoryAllocation ? OPF_E_OOM : OPF_E_CUDA;
 }
 
 static int set_status(opf_handle *h, const opf_solve_opts &o, bool keep_iter) {
@@ -1437,8 +1415,12 @@ static int run_graph(opf_handle *h, GraphCache *gc, Fn fn) {
         return read_status(h);
     }
     for (;;) {
-        fn(cudaGraphConditionalHandle{}, 0);
+        const int refused = fn(cudaGraphConditionalHandle{}, 0);
         CUDA_TRY(cudaGetLastError());
+        if (refused) {
+            g_last_error = "engine launch refused";
+            return OPF_E_CUDA;
+        }
         TRY(read_status(h));
         if (h->h_st->done) return OPF_OK;
         if (h->cancel.load() || (h->deadline > 0.0 && opf::steady_seconds() > h->deadline)) {
@@ -1459,6 +1441,7 @@ static int run_grid64(opf_handle *h, const opf_solve_opts &o) {
     IterArgs<double> a = iter_args<double>(h, rho);
     auto body = [&](cudaGraphConditionalHandle c, int use) {
         enqueue_grid_chunk<double>(h, a, h->d_u64, o.check_every, rho, c, use);
+        return 0;
     };
     if (h->g64.kind != 0 || h->g64.rho != rho || h->g64.k != o.check_every || h->g64.host_loop != hl) {
         TRY(build_while_graph(h, &h->g64, body, hl));
@@ -1582,22 +1565,23 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
                         : eng == 5 ? with_persist(iter_args<float>(h, rho), h->k32)
                         : eng == 6 ? with_persist(iter_args<float>(h, rho), h->o32)
                                    : with_plan(iter_args<float>(h, rho), h->c32);
-    int launch_rc = 0;
-    auto body = [&](cudaGraphConditionalHandle c, int use) {
+    auto body = [&](cudaGraphConditionalHandle c, int use) -> int {
+            int refused = 0;
             if (eng >= 4) {
                 const PersistPlan &pp = eng == 4 ? h->p32 : eng == 5 ? h->k32 : h->o32;
-                launch_rc |= launch_persist_engine<float>(a, pp.lay, pp.ptrs(), h->d_u32, bar_extra(o), R, k,
-                                                          h->d_st, rho, c, use, h->stream);
+                refused = launch_persist_engine<float>(a, pp.lay, pp.ptrs(), h->d_u32, bar_extra(o), R, k, h->d_st, rho,
+                                                       c, use, h->stream);
             } else if (eng == 3) {
-                launch_warp_engine<float>(a, h->w32.lay, h->w32.d_pr, h->d_u32, R, k, h->d_st, rho, c, use, h->stream);
+                refused = launch_warp_engine<float>(a, h->w32.lay, h->w32.d_pr, h->d_u32, R, k, h->d_st, rho, c, use,
+                                                    h->stream);
             } else if (eng == 2) {
-                launch_cluster_engine<float>(a, h->c32.lay, h->c32.d_pr, h->d_u32, R, k, h->d_st, rho, c, use,
-                                             h->stream);
+                refused = launch_cluster_engine<float>(a, h->c32.lay, h->c32.d_pr, h->d_u32, R, k, h->d_st, rho, c, use,
+                                                       h->stream);
             } else {
                 const int chunks = recenter ? R / k : 1;
                 for (int i = 0; i < chunks; ++i) enqueue_grid_chunk<float>(h, a, h->d_u32, k, rho, c, use);
             }
-            if (!recenter) return;
+            if (refused || !recenter) return refused;
             // re-centre on the next global update (u of the last iteration is in buffer 0)
             launch_global_x<float>(G, h->d_gseg, h->d_u32, h->d_ct32, h->d_lbt32, h->d_ubt32, h->d_xr,
                                    h->d_c64, (float)rho, h->d_xr2, h->d_objpart, h->d_st, h->stream);
@@ -1608,6 +1592,7 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
             launch_copy_if_running(G, h->d_xr2, h->d_xr, h->d_st, h->stream);
             if (eng < 4)
                 launch_make_u<float>(L, h->d_pk, h->d_ds32, h->d_mu32, (float)rho, h->d_u32, h->d_st, h->stream);
+            return 0;
     };
     // (the test hook of the bounded waits is an argument of the captured launch)
     const int planP = (eng == 6   ? 30000 + h->o32.P
@@ -1625,7 +1610,6 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
             cudaGetLastError();
             h->persist_graph_failed = true;
             hl = true;
-            launch_rc = 0;
             rc = build_while_graph(h, &h->gmix, body, true);
         }
         TRY(rc);
@@ -1634,10 +1618,6 @@ static int run_mixed(opf_handle *h, const opf_solve_opts &o, int eng, bool recen
         h->gmix.tables = tables;
     }
     TRY(run_graph(h, &h->gmix, body));
-    if (launch_rc) {
-        g_last_error = "persistent grid engine launch failed";
-        return OPF_E_CUDA;
-    }
     TRY(fault_error(h));
     // back to the unshifted FP64 state
     launch_unshift<float>(L, h->d_gk, h->d_xr, h->d_lamr, h->d_ds32, h->d_mu32, h->d_ds64, h->d_mu64, h->stream);

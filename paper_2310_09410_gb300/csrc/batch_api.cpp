@@ -258,9 +258,10 @@ BatchArgs<T> engine_args(opf_batch *b, const BPlan &p, double rho) {
 }
 
 // One pass of the loop body: re-centre, n_iters engine iterations, unshift,
-// "still running" flag (and graph condition).
+// "still running" flag (and graph condition).  0, or nonzero when the engine's
+// launch was refused.
 template <typename T>
-void enqueue_body(opf_batch *b, BPlan &p, double rho, int n_iters, int check_every,
+int enqueue_body(opf_batch *b, BPlan &p, double rho, int n_iters, int check_every,
                   cudaGraphConditionalHandle cond, int use_cond, cudaEvent_t e0 = nullptr,
                   cudaEvent_t e1 = nullptr, int ctas = -1, cudaStream_t stream = nullptr) {
     opf_handle *h = b->h;
@@ -271,24 +272,26 @@ void enqueue_body(opf_batch *b, BPlan &p, double rho, int n_iters, int check_eve
                    b->d_bbar, (T *)p.bt, (T *)p.ds, (T *)p.mu, (T *)p.lref, (T *)p.xsr, s);
     if (e0) cudaEventRecord(e0, s);
     const int grid = ctas >= 0 ? std::min(ctas, p.C) : p.C;
+    int refused = 0;
     if (p.lane) {
         // tiles of kLaneInst instances, one cluster each
         if (grid > 0)
-            lane_engine_launch(lane_args(b, p, rho), grid, p.threads, p.bytes, n_iters, check_every, s);
+            refused = lane_engine_launch(lane_args(b, p, rho), grid, p.threads, p.bytes, n_iters, check_every, s);
     } else if (grid > 0) {
         BatchArgs<T> a = engine_args<T>(b, p, rho);
-        batch_engine_launch<T>(a, p.nq, p.fg, grid, p.threads, p.bytes, n_iters, check_every, s);
+        refused = batch_engine_launch<T>(a, p.nq, p.fg, grid, p.threads, p.bytes, n_iters, check_every, s);
     }
     if (e1) cudaEventRecord(e1, s);
     launch_bunshift<T>(b->n, b->G, b->L, p.K, p.ks, p.NCH, p.d_ipos, h->d_gk, p.d_sch, b->d_xref, b->d_dref,
                        (const T *)p.ds, (const T *)p.mu, (const T *)p.xo, b->d_st, b->d_xs, b->d_lam, b->d_x, s);
     launch_bany(b->n, p.d_ipos, b->d_st, p.dbl ? b->d_flag + 1 : b->d_flag, cond, use_cond, s);
+    return refused;
 }
 
-void enqueue_body_any(opf_batch *b, BPlan &p, double rho, int n_iters, int k, cudaGraphConditionalHandle c,
+int enqueue_body_any(opf_batch *b, BPlan &p, double rho, int n_iters, int k, cudaGraphConditionalHandle c,
                       int use, cudaEvent_t e0, cudaEvent_t e1, int ctas, cudaStream_t stream) {
-    if (p.dbl) enqueue_body<double>(b, p, rho, n_iters, k, c, use, e0, e1, ctas, stream);
-    else enqueue_body<float>(b, p, rho, n_iters, k, c, use, e0, e1, ctas, stream);
+    return p.dbl ? enqueue_body<double>(b, p, rho, n_iters, k, c, use, e0, e1, ctas, stream)
+                 : enqueue_body<float>(b, p, rho, n_iters, k, c, use, e0, e1, ctas, stream);
 }
 
 int read_status(opf_batch *b) {
@@ -305,8 +308,10 @@ int run_loop(opf_batch *b, BPlan &p, double rho, int R, int k, bool host_loop) {
     if (host_loop) {
         // direct launches; the engine launches are timed alone with events
         for (;;) {
-            enqueue_body_any(b, p, rho, R, k, cudaGraphConditionalHandle{}, 0, b->eng_ev[0], b->eng_ev[1]);
+            const int refused =
+                enqueue_body_any(b, p, rho, R, k, cudaGraphConditionalHandle{}, 0, b->eng_ev[0], b->eng_ev[1]);
             BCUDA(cudaGetLastError());
+            if (refused) { set_last_error("batch: engine launch refused"); return OPF_E_CUDA; }
             int flag = 0;
             BCUDA(cudaMemcpyAsync(&flag, p.dbl ? b->d_flag + 1 : b->d_flag, sizeof(int), cudaMemcpyDeviceToHost,
                                   h->stream));
@@ -320,30 +325,14 @@ int run_loop(opf_batch *b, BPlan &p, double rho, int R, int k, bool host_loop) {
     }
     GraphCache &gc = p.graph;
     if (!gc.exec || gc.rho != rho || gc.k != k || gc.R != R) {
-        gc.reset();
-        BCUDA(cudaGraphCreate(&gc.graph, 0));
-        cudaGraphConditionalHandle cond;
-        BCUDA(cudaGraphConditionalHandleCreate(&cond, gc.graph, 1, cudaGraphCondAssignDefault));
-        alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
-        memset(raw, 0, sizeof(raw));
-        cudaGraphNodeParams *cp = reinterpret_cast<cudaGraphNodeParams *>(raw);
-        cp->type = cudaGraphNodeTypeConditional;
-        cp->conditional.handle = cond;
-        cp->conditional.type = cudaGraphCondTypeWhile;
-        cp->conditional.size = 1;
-        cudaGraphNode_t node;
-        BCUDA(cudaGraphAddNode(&node, gc.graph, nullptr, nullptr, 0, cp));
-        cudaGraph_t body = cp->conditional.phGraph_out[0];
-        BCUDA(cudaStreamBeginCaptureToGraph(h->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-        enqueue_body_any(b, p, rho, R, k, cond, 1);
-        cudaGraph_t captured = nullptr;
-        cudaError_t ec = cudaStreamEndCapture(h->stream, &captured);
-        if (ec != cudaSuccess) {
-            set_last_error(std::string("stream capture: ") + cudaGetErrorString(ec));
-            gc.reset();
-            return OPF_E_CUDA;
+        std::string why;
+        const cudaError_t e = capture_while(
+            &gc, h->stream, [&](cudaGraphConditionalHandle cond) { return enqueue_body_any(b, p, rho, R, k, cond, 1); },
+            &why);
+        if (e != cudaSuccess) {
+            set_last_error(why);
+            return e == cudaErrorMemoryAllocation ? OPF_E_OOM : OPF_E_CUDA;
         }
-        BCUDA(cudaGraphInstantiate(&gc.exec, gc.graph, 0));
         gc.rho = rho; gc.k = k; gc.R = R;
     }
     // the WHILE node tests its condition before the first pass: start it set

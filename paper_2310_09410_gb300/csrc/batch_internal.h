@@ -140,8 +140,8 @@ int plan_set_rho(opf_batch *b, BPlan *p, double rho);
 // One loop pass on the handle's stream: re-centre, n_iters engine iterations
 // (test every k), back to FP64, "still running" flag.
 // ctas >= 0 launches only the first ctas CTAs of the engine (columns packed
-// from the front).
-void enqueue_body_any(opf_batch *b, BPlan &p, double rho, int n_iters, int k, cudaGraphConditionalHandle c,
+// from the front).  Nonzero when the engine's launch was refused.
+int enqueue_body_any(opf_batch *b, BPlan &p, double rho, int n_iters, int k, cudaGraphConditionalHandle c,
                       int use, cudaEvent_t e0 = nullptr, cudaEvent_t e1 = nullptr, int ctas = -1,
                       cudaStream_t stream = nullptr);
 int read_status(opf_batch *b);

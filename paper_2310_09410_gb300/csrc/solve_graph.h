@@ -4,7 +4,9 @@
 
 #include <cuda_runtime.h>
 
+#include <cstring>
 #include <memory>
+#include <string>
 
 struct GraphCache {
     cudaGraphExec_t exec = nullptr;
@@ -32,3 +34,50 @@ struct GraphCache {
         tables.reset();
     }
 };
+
+// Captures "while (condition) body" into *gc: body(cond) enqueues one pass on
+// `s`, its kernels set the condition; it returns nonzero when a launch was
+// refused.  A launch that fails while it is captured leaves no node behind: the
+// loop would run without the kernel that ends it, for ever.  So such a graph is
+// dropped, with the launch's error.
+// cudaSuccess, or the error with *err telling where (gc is empty then).
+template <typename Body>
+cudaError_t capture_while(GraphCache *gc, cudaStream_t s, Body body, std::string *err) {
+    gc->reset();
+    gc->host_loop = false;
+    auto failed = [&](const char *where, cudaError_t e) {
+        *err = std::string(where) + ": " + cudaGetErrorString(e);
+        gc->reset();
+        return e;
+    };
+    cudaError_t e = cudaGraphCreate(&gc->graph, 0);
+    if (e != cudaSuccess) return failed("cudaGraphCreate", e);
+    cudaGraphConditionalHandle cond;
+    e = cudaGraphConditionalHandleCreate(&cond, gc->graph, 1, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return failed("cudaGraphConditionalHandleCreate", e);
+    // the parameter union has no default constructor in C++: zeroed storage
+    alignas(cudaGraphNodeParams) unsigned char raw[sizeof(cudaGraphNodeParams)];
+    memset(raw, 0, sizeof(raw));
+    cudaGraphNodeParams *cp = reinterpret_cast<cudaGraphNodeParams *>(raw);
+    cp->type = cudaGraphNodeTypeConditional;
+    cp->conditional.handle = cond;
+    cp->conditional.type = cudaGraphCondTypeWhile;
+    cp->conditional.size = 1;
+    cudaGraphNode_t node;
+    e = cudaGraphAddNode(&node, gc->graph, nullptr, nullptr, 0, cp);
+    if (e != cudaSuccess) return failed("cudaGraphAddNode", e);
+    cudaGetLastError();                  // an older error is not this capture's
+    e = cudaStreamBeginCaptureToGraph(s, cp->conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeRelaxed);
+    if (e != cudaSuccess) return failed("cudaStreamBeginCaptureToGraph", e);
+    const int refused = body(cond);
+    cudaError_t launch = cudaGetLastError();
+    if (launch == cudaSuccess && refused) launch = cudaErrorInvalidConfiguration;
+    cudaGraph_t captured = nullptr;
+    e = cudaStreamEndCapture(s, &captured);
+    if (launch != cudaSuccess) return failed("launch under stream capture", launch);
+    if (e != cudaSuccess) return failed("stream capture", e);
+    e = cudaGraphInstantiate(&gc->exec, gc->graph, 0);
+    if (e != cudaSuccess) return failed("cudaGraphInstantiate", e);
+    return cudaSuccess;
+}

@@ -2,7 +2,9 @@
 
 On the CPU, against a stand-in for the CUDA runtime: a graph captured for one
 plan's tables keeps them alive and does not match a plan built again with the
-same CTA count, in whatever order the two are freed.
+same CTA count, in whatever order the two are freed; and a capture that loses
+a launch (the runtime's error, or the launcher's refusal) gives an error and no
+graph, since the loop would lack the kernel that ends it.
 
 On the GPU: a request that does not fit between two equal single-precision
 solves (the plan, and with it its tables, is built again) leaves the iterates
@@ -21,9 +23,34 @@ RUNTIME = r"""
 #pragma once
 typedef void *cudaGraphExec_t;
 typedef void *cudaGraph_t;
-inline int destroyed = 0;
-inline int cudaGraphExecDestroy(cudaGraphExec_t) { ++destroyed; return 0; }
-inline int cudaGraphDestroy(cudaGraph_t) { ++destroyed; return 0; }
+typedef void *cudaGraphNode_t;
+typedef void *cudaStream_t;
+typedef unsigned long long cudaGraphConditionalHandle;
+enum cudaError_t { cudaSuccess, cudaErrorInvalidValue, cudaErrorInvalidConfiguration };
+enum { cudaGraphCondAssignDefault, cudaGraphNodeTypeConditional, cudaGraphCondTypeWhile, cudaStreamCaptureModeRelaxed };
+struct cudaGraphNodeParams {
+    int type;
+    struct { cudaGraphConditionalHandle handle; int type; unsigned size; cudaGraph_t *phGraph_out; } conditional;
+};
+inline int destroyed = 0, alive = 0, instantiated = 0, capturing = 0, mark;
+inline cudaError_t last = cudaSuccess;
+inline cudaGraph_t loop_body = &mark;
+inline int cudaGraphExecDestroy(cudaGraphExec_t) { ++destroyed; --alive; return 0; }
+inline int cudaGraphDestroy(cudaGraph_t) { ++destroyed; --alive; return 0; }
+inline cudaError_t cudaGraphCreate(cudaGraph_t *g, unsigned) { *g = &mark; ++alive; return cudaSuccess; }
+inline cudaError_t cudaGraphConditionalHandleCreate(cudaGraphConditionalHandle *h, cudaGraph_t, unsigned, unsigned) {
+    *h = 7; return cudaSuccess;
+}
+inline cudaError_t cudaGraphAddNode(cudaGraphNode_t *, cudaGraph_t, const cudaGraphNode_t *, const void *, unsigned,
+                                    cudaGraphNodeParams *p) { p->conditional.phGraph_out = &loop_body; return cudaSuccess; }
+inline cudaError_t cudaGetLastError() { cudaError_t e = last; last = cudaSuccess; return e; }
+inline cudaError_t cudaStreamBeginCaptureToGraph(cudaStream_t, cudaGraph_t, const cudaGraphNode_t *, const void *, unsigned,
+                                                 int) { ++capturing; return cudaSuccess; }
+inline cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) { --capturing; return cudaSuccess; }
+inline cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned) {
+    *x = &mark; ++alive; ++instantiated; return cudaSuccess;
+}
+inline const char *cudaGetErrorString(cudaError_t) { return "error"; }
 """
 
 DRIVER = r"""
@@ -49,13 +76,30 @@ int main() {
     g.reset();
     CHECK(freed == 1 && destroyed == 2 && !g.tables);         // freed with the graph, not before
     CHECK(!g.matches(4, 100.0, 50, 1000, false, 10304, plan));
+    // captures: whole; a launch that fails; a launcher that refuses; whole after an older error
+    alive = 0;
+    std::string why;
+    auto capture = [&](cudaError_t launch, int refused) {
+        return capture_while(&g, nullptr, [&](cudaGraphConditionalHandle c) {
+            if (launch != cudaSuccess) last = launch;
+            return c == 7 ? refused : 1;
+        }, &why);
+    };
+    CHECK(capture(cudaSuccess, 0) == cudaSuccess && g.exec && alive == 2 && instantiated == 1);
+    g.kind = 4;
+    CHECK(capture(cudaErrorInvalidValue, 0) == cudaErrorInvalidValue && !why.empty());
+    CHECK(!g.exec && !g.graph && alive == 0 && instantiated == 1 && capturing == 0 && g.kind == -1);
+    CHECK(capture(cudaSuccess, 1) != cudaSuccess && !g.exec && alive == 0 && instantiated == 1 && capturing == 0);
+    last = cudaErrorInvalidValue;
+    CHECK(capture(cudaSuccess, 0) == cudaSuccess && g.exec && alive == 2 && instantiated == 2);
+    g.reset();
     std::printf("ok\n");
     return 0;
 }
 """
 
 
-def test_graph_holds_its_tables(tmp_path):
+def test_graph_holds_its_tables_and_needs_its_launches(tmp_path):
     gxx = shutil.which("g++")
     if gxx is None:
         pytest.skip("no g++")
