@@ -36,6 +36,7 @@
 #include <cstdint>
 
 #include "opf_internal.h"
+#include "smem_limit.h"
 #include "test_rule.cuh"
 #include "tmem.cuh"
 
@@ -1347,7 +1348,7 @@ template <typename T>
 int batch_engine_prepare(int K, int nq, bool fg, bool tm, unsigned bytes) {
     const void *fn = engine_fn<T>(K, nq, fg, tm);
     if (!fn) return -1;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess ? 0 : -1;
+    return allow_dynamic_smem(fn, bytes);
 }
 
 template <typename T>

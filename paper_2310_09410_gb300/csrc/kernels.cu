@@ -36,6 +36,7 @@
 #include <cstring>
 
 #include "opf_internal.h"
+#include "smem_limit.h"
 #include "test_rule.cuh"
 
 namespace opf {
@@ -1145,8 +1146,7 @@ k_warp_engine(IterArgs<T> g, WarpLayout lay, const int *pr, T *u_glob, int n_ite
 
 template <typename T>
 int prepare_warp_engine(unsigned bytes) {
-    if (cudaFuncSetAttribute(k_warp_engine<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-        return -1;
+    if (allow_dynamic_smem((const void *)k_warp_engine<T>, bytes)) return -1;
     if (cudaFuncSetAttribute(k_warp_engine<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return -1;
     return 0;
@@ -1358,8 +1358,7 @@ size_t precompute_smem(int m, int n) {
 
 int launch_precompute(const PreArgs &a, int max_n, cudaStream_t st) {
     const size_t shm = precompute_smem(a.sh_m, a.sh_n);
-    if (cudaFuncSetAttribute(k_precompute, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm) != cudaSuccess)
-        return -1;
+    if (allow_dynamic_smem((const void *)k_precompute, shm)) return -1;
     // 4 warps up to 63 columns (8: 8500 buses 0.79 -> 1.23 ms), 8 above (240 blocks
     // of up to 100: 2.18 -> 1.99 ms), and one more for the right-hand side at 256
     k_precompute<<<a.S, 32 * (max_n < 64 ? 4 : max_n < 256 ? 8 : 9), shm, st>>>(a);
@@ -1399,8 +1398,7 @@ void launch_enter_shift(int L, const int *gk, const double *xr, const double *ds
 
 template <typename T>
 int prepare_cluster_engine(unsigned bytes, int P) {
-    if (cudaFuncSetAttribute(k_cluster_engine<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-        return -1;
+    if (allow_dynamic_smem((const void *)k_cluster_engine<T>, bytes)) return -1;
     if (P > 8 && cudaFuncSetAttribute(k_cluster_engine<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
         return -1;
     return 0;

@@ -36,6 +36,7 @@
 #include <cstring>
 
 #include "opf_internal.h"
+#include "smem_limit.h"
 #include "test_rule.cuh"
 #include "tmem.cuh"
 
@@ -508,8 +509,7 @@ __global__ void k_lpack(int nrec, const int4 *desc, const int4 *sub, const int4 
 }  // namespace
 
 int lane_engine_prepare(int C, unsigned bytes) {
-    if (cudaFuncSetAttribute(k_lane_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-        return -1;
+    if (allow_dynamic_smem((const void *)k_lane_engine, bytes)) return -1;
     if (C > 8 && cudaFuncSetAttribute(k_lane_engine, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
                      cudaSuccess)
         return -1;

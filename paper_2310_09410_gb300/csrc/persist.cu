@@ -93,6 +93,7 @@
 #include <type_traits>
 
 #include "opf_internal.h"
+#include "smem_limit.h"
 #include "test_rule.cuh"
 
 namespace opf {
@@ -1211,7 +1212,7 @@ static void fill_cfg(const PersistLayout &lay, cudaLaunchConfig_t *cfg, cudaLaun
 template <typename T>
 int prepare_persist_engine(const PersistLayout &lay) {
     const void *fn = persist_fn<T>(lay);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.bytes) != cudaSuccess) return -1;
+    if (allow_dynamic_smem(fn, lay.bytes)) return -1;
     if (lay.cluster && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return -1;
     return 0;
 }
