@@ -37,10 +37,13 @@ struct GraphCache {
 
 // Captures "while (condition) body" into *gc: body(cond) enqueues one pass on
 // `s`, its kernels set the condition; it returns nonzero when a launch was
-// refused.  A launch that fails while it is captured leaves no node behind: the
-// loop would run without the kernel that ends it, for ever.  So such a graph is
-// dropped, with the launch's error.
-// cudaSuccess, or the error with *err telling where (gc is empty then).
+// refused.  A graph that lacks one of its launches is dropped: the loop might
+// run without the kernel that ends it, for ever.
+// cudaSuccess, or the error with *err telling where (gc is empty then).  A
+// launch that fails under capture invalidates the capture, and ending that one
+// destroys the graph it went into: the body, which its parent would destroy a
+// second time (the process ends there, seen with a launch of too much shared
+// memory).  So the parent of an invalidated body is left alone.
 template <typename Body>
 cudaError_t capture_while(GraphCache *gc, cudaStream_t s, Body body, std::string *err) {
     gc->reset();
@@ -75,6 +78,7 @@ cudaError_t capture_while(GraphCache *gc, cudaStream_t s, Body body, std::string
     if (launch == cudaSuccess && refused) launch = cudaErrorInvalidConfiguration;
     cudaGraph_t captured = nullptr;
     e = cudaStreamEndCapture(s, &captured);
+    if (e != cudaSuccess) gc->graph = nullptr;
     if (launch != cudaSuccess) return failed("launch under stream capture", launch);
     if (e != cudaSuccess) return failed("stream capture", e);
     e = cudaGraphInstantiate(&gc->exec, gc->graph, 0);

@@ -4,7 +4,8 @@ On the CPU, against a stand-in for the CUDA runtime: a graph captured for one
 plan's tables keeps them alive and does not match a plan built again with the
 same CTA count, in whatever order the two are freed; and a capture that loses
 a launch (the runtime's error, or the launcher's refusal) gives an error and no
-graph, since the loop would lack the kernel that ends it.
+graph, since the loop would lack the kernel that ends it, and destroys no body
+twice.
 
 On the GPU: a request that does not fit between two equal single-precision
 solves (the plan, and with it its tables, is built again) leaves the iterates
@@ -32,21 +33,25 @@ struct cudaGraphNodeParams {
     int type;
     struct { cudaGraphConditionalHandle handle; int type; unsigned size; cudaGraph_t *phGraph_out; } conditional;
 };
-inline int destroyed = 0, alive = 0, instantiated = 0, capturing = 0, mark;
+inline int destroyed = 0, alive = 0, instantiated = 0, capturing = 0, broken = 0, ended_twice = 0, mark;
 inline cudaError_t last = cudaSuccess;
 inline cudaGraph_t loop_body = &mark;
 inline int cudaGraphExecDestroy(cudaGraphExec_t) { ++destroyed; --alive; return 0; }
-inline int cudaGraphDestroy(cudaGraph_t) { ++destroyed; --alive; return 0; }
-inline cudaError_t cudaGraphCreate(cudaGraph_t *g, unsigned) { *g = &mark; ++alive; return cudaSuccess; }
+inline int cudaGraphDestroy(cudaGraph_t) { ++destroyed; --alive; ended_twice += broken; return 0; }
+inline cudaError_t cudaGraphCreate(cudaGraph_t *g, unsigned) { *g = &mark; ++alive; broken = 0; return cudaSuccess; }
 inline cudaError_t cudaGraphConditionalHandleCreate(cudaGraphConditionalHandle *h, cudaGraph_t, unsigned, unsigned) {
     *h = 7; return cudaSuccess;
 }
 inline cudaError_t cudaGraphAddNode(cudaGraphNode_t *, cudaGraph_t, const cudaGraphNode_t *, const void *, unsigned,
                                     cudaGraphNodeParams *p) { p->conditional.phGraph_out = &loop_body; return cudaSuccess; }
+// a launch that fails under capture invalidates it, and its end destroys the body graph
+inline void launch_fails(cudaError_t e) { last = e; broken = 1; }
 inline cudaError_t cudaGetLastError() { cudaError_t e = last; last = cudaSuccess; return e; }
 inline cudaError_t cudaStreamBeginCaptureToGraph(cudaStream_t, cudaGraph_t, const cudaGraphNode_t *, const void *, unsigned,
                                                  int) { ++capturing; return cudaSuccess; }
-inline cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) { --capturing; return cudaSuccess; }
+inline cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *) {
+    --capturing; return broken ? cudaErrorInvalidValue : cudaSuccess;
+}
 inline cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned) {
     *x = &mark; ++alive; ++instantiated; return cudaSuccess;
 }
@@ -81,14 +86,16 @@ int main() {
     std::string why;
     auto capture = [&](cudaError_t launch, int refused) {
         return capture_while(&g, nullptr, [&](cudaGraphConditionalHandle c) {
-            if (launch != cudaSuccess) last = launch;
+            if (launch != cudaSuccess) launch_fails(launch);
             return c == 7 ? refused : 1;
         }, &why);
     };
     CHECK(capture(cudaSuccess, 0) == cudaSuccess && g.exec && alive == 2 && instantiated == 1);
     g.kind = 4;
     CHECK(capture(cudaErrorInvalidValue, 0) == cudaErrorInvalidValue && !why.empty());
-    CHECK(!g.exec && !g.graph && alive == 0 && instantiated == 1 && capturing == 0 && g.kind == -1);
+    // (the parent, whose body is gone, is left alone)
+    CHECK(!g.exec && !g.graph && alive == 1 && ended_twice == 0 && instantiated == 1 && capturing == 0 && g.kind == -1);
+    alive = 0;
     CHECK(capture(cudaSuccess, 1) != cudaSuccess && !g.exec && alive == 0 && instantiated == 1 && capturing == 0);
     last = cudaErrorInvalidValue;
     CHECK(capture(cudaSuccess, 0) == cudaSuccess && g.exec && alive == 2 && instantiated == 2);
