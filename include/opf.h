@@ -255,7 +255,8 @@ int opf_get_timing(opf_handle *h, double *ms, int n);
  *              u[seg_off[i] .. seg_off[i+1]) (at least one each)
  *   u          device, seg_off[n] doubles: rho x_k - lambda_k of every copy,
  *              grouped by global (summed in that order)
- *   c, lb, ub  device, n doubles each (bounds may be +-INFINITY)
+ *   c, lb, ub  device, n doubles each (bounds may be +-INFINITY; a bound that
+ *              is NaN bounds nothing)
  *   rho        > 0
  *   x          device, n doubles out: clip((sum u - c_i) / (rho N_i), lb_i, ub_i)
  *   objective  device, 1 double out: c^T x

@@ -55,6 +55,9 @@ __device__ __forceinline__ long long ordered(double x) {
     const long long b = __double_as_longlong(x);
     return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
+__device__ __forceinline__ bool is_nan(double x) {
+    return (unsigned long long)(__double_as_longlong(x) << 1) > 0xffe0000000000000ull;
+}
 
 // x_i = clip((sum of u over the copies of global i - c_i) / (rho N_i), lb_i, ub_i)
 __device__ __forceinline__ double global_update(int a, int b, const double *u, double c, double lb, double ub,
@@ -65,9 +68,9 @@ __device__ __forceinline__ double global_update(int a, int b, const double *u, d
     const double num = sigma - c;
     const double rcp = cnt > 0 && cnt < kRecip ? rc.r[cnt] : 0.0;
     double x = rcp != 0.0 ? quotient(num, rho * (double)cnt, rcp) : num / (rho * (double)cnt);
-    if ((unsigned long long)(__double_as_longlong(x) << 1) <= 0xffe0000000000000ull) {   // NaN stays NaN
-        if (ordered(x) < ordered(lb)) x = lb;
-        if (ordered(x) > ordered(ub)) x = ub;
+    if (!is_nan(x)) {                        // NaN stays NaN; a bound that is NaN bounds nothing
+        if (ordered(x) < ordered(lb) && !is_nan(lb)) x = lb;
+        if (ordered(x) > ordered(ub) && !is_nan(ub)) x = ub;
     }
     return x;
 }
