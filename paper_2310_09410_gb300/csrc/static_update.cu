@@ -7,6 +7,7 @@
 // framework's caching allocator that owns the whole device).  Its scratch (one
 // FP64 objective partial per block) is a file-scope __device__
 // array instead of memory from a handle, so the call allocates nothing.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -21,11 +22,23 @@
 
 namespace {
 
+namespace cg = cooperative_groups;
+
 constexpr int kThreads = 256;
-constexpr int kOneBlock = 512;       // up to so many globals run in one block, which sums the objective itself
-                                     // (between events, one block / two kernels: 181 globals 6.8 / 8.8 us, 408
-                                     // and 512 8.8 / 8.8, 800 10.9 / 8.8)
-constexpr int kBlocks = 8 * 152;     // resident blocks of the GPU: more globals than threads go round by round
+// Launch forms by the number of globals: one block, which sums the objective
+// itself; one cluster of blocks; a grid and a second launch that sums the
+// blocks' shares.  us per call in a graph and from a host that enqueues calls
+// back to back (the host is the bound there: a second launch costs it 1.9 us):
+//   globals        65       256       400       520      2000      4096      8192
+//   one block   2.5, 7.8  3.5, 7.8  4.5, 7.9  5.1, 7.8    -         -         -
+//   cluster     3.5, 7.7  3.6, 7.7  3.4, 7.7  3.5, 7.7  4.4, 7.8  5.9, 8.2  7.9, 10.2
+//   two launches   -         -         -      4.8, 9.8  5.0, 9.6  5.1, 9.7  4.9, 9.6
+constexpr int kOneBlock = 256;       // up to so many globals: one block
+constexpr int kOneCluster = 4096;    // up to so many: one cluster
+constexpr int kCluster = 8;          // its blocks, of up to kClusterThreads
+constexpr int kClusterThreads = 512;
+constexpr int kBlocks = 8 * 152;     // most blocks of the grid (a few per SM of the whole GPU): more globals than
+                                     // threads go round by round
 constexpr int kRecip = 16;           // 1 / (rho N) by copy count below this
 
 // Per-block partial sums of c^T x.  Shared by every call in a CUDA context and
@@ -91,13 +104,11 @@ __device__ __forceinline__ double block_sum(double v) {
     return v;
 }
 
-// The update of every global (round by round when there are more than threads)
-// and each block's share of c^T x in out[block] (one block: the objective).
-__global__ void __launch_bounds__(kOneBlock) k_global_update_static(int n, const int *seg_off, const double *u,
-                                                                    const double *c, const double *lb,
-                                                                    const double *ub, double rho, Recips rc, double *x,
-                                                                    double *out) {
-    cudaTriggerProgrammaticLaunchCompletion();       // the sum's block may take its place and wait there
+// The update of this thread's globals (round by round when there are more than
+// threads) and its share of c^T x.
+__device__ __forceinline__ double update_share(int n, const int *seg_off, const double *u, const double *c,
+                                               const double *lb, const double *ub, double rho, const Recips &rc,
+                                               double *x) {
     double o = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double ci = c[i];
@@ -105,8 +116,38 @@ __global__ void __launch_bounds__(kOneBlock) k_global_update_static(int n, const
         x[i] = xv;
         o = fma(ci, xv, o);
     }
-    o = block_sum(o);
+    return o;
+}
+
+// The update of every global and each block's share of c^T x in out[block] (one
+// block: the objective).
+__global__ void __launch_bounds__(kThreads) k_global_update_static(int n, const int *seg_off, const double *u,
+                                                                    const double *c, const double *lb,
+                                                                    const double *ub, double rho, Recips rc, double *x,
+                                                                    double *out) {
+    cudaTriggerProgrammaticLaunchCompletion();       // the sum's block may take its place and wait there
+    const double o = block_sum(update_share(n, seg_off, u, c, lb, ub, rho, rc, x));
     if (threadIdx.x == 0) out[blockIdx.x] = o;
+}
+
+// The same in one launch, by one cluster: the blocks' shares meet in the first
+// block's shared memory and are added there in block order.
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kClusterThreads)
+    k_global_update_cluster(int n, const int *seg_off, const double *u, const double *c, const double *lb,
+                            const double *ub, double rho, Recips rc, double *x, double *objective) {
+    __shared__ double share[kCluster];
+    cg::cluster_group cl = cg::this_cluster();
+    cl.barrier_arrive();                             // every block of the cluster has started
+    double o = update_share(n, seg_off, u, c, lb, ub, rho, rc, x);
+    o = block_sum(o);
+    cl.barrier_wait();
+    if (threadIdx.x == 0) *cl.map_shared_rank(&share[cl.block_rank()], 0) = o;
+    cl.sync();
+    if (cl.block_rank() == 0 && threadIdx.x == 0) {
+        double s = share[0];
+        for (int b = 1; b < kCluster; ++b) s += share[b];
+        *objective = s;
+    }
 }
 
 // Objective: the block partials summed in a fixed order by one block.  (By one
@@ -162,11 +203,33 @@ const Drv &drv() {
     return d;
 }
 
-// Device address of g_static_partials per CUDA context, keyed by the
-// context's process-unique id (a destroyed and re-created context, e.g. after
-// cudaDeviceReset, gets a new id, so a stale address is never reused).
+// Per CUDA context the device address of g_static_partials and whether the
+// context can hold the one-cluster launch, keyed by the context's process-unique
+// id (a destroyed and re-created context, e.g. after cudaDeviceReset, gets a new
+// id, so a stale address is never reused).
+struct CtxInfo {
+    double *partials = nullptr;
+    bool cluster = false;
+};
 std::mutex g_mu;
-std::map<unsigned long long, double *> g_dev_ptr;
+std::map<unsigned long long, CtxInfo> g_ctx;
+
+bool holds_cluster() {
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kCluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(kCluster);
+    cfg.blockDim = dim3(kClusterThreads);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_global_update_cluster, &cfg) == cudaSuccess) return n > 0;
+    cudaGetLastError();
+    return false;
+}
 
 int fail(int code, const std::string &msg) {
     opf::set_last_error("opf_global_update_static: " + msg);
@@ -204,27 +267,29 @@ extern "C" int opf_global_update_static(int32_t n, const int32_t *seg_off, const
     }
     unsigned long long id = 0;
     if (d.ctxId(ctx, &id) != CUDA_SUCCESS) return fail(OPF_E_CUDA, "cuCtxGetId failed");
-    double *partials = nullptr;
+    CtxInfo info;
     {
         // set-up, once per context with that context current: the device
         // address of the static array (host code must not use its name as an
         // address)
         std::lock_guard<std::mutex> lock(g_mu);
-        auto it = g_dev_ptr.find(id);
-        if (it != g_dev_ptr.end()) {
-            partials = it->second;
+        auto it = g_ctx.find(id);
+        if (it != g_ctx.end()) {
+            info = it->second;
         } else {
             if (d.push(ctx) != CUDA_SUCCESS) return fail(OPF_E_CUDA, "cuCtxPushCurrent failed");
             void *p = nullptr;
             cudaError_t e = cudaGetSymbolAddress(&p, g_static_partials);
+            if (e == cudaSuccess) info.cluster = holds_cluster();
             CUcontext popped = nullptr;
             d.pop(&popped);
             if (e != cudaSuccess || !p)
                 return fail(OPF_E_CUDA, std::string("cudaGetSymbolAddress: ") + cudaGetErrorString(e));
-            partials = static_cast<double *>(p);
-            g_dev_ptr[id] = partials;
+            info.partials = static_cast<double *>(p);
+            g_ctx[id] = info;
         }
     }
+    double *const partials = info.partials;
     Recips rc;
     for (int k = 0; k < kRecip; ++k) {
         const double den = rho * (double)k, r = k ? 1.0 / den : 0.0;
@@ -233,6 +298,9 @@ extern "C" int opf_global_update_static(int32_t n, const int32_t *seg_off, const
     if (n <= kOneBlock) {
         k_global_update_static<<<1, (unsigned)((n + 31) / 32 * 32), 0, s>>>(n, seg_off, u, c, lb, ub, rho, rc, x,
                                                                             objective);
+    } else if (n <= kOneCluster && info.cluster) {
+        const int threads = std::min(((n + kCluster - 1) / kCluster + 31) / 32 * 32, kClusterThreads);
+        k_global_update_cluster<<<kCluster, (unsigned)threads, 0, s>>>(n, seg_off, u, c, lb, ub, rho, rc, x, objective);
     } else {
         const int nblk = std::min((n + kThreads - 1) / kThreads, kBlocks);
         k_global_update_static<<<(unsigned)nblk, kThreads, 0, s>>>(n, seg_off, u, c, lb, ub, rho, rc, x, partials);
