@@ -771,30 +771,84 @@ static std::vector<int> warp_parts(const opf_handle *h, bool fp32, int req_P) {
     return nparts;
 }
 
-// The partition of the instance over P CTAs: parts of a depth-first order for
-// the local forms, else runs of the size-sorted order.
-static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, bool own,
-                                std::shared_ptr<PersistTables> *out) {
-    const int S = h->S, L = h->L;
+// Largest part of a split (the counts of PersistTables that it settles).
+struct PersistSizes { long long mf = 0, ms = 0, mj = 0, mt = 0, mk = 0, mv = 0; };
+
+// The split of the instance over P CTAs: parts of a depth-first order for the
+// local forms, else runs of the size-sorted order; the owner form's own.
+static void split_instance(opf_handle *h, int P, bool local, bool own, PersistOwners *owners, PersistSizes *sizes) {
+    const int S = h->S;
     std::vector<double> cost(S);
     for (int s = 0; s < S; ++s)
         cost[s] = 6.0 * h->h_sn[s] + (double)h->h_sf[s] * h->h_npad[s] + (double)h->h_sn[s] * h->h_sf[s];
-    std::vector<int> order;
-    if (local && !own) {
-        if (h->persist_order.empty()) {
+    if (own) {
+        *owners = persist_owners(P, S, h->G, cost, h->h_soff, h->h_segp, h->h_pk, h->h_gk, h->h_gstart);
+    } else {
+        if (local && h->persist_order.empty()) {
             std::vector<int> start(S);           // new trees begin in canonical order
             for (int d = 0; d < S; ++d) start[h->dev_to_canon_sub[d]] = d;
             h->persist_order = persist_order(S, h->h_soff, h->h_segp, h->h_pk, start);
         }
-        order = h->persist_order;
-    } else {
-        order.resize(S);
-        std::iota(order.begin(), order.end(), 0);
+        std::vector<int> sorted;
+        if (!local) {
+            sorted.resize(S);
+            std::iota(sorted.begin(), sorted.end(), 0);
+        }
+        owners->parts = persist_split(P, S, local ? h->persist_order : sorted, cost, h->h_soff);
     }
-    PersistOwners owners;
-    if (own) owners = persist_owners(P, S, h->G, cost, h->h_soff, h->h_segp, h->h_pk, h->h_gk, h->h_gstart);
-    else owners.parts = persist_parts(P, S, order, cost, h->h_soff, h->h_segp, h->h_pk);
-    const PersistParts &parts = owners.parts;
+    const PersistParts &parts = owners->parts;
+    PersistSizes &m = *sizes;
+    m = PersistSizes{};
+    for (int p = 0; p < P; ++p) {
+        long long f = 0, j = 0, c0 = 0, v = 0;
+        for (int i = parts.s0[p]; i < parts.s0[p + 1]; ++i) {
+            const int d = parts.sub[i], npad = h->h_npad[d], fp = local ? round4(h->h_sf[d]) : h->h_sf[d];
+            f += (long long)fp * (npad + ((npad & 7) == 0 ? 4 : 0));
+            j += h->h_sf[d];
+            c0 += fp;
+            v += npad;
+        }
+        m.mf = std::max(m.mf, f);
+        m.mj = std::max(m.mj, j);
+        m.mt = std::max(m.mt, c0);
+        m.mv = std::max(m.mv, v);
+        m.ms = std::max<long long>(m.ms, parts.s0[p + 1] - parts.s0[p]);
+        m.mk = std::max<long long>(m.mk, parts.k0[p + 1] - parts.k0[p]);
+    }
+}
+
+// False when parts of these sizes fit no CTA (T: the precision), whatever the
+// counts that are not known yet.
+template <typename T>
+static bool sizes_can_fit(const PersistSizes &m, bool local, int optin) {
+    if (local && std::max(m.mk, m.mj) > kPersistMaxThreads) return false;
+    const long long slot = local ? (long long)sizeof(T) : (long long)(persist_slot_bytes(sizeof(T)) + sizeof(T));
+    return m.mf * (long long)sizeof(T) + m.ms * (long long)sizeof(int4) + (m.mv + m.mt) * (long long)sizeof(T) +
+               (local ? 0 : m.mj * (long long)sizeof(int)) + m.mk * (slot + 3 * (long long)sizeof(double)) <= optin;
+}
+
+// The same from the averages over P parts, before any split.
+template <typename T>
+static bool average_can_fit(const opf_handle *h, int P, bool local, bool own, int optin) {
+    PersistSizes a;
+    long long f = 0, v = 0, j = 0;
+    for (int s = 0; s < h->S; ++s) {
+        f += (long long)h->h_sf[s] * h->h_npad[s];
+        v += h->h_npad[s];
+        j += h->h_sf[s];
+    }
+    a.mf = f / P; a.mv = v / P; a.mj = a.mt = j / P;
+    a.mk = h->L / P;
+    if (own && (h->G + P - 1) / P > kPersistMaxThreads) return false;
+    return sizes_can_fit<T>(a, local, optin);
+}
+
+// A split instance's tables on the device.
+static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, bool own, PersistOwners &owners,
+                                std::shared_ptr<PersistTables> *out) {
+    const int S = h->S, L = h->L;
+    PersistParts &parts = owners.parts;
+    if (local && !own) persist_lists(P, h->h_soff, h->h_segp, h->h_pk, &parts);
     auto t = std::make_shared<PersistTables>();
     t->P = P; t->S = S; t->L = L;
     t->local = local;
@@ -804,7 +858,7 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
     t->moc = owners.most_copies;
     t->fits = parts.ok;
     t->s0 = parts.s0;
-    t->remote = (long long)parts.rem.size();
+    t->remote = local ? (long long)parts.rem.size() : persist_remote(P, parts, h->h_soff, h->h_segp);
     // cluster form: a subsystem whose FP32 column products go by halves (in the
     // order of the warp engine's two warps) has its second half start at a
     // multiple of 4 rows, for 16-byte loads
@@ -860,6 +914,8 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
     }
     // one allocation and one upload, every array from a multiple of 16 bytes
     std::vector<int> all;
+    all.reserve(4 * (size_t)S + items.size() + 2 * (size_t)L + parts.rem.size() + parts.list.size() / 2 +
+                (local ? 3 * (size_t)L : 0) + 1024);
     std::vector<std::pair<void **, size_t>> at;
     auto add = [&](void *slot, const void *data, size_t bytes) {
         at.push_back({(void **)slot, all.size()});
@@ -910,9 +966,23 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     auto same = [&](const std::shared_ptr<PersistTables> &t) {
         return t && t->P == P && t->local == local && t->cluster == cluster && t->own == own;
     };
+    int optin = 0;
+    CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     if (!same(pp->tab)) {
-        if (same(other.tab)) pp->tab = other.tab;
-        else TRY(build_persist_tables(h, P, local, cluster, own, &pp->tab));
+        if (same(other.tab)) {
+            pp->tab = other.tab;
+        } else {
+            // A form that cannot fit is given up before its tables are built: the
+            // averages tell for most, the split for the rest (a new handle's first
+            // mixed solve of 500 iterations, 12,000 and 40,000 buses: 47 and 171 ms
+            // with every form that was tried built in full, 13 and 30 now).
+            if (!average_can_fit<T>(h, P, local, own, optin)) return OPF_OK;
+            PersistOwners owners;
+            PersistSizes sizes;
+            split_instance(h, P, local, own, &owners, &sizes);
+            if (!cluster && !sizes_can_fit<T>(sizes, local, optin)) return OPF_OK;
+            TRY(build_persist_tables(h, P, local, cluster, own, owners, &pp->tab));
+        }
     }
     const PersistTables &t = *pp->tab;
     PersistLayout &c = pp->lay;
@@ -997,6 +1067,7 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
                                                 : small ? (double)((at + 127) / 128 * longest)
                                                         : *std::max_element(issue, issue + 4) + sum / 4.0);
                         threads = std::max(threads, (at + 31) / 32 * 32);
+                        if (threads > kPersistMaxThreads || (cost >= 0 && worst >= cost)) break;   // no better choice
                     }
                     if (threads <= kPersistMaxThreads && (cost < 0 || worst < cost)) {
                         cost = worst;
@@ -1049,8 +1120,6 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     // flags (16 B), a DevStatus copy, the test's sums (48 B), per warp (16 warps)
     take(&c.off_misc, 64 + ((sizeof(DevStatus) + 15) & ~(size_t)15) + kPersistMaxThreads / 32 * 6 * sizeof(double));
     c.bytes = (unsigned)off;
-    int optin = 0;
-    CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     if ((long long)off > optin) return OPF_OK;
     if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
     if (persist_resident<T>(c, n_sm) < P) { cudaGetLastError(); return OPF_OK; }

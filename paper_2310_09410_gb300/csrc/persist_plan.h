@@ -118,12 +118,12 @@ inline std::vector<int> persist_order(int S, const std::vector<int> &soff, const
 }
 
 // P parts of the given order, balanced by cost[d].  Subsystems are numbered in
-// decreasing size (so a part's are sorted by number).
-inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, const std::vector<double> &cost,
-                                  const std::vector<int> &soff, const std::vector<int> &segp,
-                                  const std::vector<int> &pk) {
+// decreasing size (so a part's are sorted by number).  In two steps: the split
+// (s0, sub, k0) tells whether the parts fit a form at all, in an eighth of the
+// lists' time.
+inline PersistParts persist_split(int P, int S, const std::vector<int> &order, const std::vector<double> &cost,
+                                  const std::vector<int> &soff) {
     PersistParts t;
-    const int L = (int)pk.size();
     t.s0.assign(P + 1, S);
     t.s0[0] = 0;
     double total = 0, acc = 0;
@@ -134,26 +134,58 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
         while (p < P && acc >= total * p / P) t.s0[p++] = i + 1;
     }
     t.sub = order;
-    for (int q = 0; q < P; ++q) std::sort(t.sub.begin() + t.s0[q], t.sub.begin() + t.s0[q + 1]);
+    t.k0.assign(P + 1, 0);
+    for (int q = 0; q < P; ++q) {
+        std::sort(t.sub.begin() + t.s0[q], t.sub.begin() + t.s0[q + 1]);
+        t.k0[q + 1] = t.k0[q];
+        for (int i = t.s0[q]; i < t.s0[q + 1]; ++i) t.k0[q + 1] += soff[t.sub[i] + 1] - soff[t.sub[i]];
+    }
+    t.r0.assign(P + 1, 0);
+    t.l0.assign(P + 1, 0);
+    return t;
+}
+
+// Entries of other parts that the parts read, over all parts (rem.size() of
+// persist_lists, without the lists): per part and global of several copies, the
+// copies that are not the part's own.
+inline long long persist_remote(int P, const PersistParts &t, const std::vector<int> &soff,
+                                const std::vector<int> &segp) {
+    std::vector<int> last(segp.size(), -1);      // by first copy: the last part that counted the global
+    long long n = 0;
+    for (int q = 0; q < P; ++q)
+        for (int i = t.s0[q]; i < t.s0[q + 1]; ++i)
+            for (int k = soff[t.sub[i]]; k < soff[t.sub[i] + 1]; ++k) {
+                const int cnt = segp[k] & 255;
+                if (cnt < 2) continue;
+                --n;
+                if (last[segp[k] >> 8] == q) continue;
+                last[segp[k] >> 8] = q;
+                n += cnt;
+            }
+    return n;
+}
+
+// The slots, copy lists and exchanges of split parts.
+inline void persist_lists(int P, const std::vector<int> &soff, const std::vector<int> &segp, const std::vector<int> &pk,
+                          PersistParts *parts) {
+    PersistParts &t = *parts;
+    const int L = (int)pk.size();
     // per copy (in copy order) its part and position there, so that a list
     // reads one run of memory
     struct Place { int part, at; };
     std::vector<Place> place(L);
-    t.k0.assign(P + 1, 0);
     t.slot.resize(L);
-    for (int q = 0, j = 0; q < P; ++q) {
+    for (int q = 0, j = 0; q < P; ++q)
         for (int i = t.s0[q]; i < t.s0[q + 1]; ++i)
             for (int k = soff[t.sub[i]]; k < soff[t.sub[i] + 1]; ++k, ++j) {
                 place[pk[k]] = {q, j - t.k0[q]};
                 t.slot[j] = k;
             }
-        t.k0[q + 1] = j;
-    }
     t.seg.resize(L);
     t.out.assign(L, -1);
-    t.list.reserve(4 * (size_t)L);
-    t.r0.assign(P + 1, 0);
-    t.l0.assign(P + 1, 0);
+    t.rem.reserve(L / 4);
+    t.list.resize(4 * (size_t)L);
+    size_t used = 0;                             // entries of the lists so far
     std::vector<int> where(L, -1);               // by first copy: number of the part's list, or below l0[part]
     for (int q = 0; q < P; ++q) {
         const int nk = t.k0[q + 1] - t.k0[q], l0 = t.l0[q], r0 = t.r0[q];
@@ -164,34 +196,40 @@ inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, c
                 continue;
             }
             if (where[c0] < l0) {
-                where[c0] = (int)(t.list.size() / 8);
-                unsigned short e[8];
-                for (int c = c0, n = 0; c < c0 + cnt || n; ++c) {
-                    e[n] = 0xffff;               // past the last copy: the zero, below
-                    if (c < c0 + cnt) {
-                        if (place[c].part == q) {
-                            e[n] = (unsigned short)place[c].at;
-                        } else {
-                            e[n] = (unsigned short)(nk + (int)t.rem.size() - r0);
-                            t.rem.push_back(c);
-                            t.out[t.k0[place[c].part] + place[c].at] = c;
-                        }
-                    }
-                    if (++n == 8) {
-                        t.list.insert(t.list.end(), e, e + 8);
-                        n = 0;
+                where[c0] = (int)(used / 8);
+                const size_t end = used + ((cnt + 7) & ~7);
+                if (end > t.list.size()) t.list.resize(2 * end);
+                unsigned short *e = t.list.data() + used, *last = t.list.data() + end;
+                for (int c = c0; c < c0 + cnt; ++c) {
+                    const Place at = place[c];
+                    if (at.part == q) {
+                        *e++ = (unsigned short)at.at;
+                    } else {
+                        *e++ = (unsigned short)(nk + (int)t.rem.size() - r0);
+                        t.rem.push_back(c);
+                        t.out[t.k0[at.part] + at.at] = c;
                     }
                 }
+                while (e < last) *e++ = 0xffff;  // past the last copy: the zero, below
+                used = end;
             }
             t.seg[j] = ((where[c0] - l0) << 8) | cnt;
         }
         t.r0[q + 1] = (int)t.rem.size();
-        t.l0[q + 1] = (int)(t.list.size() / 8);
+        t.l0[q + 1] = (int)(used / 8);
         const int zero = nk + t.r0[q + 1] - r0;
         if (zero >= 0xffff) t.ok = false;
-        for (size_t i = 8 * (size_t)l0; i < t.list.size(); ++i)
-            if (t.list[i] == 0xffff) t.list[i] = (unsigned short)zero;
+        unsigned short *e = t.list.data() + 8 * (size_t)l0, *last = t.list.data() + used;
+        for (; e < last; ++e) *e = *e == 0xffff ? (unsigned short)zero : *e;
     }
+    t.list.resize(used);
+}
+
+inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, const std::vector<double> &cost,
+                                  const std::vector<int> &soff, const std::vector<int> &segp,
+                                  const std::vector<int> &pk) {
+    PersistParts t = persist_split(P, S, order, cost, soff);
+    persist_lists(P, soff, segp, pk, &t);
     return t;
 }
 
