@@ -190,8 +190,9 @@ struct PersistPtrs {
     const int *wide;               // FP64 local plans: per part the columns and the slots spread over lanes (the first)
 };
 
-// Bytes of a slot's record in a plan with several slots per thread (persist.cu).
-constexpr size_t persist_slot_bytes(size_t word) { return 6 * word + 8; }
+// Bytes per slot in a plan with several slots per thread (persist.cu): FP32 nine
+// arrays, FP64 a record.
+constexpr size_t persist_slot_bytes(size_t word) { return word == 4 ? 9 * word : 6 * word + 8; }
 
 // Shared-memory image of one CTA of the warp engine, byte offsets.
 struct WarpLayout {

@@ -48,9 +48,10 @@
 // against 6.5 on the cluster engine (12,000 stores to other CTAs' shared memory
 // twice an iteration, each behind a cluster barrier that waits for them), FP64
 // 7.4 against 8.7 in the local form.
-// k_persist_engine: the same iteration for parts that do not fit that form
-// (several slots per thread): parts are runs of the size-sorted order, slot
-// records in shared memory, and every copy of u is read from the exchange.
+// Parts that do not fit that form (several slots per thread) are runs of the
+// size-sorted order, the slots' data in shared memory, every copy of u read from
+// the exchange: k_persist_engine (FP64) by stamped words as above,
+// k_persist_slots (FP32) from plain words behind a grid barrier.
 // On tested iterations each CTA adds the Sec. III-C sums of its slots in FP64
 // and publishes them as stamped words; every CTA sums the P partials in the same
 // fixed order and takes the same stopping decision (rank 0 publishes the
@@ -530,27 +531,17 @@ __device__ __forceinline__ void place(S &s, const int4 r, int row) {
 
 // A slot's record in shared memory (k_persist_engine): the fields of Slot that
 // the rest cannot be derived from.
-template <typename T>
 struct SlotRec {
-    T f[6];                          // FP32: lam, xs, bt, ct, lo, hi; FP64: lam, rx, rbt, ct, lo, hi (bits)
+    double f[6];                     // lam, rx, rbt, ct, lo, hi (bits)
     int seg, mo;                     // (first copy's entry << 8) | copies; subsystem << 8 | row, own copy's index << 24
 };
-static_assert(sizeof(SlotRec<float>) == persist_slot_bytes(4) && sizeof(SlotRec<double>) == persist_slot_bytes(8),
-              "the layout reserves this much per slot");
+static_assert(sizeof(SlotRec) == persist_slot_bytes(8), "the layout reserves this much per slot");
 
-__device__ __forceinline__ void pack(SlotRec<float> &q, const Slot<float, false> &s) {
-    q.f[0] = s.lam; q.f[1] = s.xs; q.f[2] = s.bt; q.f[3] = s.ct; q.f[4] = s.lo; q.f[5] = s.hi;
-}
-__device__ __forceinline__ void pack(SlotRec<double> &q, const Slot<double, false> &s) {
+__device__ __forceinline__ void pack(SlotRec &q, const Slot<double, false> &s) {
     q.f[0] = s.lam; q.f[1] = s.rx; q.f[2] = s.rbt; q.f[3] = s.ct;
     q.f[4] = __longlong_as_double(s.lo); q.f[5] = __longlong_as_double(s.hi);
 }
-__device__ __forceinline__ void unpack(Slot<float, false> &s, const SlotRec<float> &q, const IterArgs<float> &g) {
-    s.lam = q.f[0]; s.xs = q.f[1]; s.bt = q.f[2]; s.ct = q.f[3]; s.lo = q.f[4]; s.hi = q.f[5];
-    s.w = __fmul_rn(s.lam, g.inv_rho);
-    s.u = g.rho * s.xs - s.lam;
-}
-__device__ __forceinline__ void unpack(Slot<double, false> &s, const SlotRec<double> &q, const IterArgs<double> &) {
+__device__ __forceinline__ void unpack(Slot<double, false> &s, const SlotRec &q) {
     s.lam = q.f[0]; s.rx = q.f[1]; s.rbt = q.f[2]; s.ct = q.f[3];
     s.lo = __double_as_longlong(q.f[4]); s.hi = __double_as_longlong(q.f[5]);
     s.u = s.rx - s.lam;
@@ -1052,10 +1043,11 @@ k_persist_local(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_
     leave(m, st, cond, use_cond);
 }
 
-template <typename T>
+// FP64, several slots per thread.
 __global__ void __launch_bounds__(kPersistMaxThreads, 2)
-k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar_extra, int n_iters, int check_every,
-                 DevStatus *st, double rho_d, cudaGraphConditionalHandle cond, int use_cond) {
+k_persist_engine(IterArgs<double> g, PersistLayout lay, PersistPtrs pp, double *U, int bar_extra, int n_iters,
+                 int check_every, DevStatus *st, double rho_d, cudaGraphConditionalHandle cond, int use_cond) {
+    using T = double;
     extern __shared__ __align__(16) unsigned char sm[];
     const int P = lay.P, rank = (int)blockIdx.x, P1 = P + 1, L = lay.L;
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -1070,9 +1062,9 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
     T *F = reinterpret_cast<T *>(sm + lay.off_F);
     int4 *srec = reinterpret_cast<int4 *>(sm + lay.off_srec);
     int *items = reinterpret_cast<int *>(sm + lay.off_items);
-    SlotRec<T> *slots = reinterpret_cast<SlotRec<T> *>(sm + lay.off_slots);
+    SlotRec *slots = reinterpret_cast<SlotRec *>(sm + lay.off_slots);
     T *rb = reinterpret_cast<T *>(sm + lay.off_r);                 // rho x of the slots
-    T *rns = reinterpret_cast<T *>(sm + lay.off_rn);               // 1 / (rho N) (FP64: 1 / N) by copy count N
+    T *rns = reinterpret_cast<T *>(sm + lay.off_rn);               // 1 / N by copy count N
     T *vb = reinterpret_cast<T *>(sm + lay.off_vb);
     T *tb = reinterpret_cast<T *>(sm + lay.off_tb);
     double *xrs = reinterpret_cast<double *>(sm + lay.off_xrs);
@@ -1083,7 +1075,7 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
     stage<int4>(srec, g.srec + s0, ns);
     stage<int>(items, g.citems + j0, nj);
     for (int i = tid; i < nv; i += nthr) vb[i] = T(0);
-    for (int i = tid; i < 256; i += nthr) rns[i] = sizeof(T) == 4 ? g.recip[i] : i ? (T)(1.0 / (double)i) : T(0);
+    for (int i = tid; i < 256; i += nthr) rns[i] = i ? 1.0 / (double)i : 0.0;
     if (tid == 0) {
         m.flags[0] = 0;
         m.flags[1] = 0;
@@ -1091,7 +1083,7 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
     }
     __syncthreads();
     stage_factors<T, false>(F, g, srec, nullptr, nullptr, s0, ns);
-    constexpr int XW = sizeof(T) == 4 ? 1 : 2;
+    constexpr int XW = 2;
     u64 *X0 = pp.xu, *X1 = pp.xu + (size_t)XW * L;
     for (int k = tid; k < nk; k += nthr) {
         const int kk = k0 + k, gi = g.gk[kk], mt = g.cmeta[kk], seg = g.segp[kk], own = g.pk[kk] - (seg >> 8);
@@ -1110,11 +1102,11 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
         }
     }
     auto fetch = [&](Slot<T, false> &s, int k, int &seg, int &own) {
-        const SlotRec<T> q = slots[k];
+        const SlotRec q = slots[k];
         seg = q.seg;
         own = (int)((unsigned)q.mo >> 24);
         place(s, srec[(q.mo & 0xffffff) >> 8], q.mo & 255);
-        unpack(s, q, g);
+        unpack(s, q);
         s.rn = rns[q.seg & 255];
         s.r = rb[k];
         s.v = vb[s.pos];
@@ -1178,10 +1170,166 @@ k_persist_engine(IterArgs<T> g, PersistLayout lay, PersistPtrs pp, T *U, int bar
     leave(m, st, cond, use_cond);
 }
 
+// FP32, several slots per thread: the slots' fields in arrays of shared memory,
+// u in two plain buffers of the exchange behind a grid barrier per iteration
+// (with every copy read through L2, polling its words costs more than the
+// barrier).  The arithmetic of a slot is Slot<float, false>'s.  us per iteration
+// with stamped words and a record per slot, and in this form: 123 buses on 2 and
+// 4 CTAs 6.5 and 4.3, 4.5 and 3.4; 1000 on 16 8.2, 4.9; 12,000 and 18,000 on two
+// CTAs per SM 8.7 and 10.5, 4.5 and 6.2.
+__global__ void __launch_bounds__(kPersistMaxThreads, 2)
+k_persist_slots(IterArgs<float> g, PersistLayout lay, PersistPtrs pp, float *U, int bar_extra, int n_iters,
+                int check_every, DevStatus *st, double rho_d, cudaGraphConditionalHandle cond, int use_cond) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int P = lay.P, rank = (int)blockIdx.x, P1 = P + 1, L = lay.L;
+    const int tid = threadIdx.x, nthr = blockDim.x;
+    if (st->done) {
+        if (use_cond && rank == 0 && tid == 0) cudaGraphSetConditional(cond, 0);
+        return;
+    }
+    const int *pr = pp.pr;
+    auto range = [&](int f, int &a, int &n) { a = pr[f * P1 + rank]; n = pr[f * P1 + rank + 1] - a; };
+    int k0, nk, s0, ns, j0, nj, v0, nv;
+    range(GR_K, k0, nk); range(GR_S, s0, ns); range(GR_J, j0, nj); range(GR_V, v0, nv);
+    float *F = reinterpret_cast<float *>(sm + lay.off_F);
+    int4 *srec = reinterpret_cast<int4 *>(sm + lay.off_srec);
+    int *items = reinterpret_cast<int *>(sm + lay.off_items);
+    int *meta = reinterpret_cast<int *>(sm + lay.off_slots);       // subsystem << 8 | row
+    int *seg = meta + nk, *pk = seg + nk;                          // copies; the slot's own place among them
+    float *lam = reinterpret_cast<float *>(pk + nk), *xs = lam + nk, *bt = xs + nk, *ct = bt + nk, *lo = ct + nk,
+          *hi = lo + nk;
+    float *rb = reinterpret_cast<float *>(sm + lay.off_r);         // x of the slots
+    float *rns = reinterpret_cast<float *>(sm + lay.off_rn);       // 1 / (rho N) by copy count N
+    float *vb = reinterpret_cast<float *>(sm + lay.off_vb);        // lambda / rho, from the global update on v
+    float *tb = reinterpret_cast<float *>(sm + lay.off_tb);
+    double *xrs = reinterpret_cast<double *>(sm + lay.off_xrs);
+    double *lrs = reinterpret_cast<double *>(sm + lay.off_lrs);
+    double *cobj = reinterpret_cast<double *>(sm + lay.off_cobj);
+    const Misc m(sm + lay.off_misc);
+    float *Y0 = reinterpret_cast<float *>(pp.xu), *Y1 = Y0 + L;    // u read by even / odd iterations
+    const float rho = g.rho, inv_rho = g.inv_rho;
+
+    stage<int4>(srec, g.srec + s0, ns);
+    stage<int>(items, g.citems + j0, nj);
+    stage<int>(meta, g.cmeta + k0, nk);
+    stage<int>(seg, g.segp + k0, nk);
+    stage<int>(pk, g.pk + k0, nk);
+    stage<float>(lam, g.mu + k0, nk);
+    stage<float>(xs, g.ds + k0, nk);
+    stage<float>(bt, g.bt + k0, nk);
+    stage<float>(rns, g.recip, 256);
+    stage<double>(lrs, g.lamr + k0, nk);
+    for (int i = tid; i < nv; i += nthr) vb[i] = 0.0f;
+    if (tid == 0) {
+        m.flags[0] = 0;
+        m.flags[1] = 0;
+        *m.loc = *st;
+    }
+    __syncthreads();
+    stage_factors<float, false>(F, g, srec, nullptr, nullptr, s0, ns);
+    for (int k = tid; k < nk; k += nthr) {
+        const int gi = g.gk[k0 + k];
+        ct[k] = g.ct[gi];
+        lo[k] = g.lbt[gi];
+        hi[k] = g.ubt[gi];
+        xrs[k] = g.xr[gi];
+        cobj[k] = pk[k] == (seg[k] >> 8) ? g.c64[gi] : 0.0;
+        vb[srec[meta[k] >> 8].y + (meta[k] & 255)] = __fmul_rn(lam[k], inv_rho);
+        __stcg(Y0 + pk[k], rho * xs[k] - lam[k]);
+    }
+    if (tid < 12) xput(pp.part, (tid / 6) * P * 6 + rank * 6 + tid % 6, 0.0, 0xffffffffu);
+    unsigned long long arrivals = (unsigned long long)(P + bar_extra);
+    bool running = grid_barrier(pp.sync, arrivals, m.flags);
+    unsigned nb = 0;
+    auto iteration = [&](int it, auto tested) -> bool {
+        constexpr bool CHK = decltype(tested)::value;
+        const float *Yin = (it & 1) ? Y1 : Y0;
+        float *Yout = (it & 1) ? Y0 : Y1;
+        double acc[6] = {0, 0, 0, 0, 0, 0};
+        for (int k = tid; k < nk; k += nthr) {
+            const int sp = seg[k], us = sp >> 8, cnt = sp & 255;
+            float sigma = 0.0f;
+            constexpr int SEGW = 8;                    // copies' loads in flight, summed in copy order
+            for (int q0 = 0; q0 < cnt; q0 += SEGW) {
+                float v[SEGW];
+#pragma unroll
+                for (int j = 0; j < SEGW; ++j) v[j] = q0 + j < cnt ? __ldcg(Yin + us + q0 + j) : 0.0f;
+#pragma unroll
+                for (int j = 0; j < SEGW; ++j)
+                    if (q0 + j < cnt) sigma += v[j];
+            }
+            float x = (sigma - ct[k]) * rns[cnt];
+            if (x < lo[k]) x = lo[k];
+            if (x > hi[k]) x = hi[k];
+            const int pos = srec[meta[k] >> 8].y + (meta[k] & 255);
+            rb[k] = x;
+            vb[pos] = x + vb[pos];
+            if constexpr (CHK) {
+                const double xd = xrs[k] + (double)x;
+                acc[2] += xd * xd;
+                acc[5] += cobj[k] * xd;
+                U[(size_t)L + pk[k]] = rho * xs[k] - lam[k];       // the u behind this global update, for the solution
+            }
+        }
+        __syncthreads();
+        for (int j = tid; j < nj; j += nthr) {
+            const int itm = items[j];
+            const int4 r = srec[itm >> 8];
+            const int npad = (r.w >> 1) & 0x1ff;
+            tb[j] = dot_col(F + r.x + (itm & 255) * fstride(npad), vb + r.y, npad);
+        }
+        __syncthreads();
+        for (int k = tid; k < nk; k += nthr) {
+            const int4 r = srec[meta[k] >> 8];
+            const int row = meta[k] & 255, f = r.w >> 10, cs = fstride((r.w >> 1) & 0x1ff), pos = r.y + row;
+            const float *Fr = F + r.x + row, *tt = tb + r.z;
+            float y0 = 0.0f, y1 = 0.0f;
+            int c = 0;
+            for (; c + 1 < f; c += 2) {
+                y0 += Fr[c * cs] * tt[c];
+                y1 += Fr[(c + 1) * cs] * tt[c + 1];
+            }
+            if (c < f) y0 += Fr[c * cs] * tt[c];
+            const float x = rb[k], old = xs[k];
+            const float xm = ((r.w & 1) ? (y0 + y1) : vb[pos] - (y0 + y1)) + bt[k];
+            const float res = x - xm;
+            const float l = lam[k] + rho * res, u = rho * xm - l;
+            xs[k] = xm;
+            lam[k] = l;
+            vb[pos] = __fmul_rn(l, inv_rho);
+            __stcg(Yout + pk[k], u);
+            if constexpr (CHK) {
+                const double rd = (double)res, dd = (double)xm - (double)old;
+                const double xsd = xrs[k] + (double)xm, lamd = lrs[k] + (double)l;
+                acc[0] += rd * rd;
+                acc[1] += dd * dd;
+                acc[3] += xsd * xsd;
+                acc[4] += lamd * lamd;
+                U[pk[k]] = u;
+            }
+        }
+        if constexpr (CHK) {
+            if (!test_iteration<false>(m, pp, 0u, acc, it, check_every, P, nb++, st, rho_d)) return false;
+        }
+        if (it + 1 == n_iters) return true;
+        arrivals += (unsigned long long)P;
+        return grid_barrier(pp.sync, arrivals, m.flags);
+    };
+    for (int it = 0; it < n_iters && running; ++it) {
+        if (((it + 1) % check_every) == 0 || it == n_iters - 1) running = iteration(it, std::true_type{});
+        else running = iteration(it, std::false_type{});
+    }
+    for (int k = tid; k < nk; k += nthr) {
+        g.mu[k0 + k] = lam[k];
+        g.ds[k0 + k] = xs[k];
+    }
+    leave(m, st, cond, use_cond);
+}
+
 // The variant of a layout (kernel attributes, occupancy and launch agree on it).
 template <typename T>
 const void *persist_fn(const PersistLayout &lay) {
-    if (!lay.local) return (const void *)k_persist_engine<T>;
+    if (!lay.local) return sizeof(T) == 4 ? (const void *)k_persist_slots : (const void *)k_persist_engine;
     return lay.own       ? (const void *)k_persist_local<T, false, true, false>
            : lay.cluster ? (const void *)k_persist_local<T, true, false, false>
            : lay.two     ? (const void *)k_persist_local<T, false, false, true>
