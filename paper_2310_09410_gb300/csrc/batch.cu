@@ -598,14 +598,15 @@ __global__ void __launch_bounds__(512, 1)
     constexpr int KQ = K < 4 ? K : 4;          // columns per global-update item
     constexpr int NQD = K / KQ;                  // items per global
     constexpr int QS = NQD == 1 ? 0 : NQD == 2 ? 1 : NQD == 4 ? 2 : 3;
-    // global-update items per thread taken together (their loads in flight
-    // together): 1 in FP32 (on the 1024 x 123-bus batch, with the first two
-    // copies' rows in the table entry and c~ in shared memory, 1 to 4 items
-    // gave 12.89, 12.97, 13.30 and 12.98 ms per launch of 2000 iterations;
-    // with the copy rows looked up in a second table and c~ read from L2, 2
-    // had been fastest: more items cost predicated instructions and
-    // registers the rest of the iteration needs), 4 for FP64 rows of 4
-    constexpr int GB = (sizeof(T) == 8 && KQ == 4) ? 4 : 1;
+    // later copies' rows of a global-update item in flight together: 4, 2 for FP64
+    // rows of four, whose registers (with four items per thread and four rows
+    // 224 bytes of a thread spilled) the rest of the iteration needs.  us per
+    // FP64 iteration, four items and four rows / one item and one row / one and
+    // two: 5, 13, 34 and 123 buses, 400 instances 11.2, 16.1, 21.4 and 90.4 / 10.0,
+    // 15.3, 21.2 and 86.5 / 9.9, 16.0, 21.0 and 86.3; 1024 instances of 34 and 123
+    // 35.5 and 180 / 35.8 and 173 / 35.6 and 173.  One item per thread at a time
+    // in FP32 too (2 to 4 were no faster).
+    constexpr int CB = (sizeof(T) == 8 && KQ == 4) ? 2 : 4;
     extern __shared__ __align__(16) unsigned char smraw[];
     T *Fsm = reinterpret_cast<T *>(smraw);
     const T *Fs = FG ? a.Fpk : Fsm;
@@ -710,95 +711,62 @@ __global__ void __launch_bounds__(512, 1)
         // its columns: sum of u over the copies, shift by c~ (bounded globals,
         // whose table entry names their bounded index; elsewhere c~ = 0),
         // 1 / N, clip to rho (bounds - x_ref), and rho x stored into every
-        // copy's slot; GB items per thread
+        // copy's slot
         // (items of many copies come first; the last round, when it is not
         // full, goes to the last threads, which had none of those)
-        auto item_of = [&](int base) { return base + (base + nthr > GQ ? nthr - 1 - tid : tid); };
-        for (int b0 = 0; b0 < GQ; b0 += GB * nthr) {
-            // the GB items of this thread advance stage by stage, so that the
-            // loads of one stage are in flight together: the table entries
-            // (with the first two copies' rows), their u; further copies
-            // (vertices of degree > 1) one by one; then the update
-            RowK<T, KQ> sum[GB];
-            int4 gtj[GB];
-            int row0[GB], row1[GB];
+        for (int b0 = 0; b0 < GQ; b0 += nthr) {
+            const int item = b0 + (b0 + nthr > GQ ? nthr - 1 - tid : tid);
+            if (item >= GQ) continue;
+            const int h = item & (NQD - 1);
+            const int4 gt = gts[item >> QS];
+            const int cnt = gt.z & 0xff;                      // (every global has a copy)
+            const int row0 = gt.x + h * KQ, row1 = gt.y + h * KQ;
+            const int st0 = (gt.z >> 8) - 2;                  // usg[st0 + q]: copy q >= 2
+            RowK<T, KQ> sum;
+            load_row<T, KQ, false>(sum, us + row0);
+            if (cnt > 1) {
+                RowK<T, KQ> u1;
+                load_row<T, KQ, false>(u1, us + row1);
 #pragma unroll
-            for (int j = 0; j < GB; ++j) {
-                const int item = item_of(b0 + j * nthr);
-                gtj[j] = make_int4(0, 0, 0, -1);
-                if (item < GQ) gtj[j] = gts[item >> QS];
-                const int hq = (item & (NQD - 1)) * KQ;
-                row0[j] = gtj[j].x + hq;
-                row1[j] = gtj[j].y + hq;
+                for (int k = 0; k < KQ; ++k) sum.v[k] += u1.v[k];
             }
+            for (int q = 2; q < cnt; q += CB) {               // CB copies' loads in flight
+                int rr[CB];
 #pragma unroll
-            for (int j = 0; j < GB; ++j) {
-                const int cnt = gtj[j].z & 0xff;
-                if constexpr (sizeof(T) == 8) {          // no add of the first copy to zero
-                    if (cnt > 0) load_row<T, KQ, false>(sum[j], us + row0[j]);
-                } else {
+                for (int c = 0; c < CB; ++c) rr[c] = q + c < cnt ? usg[st0 + q + c] : 0;
+                RowK<T, KQ> uq[CB];
 #pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] = T(0);
-                    if (cnt > 0) {
-                        RowK<T, KQ> u0;
-                        load_row<T, KQ, false>(u0, us + row0[j]);
+                for (int c = 0; c < CB; ++c)
+                    if (q + c < cnt) load_row<T, KQ, false>(uq[c], us + rr[c] + h * KQ);
 #pragma unroll
-                        for (int k = 0; k < KQ; ++k) sum[j].v[k] += u0.v[k];
-                    }
-                }
-                if (cnt > 1) {
-                    RowK<T, KQ> u1;
-                    load_row<T, KQ, false>(u1, us + row1[j]);
+                for (int c = 0; c < CB; ++c)
+                    if (q + c < cnt)
 #pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] += u1.v[k];
-                }
+                        for (int k = 0; k < KQ; ++k) sum.v[k] += uq[c].v[k];
             }
+            const T rcp = rcs[cnt];
+            if (gt.w >= 0) {
+                RowK<T, KQ> lo, hi, cr;
+                load_row<T, KQ, false>(cr, bnd + (gt.w * 3 + 2) * K + h * KQ);
+                load_row<T, KQ, false>(lo, bnd + (gt.w * 3) * K + h * KQ);
+                load_row<T, KQ, false>(hi, bnd + (gt.w * 3 + 1) * K + h * KQ);
 #pragma unroll
-            for (int j = 0; j < GB; ++j) {
-                const int item = item_of(b0 + j * nthr);
-                if (item >= GQ) continue;
-                const int h = item & (NQD - 1);
-                const int4 gt = gtj[j];
-                const int cnt = gt.z & 0xff;
-                const int st0 = (gt.z >> 8) - 2;              // usg[st0 + q]: copy q >= 2
-                for (int q = 2; q < cnt; q += 4) {            // four copies' loads in flight
-                    int rr[4];
+                for (int k = 0; k < KQ; ++k) sum.v[k] = (sum.v[k] - cr.v[k]) * rcp;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) rr[c] = q + c < cnt ? usg[st0 + q + c] : 0;
-                    RowK<T, KQ> uq[4];
+                for (int k = 0; k < KQ; ++k) sum.v[k] = clampT(sum.v[k], lo.v[k], hi.v[k]);
+            } else {
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (q + c < cnt) load_row<T, KQ, false>(uq[c], us + rr[c] + h * KQ);
+                for (int k = 0; k < KQ; ++k) sum.v[k] *= rcp;
+            }
+            store_row<T, KQ>(us + row0, sum);
+            if (cnt > 1) store_row<T, KQ>(us + row1, sum);
+            for (int q = 2; q < cnt; q += CB) {
+                int rr[CB];
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (q + c < cnt)
+                for (int c = 0; c < CB; ++c) rr[c] = q + c < cnt ? usg[st0 + q + c] : 0;
 #pragma unroll
-                            for (int k = 0; k < KQ; ++k) sum[j].v[k] += uq[c].v[k];
-                }
-                const T rcp = rcs[cnt];
-                if (gt.w >= 0) {
-                    RowK<T, KQ> lo, hi, cr;
-                    load_row<T, KQ, false>(cr, bnd + (gt.w * 3 + 2) * K + h * KQ);
-                    load_row<T, KQ, false>(lo, bnd + (gt.w * 3) * K + h * KQ);
-                    load_row<T, KQ, false>(hi, bnd + (gt.w * 3 + 1) * K + h * KQ);
-#pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] = (sum[j].v[k] - cr.v[k]) * rcp;
-#pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] = clampT(sum[j].v[k], lo.v[k], hi.v[k]);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < KQ; ++k) sum[j].v[k] *= rcp;
-                }
-                if (cnt > 0) store_row<T, KQ>(us + row0[j], sum[j]);
-                if (cnt > 1) store_row<T, KQ>(us + row1[j], sum[j]);
-                for (int q = 2; q < cnt; q += 4) {
-                    int rr[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) rr[c] = q + c < cnt ? usg[st0 + q + c] : 0;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        if (q + c < cnt) store_row<T, KQ>(us + rr[c] + h * KQ, sum[j]);
-                }
+                for (int c = 0; c < CB; ++c)
+                    if (q + c < cnt) store_row<T, KQ>(us + rr[c] + h * KQ, sum);
             }
         }
         __syncthreads();
