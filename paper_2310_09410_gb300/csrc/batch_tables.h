@@ -254,34 +254,34 @@ inline bool build_global_tables(int G, const std::vector<int> &gstart, const std
 // entries allow, the smallest first row first.  (The order of the entries is
 // free: gperm and gx list the globals of the test on their own.)
 inline void sort_global_items(GlobalTables *t, int K, int group) {
+    struct Item { int kind, row, at, bank0, bank1; };        // bank1 `group`: no second copy
     const std::vector<int> was(t->gtab);
-    auto entry = [&](int j) { return &was[4 * (size_t)j]; };
-    std::vector<int> ord(t->Gs);
-    std::iota(ord.begin(), ord.end(), 0);
-    auto kind = [&](int j) { return std::make_pair(-(entry(j)[2] & 255), entry(j)[3] < 0); };
-    std::sort(ord.begin(), ord.end(), [&](int a, int b) {
-        return std::make_tuple(kind(a), entry(a)[0]) < std::make_tuple(kind(b), entry(b)[0]);
+    std::vector<Item> ord(t->Gs);
+    for (int j = 0; j < t->Gs; ++j) {
+        const int *e = &was[4 * (size_t)j], cnt = e[2] & 255;
+        ord[j] = {2 * (255 - cnt) + (e[3] < 0), e[0], j, e[0] / K % group, cnt > 1 ? e[1] / K % group : group};
+    }
+    std::sort(ord.begin(), ord.end(), [](const Item &a, const Item &b) {
+        return std::make_tuple(a.kind, a.row, a.at) < std::make_tuple(b.kind, b.row, b.at);
     });
-    std::vector<char> bank0(group), bank1(group);
+    std::vector<int> taken0(group), taken1(group + 1);
     for (int j = 0; j < t->Gs; ++j) {
         if (j % group == 0) {
-            std::fill(bank0.begin(), bank0.end(), 0);
-            std::fill(bank1.begin(), bank1.end(), 0);
+            std::fill(taken0.begin(), taken0.end(), 0);
+            std::fill(taken1.begin(), taken1.end(), 0);
         }
-        auto clashes = [&](int i) {
-            const int *e = entry(ord[i]);
-            return bank0[e[0] / K % group] + ((e[2] & 255) > 1 ? bank1[e[1] / K % group] : 0);
-        };
-        int best = j;
-        for (int i = j; i < t->Gs && i < j + 256 && kind(ord[i]) == kind(ord[j]); ++i) {
-            if (clashes(i) < clashes(best)) best = i;
-            if (clashes(best) == 0) break;
+        auto clashes = [&](int i) { return taken0[ord[i].bank0] + taken1[ord[i].bank1]; };
+        int best = j, fewest = clashes(j);
+        for (int i = j + 1; fewest > 0 && i < t->Gs && i < j + 256 && ord[i].kind == ord[j].kind; ++i) {
+            const int c = clashes(i);
+            if (c < fewest) { best = i; fewest = c; }
         }
-        std::rotate(ord.begin() + j, ord.begin() + best, ord.begin() + best + 1);
-        const int *e = entry(ord[j]);
-        bank0[e[0] / K % group] = 1;
-        if ((e[2] & 255) > 1) bank1[e[1] / K % group] = 1;
-        for (int q = 0; q < 4; ++q) t->gtab[4 * (size_t)j + q] = e[q];
+        const Item it = ord[best];
+        for (int i = best; i > j; --i) ord[i] = ord[i - 1];
+        ord[j] = it;
+        taken0[it.bank0] = 1;
+        taken1[it.bank1] = it.bank1 < group ? 1 : 0;
+        for (int q = 0; q < 4; ++q) t->gtab[4 * (size_t)j + q] = was[4 * (size_t)it.at + q];
     }
 }
 
