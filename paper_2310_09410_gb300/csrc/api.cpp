@@ -51,9 +51,9 @@ template <typename T>
 int launch_cluster_engine(const IterArgs<T> &g, const ClusterLayout &lay, const int *pr, T *u_glob,
                           int n_iters, int check_every, DevStatus *st, double rho,
                           cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
-template <typename T> int cluster_occupancy(const ClusterLayout &lay);
+template <typename T> int cluster_occupancy(const ClusterLayout &lay, cudaStream_t s);
 template <typename T> int prepare_persist_engine(const PersistLayout &lay);
-template <typename T> long long persist_resident(const PersistLayout &lay, int n_sm);
+template <typename T> long long persist_resident(const PersistLayout &lay, int n_sm, cudaStream_t s);
 template <typename T> size_t persist_exchange_bytes(long long n);
 template <typename T>
 int launch_persist_engine(const IterArgs<T> &g, const PersistLayout &lay, const PersistPtrs &pp, T *U,
@@ -64,7 +64,7 @@ template <typename T>
 int launch_warp_engine(const IterArgs<T> &g, const WarpLayout &lay, const int *pr, T *u_glob, int n_iters,
                        int check_every, DevStatus *st, double rho, cudaGraphConditionalHandle cond, int use_cond,
                        cudaStream_t s);
-template <typename T> int warp_engine_occupancy(const WarpLayout &lay);
+template <typename T> int warp_engine_occupancy(const WarpLayout &lay, cudaStream_t s);
 template <typename T>
 void launch_make_u(int L, const int *pk, const T *ds, const T *mu, T rho, T *u, const DevStatus *st,
                    cudaStream_t s);
@@ -715,7 +715,7 @@ static int build_cluster_plan(opf_handle *h, ClusterPlan *cp, int P) {
     CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     if ((long long)c.bytes + 4096 > optin) return OPF_OK;              // does not fit: plan not ok
     if (prepare_cluster_engine<T>(c.bytes, P)) { cudaGetLastError(); return OPF_OK; }
-    if (cluster_occupancy<T>(c) < 1) { cudaGetLastError(); return OPF_OK; }
+    if (cluster_occupancy<T>(c, h->stream) < 1) { cudaGetLastError(); return OPF_OK; }
     CUDA_TRY(cudaMemcpyAsync(cp->d_pr, pr.data(), pr.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(cudaMemcpyAsync(cp->d_srec, srec.data(), srec.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream));
     if (!items.empty())
@@ -1122,7 +1122,7 @@ static int build_persist_plan(opf_handle *h, PersistPlan *pp, int P, int n_sm, b
     c.bytes = (unsigned)off;
     if ((long long)off > optin) return OPF_OK;
     if (prepare_persist_engine<T>(c)) { cudaGetLastError(); return OPF_OK; }
-    if (persist_resident<T>(c, n_sm) < P) { cudaGetLastError(); return OPF_OK; }
+    if (persist_resident<T>(c, n_sm, h->stream) < P) { cudaGetLastError(); return OPF_OK; }
     if (!wide.empty()) {
         if (!pp->d_wide) TRY(dalloc(h, &pp->d_wide, 2 * (size_t)kPersistMaxP));
         CUDA_TRY(cudaMemcpyAsync(pp->d_wide, wide.data(), wide.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
@@ -1185,8 +1185,11 @@ static int get_one_cluster_plan(opf_handle *h, PersistPlan *pp) {
     int warps = 0;
     for (int n : warp_parts(h, sizeof(T) == 4, 0)) warps += n;
     if (warps > 16 * (sizeof(T) == 4 ? kWarpEngineWarps : kWarpEngineWarps64)) return OPF_OK;
-    const int per = sizeof(T) == 4 ? 80 : 24, most = sizeof(T) == 4 ? 16 : 12;
-    return build_persist_plan<T>(h, pp, std::min(most, (h->L + per - 1) / per), 0, true, true);
+    const int per = sizeof(T) == 4 ? 80 : 24, most = sizeof(T) == 4 ? 16 : 12, P = std::min(most, (h->L + per - 1) / per);
+    TRY(build_persist_plan<T>(h, pp, P, 0, true, true));
+    // (an SM partition of any size holds no cluster of more than 8)
+    if (!pp->ok && P > 8) TRY(build_persist_plan<T>(h, pp, 8, 0, true, true));
+    return OPF_OK;
 }
 
 // Owner form: at most a CTA per subsystem; FP64 a CTA per SM of the stream (its
@@ -1367,7 +1370,7 @@ static int build_warp_plan(opf_handle *h, WarpPlan &wp, int req_P) {
     CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device));
     if ((long long)c.bytes + 4096 > optin) return OPF_OK;
     if (prepare_warp_engine<T>(c.bytes)) { cudaGetLastError(); return OPF_OK; }
-    if (warp_engine_occupancy<T>(c) < 1) { cudaGetLastError(); return OPF_OK; }
+    if (warp_engine_occupancy<T>(c, h->stream) < 1) { cudaGetLastError(); return OPF_OK; }
     if ((size_t)wdd.size() > (size_t)h->L * 16 || wrep.size() > (size_t)h->L) return OPF_OK;
     CUDA_TRY(cudaMemcpyAsync(wp.d_pr, pr.data(), pr.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(cudaMemcpyAsync(wp.d_wmap, wmap.data(), wmap.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));

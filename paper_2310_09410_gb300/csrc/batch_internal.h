@@ -94,7 +94,7 @@ namespace opf {
 // Lane engine (lane.cu): kernel attributes for clusters of C CTAs, clusters
 // the device holds at once, a launch of `tiles` clusters, factor packing.
 int lane_engine_prepare(int C, unsigned bytes);
-int lane_engine_max_clusters(int C, int threads, unsigned bytes);
+int lane_engine_max_clusters(int C, int threads, unsigned bytes, cudaStream_t s);
 int lane_engine_ctas_per_sm(int threads, unsigned bytes);
 int lane_engine_launch(const LaneArgs &a, int tiles, int threads, unsigned bytes, int n_iters, int check_every,
                        cudaStream_t s);

@@ -1180,12 +1180,14 @@ int launch_warp_engine(const IterArgs<T> &g, const WarpLayout &lay, const int *p
     return e == cudaSuccess ? 0 : -1;
 }
 
+// Clusters of this plan that the stream's SMs hold at once.  (The stream says
+// whose SMs: a partition's hold far fewer, and none of more than 8 CTAs.)
 template <typename T>
-int warp_engine_occupancy(const WarpLayout &lay) {
+int warp_engine_occupancy(const WarpLayout &lay, cudaStream_t s) {
     if (lay.warps < 1 || lay.warps > WE_WARPS) return 0;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_cluster_cfg(&cfg, attr, lay.P, 32 * lay.warps, lay.bytes, 0);
+    fill_cluster_cfg(&cfg, attr, lay.P, 32 * lay.warps, lay.bytes, s);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k_warp_engine<T>, &cfg) != cudaSuccess) return 0;
     return n;
@@ -1197,8 +1199,8 @@ template int launch_warp_engine<float>(const IterArgs<float> &, const WarpLayout
                                        DevStatus *, double, cudaGraphConditionalHandle, int, cudaStream_t);
 template int launch_warp_engine<double>(const IterArgs<double> &, const WarpLayout &, const int *, double *, int,
                                         int, DevStatus *, double, cudaGraphConditionalHandle, int, cudaStream_t);
-template int warp_engine_occupancy<float>(const WarpLayout &);
-template int warp_engine_occupancy<double>(const WarpLayout &);
+template int warp_engine_occupancy<float>(const WarpLayout &, cudaStream_t);
+template int warp_engine_occupancy<double>(const WarpLayout &, cudaStream_t);
 
 // ============================================================ small kernels
 // u[pk[k]] = rho * ds[k] - mu[k]
@@ -1426,15 +1428,16 @@ int launch_cluster_engine(const IterArgs<T> &g, const ClusterLayout &lay, const 
     return e == cudaSuccess ? 0 : -1;
 }
 
-// Largest cluster of P CTAs with `bytes` of shared memory each that can be
-// resident (0 if none).
+// Clusters of P CTAs with `bytes` of shared memory each that can be resident on
+// the stream's SMs (0 if none).
 template <typename T>
-int cluster_occupancy(const ClusterLayout &lay) {
+int cluster_occupancy(const ClusterLayout &lay, cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(lay.P, 1, 1);
     cfg.blockDim = dim3(lay.threads, 1, 1);
     cfg.dynamicSmemBytes = lay.bytes;
+    cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = lay.P;
@@ -1497,7 +1500,7 @@ void launch_recenter(int L, int G, int S, const int *gk, const double *xr_old, c
     template int launch_cluster_engine<T>(const IterArgs<T> &, const ClusterLayout &, const int *, T *,\
                                           int, int, DevStatus *, double, cudaGraphConditionalHandle,  \
                                           int, cudaStream_t);                                         \
-    template int cluster_occupancy<T>(const ClusterLayout &);                                         \
+    template int cluster_occupancy<T>(const ClusterLayout &, cudaStream_t);                           \
     template void launch_make_u<T>(int, const int *, const T *, const T *, T, T *, const DevStatus *, \
                                    cudaStream_t);                                                     \
     template int launch_global_x<T>(int, const int2 *, const T *, const T *, const T *, const T *,    \

@@ -531,11 +531,11 @@ static void lane_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int 
     cfg.numAttrs = 1;
 }
 
-// Clusters of C CTAs of this shape that the device holds at once (0: none).
-int lane_engine_max_clusters(int C, int threads, unsigned bytes) {
+// Clusters of C CTAs of this shape that the stream's SMs hold at once (0: none).
+int lane_engine_max_clusters(int C, int threads, unsigned bytes, cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    lane_config(cfg, attr, 1, C, threads, bytes, nullptr);
+    lane_config(cfg, attr, 1, C, threads, bytes, s);
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k_lane_engine, &cfg) != cudaSuccess) return 0;
     return n;

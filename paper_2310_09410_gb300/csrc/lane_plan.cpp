@@ -332,7 +332,7 @@ int build_lane_plan(opf_batch *b, BPlan *p, int WG, int maxC) {
         set_last_error("lane plan: the engine needs an SM to itself");
         return OPF_E_CAPACITY;
     }
-    if (lane_engine_max_clusters(C, p->threads, p->bytes) < 1) {
+    if (lane_engine_max_clusters(C, p->threads, p->bytes, b->h->stream) < 1) {
         set_last_error("lane plan: a cluster of this shape does not fit the device");
         return OPF_E_CAPACITY;
     }

@@ -1365,14 +1365,15 @@ int prepare_persist_engine(const PersistLayout &lay) {
     return 0;
 }
 
-// CTAs that can be resident on n_sm SMs (a cluster: its own P, or 0).
+// CTAs that can be resident on n_sm SMs (a cluster: its own P when the stream's
+// SMs hold one, else 0).
 template <typename T>
-long long persist_resident(const PersistLayout &lay, int n_sm) {
+long long persist_resident(const PersistLayout &lay, int n_sm, cudaStream_t s) {
     int n = 0;
     if (lay.cluster) {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[1];
-        fill_cfg(lay, &cfg, attr, 0);
+        fill_cfg(lay, &cfg, attr, s);
         return cudaOccupancyMaxActiveClusters(&n, persist_fn<T>(lay), &cfg) == cudaSuccess && n > 0 ? lay.P : 0;
     }
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, persist_fn<T>(lay), lay.threads, lay.bytes) != cudaSuccess)
@@ -1402,7 +1403,8 @@ int launch_persist_engine(const IterArgs<T> &g, const PersistLayout &lay, const 
 
 #define OPF_PERSIST_INST(T)                                                                                   \
     template int prepare_persist_engine<T>(const PersistLayout &);                                                        \
-    template long long persist_resident<T>(const PersistLayout &, int);   template size_t persist_exchange_bytes<T>(long long);                                                        \
+    template long long persist_resident<T>(const PersistLayout &, int, cudaStream_t);                       \
+    template size_t persist_exchange_bytes<T>(long long);                                                   \
     template int launch_persist_engine<T>(const IterArgs<T> &, const PersistLayout &, const PersistPtrs &,  \
                                           T *, int, int, int, DevStatus *, double,                            \
                                           cudaGraphConditionalHandle, int, cudaStream_t);

@@ -214,7 +214,7 @@ struct CtxInfo {
 std::mutex g_mu;
 std::map<unsigned long long, CtxInfo> g_ctx;
 
-bool holds_cluster() {
+bool holds_cluster(cudaStream_t s) {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cudaLaunchAttribute attr[1];
@@ -223,6 +223,7 @@ bool holds_cluster() {
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(kCluster);
     cfg.blockDim = dim3(kClusterThreads);
+    cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
@@ -280,7 +281,7 @@ extern "C" int opf_global_update_static(int32_t n, const int32_t *seg_off, const
             if (d.push(ctx) != CUDA_SUCCESS) return fail(OPF_E_CUDA, "cuCtxPushCurrent failed");
             void *p = nullptr;
             cudaError_t e = cudaGetSymbolAddress(&p, g_static_partials);
-            if (e == cudaSuccess) info.cluster = holds_cluster();
+            if (e == cudaSuccess) info.cluster = holds_cluster(s);
             CUcontext popped = nullptr;
             d.pop(&popped);
             if (e != cudaSuccess || !p)
