@@ -865,7 +865,7 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
     std::vector<int> two = cluster ? warp_parts(h, true, 0) : std::vector<int>(S, 1);
     std::vector<int> halves(S, 0);
     const int P1 = P + 1;
-    std::vector<int> pr(7 * P1, 0), items, meta;
+    std::vector<int> pr(6 * P1, 0), items, meta;
     auto PR = [&](int field, int p) -> int & { return pr[field * P1 + p]; };
     // per part: factors staged with column stride npad (+ 4 when npad % 8 == 0)
     std::vector<int4> srec(S);
@@ -893,16 +893,14 @@ static int build_persist_tables(opf_handle *h, int P, bool local, bool cluster, 
             t->f.push_back(h->h_sf[d]);
             fmax = std::max(fmax, h->h_sf[d]);
         }
-        t->nj.push_back((int)j);
-        t->nk.push_back(parts.k0[p + 1] - parts.k0[p]);
         t->rows32 = t->rows32 && fmax <= 32;
         t->mpair = std::max(t->mpair, ((2 * nbig + 31) & ~31LL) + j - nbig);
         PR(0, p + 1) = parts.k0[p + 1];
         PR(1, p + 1) = parts.s0[p + 1];
         PR(2, p + 1) = (int)items.size();
-        PR(4, p + 1) = PR(4, p) + (int)v;
-        PR(5, p + 1) = parts.r0[p + 1];
-        PR(6, p + 1) = parts.l0[p + 1];
+        PR(3, p + 1) = PR(3, p) + (int)v;
+        PR(4, p + 1) = parts.r0[p + 1];
+        PR(5, p + 1) = parts.l0[p + 1];
         t->mf = std::max(t->mf, f);
         t->mv = std::max(t->mv, v);
         t->mj = std::max(t->mj, j);

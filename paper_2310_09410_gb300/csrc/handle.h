@@ -36,16 +36,15 @@ struct PersistTables {
     // rounded up to 4 per subsystem), slots, vector rows, remote entries,
     // lists, destinations
     long long mf = 0, ms = 0, mj = 0, mt = 0, mk = 0, mv = 0, mr = 0, ml = 0, md = 0;
-    // per part the columns and slots, and the subsystems' sizes (FP64 lane splits);
-    // most threads of the FP32 cluster form's columns; its factors fit registers
-    std::vector<int> nj, nk;
+    // the subsystems' sizes (FP64 lane splits); most threads of the FP32 cluster
+    // form's columns; its factors fit registers
     std::vector<int> s0, npad, n, f;     // parts' first subsystem, and per subsystem in part order
     long long mog = 0, moc = 0;          // owner form: most globals and copies that a part owns
     long long mpair = 0, remote = 0;     // remote: entries read from other parts, over all parts
     bool rows32 = true;
     bool fits = true;            // indices and counts fit their fields
     int *mem = nullptr;          // one allocation: the arrays below
-    int *pr = nullptr, *items = nullptr, *meta = nullptr;   // ranges, 7 x (P + 1); per column; per slot
+    int *pr = nullptr, *items = nullptr, *meta = nullptr;   // ranges, 6 x (P + 1); per column; per slot
     int *sub = nullptr, *slot = nullptr, *seg = nullptr, *out = nullptr, *rem = nullptr;
     uint4 *list = nullptr;
     int *dst = nullptr, *dr = nullptr, *dseg = nullptr, *halves = nullptr, *g0 = nullptr, *gfirst = nullptr;

@@ -170,7 +170,7 @@ struct PersistLayout {
 
 // Device arrays of a persistent grid engine plan.
 struct PersistPtrs {
-    const int *pr;                 // part ranges, 7 fields x (P + 1)
+    const int *pr;                 // part ranges, 6 fields x (P + 1)
     unsigned long long *part;      // Sec. III-C partial sums, stamped FP64 words, 2 x P x 6
     unsigned long long *sync;      // grid barrier counter
     unsigned long long *xu;        // exchange of u: two buffers of L stamped entries

@@ -210,7 +210,7 @@ __device__ __forceinline__ double dot_rows(const double *f, const double *v, int
 __host__ __device__ __forceinline__ int fstride(int npad) { return npad + ((npad & 7) == 0 ? 4 : 0); }
 
 // Part ranges: pr[field * (P + 1) + rank].
-enum { GR_K = 0, GR_S, GR_J, GR_F, GR_V, GR_R, GR_L, GR_NFIELDS };
+enum { GR_K = 0, GR_S, GR_J, GR_V, GR_R, GR_L };
 
 // ---- exchange entries: value and iteration number in one word
 using u64 = unsigned long long;
