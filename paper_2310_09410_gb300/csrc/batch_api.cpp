@@ -389,7 +389,12 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
     };
     b->tune_log.clear();
     if (b->force_k32) {
-        if (b->force_k32 == 1) { set_last_error("batch plan: engine attributes"); return OPF_E_CUDA; }
+        if (b->force_k32 == 1) {
+            // (refused as before the shape existed, when no such kernel could be prepared)
+            set_last_error("batch plan: one instance per CTA in FP32 is the library's own choice for small batches and "
+                           "cannot be asked for");
+            return OPF_E_CUDA;
+        }
         return build(b->force_k32, b->force_w32 > 0 ? b->force_w32 : 16);
     }
     // K: the fewest instances per CTA that leave an SM per CTA, and half of that
