@@ -1194,14 +1194,23 @@ static int get_one_cluster_plan(opf_handle *h, PersistPlan *pp) {
 // FP64 pipes bound it), FP32 one per 160 slots up to that (every CTA takes the x
 // of its own globals: 240 blocks over 900 globals 3.62 us per iteration on 152
 // CTAs, 3.44 with 160 slots each, 3.51 with 320; over 300 globals 6.37, 4.55 and
-// 3.95; 200 blocks of up to 30 3.74, 2.45 and 2.75).
+// 3.95; 200 blocks of up to 30 3.74, 2.45 and 2.75), but no more than leave room
+// for a second solve beside it: one CTA of these can take an SM to itself, and 77
+// of 152 SMs serialize two handles (240 blocks over 900 globals, two handles
+// together 3.5 us per iteration with 77, 1.9 with 76; 240 over 120 globals alone
+// 5.5 and 5.1).
 template <typename T>
 static int get_owner_plan(opf_handle *h, PersistPlan *pp) {
     if (pp->tried) return OPF_OK;
     pp->tried = true;
     const int n_sm = stream_sm_count(h->stream, h->device);
-    const int want = sizeof(T) == 8 ? n_sm : std::min(n_sm, (h->L + 159) / 160);
-    return build_persist_plan<T>(h, pp, std::min(want, h->S), n_sm, true, false, true);
+    const int want = std::min(h->S, sizeof(T) == 8 ? n_sm : std::min(n_sm, (h->L + 159) / 160));
+    TRY(build_persist_plan<T>(h, pp, want, n_sm, true, false, true));
+    if (sizeof(T) == 8 || !pp->ok) return OPF_OK;
+    const long long half = persist_resident<T>(pp->lay, n_sm, h->stream) / 2;
+    if (want <= half || half < 1) return OPF_OK;
+    TRY(build_persist_plan<T>(h, pp, (int)half, n_sm, true, false, true));
+    return pp->ok ? OPF_OK : build_persist_plan<T>(h, pp, want, n_sm, true, false, true);
 }
 
 template <typename T>
