@@ -375,16 +375,9 @@ __device__ __forceinline__ void batch_task(const BatchTask &tk, const double *Fs
 // loop over them took 90 cycles per level, twice the shuffle and the add);
 // every tensor-memory load of a task before one wait; a slot array free of
 // bank conflicts at each K; global-update items sorted so that a warp's lanes
-// take the same branches.  us per iteration with a test every 50, before and
-// now: 123 buses, 20 instances (K = 2) 4.11 -> 2.97; 34 buses, 201 instances
-// (K = 2) 2.47 -> 1.71; 123 buses, 1024 instances (K = 8) 6.57 -> 6.16, of which
-// the tests take 0.42 -> 0.26.  Single parts: the plan's chunks per lane
-// (task_chunks) 3.37 -> 3.10 and 1.98 -> 1.71, a lane's places in the slot array
-// kept instead of recomputed 6.39 -> 6.29, the items' rows on distinct banks
-// (sort_global_items) 6.29 -> 6.16 and 3.08 -> 2.97.  Tried and slower: four rows per step
-// (K = 8 6.19 -> 7.4), 20 or 24 warps (6.24 -> 6.46, 7.42), the next rows'
-// factors prefetched (spills), two chains per row (K = 2 3.19 -> 3.35), whole rows of 8 columns
-// per global-update item (6.29 -> 7.63: two-way conflicts).
+// take the same branches.  us per iteration with a test every 100, against scalar
+// multiply-adds: 123 buses, 40 instances (K = 2) 3.80 -> 2.52; 34 buses, 200
+// instances (K = 2) 2.26 -> 1.59; 123 buses, 1024 instances (K = 8) 6.53 -> 6.14.
 using u64 = unsigned long long;
 __device__ __forceinline__ u64 pk(float a, float b) {
     u64 r;

@@ -416,7 +416,11 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
     BCUDA(cudaMemcpyAsync(b->d_st_save, b->d_st, b->n * sizeof(DevStatus), cudaMemcpyDeviceToDevice, h->stream));
     double best = 1e300;
     int bk = 0, bw = 0;
-    const int iters = 2 * std::max(k, 2);
+    // 100 iterations at least, with the solve's tests: 20 iterations without tests
+    // take 35 to 41 us, the events tell 2 us, and tests cost the shapes unlike
+    // (tests every 10, 40 buses, 21 instances: 16 warps picked over 8 by chance,
+    // a pass 7.7 instead of 7.3 ms)
+    const int iters = 2 * std::max(k, 50);
     int lk = 0, lw = 0;      // the shape p holds
     auto timed = [&](int K, int W) -> int {
         lk = 0;
@@ -431,10 +435,10 @@ int ensure_plan(opf_batch *b, bool dbl, double rho, int k) {
                            h->d_F64, h->d_gk, p.d_sch, b->d_bbar, (float *)p.bt, (float *)p.ds, (float *)p.mu,
                            (float *)p.lref, (float *)p.xsr, h->stream);
         auto run = [&](int n_it) {
-            batch_engine_launch<float>(engine_args<float>(b, p, rho), p.nq, false, p.C, p.threads, p.bytes, n_it, 0,
+            batch_engine_launch<float>(engine_args<float>(b, p, rho), p.nq, false, p.C, p.threads, p.bytes, n_it, k,
                                        h->stream);
         };
-        run(4);   // warm-up
+        run(1);   // warm-up
         BCUDA(cudaEventRecord(b->ev[0], h->stream));
         run(iters);
         BCUDA(cudaEventRecord(b->ev[1], h->stream));

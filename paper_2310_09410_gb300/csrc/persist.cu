@@ -70,22 +70,10 @@
 // the warp engine's order of every sum (the iterates are its, bit for bit) with
 // the factor rows in registers, columns on one lane each and those of more than
 // 32 rows on two.  FP64 (every form) spreads the long columns and rows over lanes.
-// Measured per iteration with a test every 50, grid form, before (every copy of
-// u through L2 behind a grid barrier, parts of the size-sorted order, FP64 sums
-// of the test by butterflies) and now: 8500 buses FP32 4.23 -> 3.0 us, FP64
-// 10.5 -> 7.3 us; 123 buses FP64 4.7 -> 2.8 us.  Of the 8500-bus steps: stamped
-// entries alone, all copies through L2, 6.1 us FP32 (every slot polls, and the
-// polls fill the L1) and 8.4 us FP64; local parts 3.6 and 8.8 us; the copies'
-// places in registers, loops unrolled, long warps of co-resident CTAs on
-// different sub-partitions, and the test's sums spread over lanes and warps
-// 3.1 and 7.7 us (a test cost some 40 us, now 12); FP64 with the longest columns
-// and rows on several lanes in warps of their own 7.3.
-// One-cluster form against the warp engine: FP32 13 / 34 / 123 buses 0.92 /
-// 1.00 / 1.11 us against 1.71 / 1.80 / 2.31; FP64 13 / 34 buses 1.93 / 2.07
-// against 2.92 / 3.03.  Its FP32 phases before the last changes (123 buses,
-// 1.91 us): column products 1950 of 3700 cycles (scalar reads of strided
-// columns, 8-way bank conflicts; 16-byte reads, all of a column's in flight),
-// local update 940 (the row from registers, the products as 16-byte reads).
+// us per iteration with a test every 50: 8500 buses FP32 4.4 -> 3.1, FP64 10.7 ->
+// 7.3, 123 buses FP64 4.6 -> 2.6 (before: every copy of u through L2 behind a
+// grid barrier); one cluster against the warp engine, FP32 13 / 34 / 123 buses
+// 1.5 / 1.6 / 2.1 -> 0.93 / 0.93 / 1.06, FP64 13 / 34 buses 2.4 -> 1.8.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
