@@ -76,7 +76,7 @@ FP32_LANES = 128
 # DRAM bytes per launch of the dominant kernels, copied from the ncu captures
 # summarised in profiles/ (a copied constant, labelled so in the line; None
 # once the kernel has changed since the capture).
-BATCH_ENGINE_TRAFFIC_PER_LAUNCH = 76636928 + 2526208
+BATCH_ENGINE_TRAFFIC_PER_LAUNCH = 76567808 + 2186240
 BATCH_ENGINE_TRAFFIC_SOURCE = "profiles/k_batch_engine_123bus_x1024.md"
 # Warp instructions per instance-iteration of the batched engine in the
 # shape the autotune picks for the 1024 x 123-bus batch (8 instances per CTA,
@@ -85,7 +85,7 @@ BATCH_ENGINE_TRAFFIC_SOURCE = "profiles/k_batch_engine_123bus_x1024.md"
 # The first value is an earlier capture's (the default of issue_roofline), the
 # second the current kernel's, which the bench lines use.
 BATCH_ENGINE_INST_PER_INSTANCE_ITER = 16.7984e9 / (4000 * 1024)
-BATCH_ENGINE_INST_PER_INSTANCE_ITER_NOW = 14.6856e9 / (4000 * 1024)
+BATCH_ENGINE_INST_PER_INSTANCE_ITER_NOW = 13.9053e9 / (4000 * 1024)
 BATCH_ENGINE_INST_SHAPE = {"k_inst": 8, "warps": 16, "tmem": 1}
 ITERS_PER_LAUNCH = 1000
 
