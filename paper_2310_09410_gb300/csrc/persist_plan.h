@@ -14,6 +14,8 @@
 #include <algorithm>
 #include <functional>
 #include <numeric>
+#include <system_error>
+#include <thread>
 #include <utility>
 #include <vector>
 
@@ -183,46 +185,92 @@ inline void persist_lists(int P, const std::vector<int> &soff, const std::vector
             }
     t.seg.resize(L);
     t.out.assign(L, -1);
-    t.rem.reserve(L / 4);
-    t.list.resize(4 * (size_t)L);
-    size_t used = 0;                             // entries of the lists so far
-    std::vector<int> where(L, -1);               // by first copy: number of the part's list, or below l0[part]
-    for (int q = 0; q < P; ++q) {
-        const int nk = t.k0[q + 1] - t.k0[q], l0 = t.l0[q], r0 = t.r0[q];
-        for (int j = t.k0[q]; j < t.k0[q + 1]; ++j) {
-            const int sp = segp[t.slot[j]], c0 = sp >> 8, cnt = sp & 255;
-            if (cnt == 1) {
-                t.seg[j] = 1;
-                continue;
-            }
-            if (where[c0] < l0) {
-                where[c0] = (int)(used / 8);
-                const size_t end = used + ((cnt + 7) & ~7);
-                if (end > t.list.size()) t.list.resize(2 * end);
-                unsigned short *e = t.list.data() + used, *last = t.list.data() + end;
-                for (int c = c0; c < c0 + cnt; ++c) {
-                    const Place at = place[c];
-                    if (at.part == q) {
-                        *e++ = (unsigned short)at.at;
-                    } else {
-                        *e++ = (unsigned short)(nk + (int)t.rem.size() - r0);
-                        t.rem.push_back(c);
-                        t.out[t.k0[at.part] + at.at] = c;
-                    }
+    // Ranges of parts with about as many slots each, on threads of their own when
+    // there are many (8500 buses, 119,000 slots: 1.25 ms on one, 0.45 on four).
+    // Parts do not depend on each other: a range has its own lists and remote
+    // entries, appended in order below, and an export that several ranges mark
+    // gets the same value from each.
+    struct Range {
+        int p0 = 0, p1 = 0;
+        bool ok = true;
+        std::vector<int> rem;
+        std::vector<unsigned short> list;
+    };
+    auto fill = [&](Range &r) {
+        const int slots = t.k0[r.p1] - t.k0[r.p0];
+        r.list.resize(4 * (size_t)slots + 8);
+        r.rem.reserve(slots / 4);
+        size_t used = 0;                             // entries of the lists so far
+        std::vector<int> where(L, -1);               // by first copy: number of the part's list, or below the part's first
+        for (int q = r.p0; q < r.p1; ++q) {
+            const int nk = t.k0[q + 1] - t.k0[q], l0 = (int)(used / 8), r0 = (int)r.rem.size();
+            for (int j = t.k0[q]; j < t.k0[q + 1]; ++j) {
+                const int sp = segp[t.slot[j]], c0 = sp >> 8, cnt = sp & 255;
+                if (cnt == 1) {
+                    t.seg[j] = 1;
+                    continue;
                 }
-                while (e < last) *e++ = 0xffff;  // past the last copy: the zero, below
-                used = end;
+                if (where[c0] < l0) {
+                    where[c0] = (int)(used / 8);
+                    const size_t end = used + ((cnt + 7) & ~7);
+                    if (end > r.list.size()) r.list.resize(2 * end);
+                    unsigned short *e = r.list.data() + used, *last = r.list.data() + end;
+                    for (int c = c0; c < c0 + cnt; ++c) {
+                        const Place at = place[c];
+                        if (at.part == q) {
+                            *e++ = (unsigned short)at.at;
+                        } else {
+                            *e++ = (unsigned short)(nk + (int)r.rem.size() - r0);
+                            r.rem.push_back(c);
+                            __atomic_store_n(&t.out[t.k0[at.part] + at.at], c, __ATOMIC_RELAXED);
+                        }
+                    }
+                    while (e < last) *e++ = 0xffff;  // past the last copy: the zero, below
+                    used = end;
+                }
+                t.seg[j] = ((where[c0] - l0) << 8) | cnt;
             }
-            t.seg[j] = ((where[c0] - l0) << 8) | cnt;
+            t.r0[q + 1] = (int)r.rem.size() - r0;    // counts here, places below
+            t.l0[q + 1] = (int)(used / 8) - l0;
+            const int zero = nk + t.r0[q + 1];
+            if (zero >= 0xffff) r.ok = false;
+            unsigned short *e = r.list.data() + 8 * (size_t)l0, *last = r.list.data() + used;
+            for (; e < last; ++e) *e = *e == 0xffff ? (unsigned short)zero : *e;
         }
-        t.r0[q + 1] = (int)t.rem.size();
-        t.l0[q + 1] = (int)(used / 8);
-        const int zero = nk + t.r0[q + 1] - r0;
-        if (zero >= 0xffff) t.ok = false;
-        unsigned short *e = t.list.data() + 8 * (size_t)l0, *last = t.list.data() + used;
-        for (; e < last; ++e) *e = *e == 0xffff ? (unsigned short)zero : *e;
+        r.list.resize(used);
+    };
+    const int n_ranges = std::max(1, std::min(4, L / 15000));
+    std::vector<Range> ranges(n_ranges);
+    for (int i = 0, p = 0; i < n_ranges; ++i) {
+        ranges[i].p0 = p;
+        while (p < P && (i + 1 == n_ranges || (long long)t.k0[p] * n_ranges < (long long)L * (i + 1))) ++p;
+        ranges[i].p1 = p;
     }
-    t.list.resize(used);
+    std::vector<std::thread> threads;
+    int started = 1;                                 // the first range is this thread's
+    try {
+        for (; started < n_ranges; ++started) threads.emplace_back(fill, std::ref(ranges[started]));
+    } catch (const std::system_error &) {            // no thread to be had: the rest here
+    }
+    fill(ranges[0]);
+    for (int i = started; i < n_ranges; ++i) fill(ranges[i]);
+    for (std::thread &th : threads) th.join();
+    size_t rems = 0, lists = 0;
+    for (const Range &r : ranges) {
+        rems += r.rem.size();
+        lists += r.list.size();
+        t.ok = t.ok && r.ok;
+    }
+    t.rem.reserve(rems);
+    t.list.reserve(lists);
+    for (const Range &r : ranges) {
+        t.rem.insert(t.rem.end(), r.rem.begin(), r.rem.end());
+        t.list.insert(t.list.end(), r.list.begin(), r.list.end());
+    }
+    for (int q = 0; q < P; ++q) {
+        t.r0[q + 1] += t.r0[q];
+        t.l0[q + 1] += t.l0[q];
+    }
 }
 
 inline PersistParts persist_parts(int P, int S, const std::vector<int> &order, const std::vector<double> &cost,

@@ -1,7 +1,8 @@
 """The two steps of the persistent engine's partition (`csrc/persist_plan.h`),
 compiled with g++: the split's slot ranges are those of the whole partition, and
 the remote entries counted without the lists are the lists', on random consensus
-structures and part counts in any order of the subsystems.
+structures and part counts in any order of the subsystems; lists built on
+several threads (many slots) are those of a plain pass over the parts.
 
 On the GPU: a request that does not fit in double precision falls back to the
 automatic CTA count, with its iterates."""
@@ -20,17 +21,68 @@ DRIVER = r"""
 #include <cstdio>
 #include <random>
 using namespace opf;
+static bool plain_lists(int P, const PersistParts &t, const std::vector<int> &soff, const std::vector<int> &segp,
+                        const std::vector<int> &pk) {
+    const int L = (int)pk.size();
+    std::vector<int> part(L), at(L), rem, out(L, -1), seg(L), r0{0}, l0{0};
+    std::vector<unsigned short> list;
+    for (int q = 0, j = 0; q < P; ++q)
+        for (int i = t.s0[q]; i < t.s0[q + 1]; ++i)
+            for (int k = soff[t.sub[i]]; k < soff[t.sub[i] + 1]; ++k, ++j) {
+                if (t.slot[j] != k) return false;
+                part[pk[k]] = q;
+                at[pk[k]] = j - t.k0[q];
+            }
+    for (int q = 0; q < P; ++q) {
+        const int nk = t.k0[q + 1] - t.k0[q];
+        std::vector<std::vector<int>> lists;
+        std::vector<int> number(L, -1);
+        for (int j = t.k0[q]; j < t.k0[q + 1]; ++j) {
+            const int c0 = segp[t.slot[j]] >> 8, cnt = segp[t.slot[j]] & 255;
+            seg[j] = 1;
+            if (cnt == 1) continue;
+            if (number[c0] < 0) {
+                number[c0] = (int)lists.size();
+                std::vector<int> e;
+                for (int c = c0; c < c0 + cnt; ++c) {
+                    if (part[c] == q) { e.push_back(at[c]); continue; }
+                    e.push_back(nk + (int)rem.size() - r0[q]);
+                    rem.push_back(c);
+                    out[t.k0[part[c]] + at[c]] = c;
+                }
+                while (e.size() % 8) e.push_back(-1);
+                for (size_t i = 0; i < e.size(); i += 8) lists.emplace_back(e.begin() + i, e.begin() + i + 8);
+            }
+            seg[j] = (number[c0] << 8) | cnt;
+        }
+        r0.push_back((int)rem.size());
+        for (const auto &e : lists)
+            for (int v : e) list.push_back((unsigned short)(v < 0 ? nk + r0[q + 1] - r0[q] : v));
+        l0.push_back((int)(list.size() / 8));
+    }
+    return rem == t.rem && out == t.out && seg == t.seg && r0 == t.r0 && l0 == t.l0 && list == t.list;
+}
 int main() {
     std::mt19937 rng(5);
-    for (int seed = 0; seed < 400; ++seed) {
-        const int S = 1 + rng() % 60, G = 1 + rng() % 90, P = 1 + rng() % 20;
+    for (int seed = 0; seed < 404; ++seed) {
+        const bool many = seed >= 400;           // 36,000 and 66,000 slots: several threads
+        const int S = many ? 6000 + 5000 * (seed & 1) : 1 + rng() % 60, G = many ? 20000 : 1 + rng() % 90,
+                  P = many ? 1 + 60 * (seed - 400) : 1 + rng() % 20;
         std::vector<int> soff{0}, gk;
         for (int d = 0; d < S; ++d) {
-            std::vector<int> g(G);
-            std::iota(g.begin(), g.end(), 0);
-            std::shuffle(g.begin(), g.end(), rng);
             const int n = std::min<int>(G, 1 + rng() % 12);
-            gk.insert(gk.end(), g.begin(), g.begin() + n);
+            std::vector<int> g;
+            if (many) {                          // neighbours share most globals
+                for (int i = 0; i < n; ++i) g.push_back((d * 3 + 17 * i + (int)(rng() % 3 ? 0 : rng() % G)) % G);
+                std::sort(g.begin(), g.end());
+                g.erase(std::unique(g.begin(), g.end()), g.end());
+            } else {
+                g.resize(G);
+                std::iota(g.begin(), g.end(), 0);
+                std::shuffle(g.begin(), g.end(), rng);
+                g.resize(n);
+            }
+            gk.insert(gk.end(), g.begin(), g.end());
             soff.push_back((int)gk.size());
         }
         const int L = (int)gk.size();
@@ -49,7 +101,8 @@ int main() {
         const PersistParts split = persist_split(P, S, order, cost, soff);
         const PersistParts all = persist_parts(P, S, order, cost, soff, segp, pk);
         if (split.s0 != all.s0 || split.k0 != all.k0 || split.sub != all.sub || all.k0[P] != L ||
-            persist_remote(P, split, soff, segp) != (long long)all.rem.size()) {
+            persist_remote(P, split, soff, segp) != (long long)all.rem.size() ||
+            (P <= 200 && !plain_lists(P, all, soff, segp, pk))) {
             std::printf("FAIL seed %d\n", seed);
             return 1;
         }
